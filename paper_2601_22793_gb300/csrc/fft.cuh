@@ -80,15 +80,28 @@ __device__ __forceinline__ float2 mul_i(float2 a)
     return DIR < 0 ? make_float2(a.y, -a.x) : make_float2(-a.y, a.x);
 }
 
+// p = a + DIR i b, m = a - DIR i b: the swap of parts makes scalar additions
+// cheaper than the moves a packed form would need
+template <int DIR>
+__device__ __forceinline__ void addsub_i(float2 a, float2 b, float2& p, float2& m)
+{
+    if (DIR < 0) {
+        p = make_float2(a.x + b.y, a.y - b.x);
+        m = make_float2(a.x - b.y, a.y + b.x);
+    } else {
+        p = make_float2(a.x - b.y, a.y + b.x);
+        m = make_float2(a.x + b.y, a.y - b.x);
+    }
+}
+
 template <int DIR>
 __device__ __forceinline__ void dft4(float2& a0, float2& a1, float2& a2, float2& a3)
 {
     float2 t0 = cadd(a0, a2), t1 = csub(a0, a2);
-    float2 t2 = cadd(a1, a3), t3 = mul_i<DIR>(csub(a1, a3));
+    float2 t2 = cadd(a1, a3), t3 = csub(a1, a3);
     a0 = cadd(t0, t2);
     a2 = csub(t0, t2);
-    a1 = cadd(t1, t3);
-    a3 = csub(t1, t3);
+    addsub_i<DIR>(t1, t3, a1, a3);
 }
 
 template <int DIR>
@@ -102,8 +115,6 @@ __device__ __forceinline__ void dft8(float2* v)
     float2 o1 = v[3], o2 = v[5], o3 = v[7];
     // k = 1: (h, DIR h)
     o1 = make_float2(h * (o1.x - (float)DIR * o1.y), h * (o1.y + (float)DIR * o1.x));
-    // k = 2: DIR i
-    o2 = mul_i<DIR>(o2);
     // k = 3: (-h, DIR h)
     o3 = make_float2(-h * (o3.x + (float)DIR * o3.y), h * ((float)DIR * o3.x - o3.y));
     float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
@@ -112,8 +123,7 @@ __device__ __forceinline__ void dft8(float2* v)
     v[4] = csub(e0, q0);
     v[1] = cadd(e1, o1);
     v[5] = csub(e1, o1);
-    v[2] = cadd(e2, o2);
-    v[6] = csub(e2, o2);
+    addsub_i<DIR>(e2, o2, v[2], v[6]);   // k = 2: DIR i
     v[3] = cadd(e3, o3);
     v[7] = csub(e3, o3);
 }

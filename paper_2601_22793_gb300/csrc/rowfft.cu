@@ -437,6 +437,34 @@ __host__ __device__ constexpr int ct_lg(int v) { return v <= 1 ? 0 : 1 + ct_lg<N
 template <int NX, int RP>
 __device__ __forceinline__ int row_of(int e) { return RP == 1 ? 0 : (int)((unsigned)e / NX); }
 
+// The gather of one pixel with any mapped point: corners outside the grid
+// read 0 (Eq. 4); a shift that is not finite or beyond the grid reads only 0.
+__device__ __noinline__ float gather_guarded(const float* R, int y, int x, float uy, float ux, int ny,
+                                             int nx)
+{
+    const float lim = 2.f * (float)(nx > ny ? nx : ny);
+    ux = fminf(fmaxf(ux, -lim), lim);
+    uy = fminf(fmaxf(uy, -lim), lim);
+    const float fx = floorf(ux), fy = floorf(uy);
+    const float dx = ux - fx, dy = uy - fy;
+    const int cx = x + (int)fx, cy = y + (int)fy;
+    const bool x0 = (unsigned)cx < (unsigned)nx, x1 = (unsigned)(cx + 1) < (unsigned)nx;
+    float r00 = 0.f, r10 = 0.f, r01 = 0.f, r11 = 0.f;
+    if ((unsigned)cy < (unsigned)ny) {
+        const float* r = R + (size_t)cy * nx + cx;
+        if (x0) r00 = __ldg(r);
+        if (x1) r10 = __ldg(r + 1);
+    }
+    if ((unsigned)(cy + 1) < (unsigned)ny) {
+        const float* r = R + (size_t)(cy + 1) * nx + cx;
+        if (x0) r01 = __ldg(r);
+        if (x1) r11 = __ldg(r + 1);
+    }
+    const float top = r00 + dx * (r10 - r00);
+    const float bot = r01 + dx * (r11 - r01);
+    return (1.f - dy) * top + dy * bot;
+}
+
 // Shared memory: the thickness rows yb - 1 .. yb + 2 RP, staged for the
 // gradient, alias the FFT rows, which are written only after the last
 // thickness read (row_fwd_mono_smem).  256-thread monochromatic blocks run
@@ -489,70 +517,113 @@ k_row_fwd_mono(const EprConsts C, const RowArgs A)
         cp_async_wait_all();   // no copy may land after the block has left
         return;
     }
-    cp_async_wait_all();
-    __syncthreads();
     const float cs = POLY ? line_const(C.c, A.line0 + sl) : C.c[0];
     // residual D - P (one line) or the line's split residual
     const float* Rb = POLY ? A.Ps + (pb * C.ns + (size_t)(A.line0 + sl) * npix) : A.P + pb;
     const float* Rt = A.P + pb;   // D - P, for |D - P|^2
+    // |D - P|^2 of the block's rows, while the thickness rows arrive; for one
+    // line this also brings into L1 the rows that most corners lie in (and
+    // the two next to them are asked for), so the gather below finds them
     float ra = 0.f;
+    if (!POLY || sl == 0) {
+        float2 own[EPT];
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) {
+            const int e = tid + k * T;
+            const int m = row_of<NX, RP>(e), x = e - m * NX;
+            const float* q = Rt + (size_t)(yb + 2 * m) * NX + x;
+            own[k] = make_float2(__ldg(q), __ldg(q + NX));
+        }
+        if (GATHER && !POLY && tid < 2 * (NX / 32)) {
+            const int y = tid < NX / 32 ? yb - 1 : yb + 2 * RP;
+            if (y >= 0 && y < ny) prefetch_l1(Rb + (size_t)y * NX + 32 * (tid % (NX / 32)));
+        }
+        float2 r2 = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) r2 = fma2(own[k], own[k], r2);
+        ra = r2.x + r2.y;
+    }
+    if (GATHER && POLY) {   // a line's own rows and the two next to them
+        for (int i = tid; i < (2 * RP + 2) * (NX / 32); i += T) {
+            const int y = yb - 1 + i / (NX / 32);
+            if (y >= 0 && y < ny) prefetch_l1(Rb + (size_t)y * NX + 32 * (i % (NX / 32)));
+        }
+    }
+    cp_async_wait_all();
+    __syncthreads();
     float2 vk[EPT];   // the packed row pair values, stored once the thickness is dead
+    // The gather of a row pair's two pixels (y0, x) and (y0 + 1, x), packed:
+    // 126 -> 92 thread instructions per pixel of this kernel, 148 -> 133 us for
+    // eight 2048^2 projections (with the loads ahead of the gather above).
+    // Pixels whose four corners all lie on the grid load them unconditionally
+    // on the spot; the others (the rim of the field) are flagged and redone
+    // with guarded loads after the loop, so the loop has no branch between
+    // one element's loads and the next's.
+    unsigned int rim = 0u;   // bits 2 k + r0
+    auto shift2 = [&](int k, int& x, int& y0, float2& ux, float2& uy) {
+        const int e = tid + k * T;
+        const int m = row_of<NX, RP>(e);
+        x = e - m * NX;
+        y0 = yb + 2 * m;
+        const float* tr = kStageT ? Ts + (2 * m + 1) * NX + x : A.T + pb + (size_t)y0 * NX + x;
+        auto ld = [&](int o) { return kStageT ? tr[o] : __ldg(tr + o); };
+        // edges (one-sided differences): with one row pair per block only the
+        // first and last element of a thread can be an edge column, and only
+        // the first (last) row of the pair the top (bottom) row
+        const bool xlo = (RP > 1 || k == 0) && x == 0;
+        const bool xhi = (RP > 1 || k == EPT - 1) && x == NX - 1;
+        const bool ylo = y0 == 0, yhi = y0 + 1 == ny - 1;
+        const float2 t = make_float2(ld(0), ld(NX));
+        const float2 l = xlo ? t : make_float2(ld(-1), ld(NX - 1));
+        const float2 r = xhi ? t : make_float2(ld(1), ld(NX + 1));
+        const float2 up = make_float2(ylo ? t.x : ld(-NX), t.x);
+        const float2 dn = make_float2(t.y, yhi ? t.y : ld(2 * NX));
+        // half the shift constant multiplies the doubled central difference
+        // (0.5 scales exactly), the whole one a one-sided difference
+        const float csx = XT ? xt_get(C, EPR_XT_C, A.line0 + sl, x) : cs;
+        const float ch = 0.5f * csx;
+        ux = mul2(both(xlo || xhi ? csx : ch), sub2(r, l));
+        uy = mul2(make_float2(ylo ? csx : ch, yhi ? csx : ch), sub2(dn, up));
+    };
 #pragma unroll
     for (int k = 0; k < EPT; ++k) {
-        const int e = tid + k * T;
-        const int m = row_of<NX, RP>(e), x = e - m * NX;
-        const int y0 = yb + 2 * m;
-        float v[2];
-#pragma unroll
-        for (int r0 = 0; r0 < 2; ++r0) {
-            const int y = y0 + r0;
-            if constexpr (!GATHER) {   // identity back-transport of the local closure
-                v[r0] = __ldg(Rb + (size_t)y * NX + x);
-            } else {
-            const float* tr = kStageT ? Ts + (2 * m + r0 + 1) * NX : A.T + pb + (size_t)y * NX;
-            const float t = kStageT ? tr[x] : __ldg(tr + x);
-            // edges (one-sided differences): with one row pair per block only
-            // the first and last element of a thread can be an edge column,
-            // and only the first (last) row of the pair the top (bottom) row
-            const bool xlo = (RP > 1 || k == 0) && x == 0;
-            const bool xhi = (RP > 1 || k == EPT - 1) && x == NX - 1;
-            const bool ylo = r0 == 0 && y == 0, yhi = r0 == 1 && y == ny - 1;
-            float gx, gy;
-            if (xlo) gx = tr[1] - t;
-            else if (xhi) gx = t - tr[x - 1];
-            else gx = 0.5f * (tr[x + 1] - tr[x - 1]);
-            if (ylo) gy = tr[NX + x] - t;
-            else if (yhi) gy = t - tr[x - NX];
-            else gy = 0.5f * (tr[NX + x] - tr[x - NX]);   // rows y - 1 and y + 1 exist here
-            const float lim = 2.f * (float)(NX > ny ? NX : ny);
-            const float csx = XT ? xt_get(C, EPR_XT_C, A.line0 + sl, x) : cs;
-            const float ux = fminf(fmaxf(csx * gx, -lim), lim);
-            const float uy = fminf(fmaxf(csx * gy, -lim), lim);
-            const float fx = floorf(ux), fy = floorf(uy);
-            const float dx = ux - fx, dy = uy - fy;
-            const int cx = x + (int)fx, cy = y + (int)fy;
-            const bool x0 = (unsigned)cx < (unsigned)NX, x1 = (unsigned)(cx + 1) < (unsigned)NX;
-            float r00 = 0.f, r10 = 0.f, r01 = 0.f, r11 = 0.f;
-            if ((unsigned)cy < (unsigned)ny) {
-                const float* rr = Rb + (size_t)cy * NX + cx;
-                if (x0) r00 = __ldg(rr);
-                if (x1) r10 = __ldg(rr + 1);
-            }
-            if ((unsigned)(cy + 1) < (unsigned)ny) {
-                const float* rr = Rb + (size_t)(cy + 1) * NX + cx;
-                if (x0) r01 = __ldg(rr);
-                if (x1) r11 = __ldg(rr + 1);
-            }
-            const float top = r00 + dx * (r10 - r00);
-            const float bot = r01 + dx * (r11 - r01);
-            v[r0] = (1.f - dy) * top + dy * bot;
-            }
-            if (!POLY || sl == 0) {
-                const float own = __ldg(Rt + (size_t)y * NX + x);
-                ra += own * own;
-            }
+        if constexpr (!GATHER) {   // identity back-transport of the local closure
+            const int e = tid + k * T;
+            const int m = row_of<NX, RP>(e), x = e - m * NX;
+            const size_t q = (size_t)(yb + 2 * m) * NX + x;
+            vk[k] = make_float2(__ldg(Rb + q), __ldg(Rb + q + NX));
+        } else {
+            int x, y0;
+            float2 ux, uy;
+            shift2(k, x, y0, ux, uy);
+            int ix0, ix1, iy0, iy1;
+            const float2 dx = floor_frac2(ux, ix0, ix1), dy = floor_frac2(uy, iy0, iy1);
+            const int cx0 = x + ix0, cx1 = x + ix1, cy0 = y0 + iy0, cy1 = y0 + 1 + iy1;
+            const bool in0 = (unsigned)cx0 < (unsigned)(NX - 1) && (unsigned)cy0 < (unsigned)(ny - 1);
+            const bool in1 = (unsigned)cx1 < (unsigned)(NX - 1) && (unsigned)cy1 < (unsigned)(ny - 1);
+            if (!in0) rim |= 1u << (2 * k);
+            if (!in1) rim |= 2u << (2 * k);
+            const float* p0 = Rb + (in0 ? cy0 * NX + cx0 : 0);
+            const float* p1 = Rb + (in1 ? cy1 * NX + cx1 : 0);
+            const float2 r00 = make_float2(__ldg(p0), __ldg(p1));
+            const float2 r10 = make_float2(__ldg(p0 + 1), __ldg(p1 + 1));
+            const float2 r01 = make_float2(__ldg(p0 + NX), __ldg(p1 + NX));
+            const float2 r11 = make_float2(__ldg(p0 + NX + 1), __ldg(p1 + NX + 1));
+            const float2 top = fma2(dx, sub2(r10, r00), r00);
+            const float2 bot = fma2(dx, sub2(r11, r01), r01);
+            vk[k] = fma2(dy, bot, mul2(sub2(both(1.f), dy), top));
         }
-        vk[k] = make_float2(v[0], v[1]);
+    }
+    if (GATHER && rim) {
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) {
+            if (!((rim >> (2 * k)) & 3u)) continue;
+            int x, y0;
+            float2 ux, uy;
+            shift2(k, x, y0, ux, uy);
+            if ((rim >> (2 * k)) & 1u) vk[k].x = gather_guarded(Rb, y0, x, uy.x, ux.x, ny, NX);
+            if ((rim >> (2 * k)) & 2u) vk[k].y = gather_guarded(Rb, y0 + 1, x, uy.y, ux.y, ny, NX);
+        }
     }
     if constexpr (GATHER && kStageT) __syncthreads();   // every thickness read is done
     if constexpr (RP == 1 && eprfft::ct_radix(NX, 0, MAXR) == EPT) {
