@@ -7,16 +7,20 @@
 //  * A block owns one TH x TW destination tile of one projection and holds
 //    its accumulators (one per line) in shared memory.
 //  * It scans every source pixel whose shifted corners can land in the tile:
-//    the tile grown by R = reach + 1 pixels on each side.  The thickness of
-//    that region plus a one-pixel ring (for the gradient) is staged in shared
-//    memory with coalesced loads.  Blocks whose staged region lies inside the
-//    grid take a path without edge tests.
+//    the tile grown by the reach on each side (a shift of exactly +reach
+//    gives its far corner weight 0, so no further pixel contributes).  The
+//    thickness of that region plus a one-pixel ring (for the gradient) is
+//    staged in shared memory with asynchronous copies; beyond the grid the
+//    edge value is replicated, which makes the central difference half the
+//    one-sided one.  Blocks whose staged region lies inside the grid take a
+//    path without edge tests.
 //  * Per source and line it forms the shift u = c_s G[T] (central
 //    differences, one-sided at the grid edges), splits u into floor and
-//    fraction (the integer pixel index never passes through float), and adds
-//    f_s exp(-mu_s T) times the four bilinear weights to the corners inside
-//    the tile with shared-memory atomics.  exp is evaluated only when the
-//    source reaches the tile.
+//    fraction, and adds f_s exp(-mu_s T) times the four bilinear weights to
+//    the corners inside the tile with shared-memory atomics.  exp is
+//    evaluated only when the source reaches the tile.  A thread takes four
+//    vertically adjacent sources as two packed pairs; a quad that holds a
+//    long shift is done source by source instead.
 //  * The shared accumulators are integers, because integer shared-memory
 //    atomics are single instructions while float ones are not.  The float
 //    mode adds round(v * 2^S) in uint32 with S chosen from the reach so that
@@ -39,9 +43,14 @@
 //    kernel adds those contributions with global atomics.  No mass is lost,
 //    whatever the shift.  The list fill counter alternates between two slots
 //    by iteration parity, so the overflow kernel can clear the next slot.
-//  * Fixed-point mode accumulates round(v * 2^40) in uint64 (contributions
-//    are non-negative) in shared and global memory: integer addition is
-//    associative, so the result is bit-identical across runs.
+//  * Fixed-point mode accumulates round(v * 2^40) (contributions are
+//    non-negative), as uint64 in global memory: integer addition is
+//    associative, so the result is bit-identical across runs.  In shared
+//    memory the sums are kept as two uint32 planes, q = hi 2^L + lo, because
+//    64-bit shared-memory atomics are compare-and-swap loops: with at most
+//    W = (2 reach + 3)^2 sources per pixel of at most 2^41 each, W 2^L and
+//    W 2^(41 - L) both fit in 32 bits for L = 32 - ceil(log2 W) and
+//    W <= 2^11 (reach <= 21); a longer reach keeps the uint64 sums.
 #include <type_traits>
 
 #include "epr_internal.cuh"
@@ -71,55 +80,98 @@ struct SplatArgs {
     int parity;
     int check_done;
     float fxs, fxs_inv;      // float mode: scale 2^S of the uint32 accumulators
+    int fx_lo;               // fixed-point mode: bits L of the low plane, 0 = uint64 sums
+    float fx_lo_s, fx_lo_inv;   // 2^L, 2^-L
+    float ch_max, tneg_max;  // largest |c_s| / 2 and largest tneg of the lines
 };
-
-// numpy.gradient semantics along one axis from three neighbours.
-__device__ __forceinline__ float grad1(float lo, float mid, float hi, int i, int n)
-{
-    if (i == 0) return hi - mid;
-    if (i == n - 1) return mid - lo;
-    return 0.5f * (hi - lo);
-}
 
 // i / d for 0 <= i < 2^20 and d < 2^12 without an integer division
 __device__ __forceinline__ int fdiv(int i, float inv_d) { return (int)(((float)i + 0.5f) * inv_d); }
 
-// v is already scaled by the accumulator's 2^S
-template <bool DET>
-__device__ __forceinline__ void acc_add(void* acc, int idx, float v)
+__device__ __forceinline__ float exp2_approx(float x)
 {
-    if constexpr (DET) {
-        unsigned long long q = (unsigned long long)__float2ll_rn(v);
-        atomicAdd(reinterpret_cast<unsigned long long*>(acc) + idx, q);
-    } else {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// largest magnitude of three, and the smaller of two; NaN if one is NaN
+__device__ __forceinline__ float max_abs3(float a, float b, float c)
+{
+    float r;
+    asm("max.ftz.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float min_nan(float a, float b)
+{
+    float r;
+    asm("min.ftz.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+// Accumulator modes: float (uint32 of value * 2^S), fixed point as two uint32
+// planes, fixed point as uint64.
+enum { ACC_F32 = 0, ACC_FX2 = 1, ACC_FX64 = 2 };
+
+// v is already scaled by the accumulator's 2^S (2^40 in fixed point); the
+// second plane of ACC_FX2 follows the first at `plane` words.
+template <int MODE>
+__device__ __forceinline__ void acc_add(void* acc, int idx, int plane, float v, const SplatArgs& A)
+{
+    if constexpr (MODE == ACC_F32) {
         atomicAdd(reinterpret_cast<unsigned int*>(acc) + idx, __float2uint_rn(v));
+    } else if constexpr (MODE == ACC_FX2) {
+        // hi = floor(v / 2^L); v - hi 2^L is exact (v has 24 bits), and its
+        // rounding is that of v to an integer
+        const unsigned int hi = __float2uint_rz(v * A.fx_lo_inv);
+        const unsigned int lo = __float2uint_rn(fmaf(-(float)hi, A.fx_lo_s, v));
+        unsigned int* a = reinterpret_cast<unsigned int*>(acc) + idx;
+        atomicAdd(a, lo);
+        atomicAdd(a + plane, hi);
+    } else {
+        atomicAdd(reinterpret_cast<unsigned long long*>(acc) + idx,
+                  (unsigned long long)__float2ll_rn(v));
     }
 }
 
-// NS = 1: single line known at compile time; NS = 0: C.ns lines.
-// Shared layout: accumulators [ns][TH + 2][TW + 2]; the staged thickness window
-// [SH][SWa] whose first column ax0 = tx0 - HX is 16-byte aligned (HX = R + 1
-// rounded up to 4) so rows load as float4; a list of far sources.
+template <int MODE>
+__device__ __forceinline__ unsigned long long acc_fx(const void* acc, int idx, int plane, int L)
+{
+    if constexpr (MODE == ACC_FX2) {
+        const unsigned int* a = reinterpret_cast<const unsigned int*>(acc) + idx;
+        return (unsigned long long)a[0] + ((unsigned long long)a[plane] << L);
+    } else {
+        return reinterpret_cast<const unsigned long long*>(acc)[idx];
+    }
+}
+
 constexpr int kFarList = 256;
 constexpr int kQuad = 4;   // sources per scan work item
+constexpr int kAccX = 4;   // accumulator column of tile column 0 (16-byte aligned rows)
 
+// NS = 1: single line known at compile time; NS = 0: C.ns lines.
+// Shared layout: accumulators [ns][TH + 2][TW + 8], the tile with a one-pixel
+// apron (its rows start at a 16-byte boundary, so the flush reads four pixels
+// at once); the staged thickness window [SH][SWa] whose first column
+// ax0 = tx0 - HX is 16-byte aligned (HX = reach + 1 rounded up to 4); a list
+// of far sources.
+//
 // The tile shape is a compile-time parameter (64 x 64, 32 x 64, 64 x 32 or
-// 32 x 32, chosen on the host), and so is the reach RC of the float solves
-// for the reaches the tuner tries (3, 4, 6; RC = 0 takes C.smax), so every
-// tile- and reach-derived index, stride and offset folds into immediates.
-// Five blocks per SM (48 registers; a 64 x 64 tile at reach 4 takes 44 KB of
-// shared memory); the mono residual kernel with a runtime reach needs more
-// registers and runs four.
+// 32 x 32, chosen on the host), and so is the reach RC for the reaches the
+// tuner tries (RC = 0 takes C.smax), so every tile- and reach-derived index,
+// stride and offset folds into immediates.  Five blocks per SM (48 registers;
+// a 64 x 64 tile at reach 4 takes 43 KB of shared memory).
 // XT: an x-dependent spectrum, the line constants read per source column
 // from the plan's table (runtime line count and reach only).
 // OCC > 0: that many blocks per SM (six for the one-line residual kernels of
-// the tiles smaller than 64 x 64 at reach 3 and 4: 40 registers, no spills).
-template <int NS, bool DET, bool RESID, int TH, int TW, int RC = 0, bool XT = false, int OCC = 0>
+// the tiles smaller than 64 x 64 at reach 3 and 4: 40 registers).
+template <int NS, int MODE, bool RESID, int TH, int TW, int RC = 0, bool XT = false, int OCC = 0>
 __global__ void __launch_bounds__(splat_threads(NS),
                                   OCC > 0 ? OCC : NS != 1 ? 2 : ((RESID && RC == 0) ? 4 : 5))
 k_splat(const EprConsts C, const SplatArgs A)
 {
     constexpr int kSplatThreads = splat_threads(NS);
+    constexpr bool DET = MODE != ACC_F32;
     static_assert((TW & (TW - 1)) == 0 && TH * TW <= 4 * 4 * kSplatThreads, "tile shape");
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_far_idx[kFarList];
@@ -129,17 +181,15 @@ k_splat(const EprConsts C, const SplatArgs A)
     const int nx = C.nx, ny = C.ny;
     const int ns = NS ? NS : C.ns;
     const int ty0 = blockIdx.y * TH, tx0 = blockIdx.x * TW;
-    const int smax = RC > 0 ? RC : C.smax;
-    const int R = smax + 1;
+    const int R = RC > 0 ? RC : C.smax;
     const int RH = TH + 2 * R, RW = TW + 2 * R;     // source region
     const int RHq = (RH + kQuad - 1) / kQuad;         // its rows in quads
     const int HX = (R + 1 + 3) & ~3;
     const int SH = RHq * kQuad + 2, SWa = TW + 2 * HX;   // staged thickness
     const int coff = HX - R - 1;                     // staged column of source column tx0 - R - 1
     constexpr int tile = TH * TW;
-    // accumulators [ns][TH + 2][TW + 2]: the tile with a one-pixel apron, so
-    // the four corners of any source that touches the tile have a slot
-    constexpr int AP = TW + 2, ACC = (TH + 2) * AP;
+    constexpr int AP = TW + 2 * kAccX, ACC = (TH + 2) * AP;
+    const int plane = ns * ACC;                       // words of one plane (ACC_FX2)
     const size_t npix = (size_t)nx * ny;
     const int tid = threadIdx.x;
 
@@ -149,31 +199,22 @@ k_splat(const EprConsts C, const SplatArgs A)
     const float* Tb = A.T + (size_t)b * npix;
     if (tid == 0) s_far_n = 0;
 
-    // the detector data of the tile, fetched before the scan (residual output)
+    // the detector data of the tile (residual output): its lines are asked for
+    // here and loaded after the scan, whose registers they would take
     constexpr int kDq = 4;   // float4 per thread: tiles up to 64 x 64
-    float4 dreg[kDq];
     constexpr int nq = tile >> 2;
     constexpr int tw4 = TW >> 2;
     if constexpr (RESID) {
-#pragma unroll
-        for (int k = 0; k < kDq; ++k) {
-            const int i4 = tid + k * kSplatThreads;
-            dreg[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (i4 < nq) {
-                const int ly = i4 / tw4, lx = (i4 - ly * tw4) << 2;
-                const int gy = ty0 + ly, gx = tx0 + lx;
-                if (gy < ny && gx < nx)
-                    dreg[k] = __ldg(reinterpret_cast<const float4*>(A.D + (size_t)b * npix + (size_t)gy * nx + gx));
-            }
+        constexpr int kLine = TW / 32;   // 128-byte lines of a row
+        if (tid < TH * kLine) {
+            const int gy = ty0 + tid / kLine, gx = tx0 + 32 * (tid % kLine);
+            if (gy < ny && gx < nx) prefetch_l2(A.D + (size_t)b * npix + (size_t)gy * nx + gx);
         }
     }
 
-    if constexpr (DET) {
-        unsigned long long* a = reinterpret_cast<unsigned long long*>(acc);
-        for (int i = tid; i < ns * ACC; i += kSplatThreads) a[i] = 0ull;
-    } else {   // ACC = 4 (TH/2 + 1)(TW/2 + 1)
+    {   // ACC = 2 (TH + 2)(TW / 2 + 4), a multiple of 4
         uint4* a = reinterpret_cast<uint4*>(acc);
-        for (int i = tid; i < ns * ACC / 4; i += kSplatThreads) a[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = tid; i < ns * ACC / (DET ? 2 : 4); i += kSplatThreads) a[i] = make_uint4(0u, 0u, 0u, 0u);
     }
     // T, the done flags and the overflow counters come from earlier kernels
     epr_grid_wait();
@@ -186,47 +227,53 @@ k_splat(const EprConsts C, const SplatArgs A)
         const float inv_q = 1.f / (float)q;
         for (int i = tid; i < SH * q; i += kSplatThreads) {
             const int ly = fdiv(i, inv_q), c4 = i - ly * q;
-            const int gy = sy0 + ly, gx = ax0 + 4 * c4;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (gy >= 0 && gy < ny && gx >= 0 && gx < nx)   // nx % 4 == 0: all four or none
-                v = __ldg(reinterpret_cast<const float4*>(Tb + (size_t)gy * nx + gx));
-            reinterpret_cast<float4*>(Ts)[i] = v;
+            const int gy = min(max(sy0 + ly, 0), ny - 1), gx = ax0 + 4 * c4;
+            const float* src = Tb + (size_t)gy * nx;
+            if (gx >= 0 && gx < nx) {   // nx % 4 == 0: all four or none
+                cp_async16(reinterpret_cast<float4*>(Ts) + i, src + gx);
+            } else {                     // the edge value (only the nearest column is read)
+                const float v = __ldg(src + (gx < 0 ? 0 : nx - 1));
+                reinterpret_cast<float4*>(Ts)[i] = make_float4(v, v, v, v);
+            }
         }
+        cp_async_commit();
+        cp_async_wait_all();
     }
     __syncthreads();
 
-    const float fsmax = (float)smax;
+    const float fsmax = (float)R;
     // the accumulator scale 2^S is folded into the line weight: a power of two
     // scales exactly, so each contribution rounds to the same integer
     const float fxs = DET ? EPR_FX_SCALE : A.fxs;
-    // One source at tile-local (ly, lx) with thickness t and twice its
+    constexpr float kLog2e = 1.4426950408889634f;
+    // One source at region-local (ly, lx) with thickness t and twice its
     // gradient: every line's shift, contributions and far flag.  Gradients
     // are kept doubled (hi - lo), and half the shift constant multiplies
     // them: 0.5 scales exactly, so u is the same float.
     auto source = [&](int ly, int lx, float t, float gx2, float gy2) {
         unsigned int far = 0u;
         const int sxc = XT ? tx0 - R + lx : 0;   // source column (inside the grid)
-#pragma unroll(NS ? NS : 1)
+#pragma unroll 1
         for (int s = 0; s < ns; ++s) {
-            const float ch = 0.5f * (XT ? xt_get(C, EPR_XT_C, s, sxc) : C.c[s]);
+            const float ch = 0.5f * (XT ? xt_get(C, EPR_XT_C, s, sxc) : line_const(C.c, s));
             const float ux = ch * gx2, uy = ch * gy2;
-            const float tneg = XT ? xt_get(C, EPR_XT_TNEG, s, sxc) : C.tneg[s];
+            const float tneg = XT ? xt_get(C, EPR_XT_TNEG, s, sxc) : line_const(C.tneg, s);
             if (fabsf(ux) <= fsmax && fabsf(uy) <= fsmax && t >= tneg) {
-                const float fx = floorf(ux), fy = floorf(uy);
-                const int cx = lx - R + (int)fx, cy = ly - R + (int)fy;  // corner 00, tile-local
+                int ix, iy;
+                const float2 d = floor_frac2(make_float2(ux, uy), ix, iy);
+                const int cx = lx - R + ix, cy = ly - R + iy;   // corner 00, tile-local
                 // all four corners have a slot (apron) when one is in the tile
                 if ((unsigned)(cx + 1) <= (unsigned)TW && (unsigned)(cy + 1) <= (unsigned)TH) {
-                    const float dx = ux - fx, dy = uy - fy;
-                    const float fs = XT ? xt_get(C, EPR_XT_F, s, sxc) : C.f[s];
-                    const float mus = XT ? xt_get(C, EPR_XT_MU, s, sxc) : C.mu[s];
-                    const float m = (fs * fxs) * __expf(-mus * t);   // 2^S f e^(-mu t)
-                    const float mx1 = m * dx, mx0 = m - mx1;          // m (1 - dx), m dx
-                    const float w = 1.f - dy;
-                    const int idx = s * ACC + (cy + 1) * AP + (cx + 1);
-                    acc_add<DET>(acc, idx, mx0 * w);
-                    acc_add<DET>(acc, idx + 1, mx1 * w);
-                    acc_add<DET>(acc, idx + AP, mx0 * dy);
-                    acc_add<DET>(acc, idx + AP + 1, mx1 * dy);
+                    const float fs = XT ? xt_get(C, EPR_XT_F, s, sxc) : line_const(C.f, s);
+                    const float mus = XT ? xt_get(C, EPR_XT_MU, s, sxc) : line_const(C.mu, s);
+                    const float m = (fs * fxs) * exp2_approx((-mus * kLog2e) * t);   // 2^S f e^(-mu t)
+                    const float mx1 = m * d.x, mx0 = m - mx1;          // m dx, m (1 - dx)
+                    const float w = 1.f - d.y;
+                    const int idx = s * ACC + (cy + 1) * AP + (cx + kAccX);
+                    acc_add<MODE>(acc, idx, plane, mx0 * w, A);
+                    acc_add<MODE>(acc, idx + 1, plane, mx1 * w, A);
+                    acc_add<MODE>(acc, idx + AP, plane, mx0 * d.y, A);
+                    acc_add<MODE>(acc, idx + AP + 1, plane, mx1 * d.y, A);
                 }
             } else {
                 far |= 1u << s;
@@ -253,10 +300,18 @@ k_splat(const EprConsts C, const SplatArgs A)
     // The scan: a thread takes kQuad vertically adjacent sources of one
     // column (rows ly0 .. ly0 + kQuad - 1 of the region, padded to a multiple
     // of kQuad; padding rows cannot reach the tile and are not owned by it),
-    // reusing the column's thickness values.  Specialised for blocks whose
-    // staged region lies inside the grid (central differences everywhere, no
-    // edge tests) and for edge blocks.  Work item (qy, lx) is advanced by
-    // kSplatThreads = dly quad rows + dlx columns.
+    // reusing the column's thickness values.  Sources 0, 1 and 2, 3 of the
+    // quad are the two lanes of packed arithmetic: the column's six values
+    // form the pairs (c0, c1), (c2, c3), (c4, c5), whose differences are the
+    // row gradients of both pairs.  The scan was bound by instruction issue
+    // (75 % active in a batch): the packed forms, the floor by rounding mode
+    // (FRND and F2I run at an eighth of the FMA rate) and one long-shift test
+    // per quad took it from 123 to 91 thread instructions per pixel, and the
+    // kernel from 142 to 103 us for eight 2048^2 projections; what bounds it
+    // now is the shared-memory data pipe (80 % busy: the loads of the staged
+    // window and the accumulator atomics).
+    // Work item (qy, lx) is advanced by kSplatThreads = dly quad rows +
+    // dlx columns.
     const int nitem = RHq * RW;
     const int dly = kSplatThreads / RW, dlx = kSplatThreads - dly * RW;
     auto scan = [&](auto interior_tag) {
@@ -266,28 +321,101 @@ k_splat(const EprConsts C, const SplatArgs A)
                  qy += dly + (lx >= RW ? 1 : 0), lx -= (lx >= RW ? RW : 0)) {
             const int ly0 = qy * kQuad;
             const float* tp = Ts + (ly0 + 1) * SWa + (lx + 1 + coff);   // source (ly0, lx)
-            float col[kQuad + 2];   // the column, rows ly0 - 1 .. ly0 + kQuad
+            float2 c[kQuad / 2 + 1], g_x[kQuad / 2], g_y[kQuad / 2];   // column pairs, twice the gradients
 #pragma unroll
-            for (int j = 0; j < kQuad + 2; ++j) col[j] = tp[(j - 1) * SWa];
+            for (int j = 0; j < kQuad / 2 + 1; ++j)
+                c[j] = make_float2(tp[(2 * j - 1) * SWa], tp[2 * j * SWa]);
+            const int sx = tx0 - R + lx;
+            if (!IN && (sx < 0 || sx >= nx)) continue;
 #pragma unroll
-            for (int j = 0; j < kQuad; ++j) {
-                const float t = col[j + 1];
-                float gx2, gy2;   // twice the gradient
-                if constexpr (IN) {
-                    gx2 = tp[j * SWa + 1] - tp[j * SWa - 1];
-                    gy2 = col[j + 2] - col[j];
-                } else {
-                    const int sy = ty0 - R + ly0 + j, sx = tx0 - R + lx;
-                    if (sy < 0 || sy >= ny || sx < 0 || sx >= nx) continue;
-                    gx2 = 2.f * grad1(tp[j * SWa - 1], t, tp[j * SWa + 1], sx, nx);
-                    gy2 = 2.f * grad1(col[j], t, col[j + 2], sy, ny);
+            for (int j = 0; j < kQuad / 2; ++j) {
+                g_x[j] = sub2(make_float2(tp[2 * j * SWa + 1], tp[(2 * j + 1) * SWa + 1]),
+                              make_float2(tp[2 * j * SWa - 1], tp[(2 * j + 1) * SWa - 1]));
+                g_y[j] = sub2(c[j + 1], c[j]);
+                if constexpr (!IN) {   // one-sided differences are not halved
+                    if (sx == 0 || sx == nx - 1) g_x[j] = add2(g_x[j], g_x[j]);
+                    const int sy = ty0 - R + ly0 + 2 * j;
+                    if (sy == 0 || sy == ny - 1) g_y[j].x += g_y[j].x;
+                    if (sy + 1 == 0 || sy + 1 == ny - 1) g_y[j].y += g_y[j].y;
                 }
-                source(ly0 + j, lx, t, gx2, gy2);
+            }
+            bool ok[kQuad];   // sources on the grid
+#pragma unroll
+            for (int j = 0; j < kQuad; ++j) ok[j] = IN || (unsigned)(ty0 - R + ly0 + j) < (unsigned)ny;
+            const float t[kQuad] = {c[0].y, c[1].x, c[1].y, c[2].x};
+            // no line's shift is long when that of the largest |c_s| is not;
+            // a NaN fails the test and goes to the source path
+            const float um = max_abs3(max_abs3(max_abs3(g_x[0].x, g_x[0].y, g_x[1].x), g_x[1].y, g_y[0].x),
+                                      g_y[0].y, max_abs3(g_y[1].x, g_y[1].y, 0.f));
+            const bool all_near = A.ch_max * um <= fsmax &&
+                                  min_nan(min_nan(t[0], t[1]), min_nan(t[2], t[3])) >= A.tneg_max;
+            if (XT || !all_near) {
+#pragma unroll 1
+                for (int j = 0; j < kQuad; ++j) {
+                    const bool hi = j >= 2, od = j & 1;
+                    const float2 gx = hi ? g_x[1] : g_x[0], gy = hi ? g_y[1] : g_y[0];
+                    const bool on = IN || (unsigned)(ty0 - R + ly0 + j) < (unsigned)ny;
+                    if (on) source(ly0 + j, lx, tp[j * SWa], od ? gx.y : gx.x, od ? gy.y : gy.x);
+                }
+                continue;
+            }
+#pragma unroll(NS ? NS : 1)
+            for (int s = 0; s < ns; ++s) {
+                const float2 ch = both(0.5f * C.c[s]);
+#pragma unroll
+                for (int j = 0; j < kQuad / 2; ++j) {
+                    int ix0, ix1, iy0, iy1;
+                    const float2 dx = floor_frac2(mul2(ch, g_x[j]), ix0, ix1);
+                    const float2 dy = floor_frac2(mul2(ch, g_y[j]), iy0, iy1);
+                    // corner 00, counted from the apron
+                    const int cx0 = lx - R + 1 + ix0, cx1 = lx - R + 1 + ix1;
+                    const int cy0 = ly0 + 2 * j - R + 1 + iy0, cy1 = ly0 + 2 * j - R + 2 + iy1;
+                    const bool in0 = ok[2 * j] && (unsigned)cx0 <= (unsigned)TW && (unsigned)cy0 <= (unsigned)TH;
+                    const bool in1 = ok[2 * j + 1] && (unsigned)cx1 <= (unsigned)TW && (unsigned)cy1 <= (unsigned)TH;
+                    if (in0 || in1) {
+                        const float mk = -C.mu[s] * kLog2e;
+                        // 2^S f e^(-mu t)
+                        const float2 m = mul2(both(C.f[s] * fxs),
+                                              make_float2(exp2_approx(mk * t[2 * j]), exp2_approx(mk * t[2 * j + 1])));
+                        const float2 mx1 = mul2(m, dx), mx0 = sub2(m, mx1);
+                        const float2 w = sub2(both(1.f), dy);
+                        const float2 v00 = mul2(mx0, w), v10 = mul2(mx1, w);
+                        const float2 v01 = mul2(mx0, dy), v11 = mul2(mx1, dy);
+                        if (in0) {
+                            const int idx = s * ACC + cy0 * AP + cx0 + kAccX - 1;
+                            acc_add<MODE>(acc, idx, plane, v00.x, A);
+                            acc_add<MODE>(acc, idx + 1, plane, v10.x, A);
+                            acc_add<MODE>(acc, idx + AP, plane, v01.x, A);
+                            acc_add<MODE>(acc, idx + AP + 1, plane, v11.x, A);
+                        }
+                        if (in1) {
+                            const int idx = s * ACC + cy1 * AP + cx1 + kAccX - 1;
+                            acc_add<MODE>(acc, idx, plane, v00.y, A);
+                            acc_add<MODE>(acc, idx + 1, plane, v10.y, A);
+                            acc_add<MODE>(acc, idx + AP, plane, v01.y, A);
+                            acc_add<MODE>(acc, idx + AP + 1, plane, v11.y, A);
+                        }
+                    }
+                }
             }
         }
     };
     if (interior) scan(std::true_type{});
     else scan(std::false_type{});
+    float4 dreg[kDq];
+    if constexpr (RESID) {   // under way while the block meets at the barrier
+#pragma unroll
+        for (int k = 0; k < kDq; ++k) {
+            const int i4 = tid + k * kSplatThreads;
+            dreg[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (i4 < nq) {
+                const int ly = i4 / tw4, lx = (i4 - ly * tw4) << 2;
+                const int gy = ty0 + ly, gx = tx0 + lx;
+                if (gy < ny && gx < nx)
+                    dreg[k] = __ldg(reinterpret_cast<const float4*>(A.D + (size_t)b * npix + (size_t)gy * nx + gx));
+            }
+        }
+    }
     __syncthreads();
     epr_grid_release();
 
@@ -306,14 +434,9 @@ k_splat(const EprConsts C, const SplatArgs A)
                 const int ly = sy - ty0 + R, lx = sx - tx0 + R;   // in the source region
                 const float* tp = Ts + (ly + 1) * SWa + (lx + 1 + coff);
                 const float t = tp[0];
-                float gx2, gy2;
-                if (interior) {
-                    gx2 = tp[1] - tp[-1];
-                    gy2 = tp[SWa] - tp[-SWa];
-                } else {
-                    gx2 = 2.f * grad1(tp[-1], t, tp[1], sx, nx);
-                    gy2 = 2.f * grad1(tp[-SWa], t, tp[SWa], sy, ny);
-                }
+                float gx2 = tp[1] - tp[-1], gy2 = tp[SWa] - tp[-SWa];
+                if (sx == 0 || sx == nx - 1) gx2 += gx2;
+                if (sy == 0 || sy == ny - 1) gy2 += gy2;
                 A.ovf_idx[(size_t)b * C.ovf_cap + gpos] = pix;
                 A.ovf_mask[(size_t)b * C.ovf_cap + gpos] = s_far_mask[e];
                 A.ovf_tg[(size_t)b * C.ovf_cap + gpos] = make_float4(t, gx2, gy2, 0.f);
@@ -323,9 +446,10 @@ k_splat(const EprConsts C, const SplatArgs A)
         }
     }
 
-    // flush: every pixel of the tile inside the grid, once, coalesced
-    if constexpr (RESID) {
-        const unsigned int* a = reinterpret_cast<const unsigned int*>(acc);
+    // flush: every pixel of the tile inside the grid, once, coalesced, four
+    // at a time
+    if constexpr (!DET) {
+        const uint4* a = reinterpret_cast<const uint4*>(acc);
         const float inv = A.fxs_inv;
 #pragma unroll
         for (int k = 0; k < kDq; ++k) {
@@ -334,11 +458,27 @@ k_splat(const EprConsts C, const SplatArgs A)
             const int ly = i4 / tw4, lx = (i4 - ly * tw4) << 2;
             const int gy = ty0 + ly, gx = tx0 + lx;
             if (gy >= ny || gx >= nx) continue;
-            const unsigned int* v = a + (ly + 1) * AP + lx + 1;
-            const float4 d = dreg[k];
-            *reinterpret_cast<float4*>(A.P + (size_t)b * npix + (size_t)gy * nx + gx) =
-                make_float4(d.x - (float)v[0] * inv, d.y - (float)v[1] * inv,
-                            d.z - (float)v[2] * inv, d.w - (float)v[3] * inv);
+            const size_t o = (size_t)b * npix + (size_t)gy * nx + gx;
+            const int i0 = ((ly + 1) * AP + lx + kAccX) >> 2;
+            if constexpr (RESID) {
+                const uint4 v = a[i0];
+                const float4 d = dreg[k];
+                *reinterpret_cast<float4*>(A.P + o) =
+                    make_float4(d.x - (float)v.x * inv, d.y - (float)v.y * inv,
+                                d.z - (float)v.z * inv, d.w - (float)v.w * inv);
+            } else {
+                // sum <= 2 (2 reach + 3)^2 sum_s f_s: no overflow either
+                uint4 sum = make_uint4(0u, 0u, 0u, 0u);
+                for (int s = 0; s < ns; ++s) {
+                    const uint4 v = a[s * (ACC / 4) + i0];
+                    sum = make_uint4(sum.x + v.x, sum.y + v.y, sum.z + v.z, sum.w + v.w);
+                    if (ns > 1)
+                        *reinterpret_cast<float4*>(A.Ps + (size_t)s * npix + o + (size_t)b * (ns - 1) * npix) =
+                            make_float4((float)v.x * inv, (float)v.y * inv, (float)v.z * inv, (float)v.w * inv);
+                }
+                *reinterpret_cast<float4*>(A.P + o) = make_float4((float)sum.x * inv, (float)sum.y * inv,
+                                                                  (float)sum.z * inv, (float)sum.w * inv);
+            }
         }
     } else {
         for (int i = tid; i < tile; i += kSplatThreads) {
@@ -346,27 +486,14 @@ k_splat(const EprConsts C, const SplatArgs A)
             const int gy = ty0 + ly, gx = tx0 + lx;
             if (gy >= ny || gx >= nx) continue;
             const size_t o = (size_t)b * npix + (size_t)gy * nx + gx;
-            if constexpr (DET) {
-                const unsigned long long* a = reinterpret_cast<const unsigned long long*>(acc);
-                unsigned long long sum = 0ull;
-                for (int s = 0; s < ns; ++s) {
-                    const unsigned long long q = a[s * ACC + (ly + 1) * AP + lx + 1];
-                    sum += q;
-                    if (ns > 1) A.Psq[(size_t)s * npix + o + (size_t)b * (ns - 1) * npix] = q;
-                }
-                A.Pq[o] = sum;
-            } else {
-                // sum <= 2 (2 reach + 3)^2 sum_s f_s: no overflow either
-                const unsigned int* a = reinterpret_cast<const unsigned int*>(acc);
-                unsigned int sum = 0u;
-                for (int s = 0; s < ns; ++s) {
-                    const unsigned int q = a[s * ACC + (ly + 1) * AP + lx + 1];
-                    sum += q;
-                    if (ns > 1)
-                        A.Ps[(size_t)s * npix + o + (size_t)b * (ns - 1) * npix] = (float)q * A.fxs_inv;
-                }
-                A.P[o] = (float)sum * A.fxs_inv;
+            unsigned long long sum = 0ull;
+            for (int s = 0; s < ns; ++s) {
+                const unsigned long long q =
+                    acc_fx<MODE>(acc, s * ACC + (ly + 1) * AP + lx + kAccX, plane, A.fx_lo);
+                sum += q;
+                if (ns > 1) A.Psq[(size_t)s * npix + o + (size_t)b * (ns - 1) * npix] = q;
             }
+            A.Pq[o] = sum;
         }
     }
 }
@@ -603,85 +730,107 @@ __global__ void __launch_bounds__(256) k_bin_os(const EprConsts C, const SplatAr
     }
 }
 
-template <int NS, bool DET, bool RESID, int TH, int TW, int RC = 0, bool XT = false, int OCC = 0>
+template <int NS, int MODE, bool RESID, int TH, int TW, int RC = 0, bool XT = false, int OCC = 0>
 cudaError_t launch_t(const EprConsts& C, const SplatArgs& A, dim3 grid, size_t smem, int batch,
                      cudaStream_t stream)
 {
     const bool pdl = C.pdl != 0;
-    const cudaError_t e = epr_launch_kernel(pdl, k_splat<NS, DET, RESID, TH, TW, RC, XT, OCC>, grid,
+    const cudaError_t e = epr_launch_kernel(pdl, k_splat<NS, MODE, RESID, TH, TW, RC, XT, OCC>, grid,
                                             dim3(splat_threads(NS)), smem, stream, C, A);
     if (e != cudaSuccess) return e;
-    return epr_launch_kernel(pdl, k_splat_overflow<DET, RESID, XT>, dim3(128, batch), dim3(128), 0,
-                             stream, C, A);
+    return epr_launch_kernel(pdl, k_splat_overflow<MODE != ACC_F32, RESID, XT>, dim3(128, batch),
+                             dim3(128), 0, stream, C, A);
 }
 
 // Tiles whose one-line residual kernel has a six-blocks-per-SM variant.
 template <int TH, int TW>
 constexpr bool has_occ6() { return TH * TW < 64 * 64; }
 
+template <int TH, int TW, int MODE>
+cudaError_t launch_fx(const EprConsts& C, const SplatArgs& A, dim3 grid, size_t smem, int batch,
+                      cudaStream_t stream)
+{
+    if (C.xt) return launch_t<0, MODE, false, TH, TW, 0, true>(C, A, grid, smem, batch, stream);
+    const bool r4 = MODE == ACC_FX2 && C.smax == 4;   // the default reach
+    if (C.ns == 1)
+        return r4 ? launch_t<1, MODE, false, TH, TW, MODE == ACC_FX2 ? 4 : 0>(C, A, grid, smem, batch, stream)
+                  : launch_t<1, MODE, false, TH, TW>(C, A, grid, smem, batch, stream);
+    return r4 ? launch_t<0, MODE, false, TH, TW, MODE == ACC_FX2 ? 4 : 0>(C, A, grid, smem, batch, stream)
+              : launch_t<0, MODE, false, TH, TW>(C, A, grid, smem, batch, stream);
+}
+
 template <int TH, int TW>
 cudaError_t launch_shape(const EprConsts& C, const SplatArgs& A, int resid, bool occ6, dim3 grid,
                          size_t smem, int batch, cudaStream_t stream)
 {
     const bool mono = C.ns == 1;
-    if (C.xt)   // x-dependent spectrum: the generic kernels with per-column constants
-        return C.det ? launch_t<0, true, false, TH, TW, 0, true>(C, A, grid, smem, batch, stream)
-                     : launch_t<0, false, false, TH, TW, 0, true>(C, A, grid, smem, batch, stream);
     if (C.det)
-        return mono ? launch_t<1, true, false, TH, TW>(C, A, grid, smem, batch, stream)
-                    : launch_t<0, true, false, TH, TW>(C, A, grid, smem, batch, stream);
+        return A.fx_lo > 0 ? launch_fx<TH, TW, ACC_FX2>(C, A, grid, smem, batch, stream)
+                           : launch_fx<TH, TW, ACC_FX64>(C, A, grid, smem, batch, stream);
+    if (C.xt)   // x-dependent spectrum: the generic kernels with per-column constants
+        return launch_t<0, ACC_F32, false, TH, TW, 0, true>(C, A, grid, smem, batch, stream);
     if constexpr (has_occ6<TH, TW>()) {
         if (resid && mono && occ6 && C.smax == 3)
-            return launch_t<1, false, true, TH, TW, 3, false, 6>(C, A, grid, smem, batch, stream);
+            return launch_t<1, ACC_F32, true, TH, TW, 3, false, 6>(C, A, grid, smem, batch, stream);
         if (resid && mono && occ6 && C.smax == 4)
-            return launch_t<1, false, true, TH, TW, 4, false, 6>(C, A, grid, smem, batch, stream);
+            return launch_t<1, ACC_F32, true, TH, TW, 4, false, 6>(C, A, grid, smem, batch, stream);
     }
     if (resid && mono) {
         switch (C.smax) {
-        case 3: return launch_t<1, false, true, TH, TW, 3>(C, A, grid, smem, batch, stream);
-        case 4: return launch_t<1, false, true, TH, TW, 4>(C, A, grid, smem, batch, stream);
-        case 6: return launch_t<1, false, true, TH, TW, 6>(C, A, grid, smem, batch, stream);
-        default: return launch_t<1, false, true, TH, TW>(C, A, grid, smem, batch, stream);
+        case 3: return launch_t<1, ACC_F32, true, TH, TW, 3>(C, A, grid, smem, batch, stream);
+        case 4: return launch_t<1, ACC_F32, true, TH, TW, 4>(C, A, grid, smem, batch, stream);
+        case 6: return launch_t<1, ACC_F32, true, TH, TW, 6>(C, A, grid, smem, batch, stream);
+        default: return launch_t<1, ACC_F32, true, TH, TW>(C, A, grid, smem, batch, stream);
         }
     }
-    if (mono) return launch_t<1, false, false, TH, TW>(C, A, grid, smem, batch, stream);
+    if (mono)
+        return C.smax == 4 ? launch_t<1, ACC_F32, false, TH, TW, 4>(C, A, grid, smem, batch, stream)
+                           : launch_t<1, ACC_F32, false, TH, TW>(C, A, grid, smem, batch, stream);
     if (C.ns == 8)   // the common polychromatic counts with an unrolled line loop
-        return C.smax == 4 ? launch_t<8, false, false, TH, TW, 4>(C, A, grid, smem, batch, stream)
-                           : launch_t<8, false, false, TH, TW>(C, A, grid, smem, batch, stream);
+        return C.smax == 4 ? launch_t<8, ACC_F32, false, TH, TW, 4>(C, A, grid, smem, batch, stream)
+                           : launch_t<8, ACC_F32, false, TH, TW>(C, A, grid, smem, batch, stream);
     if (C.ns == 4)
-        return C.smax == 4 ? launch_t<4, false, false, TH, TW, 4>(C, A, grid, smem, batch, stream)
-                           : launch_t<4, false, false, TH, TW>(C, A, grid, smem, batch, stream);
+        return C.smax == 4 ? launch_t<4, ACC_F32, false, TH, TW, 4>(C, A, grid, smem, batch, stream)
+                           : launch_t<4, ACC_F32, false, TH, TW>(C, A, grid, smem, batch, stream);
     switch (C.smax) {
-    case 3: return launch_t<0, false, false, TH, TW, 3>(C, A, grid, smem, batch, stream);
-    case 4: return launch_t<0, false, false, TH, TW, 4>(C, A, grid, smem, batch, stream);
-    case 6: return launch_t<0, false, false, TH, TW, 6>(C, A, grid, smem, batch, stream);
-    default: return launch_t<0, false, false, TH, TW>(C, A, grid, smem, batch, stream);
+    case 3: return launch_t<0, ACC_F32, false, TH, TW, 3>(C, A, grid, smem, batch, stream);
+    case 4: return launch_t<0, ACC_F32, false, TH, TW, 4>(C, A, grid, smem, batch, stream);
+    case 6: return launch_t<0, ACC_F32, false, TH, TW, 6>(C, A, grid, smem, batch, stream);
+    default: return launch_t<0, ACC_F32, false, TH, TW>(C, A, grid, smem, batch, stream);
     }
 }
 
 template <int TH, int TW>
 cudaError_t init_shape()
 {
-    cudaError_t e = epr_allow_max_smem(k_splat<1, true, false, TH, TW>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<0, true, false, TH, TW>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<1, false, true, TH, TW>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<1, false, true, TH, TW, 3>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<1, false, true, TH, TW, 4>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<1, false, true, TH, TW, 6>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<1, false, false, TH, TW>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<0, false, false, TH, TW>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<0, false, false, TH, TW, 3>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<0, false, false, TH, TW, 4>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<0, false, false, TH, TW, 6>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<8, false, false, TH, TW, 4>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<8, false, false, TH, TW>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<4, false, false, TH, TW, 4>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<4, false, false, TH, TW>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<0, true, false, TH, TW, 0, true>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<0, false, false, TH, TW, 0, true>);
+    cudaError_t e = cudaSuccess;
+    auto allow = [&](auto kernel) { if (e == cudaSuccess) e = epr_allow_max_smem(kernel); };
+    allow(k_splat<1, ACC_FX2, false, TH, TW, 4>);
+    allow(k_splat<0, ACC_FX2, false, TH, TW, 4>);
+    allow(k_splat<1, ACC_FX2, false, TH, TW>);
+    allow(k_splat<0, ACC_FX2, false, TH, TW>);
+    allow(k_splat<1, ACC_FX64, false, TH, TW>);
+    allow(k_splat<0, ACC_FX64, false, TH, TW>);
+    allow(k_splat<1, ACC_F32, true, TH, TW>);
+    allow(k_splat<1, ACC_F32, true, TH, TW, 3>);
+    allow(k_splat<1, ACC_F32, true, TH, TW, 4>);
+    allow(k_splat<1, ACC_F32, true, TH, TW, 6>);
+    allow(k_splat<1, ACC_F32, false, TH, TW, 4>);
+    allow(k_splat<1, ACC_F32, false, TH, TW>);
+    allow(k_splat<0, ACC_F32, false, TH, TW>);
+    allow(k_splat<0, ACC_F32, false, TH, TW, 3>);
+    allow(k_splat<0, ACC_F32, false, TH, TW, 4>);
+    allow(k_splat<0, ACC_F32, false, TH, TW, 6>);
+    allow(k_splat<8, ACC_F32, false, TH, TW, 4>);
+    allow(k_splat<8, ACC_F32, false, TH, TW>);
+    allow(k_splat<4, ACC_F32, false, TH, TW, 4>);
+    allow(k_splat<4, ACC_F32, false, TH, TW>);
+    allow(k_splat<0, ACC_FX2, false, TH, TW, 0, true>);
+    allow(k_splat<0, ACC_FX64, false, TH, TW, 0, true>);
+    allow(k_splat<0, ACC_F32, false, TH, TW, 0, true>);
     if constexpr (has_occ6<TH, TW>()) {
-        if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<1, false, true, TH, TW, 3, false, 6>);
-        if (e == cudaSuccess) e = epr_allow_max_smem(k_splat<1, false, true, TH, TW, 4, false, 6>);
+        allow(k_splat<1, ACC_F32, true, TH, TW, 3, false, 6>);
+        allow(k_splat<1, ACC_F32, true, TH, TW, 4, false, 6>);
     }
     return e;
 }
@@ -693,10 +842,10 @@ bool epr_splat_has_occ6(int TH, int TW, int reach) { return TH * TW < 64 * 64 &&
 
 size_t epr_splat_smem(const EprConsts& C, int TH, int TW)
 {
-    const int R = C.smax + 1;
+    const int R = C.smax;
     const int HX = (R + 1 + 3) & ~3;
     const int SH = (TH + 2 * R + kQuad - 1) / kQuad * kQuad + 2;
-    const size_t acc_bytes = (size_t)C.ns * (TH + 2) * (TW + 2) * (C.det ? 8 : 4);
+    const size_t acc_bytes = (size_t)C.ns * (TH + 2) * (TW + 2 * kAccX) * (C.det ? 8 : 4);
     return ((acc_bytes + 15) & ~size_t(15)) + (size_t)SH * (TW + 2 * HX) * sizeof(float);
 }
 
@@ -727,6 +876,16 @@ cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* 
         while ((1 << bits) < win) ++bits;
         A.fxs = ldexpf(1.f, 32 - bits);
         A.fxs_inv = ldexpf(1.f, bits - 32);
+        // fixed point: W 2^L and W 2^(41 - L) < 2^32 with W < 2^(bits - 1)
+        A.fx_lo = bits - 1 <= 11 ? 32 - (bits - 1) : 0;
+        A.fx_lo_s = ldexpf(1.f, A.fx_lo);
+        A.fx_lo_inv = ldexpf(1.f, -A.fx_lo);
+        A.ch_max = 0.f;
+        A.tneg_max = C.tneg[0];
+        for (int i = 0; i < C.ns; ++i) {
+            A.ch_max = fmaxf(A.ch_max, 0.5f * fabsf(C.c[i]));
+            A.tneg_max = fmaxf(A.tneg_max, C.tneg[i]);
+        }
     }
     const size_t smem = epr_splat_smem(C, TH, TW);
     dim3 grid((C.nx + TW - 1) / TW, (C.ny + TH - 1) / TH, batch);
