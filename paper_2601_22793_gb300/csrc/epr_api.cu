@@ -38,8 +38,9 @@ cudaError_t epr_launch_row_fwd(const EprConsts& C, const EprWork& W, int mode, c
                                float tol, int batch, int check_done, cudaStream_t stream);
 cudaError_t epr_launch_split(const EprConsts& C, const EprWork& W, const float* D, int batch,
                              int fixed_point, int check_done, cudaStream_t stream);
-cudaError_t epr_launch_dnorm(const EprConsts& C, const EprWork& W, const float* D, int batch,
-                             size_t npix, double scale, cudaStream_t stream);
+cudaError_t epr_launch_solve_begin(const EprConsts& C, const EprWork& W, const float* D, float* T,
+                                   int batch, size_t npd, size_t npix, double scale,
+                                   cudaStream_t stream);
 cudaError_t epr_launch_split_os(const EprConsts& C, const EprWork& W, const float* D, int batch,
                                 int fixed_point, int check_done, cudaStream_t stream);
 cudaError_t epr_launch_bin_os(const EprConsts& C, const EprWork& W, int fixed_point, float* out,
@@ -47,13 +48,14 @@ cudaError_t epr_launch_bin_os(const EprConsts& C, const EprWork& W, int fixed_po
 cudaError_t epr_launch_row_inv(const EprConsts& C, const EprWork& W, int mode, float* Out, int line0,
                                int nl, int it, float omega, float eps, float tol, int batch,
                                int check_done, cudaStream_t stream);
-cudaError_t epr_row_init();
+cudaError_t epr_row_init(int nx);
 bool epr_col_make_map(const EprConsts& C, const float2* S, long long rows, CUtensorMap* out);
 cudaError_t epr_launch_col(const EprConsts& C, const EprWork& W, int line0, int nl, int batch,
                            int check_done, int cw_hint, int rho_it, cudaStream_t stream);
 cudaError_t epr_launch_finalize_kappa(const EprConsts& C, const EprWork& W, int it, float tol,
                                       int batch, cudaStream_t stream);
 cudaError_t epr_col_init();
+cudaError_t epr_col_init_tma(int ny);
 cudaError_t epr_launch_gather(const EprConsts& C, const float* T, const float* r, float* g, int line,
                               int batch, cudaStream_t stream);
 cudaError_t epr_launch_fx_to_float(const unsigned long long* q, float* out, size_t n, cudaStream_t stream);
@@ -120,7 +122,7 @@ struct epr_plan_s {
     double E[EPR_MAX_LINES], delta[EPR_MAX_LINES], beta[EPR_MAX_LINES], w[EPR_MAX_LINES];
     // workspace
     EprWork W;
-    alignas(64) CUtensorMap col_map;   // S for the column pass's bulk copies
+    CUtensorMap col_map[2];   // S for the column pass's bulk copies: wide, two-column tile
     int cap_batch;       // batch the workspace is sized for
     int cap_hist;        // history length it is sized for
     std::vector<void*> allocs;
@@ -283,9 +285,7 @@ epr_status ensure_workspace(epr_plan_s* p, int batch, int hist)
     }
     W.tw_x = p->tw_x;
     W.tw_y = p->tw_y;
-    if (p->opt.fft_radix == 16) W.col_radix16 = 1;
-    W.col_map = epr_col_make_map(C, W.S, (long long)nb * C.ns * C.ny, &p->col_map) ? &p->col_map
-                                                                                   : nullptr;
+    W.col_map = epr_col_make_map(C, W.S, (long long)nb * C.ns * C.ny, p->col_map) ? p->col_map : nullptr;
     p->cap_batch = nb;
     p->cap_hist = nh;
     // pinned host mirrors for solve info
@@ -411,15 +411,15 @@ epr_status launch_solve(epr_plan_s* p, const float* D, float* T, int batch, cons
 {
     const EprConsts& C = p->C;
     const size_t npix = (size_t)C.nx * C.ny;
-    EPR_TRY(cudaMemsetAsync(p->W.st, 0, (size_t)batch * sizeof(EprProjState), s));
-    EPR_TRY(cudaMemsetAsync(p->W.err, 0, sizeof(unsigned int), s));
-    if (o->init == 0) EPR_TRY(cudaMemsetAsync(T, 0, (size_t)batch * npix * sizeof(float), s));
     {
         ProfScope ps(p, EPR_KERNEL_OTHER, s);
-        // |D|^2 at detector resolution; with oversampling the norm of the
-        // residual is taken over its o^2-fold replication, so scale by o^2
+        // the solver state and error word cleared, T := 0 where the solve starts
+        // from the flat field, and |D|^2 at detector resolution; with
+        // oversampling the norm of the residual is taken over its o^2-fold
+        // replication, so scale by o^2
         const size_t npd = npix / ((size_t)C.os * C.os);
-        EPR_TRY(epr_launch_dnorm(C, p->W, D, batch, npd, (double)C.os * C.os, s));
+        EPR_TRY(epr_launch_solve_begin(C, p->W, D, o->init == 0 ? T : nullptr, batch, npd, npix,
+                                       (double)C.os * C.os, s));
     }
     // the non-local models back-transport with the gather, the local closures
     // with the identity
@@ -817,12 +817,11 @@ bool line_constants(epr_plan_s* p, double L_m, const double* delta, const double
 std::mutex g_init_mu;
 int g_init_done[64];
 
-epr_status init_kernels(int dev)
+epr_status init_kernels(int dev, int nx, int ny)
 {
     std::lock_guard<std::mutex> lk(g_init_mu);
     if (dev >= 0 && dev < 64 && g_init_done[dev]) return EPR_OK;
     EPR_TRY(epr_splat_init());
-    EPR_TRY(epr_row_init());
     EPR_TRY(epr_col_init());
     EPR_TRY(epr_local_init());
     if (dev >= 0 && dev < 64) g_init_done[dev] = 1;
@@ -837,6 +836,8 @@ extern "C" {
 const char* epr_status_string(epr_status s)
 {
     switch (s) {
+    EPR_TRY(epr_row_init(nx));
+    EPR_TRY(epr_col_init_tma(ny));
     case EPR_OK: return "ok";
     case EPR_ERR_INVALID_ARG: return "invalid argument";
     case EPR_ERR_UNSUPPORTED_SIZE:
@@ -919,7 +920,7 @@ epr_status epr_plan_create(epr_plan_t* out, int nx, int ny, double pixel_m, doub
         return EPR_ERR_INVALID_ARG;  // no line both weighted and absorbing
     }
 
-    epr_status st = init_kernels(p->device);
+    epr_status st = init_kernels(p->device, nx, ny);
     if (st != EPR_OK) {
         delete p;
         return st;
@@ -947,7 +948,7 @@ epr_status epr_plan_create(epr_plan_t* out, int nx, int ny, double pixel_m, doub
     }
     p->W.tw_x = p->tw_x;
     p->W.tw_y = p->tw_y;
-    p->W.col_radix16 = p->opt.fft_radix == 16;   // the choice the tuning calls report
+    p->W.col_radix16 = p->opt.fft_radix != 8;   // the choice the tuning calls report
     choose_splat_tiles(p);
     *out = p;
     return EPR_OK;

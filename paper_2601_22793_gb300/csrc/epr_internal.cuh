@@ -188,19 +188,31 @@ __device__ __forceinline__ float2 cscale(float2 a, float s) { return mul2(a, bot
 // `red` must hold 2 * 32 floats of shared memory.
 __device__ __forceinline__ void block_sum2(float& a, float& b, float* red)
 {
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-    }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = (blockDim.x + 31) >> 5;
+    const int left = (int)blockDim.x - 32 * wid;   // threads from this warp on
+    if (left >= 32) {
+        for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_down_sync(0xffffffffu, a, o);
+            b += __shfl_down_sync(0xffffffffu, b, o);
+        }
+    } else {   // a last warp that is not full: only its own lanes count
+        const unsigned int mask = (1u << left) - 1u;
+        for (int o = 16; o > 0; o >>= 1) {
+            const float x = __shfl_down_sync(mask, a, o), y = __shfl_down_sync(mask, b, o);
+            if (lane + o < left) {
+                a += x;
+                b += y;
+            }
+        }
+    }
     __syncthreads();
     if (lane == 0) {
         red[wid] = a;
         red[32 + wid] = b;
     }
     __syncthreads();
-    if (wid == 0) {
+    if (wid == 0 && nw > 1) {   // one warp holds its totals already
         a = lane < nw ? red[lane] : 0.f;
         b = lane < nw ? red[32 + lane] : 0.f;
         for (int o = 16; o > 0; o >>= 1) {
@@ -214,9 +226,18 @@ __device__ __forceinline__ void block_sum2(float& a, float& b, float* red)
 // block size); the total is returned to every thread.  `red` holds 32 doubles.
 __device__ __forceinline__ double block_sum_d(double v, double* red)
 {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = (blockDim.x + 31) >> 5;
+    const int left = (int)blockDim.x - 32 * wid;
+    if (left >= 32) {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    } else {
+        const unsigned int mask = (1u << left) - 1u;
+        for (int o = 16; o > 0; o >>= 1) {
+            const double x = __shfl_down_sync(mask, v, o);
+            if (lane + o < left) v += x;
+        }
+    }
     __syncthreads();
     if (lane == 0) red[wid] = v;
     __syncthreads();

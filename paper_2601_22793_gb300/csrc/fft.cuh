@@ -179,12 +179,81 @@ __device__ __forceinline__ void dft16(float2* v)
     for (int k = 0; k < 16; ++k) v[k] = o[k];
 }
 
+// 6 and 12 points as 2 x 3 and 4 x 3 by the prime-factor map (Good), which
+// needs no twiddles: with n = 3 n1 + 2 n2 mod 6, k = 3 k1 + 4 k2 mod 6, and
+// n = 3 n1 + 4 n2 mod 12, k = 9 k1 + 4 k2 mod 12, n k splits into n1 k1 over
+// the first factor and n2 k2 over the second.
+template <int DIR>
+__device__ __forceinline__ void dft6(float2* v)
+{
+    dft3<DIR>(v[0], v[2], v[4]);   // n1 = 0: n = 0, 2, 4
+    dft3<DIR>(v[3], v[5], v[1]);   // n1 = 1: n = 3, 5, 1
+    dft2<DIR>(v[0], v[3]);         // k2 = 0: k = 0, 3
+    dft2<DIR>(v[2], v[5]);         // k2 = 1: k = 4, 1
+    dft2<DIR>(v[4], v[1]);         // k2 = 2: k = 2, 5
+    const float2 x1 = v[5], x2 = v[4], x4 = v[2], x5 = v[1];
+    v[1] = x1;
+    v[2] = x2;
+    v[4] = x4;
+    v[5] = x5;
+}
+
+template <int DIR>
+__device__ __forceinline__ void dft12(float2* v)
+{
+    float2 a[3][4];   // [n2][n1], then [k2][k1]
+#pragma unroll
+    for (int n1 = 0; n1 < 4; ++n1)
+#pragma unroll
+        for (int n2 = 0; n2 < 3; ++n2) a[n2][n1] = v[(3 * n1 + 4 * n2) % 12];
+#pragma unroll
+    for (int n1 = 0; n1 < 4; ++n1) dft3<DIR>(a[0][n1], a[1][n1], a[2][n1]);
+#pragma unroll
+    for (int k2 = 0; k2 < 3; ++k2) dft4<DIR>(a[k2][0], a[k2][1], a[k2][2], a[k2][3]);
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1)
+#pragma unroll
+        for (int k2 = 0; k2 < 3; ++k2) v[(9 * k1 + 4 * k2) % 12] = a[k2][k1];
+}
+
+// 9 points as 3 x 3: n = 3 n1 + n2, k = k1 + 3 k2, twiddles W9^(n2 k1).
+template <int DIR>
+__device__ __forceinline__ void dft9(float2* v)
+{
+    const float d = (float)DIR;
+    const float c1 = 0.76604444311897803520f, s1 = 0.64278760968653932632f;    // 2 pi / 9
+    const float c2 = 0.17364817766693034885f, s2 = 0.98480775301220805937f;    // 4 pi / 9
+    const float c4 = -0.93969262078590838405f, s4 = 0.34202014332566873304f;   // 8 pi / 9
+    auto rot = [](float2 a, float c, float s) {   // a (c + i s)
+        return make_float2(a.x * c - a.y * s, a.x * s + a.y * c);
+    };
+#pragma unroll
+    for (int n2 = 0; n2 < 3; ++n2) dft3<DIR>(v[n2], v[n2 + 3], v[n2 + 6]);
+    v[1 + 3] = rot(v[1 + 3], c1, d * s1);   // n2 k1 = 1
+    v[1 + 6] = rot(v[1 + 6], c2, d * s2);   // 2
+    v[2 + 3] = rot(v[2 + 3], c2, d * s2);   // 2
+    v[2 + 6] = rot(v[2 + 6], c4, d * s4);   // 4
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) dft3<DIR>(v[3 * k1], v[3 * k1 + 1], v[3 * k1 + 2]);
+    // v[3 k1 + k2] holds X[k1 + 3 k2]
+    const float2 x1 = v[3], x2 = v[6], x3 = v[1], x5 = v[7], x6 = v[2], x7 = v[5];
+    v[1] = x1;
+    v[2] = x2;
+    v[3] = x3;
+    v[5] = x5;
+    v[6] = x6;
+    v[7] = x7;
+}
+
 template <int R, int DIR>
 __device__ __forceinline__ void dft(float2* v)
 {
     if constexpr (R == 2) dft2<DIR>(v[0], v[1]);
     else if constexpr (R == 3) dft3<DIR>(v[0], v[1], v[2]);
     else if constexpr (R == 4) dft4<DIR>(v[0], v[1], v[2], v[3]);
+    else if constexpr (R == 6) dft6<DIR>(v);
+    else if constexpr (R == 9) dft9<DIR>(v);
+    else if constexpr (R == 12) dft12<DIR>(v);
     else if constexpr (R == 16) dft16<DIR>(v);
     else dft8<DIR>(v);
 }
@@ -270,8 +339,7 @@ __device__ void fft(float2* buf, int N, int lgseq, int sj, int sm, const float2*
 // template parameters, so every stage is unrolled, strides fold into address
 // offsets, the first stage (Ns = 1) needs no twiddle, and a radix-R stage
 // loads one twiddle w = exp(DIR 2 pi i jm / (Ns R)) and forms w^2 .. w^(R-1)
-// by the Chebyshev three-term recurrence of cos and sin (a few ulp for
-// R <= 8, well inside the transform's error).
+// as products (apply_twiddles).
 // ---------------------------------------------------------------------------
 namespace eprfft {
 
@@ -282,29 +350,41 @@ __host__ __device__ constexpr int ct_pow2_part(int n)
 }
 // Stage plans: as many stages of the largest radix maxr (8, or 16 for blocks
 // with 16 elements per thread) as divide the power of two, then one stage of
-// the remaining power of two, then the factors of 3.
-__host__ __device__ constexpr int ct_n_stages(int n, int maxr = 8)
-{
-    int p = ct_pow2_part(n), c = 0;
-    while (p >= maxr) { p /= maxr; ++c; }
-    if (p > 1) ++c;
-    int t = n / ct_pow2_part(n);
-    while (t > 1) { t /= 3; ++c; }
-    return c;
-}
+// the remaining power of two (2, 4 or 8), times 3 when the power of three is
+// odd and that gives 6 or 12, then the factors of 9 and a last 3.  A merged
+// stage saves a round trip through shared memory: 1728 = 8 8 9 3 instead of
+// 8 8 3 3 3, 864 = 8 12 9 instead of 8 4 3 3 3.
 __host__ __device__ constexpr int ct_radix(int n, int s, int maxr = 8)
 {
-    int p = ct_pow2_part(n), k = 0;
+    int p = ct_pow2_part(n), t = n / p, k = 0;
     while (p >= maxr) {
         if (k == s) return maxr;
         p /= maxr;
         ++k;
     }
-    if (p > 1) {
+    int odd = 1;   // 3 when the power of three is odd
+    for (int u = t; u > 1; u /= 3) odd = 4 - odd;
+    t /= odd;
+    if (odd == 3 && (p == 2 || p == 4)) {
+        if (k == s) return 3 * p;
+        ++k;
+        odd = 1;
+    } else if (p > 1) {
         if (k == s) return p;
         ++k;
     }
-    return 3;
+    while (t > 1) {
+        if (k == s) return 9;
+        t /= 9;
+        ++k;
+    }
+    return k == s && odd == 3 ? 3 : 1;   // 1: past the last stage
+}
+__host__ __device__ constexpr int ct_n_stages(int n, int maxr = 8)
+{
+    int c = 0;
+    while (ct_radix(n, c, maxr) > 1) ++c;
+    return c;
 }
 __host__ __device__ constexpr int ct_ns(int n, int s, int maxr = 8)
 {
@@ -324,6 +404,33 @@ __host__ __device__ constexpr int ct_ns_rev(int n, int s, int maxr = 8)
     int v = 1;
     for (int i = 0; i < s; ++i) v *= ct_radix_rev(n, i, maxr);
     return v;
+}
+
+// v[r] *= w^r with w = exp(DIR 2 pi i i / N).  The powers come from products
+// of two lower ones (w^2 = w w, w^3 = w^2 w, w^4 = w^2 w^2, ...), so each is
+// at most 4 roundings deep: a transform of 2048 points is off by 1.8e-7 (radix
+// 8) and 2.5e-7 (radix 16) of its norm, where the three-term recurrence of
+// cos and sin (half the operations, 3 % of a 2048^2 solve) gives 4.2e-7 and
+// 6.5e-7: its error grows with r^2.  Taking w^4 and w^8 from the table as well
+// halves the error again and costs 3 %, in a kernel bound by its loads.
+template <int R, int DIR>
+__device__ __forceinline__ void apply_twiddles(float2 (&v)[R], const float2* __restrict__ tw, int i)
+{
+    float2 p[R];
+    p[1] = __ldg(&tw[i]);
+    if (DIR > 0) p[1].y = -p[1].y;
+    v[1] = cmul(v[1], p[1]);
+#pragma unroll
+    for (int r = 2; r < R; ++r) {
+        const int h = r >= 8 ? 8 : r >= 4 ? 4 : 2;
+        if (h == r) {
+            const float2 q = p[r / 2];
+            p[r] = make_float2(q.x * q.x - q.y * q.y, (q.x + q.x) * q.y);
+        } else {
+            p[r] = cmul(p[h], p[r - h]);
+        }
+        v[r] = cmul(v[r], p[r]);
+    }
 }
 
 // Output map of a stage: out = post(value, e) with e = j * SJ + m * SM the
@@ -369,29 +476,7 @@ __device__ __forceinline__ void stage_ct(const float2* in, float2* buf, const fl
                 for (int r = 0; r < R; ++r) v[k][r] = in[PADI::idx((j + r * NR) * SJ + base)];
             }
             if constexpr (NS > 1) {
-                // w^r = (cos r theta, sin r theta) by the three-term recurrence
-                // x_{r+1} = 2 cos(theta) x_r - x_{r-1} (two multiply-adds per power);
-                // a radix-16 stage runs it to w^7 only and takes w^8 = (w^4)^2 and
-                // w^(8 + r) = w^8 w^r, which keeps every power within a few ulp
-                float2 w = __ldg(&tw[jm * TWSTEP]);
-                if (DIR > 0) w.y = -w.y;
-                const float c2 = w.x + w.x;
-                constexpr int RREC = R > 8 ? 8 : R;
-                float2 wpow[RREC];
-                wpow[0] = make_float2(1.f, 0.f);
-                if constexpr (RREC > 1) wpow[1] = w;
-#pragma unroll
-                for (int r = 2; r < RREC; ++r)
-                    wpow[r] = make_float2(fmaf(c2, wpow[r - 1].x, -wpow[r - 2].x),
-                                          fmaf(c2, wpow[r - 1].y, -wpow[r - 2].y));
-#pragma unroll
-                for (int r = 1; r < RREC; ++r) v[k][r] = cmul(v[k][r], wpow[r]);
-                if constexpr (R > 8) {
-                    const float2 w8 = cmul(wpow[4], wpow[4]);
-                    v[k][8] = cmul(v[k][8], w8);
-#pragma unroll
-                    for (int r = 9; r < R; ++r) v[k][r] = cmul(v[k][r], cmul(w8, wpow[r - 8]));
-                }
+                apply_twiddles<R, DIR>(v[k], tw, jm * TWSTEP);
             }
             dst[k] = (jd * NS * R + jm) * SJ + base;
         }
@@ -513,25 +598,7 @@ __device__ __forceinline__ void stage_turn(float2* buf, const float2* __restrict
 #pragma unroll
             for (int r = 0; r < R; ++r) v[k][r] = buf[PAD::idx((j + r * NR) * SJ + base)];
             if constexpr (NS > 1) {
-                float2 w = __ldg(&tw[j * TWSTEP]);
-                if (DIRF > 0) w.y = -w.y;
-                const float c2 = w.x + w.x;
-                constexpr int RREC = R > 8 ? 8 : R;
-                float2 wpow[RREC];
-                wpow[0] = make_float2(1.f, 0.f);
-                if constexpr (RREC > 1) wpow[1] = w;
-#pragma unroll
-                for (int r = 2; r < RREC; ++r)
-                    wpow[r] = make_float2(fmaf(c2, wpow[r - 1].x, -wpow[r - 2].x),
-                                          fmaf(c2, wpow[r - 1].y, -wpow[r - 2].y));
-#pragma unroll
-                for (int r = 1; r < RREC; ++r) v[k][r] = cmul(v[k][r], wpow[r]);
-                if constexpr (R > 8) {
-                    const float2 w8 = cmul(wpow[4], wpow[4]);
-                    v[k][8] = cmul(v[k][8], w8);
-#pragma unroll
-                    for (int r = 9; r < R; ++r) v[k][r] = cmul(v[k][r], cmul(w8, wpow[r - 8]));
-                }
+                apply_twiddles<R, DIRF>(v[k], tw, j * TWSTEP);
             }
             j_of[k] = j;
             m_of[k] = m;

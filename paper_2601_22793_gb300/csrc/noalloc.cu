@@ -45,7 +45,7 @@ cudaError_t epr_launch_row_inv(const EprConsts& C, const EprWork& W, int mode, f
                                int batch, int check_done, cudaStream_t stream);
 cudaError_t epr_launch_col(const EprConsts& C, const EprWork& W, int line0, int nl, int batch,
                            int check_done, int cw_hint, int rho_it, cudaStream_t stream);
-cudaError_t epr_row_init();
+cudaError_t epr_row_init(int nx);
 cudaError_t epr_col_init();
 
 namespace {
@@ -76,7 +76,7 @@ cudaError_t setup(int dev, unsigned char** out)
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lk(g_mu);
     if (!g_attr_ready[dev]) {
-        e = epr_row_init();
+        e = epr_row_init(0);
         if (e != cudaSuccess) return e;
         e = epr_col_init();
         if (e != cudaSuccess) return e;
