@@ -84,10 +84,10 @@ cudaError_t epr_launch_sv_split_adj(const EprConsts& C, float* RSB, const float*
 cudaError_t epr_launch_sv_gT(const EprConsts& C, const float* vx, const float* vy, float* tn, int B,
                              cudaStream_t s);
 cudaError_t epr_launch_sv_accum(const double* part, size_t npix, int nslot, int slot, double* acc,
+size_t epr_vjp_part_len(int ns, int batch);
                                 int nacc, int slot_acc, double scale, int B, cudaStream_t s);
 cudaError_t epr_launch_vjp(const EprConsts& C, const float* T, const float* gbar, float* Tbar,
-                           float* vx, float* vy, double* part, int nblk, int batch,
-                           cudaStream_t stream);
+                           double* part, double* sums, int batch, cudaStream_t stream);
 
 // --- launch accounting -------------------------------------------------------
 static std::atomic<long long> g_launches(0);
@@ -155,10 +155,8 @@ struct epr_plan_s {
     cudaGraphExec_t prof_exec;   // last profiled solve
     bool tuned;                  // autotuner has run
     // vector-Jacobian product workspace (allocated on first use)
-    float* vjp_vx;
-    float* vjp_vy;
-    double* vjp_part;
-    double* h_vjp_part;
+    double* vjp_part;      // block partials and their sums
+    double* h_vjp_part;    // pinned copy of the sums
     int vjp_cap;
     // x-dependent spectrum: per-column constants on the device (C.xt points
     // here while a table is set) and the uniform preconditioner constants
@@ -836,9 +834,9 @@ extern "C" {
 const char* epr_status_string(epr_status s)
 {
     switch (s) {
+    case EPR_OK: return "ok";
     EPR_TRY(epr_row_init(nx));
     EPR_TRY(epr_col_init_tma(ny));
-    case EPR_OK: return "ok";
     case EPR_ERR_INVALID_ARG: return "invalid argument";
     case EPR_ERR_UNSUPPORTED_SIZE:
         return "unsupported size (need 2^a 3^b, a >= 3, 16..4096; internal grids of an "
@@ -967,8 +965,6 @@ void epr_plan_destroy(epr_plan_t p)
     if (p->h_st) cudaFreeHost(p->h_st);
     if (p->h_hist) cudaFreeHost(p->h_hist);
     if (p->prof_exec) cudaGraphExecDestroy(p->prof_exec);
-    if (p->vjp_vx) cudaFree(p->vjp_vx);
-    if (p->vjp_vy) cudaFree(p->vjp_vy);
     if (p->vjp_part) cudaFree(p->vjp_part);
     if (p->h_vjp_part) cudaFreeHost(p->h_vjp_part);
     if (p->xt_dev) cudaFree(p->xt_dev);
@@ -1103,20 +1099,15 @@ epr_status epr_vjp(epr_plan_t p, const float* T, const float* gbar, float* Tbar,
     cudaStream_t s = (cudaStream_t)stream;
     const EprConsts& C = p->C;
     const size_t npix = (size_t)C.nx * C.ny, n = (size_t)batch * npix;
-    const int nblk = 256;
+    const size_t part_len = epr_vjp_part_len(C.ns, batch), nsum = (size_t)batch * 2 * C.ns;
     if (batch > p->vjp_cap) {
         EPR_TRY(cudaStreamSynchronize(s));
-        if (p->vjp_vx) cudaFree(p->vjp_vx);
-        if (p->vjp_vy) cudaFree(p->vjp_vy);
         if (p->vjp_part) cudaFree(p->vjp_part);
         if (p->h_vjp_part) cudaFreeHost(p->h_vjp_part);
-        p->vjp_vx = p->vjp_vy = nullptr;
         p->vjp_part = p->h_vjp_part = nullptr;
         p->vjp_cap = 0;
-        EPR_TRY(cudaMalloc((void**)&p->vjp_vx, n * sizeof(float)));
-        EPR_TRY(cudaMalloc((void**)&p->vjp_vy, n * sizeof(float)));
-        EPR_TRY(cudaMalloc((void**)&p->vjp_part, (size_t)batch * nblk * 2 * C.ns * sizeof(double)));
-        EPR_TRY(cudaMallocHost((void**)&p->h_vjp_part, (size_t)batch * nblk * 2 * C.ns * sizeof(double)));
+        EPR_TRY(cudaMalloc((void**)&p->vjp_part, part_len * sizeof(double)));
+        EPR_TRY(cudaMallocHost((void**)&p->h_vjp_part, nsum * sizeof(double)));
         p->vjp_cap = batch;
     }
     float *Td, *gd, *Tbd;
@@ -1127,27 +1118,19 @@ epr_status epr_vjp(epr_plan_t p, const float* T, const float* gbar, float* Tbar,
     if (st != EPR_OK) return st;
     {
         ProfScope ps(p, EPR_KERNEL_OTHER, s);
-        EPR_TRY(epr_launch_vjp(C, Td, gd, Tbd, p->vjp_vx, p->vjp_vy, p->vjp_part, nblk, batch, s));
+        EPR_TRY(epr_launch_vjp(C, Td, gd, Tbd, p->vjp_part, scalars ? sums : nullptr, batch, s));
     }
     if (sTb) EPR_TRY(cudaMemcpyAsync(Tbar, Tbd, n * sizeof(float), cudaMemcpyDeviceToHost, s));
-    const bool scalars = delta_bar || beta_bar || L_bar;
-    if (scalars) {
-        const size_t np = (size_t)batch * nblk * 2 * C.ns;
-        EPR_TRY(cudaMemcpyAsync(p->h_vjp_part, p->vjp_part, np * sizeof(double),
-                                cudaMemcpyDeviceToHost, s));
-    }
+    if (scalars)
+        EPR_TRY(cudaMemcpyAsync(p->h_vjp_part, sums, nsum * sizeof(double), cudaMemcpyDeviceToHost, s));
     if (scalars || sTb) EPR_TRY(cudaStreamSynchronize(s));
     if (scalars) {
         const double p2 = p->pixel * p->pixel;
         for (int b = 0; b < batch; ++b) {
             double lbar = 0.0;
             for (int l = 0; l < C.ns; ++l) {
-                double cbar = 0.0, mubar = 0.0;
-                for (int k = 0; k < nblk; ++k) {
-                    const double* q = p->h_vjp_part + ((size_t)b * nblk + k) * 2 * C.ns;
-                    cbar += q[2 * l];
-                    mubar += q[2 * l + 1];
-                }
+                const double cbar = p->h_vjp_part[((size_t)b * C.ns + l) * 2];
+                const double mubar = p->h_vjp_part[((size_t)b * C.ns + l) * 2 + 1];
                 const double lam = kHcEvM / (p->E[l] * 1e3);
                 const double kk = 2.0 * kPi / lam;
                 if (delta_bar) delta_bar[(size_t)b * C.ns + l] = -p->L / p2 * cbar;
@@ -1160,6 +1143,8 @@ epr_status epr_vjp(epr_plan_t p, const float* T, const float* gbar, float* Tbar,
     return EPR_OK;
 }
 
+    const bool scalars = delta_bar || beta_bar || L_bar;
+    double* sums = p->vjp_part + (part_len - nsum);
 }  // extern "C"
 
 // --- reverse mode through the unrolled non-local solve ----------------------

@@ -13,99 +13,145 @@
 //   cbar_s   += ubar . G[T],   mubar_s += -T I_s a         (scalars)
 // then Tbar += G^T[vx, vy], the transpose of the numpy-gradient stencil.
 // The host turns cbar, mubar into dF/dL, dF/ddelta_s, dF/dbeta_s.
+//
+// A warp marches down a strip of 30 output columns (32 lanes): vx of the
+// neighbouring columns comes by warp shuffle and the last three rows of vy
+// stay in registers, so G^T needs no maps of vx and vy and no second pass.
+// Bound by the gather's loads (four corners per line and pixel, from L1 and
+// L2); the two-pass form it replaces also wrote and read vx, vy and Tbar and
+// kept its per-line sums in local memory.
 #include "epr_internal.cuh"
 
 namespace {
 
+constexpr int kVjpThreads = 256;
+constexpr int kVjpRows = 32;       // rows of a strip unit
+constexpr int kVjpMaxBlocks = 608; // per projection: 4 per SM on 152 SMs
+
 struct VjpArgs {
     const float* T;
     const float* gbar;
-    float* Tbar;         // receives -sum mu I a, then the full gradient
-    float* vx;           // [B][ny][nx]
-    float* vy;
-    double* part;        // [B][nblk][2 ns]  (cbar_s, mubar_s) per block
-    int nblk;
+    float* Tbar;
+    double* part;        // [B][kVjpMaxBlocks][2 ns]  (cbar_s, mubar_s) per block
+    int strips, units;   // of one projection
 };
 
-__device__ __forceinline__ float grad_v(const float* Tb, int y, int x, int ny, int nx, bool along_x)
+// corners of gbar at a mapped point on the rim of the field or beyond it
+// (0 outside the grid), and the fractions of the clamped shift
+__device__ __noinline__ void vjp_corners(const float* G, int y, int x, float uy, float ux, int ny, int nx,
+                                         float (&g)[4], float& dx, float& dy)
 {
-    const size_t o = (size_t)y * nx + x;
-    if (along_x) {
-        if (x == 0) return __ldg(&Tb[o + 1]) - __ldg(&Tb[o]);
-        if (x == nx - 1) return __ldg(&Tb[o]) - __ldg(&Tb[o - 1]);
-        return 0.5f * (__ldg(&Tb[o + 1]) - __ldg(&Tb[o - 1]));
+    const float lim = 2.f * (float)(nx > ny ? nx : ny);
+    ux = fminf(fmaxf(ux, -lim), lim);
+    uy = fminf(fmaxf(uy, -lim), lim);
+    const float fx = floorf(ux), fy = floorf(uy);
+    dx = ux - fx;
+    dy = uy - fy;
+    const int cx = x + (int)fx, cy = y + (int)fy;
+    const bool x0 = (unsigned)cx < (unsigned)nx, x1 = (unsigned)(cx + 1) < (unsigned)nx;
+    g[0] = g[1] = g[2] = g[3] = 0.f;
+    if ((unsigned)cy < (unsigned)ny) {
+        const float* r = G + (size_t)cy * nx + cx;
+        if (x0) g[0] = __ldg(r);
+        if (x1) g[1] = __ldg(r + 1);
     }
-    if (y == 0) return __ldg(&Tb[o + nx]) - __ldg(&Tb[o]);
-    if (y == ny - 1) return __ldg(&Tb[o]) - __ldg(&Tb[o - nx]);
-    return 0.5f * (__ldg(&Tb[o + nx]) - __ldg(&Tb[o - nx]));
+    if ((unsigned)(cy + 1) < (unsigned)ny) {
+        const float* r = G + (size_t)(cy + 1) * nx + cx;
+        if (x0) g[2] = __ldg(r);
+        if (x1) g[3] = __ldg(r + 1);
+    }
 }
 
-constexpr int kVjpThreads = 256;
-
-__global__ void __launch_bounds__(kVjpThreads) k_vjp_pix(const EprConsts C, const VjpArgs A)
+// NSM: bound of the line count at compile time (the sums stay in registers)
+template <int NSM>
+__global__ void __launch_bounds__(kVjpThreads) k_vjp(const __grid_constant__ EprConsts C, const VjpArgs A)
 {
-    __shared__ float s_c[EPR_MAX_LINES], s_f[EPR_MAX_LINES], s_mu[EPR_MAX_LINES];
-    __shared__ float red[2 * EPR_MAX_LINES][kVjpThreads / 32];
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int s = 0; s < EPR_MAX_LINES; ++s) {
-            s_c[s] = C.c[s];
-            s_f[s] = C.f[s];
-            s_mu[s] = C.mu[s];
-        }
-    }
-    __syncthreads();
+    __shared__ float red[2 * NSM][kVjpThreads / 32];
     const int nx = C.nx, ny = C.ny, ns = C.ns, b = blockIdx.y;
     const size_t npix = (size_t)nx * ny, pb = (size_t)b * npix;
     const float* Tb = A.T + pb;
     const float* Gb = A.gbar + pb;
-    float cacc[EPR_MAX_LINES], macc[EPR_MAX_LINES];
-    for (int s = 0; s < ns; ++s) {
-        cacc[s] = 0.f;
-        macc[s] = 0.f;
-    }
-    for (size_t i = blockIdx.x * (size_t)kVjpThreads + threadIdx.x; i < npix;
-         i += (size_t)gridDim.x * kVjpThreads) {
-        const int y = (int)(i / nx), x = (int)(i - (size_t)y * nx);
-        const float t = __ldg(&Tb[i]);
-        const float gxv = grad_v(Tb, y, x, ny, nx, true), gyv = grad_v(Tb, y, x, ny, nx, false);
-        const float lim = 2.f * (float)(nx > ny ? nx : ny);
-        float tb = 0.f, vxs = 0.f, vys = 0.f;
-        for (int s = 0; s < ns; ++s) {
-            const float cs = s_c[s];
-            const float ux = fminf(fmaxf(cs * gxv, -lim), lim), uy = fminf(fmaxf(cs * gyv, -lim), lim);
-            const float fx = floorf(ux), fy = floorf(uy);
-            const float dx = ux - fx, dy = uy - fy;
-            const int cx = x + (int)fx, cy = y + (int)fy;
-            const bool x0 = (unsigned)cx < (unsigned)nx, x1 = (unsigned)(cx + 1) < (unsigned)nx;
-            float g00 = 0.f, g10 = 0.f, g01 = 0.f, g11 = 0.f;
-            if ((unsigned)cy < (unsigned)ny) {
-                const float* r = Gb + (size_t)cy * nx + cx;
-                if (x0) g00 = __ldg(r);
-                if (x1) g10 = __ldg(r + 1);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    float cacc[NSM], macc[NSM];
+#pragma unroll
+    for (int s = 0; s < NSM; ++s) cacc[s] = macc[s] = 0.f;
+    for (int w = blockIdx.x * (kVjpThreads / 32) + wid; w < A.units; w += gridDim.x * (kVjpThreads / 32)) {
+        const int y0 = (w / A.strips) * kVjpRows, y1 = min(y0 + kVjpRows, ny);
+        const int x = (w % A.strips) * 30 - 1 + lane;
+        const bool on = x >= 0 && x < nx;                    // on the grid
+        const bool own = on && lane >= 1 && lane < 31;       // an output column
+        const int xc = min(max(x, 0), nx - 1);
+        const float* Tc = Tb + xc;
+        auto ldT = [&](int y) { return __ldg(Tc + (size_t)min(max(y, 0), ny - 1) * nx); };
+        float tm = 0.f, tc = ldT(y0 - 2), tp = ldT(y0 - 1), ahead = ldT(y0);
+        float vym = 0.f, vyc = 0.f, out = 0.f;   // v'_y of rows r - 2, r - 1; Tbar of row r - 1 so far
+        for (int r = y0 - 1; r <= y1; ++r) {   // v of row r; row r - 1 is complete
+            tm = tc;
+            tc = tp;
+            tp = ahead;
+            ahead = ldT(r + 2);
+            float l = __shfl_up_sync(0xffffffffu, tc, 1), h = __shfl_down_sync(0xffffffffu, tc, 1);
+            // the halo lanes' outer neighbours
+            if (lane == 0) l = __ldg(Tb + (size_t)min(max(r, 0), ny - 1) * nx + max(xc - 1, 0));
+            if (lane == 31) h = __ldg(Tb + (size_t)min(max(r, 0), ny - 1) * nx + min(xc + 1, nx - 1));
+            const bool xe = x == 0 || x == nx - 1, ye = r == 0 || r == ny - 1;
+            const float sx = xe ? 1.f : 0.5f, sy = ye ? 1.f : 0.5f;
+            const float gx = ((x == nx - 1 ? tc : h) - (x == 0 ? tc : l)) * sx;
+            const float gy = ((r == ny - 1 ? tc : tp) - (r == 0 ? tc : tm)) * sy;
+            float tb = 0.f, vx = 0.f, vy = 0.f;
+            if (on && r >= 0 && r < ny) {
+                const bool mine = own && r >= y0 && r < y1;   // counted in the sums once
+#pragma unroll
+                for (int s = 0; s < NSM; ++s) {
+                    if (s >= ns) break;
+                    const float cs = C.c[s];
+                    const float ux = cs * gx, uy = cs * gy;
+                    int ix, iy;
+                    const float2 d = floor_frac2(make_float2(ux, uy), ix, iy);
+                    float dx = d.x, dy = d.y;
+                    const int cx = x + ix, cy = r + iy;
+                    float g[4];
+                    if ((unsigned)cx < (unsigned)(nx - 1) && (unsigned)cy < (unsigned)(ny - 1)) {
+                        const float* q = Gb + (size_t)cy * nx + cx;
+                        g[0] = __ldg(q);
+                        g[1] = __ldg(q + 1);
+                        g[2] = __ldg(q + nx);
+                        g[3] = __ldg(q + nx + 1);
+                    } else {
+                        vjp_corners(Gb, r, x, uy, ux, ny, nx, g, dx, dy);
+                    }
+                    const float a = (1.f - dy) * ((1.f - dx) * g[0] + dx * g[1]) +
+                                    dy * ((1.f - dx) * g[2] + dx * g[3]);
+                    const float Is = C.f[s] * __expf(-C.mu[s] * tc);
+                    const float ubx = Is * ((1.f - dy) * (g[1] - g[0]) + dy * (g[3] - g[2]));
+                    const float uby = Is * ((1.f - dx) * (g[2] - g[0]) + dx * (g[3] - g[1]));
+                    tb += -C.mu[s] * Is * a;
+                    vx += cs * ubx;
+                    vy += cs * uby;
+                    if (mine) {
+                        cacc[s] += ubx * gx + uby * gy;
+                        macc[s] += -tc * Is * a;
+                    }
+                }
             }
-            if ((unsigned)(cy + 1) < (unsigned)ny) {
-                const float* r = Gb + (size_t)(cy + 1) * nx + cx;
-                if (x0) g01 = __ldg(r);
-                if (x1) g11 = __ldg(r + 1);
-            }
-            const float a = (1.f - dy) * ((1.f - dx) * g00 + dx * g10) + dy * ((1.f - dx) * g01 + dx * g11);
-            const float Is = s_f[s] * __expf(-s_mu[s] * t);
-            const float ubx = Is * ((1.f - dy) * (g10 - g00) + dy * (g11 - g01));
-            const float uby = Is * ((1.f - dx) * (g01 - g00) + dx * (g11 - g10));
-            tb += -s_mu[s] * Is * a;
-            vxs += cs * ubx;
-            vys += cs * uby;
-            cacc[s] += ubx * gxv + uby * gyv;
-            macc[s] += -t * Is * a;
+            // G^T: with v' = v at the edges and v / 2 elsewhere, row and column
+            // i add v'(i - 1) - v'(i + 1), where a neighbour beyond the grid is
+            // minus the edge value
+            const float vxs = vx * sx, vys = vy * sy;
+            const float vl = __shfl_up_sync(0xffffffffu, vxs, 1), vh = __shfl_down_sync(0xffffffffu, vxs, 1);
+            const float row = tb + ((x == 0 ? -vxs : vl) - (x == nx - 1 ? -vxs : vh));
+            const int yo = r - 1;
+            if (own && yo >= y0 && yo < y1)
+                A.Tbar[pb + (size_t)yo * nx + x] =
+                    out + ((yo == 0 ? -vyc : vym) - (yo == ny - 1 ? -vyc : vys));
+            out = row;
+            vym = vyc;
+            vyc = vys;
         }
-        A.Tbar[pb + i] = tb;
-        A.vx[pb + i] = vxs;
-        A.vy[pb + i] = vys;
     }
     // deterministic block partials: warp shuffles, then warps in order
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int s = 0; s < ns; ++s) {
+#pragma unroll
+    for (int s = 0; s < NSM; ++s) {
         float c = cacc[s], m = macc[s];
         for (int o = 16; o > 0; o >>= 1) {
             c += __shfl_down_sync(0xffffffffu, c, o);
@@ -119,55 +165,51 @@ __global__ void __launch_bounds__(kVjpThreads) k_vjp_pix(const EprConsts C, cons
     __syncthreads();
     if (threadIdx.x < 2 * ns) {
         double acc = 0.0;
-        for (int w = 0; w < kVjpThreads / 32; ++w) acc += (double)red[threadIdx.x][w];
-        A.part[((size_t)b * A.nblk + blockIdx.x) * 2 * ns + threadIdx.x] = acc;
+        for (int i = 0; i < kVjpThreads / 32; ++i) acc += (double)red[threadIdx.x][i];
+        A.part[((size_t)b * kVjpMaxBlocks + blockIdx.x) * 2 * ns + threadIdx.x] = acc;
     }
 }
 
-// transpose of the unit-spacing numpy-gradient stencil along one axis
-__device__ __forceinline__ float gT1(const float* v, size_t st, int n, int x)
+// sums[b][k] of the nblk block partials, in a fixed order: one block per
+// scalar and projection
+__global__ void __launch_bounds__(256) k_vjp_sum(const double* part, int nblk, int n, double* sums)
 {
-    float acc = 0.f;
-    if (x - 1 >= 1 && x - 1 <= n - 2) acc += 0.5f * v[(size_t)(x - 1) * st];
-    if (x + 1 >= 1 && x + 1 <= n - 2) acc -= 0.5f * v[(size_t)(x + 1) * st];
-    if (x == 1) acc += v[0];
-    if (x == 0) acc -= v[0];
-    if (x == n - 1) acc += v[(size_t)(n - 1) * st];
-    if (x == n - 2) acc -= v[(size_t)(n - 1) * st];
-    return acc;
-}
-
-__global__ void k_vjp_gT(const EprConsts C, const VjpArgs A)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int b = blockIdx.z;
-    const int nx = C.nx, ny = C.ny;
-    if (x >= nx || y >= ny) return;
-    const size_t pb = (size_t)b * nx * ny;
-    const float* vx = A.vx + pb + (size_t)y * nx;
-    const float* vy = A.vy + pb + x;
-    const size_t o = pb + (size_t)y * nx + x;
-    A.Tbar[o] += gT1(vx, 1, nx, x) + gT1(vy, (size_t)nx, ny, y);
+    __shared__ double red[32];
+    const int k = blockIdx.x, b = blockIdx.y;
+    double v = 0.0;
+    for (int i = threadIdx.x; i < nblk; i += blockDim.x) v += part[((size_t)b * kVjpMaxBlocks + i) * n + k];
+    const double t = block_sum_d(v, red);
+    if (threadIdx.x == 0) sums[(size_t)b * n + k] = t;
 }
 
 }  // namespace
 
-// Two kernels; the per-block scalar partials land in `part` ([batch][nblk][2 ns]).
+// Doubles of workspace: the block partials, then the sums ([batch][2 ns]).
+size_t epr_vjp_part_len(int ns, int batch) { return (size_t)batch * (kVjpMaxBlocks + 1) * 2 * ns; }
+
+// The gradient, and with `sums` (device, [batch][2 ns]: cbar_s, mubar_s) the
+// scalars.
 cudaError_t epr_launch_vjp(const EprConsts& C, const float* T, const float* gbar, float* Tbar,
-                           float* vx, float* vy, double* part, int nblk, int batch,
-                           cudaStream_t stream)
+                           double* part, double* sums, int batch, cudaStream_t stream)
 {
     VjpArgs A;
     A.T = T;
     A.gbar = gbar;
     A.Tbar = Tbar;
-    A.vx = vx;
-    A.vy = vy;
     A.part = part;
-    A.nblk = nblk;
-    k_vjp_pix<<<dim3(nblk, batch), kVjpThreads, 0, stream>>>(C, A);
-    k_vjp_gT<<<dim3((C.nx + 63) / 64, (C.ny + 3) / 4, batch), dim3(64, 4), 0, stream>>>(C, A);
-    epr_count_launch(2);
+    A.strips = (C.nx + 29) / 30;
+    A.units = A.strips * ((C.ny + kVjpRows - 1) / kVjpRows);
+    int nblk = (A.units + kVjpThreads / 32 - 1) / (kVjpThreads / 32);
+    if (nblk > kVjpMaxBlocks) nblk = kVjpMaxBlocks;
+    const dim3 grid(nblk, batch), blk(kVjpThreads);
+    if (C.ns == 1) k_vjp<1><<<grid, blk, 0, stream>>>(C, A);
+    else if (C.ns <= 4) k_vjp<4><<<grid, blk, 0, stream>>>(C, A);
+    else if (C.ns <= 8) k_vjp<8><<<grid, blk, 0, stream>>>(C, A);
+    else k_vjp<16><<<grid, blk, 0, stream>>>(C, A);
+    epr_count_launch(1);
+    if (sums) {
+        k_vjp_sum<<<dim3(2 * C.ns, batch), 256, 0, stream>>>(part, nblk, 2 * C.ns, sums);
+        epr_count_launch(1);
+    }
     return cudaGetLastError();
 }
