@@ -1,502 +1,11 @@
-// Forward non-local transport: the conservative bilinear redistribution of
-// the object intensity of every spectral line onto the detector grid
-// (arXiv 2601.22793, Eq. 3 and "Discrete implementation: conservative
-// bilinear redistribution"), with the polychromatic sum of Eq. 5.
-//
-// Design (destination-tile binning):
-//  * A block owns one TH x TW destination tile of one projection and holds
-//    its accumulators (one per line) in shared memory.
-//  * It scans every source pixel whose shifted corners can land in the tile:
-//    the tile grown by the reach on each side (a shift of exactly +reach
-//    gives its far corner weight 0, so no further pixel contributes).  The
-//    thickness of that region plus a one-pixel ring (for the gradient) is
-//    staged in shared memory with asynchronous copies; beyond the grid the
-//    edge value is replicated, which makes the central difference half the
-//    one-sided one.  Blocks whose staged region lies inside the grid take a
-//    path without edge tests.
-//  * Per source and line it forms the shift u = c_s G[T] (central
-//    differences, one-sided at the grid edges), splits u into floor and
-//    fraction, and adds f_s exp(-mu_s T) times the four bilinear weights to
-//    the corners inside the tile with shared-memory atomics.  exp is
-//    evaluated only when the source reaches the tile.  A thread takes four
-//    vertically adjacent sources as two packed pairs; a quad that holds a
-//    long shift is done source by source instead.
-//  * The shared accumulators are integers, because integer shared-memory
-//    atomics are single instructions while float ones are not.  The float
-//    mode adds round(v * 2^S) in uint32 with S chosen from the reach so that
-//    no pixel can overflow: at most (2 reach + 3)^2 sources reach a pixel,
-//    each with a contribution <= f_s <= 1, so 2^(32-S) >= (2 reach + 3)^2.
-//    With a factor 2 of headroom, 2^(32-S) >= 2 (2 reach + 3)^2 holds for
-//    contributions up to 2 f_s, and a source whose intensity exceeds that
-//    (T < -ln 2 / mu_s, a negative thickness far outside any physical
-//    iterate) takes the overflow path with the long shifts.  For reach 4,
-//    S = 24: a rounding error of at most 3e-8 per contribution, half an fp32
-//    ulp of a unit intensity.
-//  * Every destination pixel is written exactly once, with plain coalesced
-//    stores: no zero fill and no global atomics on the fast path.  In the
-//    monochromatic float solve the flush stores the residual D - P instead
-//    of P (the adjoint gather then reads one value per corner).
-//  * A source-line with |u| > reach in either axis (or T below the bound
-//    above) is never splatted by the scan; the block that owns the source
-//    pixel appends it (with a bit mask of its long lines, its thickness and
-//    twice its gradient) to a per-projection overflow list, and a second
-//    kernel adds those contributions with global atomics.  No mass is lost,
-//    whatever the shift.  The list fill counter alternates between two slots
-//    by iteration parity, so the overflow kernel can clear the next slot.
-//  * Fixed-point mode accumulates round(v * 2^40) (contributions are
-//    non-negative), as uint64 in global memory: integer addition is
-//    associative, so the result is bit-identical across runs.  In shared
-//    memory the sums are kept as two uint32 planes, q = hi 2^L + lo, because
-//    64-bit shared-memory atomics are compare-and-swap loops: with at most
-//    W = (2 reach + 3)^2 sources per pixel of at most 2^41 each, W 2^L and
-//    W 2^(41 - L) both fit in 32 bits for L = 32 - ceil(log2 W) and
-//    W <= 2^11 (reach <= 21); a longer reach keeps the uint64 sums.
-#include <type_traits>
-
-#include "epr_internal.cuh"
+// Forward non-local transport around the tile kernel (splat_tile.cuh, which
+// describes it): the long-shift sources, the residual split, the oversampled
+// forms, and the host launchers.
+#include "splat_tile.cuh"
 
 namespace {
 
-// Threads of a splat block: 256 for one line; 512 for several lines (a
-// runtime count, or 4 or 8 at compile time), whose per-line accumulators
-// limit a 32 x 64 tile to two blocks per SM: the wider block doubles the
-// warps that hide the latency of the shared-memory atomics.  With the line
-// count known at compile time the line loop unrolls, so the compiler can
-// interleave the lines' dependency chains.
-__host__ __device__ constexpr int splat_threads(int NS) { return NS == 1 ? 256 : 512; }
-
-struct SplatArgs {
-    const float* T;          // [B][ny][nx]
-    const float* D;          // [B][ny][nx] (residual output)
-    float* P;                // [B][ny][nx]   P, or D - P (residual output)
-    float* Ps;               // [B][ns][ny][nx] or NULL (float mode, ns > 1)
-    unsigned long long* Pq;  // fixed-point mode
-    unsigned long long* Psq;
-    int* ovf_idx;
-    unsigned int* ovf_mask;
-    float4* ovf_tg;          // (T, twice the gradient x, y, 0) of each entry
-    EprProjState* st;
-    unsigned int* err;
-    int parity;
-    int check_done;
-    float fxs, fxs_inv;      // float mode: scale 2^S of the uint32 accumulators
-    int fx_lo;               // fixed-point mode: bits L of the low plane, 0 = uint64 sums
-    float fx_lo_s, fx_lo_inv;   // 2^L, 2^-L
-    float ch_max, tneg_max;  // largest |c_s| / 2 and largest tneg of the lines
-};
-
-// i / d for 0 <= i < 2^20 and d < 2^12 without an integer division
-__device__ __forceinline__ int fdiv(int i, float inv_d) { return (int)(((float)i + 0.5f) * inv_d); }
-
-__device__ __forceinline__ float exp2_approx(float x)
-{
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-// largest magnitude of three, and the smaller of two; NaN if one is NaN
-__device__ __forceinline__ float max_abs3(float a, float b, float c)
-{
-    float r;
-    asm("max.ftz.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-__device__ __forceinline__ float min_nan(float a, float b)
-{
-    float r;
-    asm("min.ftz.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-
-// Accumulator modes: float (uint32 of value * 2^S), fixed point as two uint32
-// planes, fixed point as uint64.
-enum { ACC_F32 = 0, ACC_FX2 = 1, ACC_FX64 = 2 };
-
-// v is already scaled by the accumulator's 2^S (2^40 in fixed point); the
-// second plane of ACC_FX2 follows the first at `plane` words.
-template <int MODE>
-__device__ __forceinline__ void acc_add(void* acc, int idx, int plane, float v, const SplatArgs& A)
-{
-    if constexpr (MODE == ACC_F32) {
-        atomicAdd(reinterpret_cast<unsigned int*>(acc) + idx, __float2uint_rn(v));
-    } else if constexpr (MODE == ACC_FX2) {
-        // hi = floor(v / 2^L); v - hi 2^L is exact (v has 24 bits), and its
-        // rounding is that of v to an integer
-        const unsigned int hi = __float2uint_rz(v * A.fx_lo_inv);
-        const unsigned int lo = __float2uint_rn(fmaf(-(float)hi, A.fx_lo_s, v));
-        unsigned int* a = reinterpret_cast<unsigned int*>(acc) + idx;
-        atomicAdd(a, lo);
-        atomicAdd(a + plane, hi);
-    } else {
-        atomicAdd(reinterpret_cast<unsigned long long*>(acc) + idx,
-                  (unsigned long long)__float2ll_rn(v));
-    }
-}
-
-template <int MODE>
-__device__ __forceinline__ unsigned long long acc_fx(const void* acc, int idx, int plane, int L)
-{
-    if constexpr (MODE == ACC_FX2) {
-        const unsigned int* a = reinterpret_cast<const unsigned int*>(acc) + idx;
-        return (unsigned long long)a[0] + ((unsigned long long)a[plane] << L);
-    } else {
-        return reinterpret_cast<const unsigned long long*>(acc)[idx];
-    }
-}
-
-constexpr int kFarList = 256;
-constexpr int kQuad = 4;   // sources per scan work item
-constexpr int kAccX = 4;   // accumulator column of tile column 0 (16-byte aligned rows)
-
-// NS = 1: single line known at compile time; NS = 0: C.ns lines.
-// Shared layout: accumulators [ns][TH + 2][TW + 8], the tile with a one-pixel
-// apron (its rows start at a 16-byte boundary, so the flush reads four pixels
-// at once); the staged thickness window [SH][SWa] whose first column
-// ax0 = tx0 - HX is 16-byte aligned (HX = reach + 1 rounded up to 4); a list
-// of far sources.
-//
-// The tile shape is a compile-time parameter (64 x 64, 32 x 64, 64 x 32 or
-// 32 x 32, chosen on the host), and so is the reach RC for the reaches the
-// tuner tries (RC = 0 takes C.smax), so every tile- and reach-derived index,
-// stride and offset folds into immediates.  Five blocks per SM (48 registers;
-// a 64 x 64 tile at reach 4 takes 43 KB of shared memory).
-// XT: an x-dependent spectrum, the line constants read per source column
-// from the plan's table (runtime line count and reach only).
-// OCC > 0: that many blocks per SM (six for the one-line residual kernels of
-// the tiles smaller than 64 x 64 at reach 3 and 4: 40 registers).
-template <int NS, int MODE, bool RESID, int TH, int TW, int RC = 0, bool XT = false, int OCC = 0>
-__global__ void __launch_bounds__(splat_threads(NS),
-                                  OCC > 0 ? OCC : NS != 1 ? 2 : ((RESID && RC == 0) ? 4 : 5))
-k_splat(const EprConsts C, const SplatArgs A)
-{
-    constexpr int kSplatThreads = splat_threads(NS);
-    constexpr bool DET = MODE != ACC_F32;
-    static_assert((TW & (TW - 1)) == 0 && TH * TW <= 4 * 4 * kSplatThreads, "tile shape");
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_far_idx[kFarList];
-    __shared__ unsigned int s_far_mask[kFarList];
-    __shared__ int s_far_n, s_far_base;
-    const int b = blockIdx.z;
-    const int nx = C.nx, ny = C.ny;
-    const int ns = NS ? NS : C.ns;
-    const int ty0 = blockIdx.y * TH, tx0 = blockIdx.x * TW;
-    const int R = RC > 0 ? RC : C.smax;
-    const int RH = TH + 2 * R, RW = TW + 2 * R;     // source region
-    const int RHq = (RH + kQuad - 1) / kQuad;         // its rows in quads
-    const int HX = (R + 1 + 3) & ~3;
-    const int SH = RHq * kQuad + 2, SWa = TW + 2 * HX;   // staged thickness
-    const int coff = HX - R - 1;                     // staged column of source column tx0 - R - 1
-    constexpr int tile = TH * TW;
-    constexpr int AP = TW + 2 * kAccX, ACC = (TH + 2) * AP;
-    const int plane = ns * ACC;                       // words of one plane (ACC_FX2)
-    const size_t npix = (size_t)nx * ny;
-    const int tid = threadIdx.x;
-
-    void* acc = smem;
-    const size_t acc_bytes = (size_t)ns * ACC * (DET ? 8 : 4);
-    float* Ts = reinterpret_cast<float*>(smem + ((acc_bytes + 15) & ~size_t(15)));
-    const float* Tb = A.T + (size_t)b * npix;
-    if (tid == 0) s_far_n = 0;
-
-    // the detector data of the tile (residual output): its lines are asked for
-    // here and loaded after the scan, whose registers they would take
-    constexpr int kDq = 4;   // float4 per thread: tiles up to 64 x 64
-    constexpr int nq = tile >> 2;
-    constexpr int tw4 = TW >> 2;
-    if constexpr (RESID) {
-        constexpr int kLine = TW / 32;   // 128-byte lines of a row
-        if (tid < TH * kLine) {
-            const int gy = ty0 + tid / kLine, gx = tx0 + 32 * (tid % kLine);
-            if (gy < ny && gx < nx) prefetch_l2(A.D + (size_t)b * npix + (size_t)gy * nx + gx);
-        }
-    }
-
-    {   // ACC = 2 (TH + 2)(TW / 2 + 4), a multiple of 4
-        uint4* a = reinterpret_cast<uint4*>(acc);
-        for (int i = tid; i < ns * ACC / (DET ? 2 : 4); i += kSplatThreads) a[i] = make_uint4(0u, 0u, 0u, 0u);
-    }
-    // T, the done flags and the overflow counters come from earlier kernels
-    epr_grid_wait();
-    if (A.check_done && A.st[b].done) return;
-
-    const int sy0 = ty0 - R - 1, sx0 = tx0 - R - 1, ax0 = tx0 - HX;
-    const bool interior = sy0 >= 0 && sx0 >= 0 && sy0 + SH <= ny && sx0 + RW + 2 <= nx;
-    {
-        const int q = SWa >> 2;
-        const float inv_q = 1.f / (float)q;
-        for (int i = tid; i < SH * q; i += kSplatThreads) {
-            const int ly = fdiv(i, inv_q), c4 = i - ly * q;
-            const int gy = min(max(sy0 + ly, 0), ny - 1), gx = ax0 + 4 * c4;
-            const float* src = Tb + (size_t)gy * nx;
-            if (gx >= 0 && gx < nx) {   // nx % 4 == 0: all four or none
-                cp_async16(reinterpret_cast<float4*>(Ts) + i, src + gx);
-            } else {                     // the edge value (only the nearest column is read)
-                const float v = __ldg(src + (gx < 0 ? 0 : nx - 1));
-                reinterpret_cast<float4*>(Ts)[i] = make_float4(v, v, v, v);
-            }
-        }
-        cp_async_commit();
-        cp_async_wait_all();
-    }
-    __syncthreads();
-
-    const float fsmax = (float)R;
-    // the accumulator scale 2^S is folded into the line weight: a power of two
-    // scales exactly, so each contribution rounds to the same integer
-    const float fxs = DET ? EPR_FX_SCALE : A.fxs;
-    constexpr float kLog2e = 1.4426950408889634f;
-    // One source at region-local (ly, lx) with thickness t and twice its
-    // gradient: every line's shift, contributions and far flag.  Gradients
-    // are kept doubled (hi - lo), and half the shift constant multiplies
-    // them: 0.5 scales exactly, so u is the same float.
-    auto source = [&](int ly, int lx, float t, float gx2, float gy2) {
-        unsigned int far = 0u;
-        const int sxc = XT ? tx0 - R + lx : 0;   // source column (inside the grid)
-#pragma unroll 1
-        for (int s = 0; s < ns; ++s) {
-            const float ch = 0.5f * (XT ? xt_get(C, EPR_XT_C, s, sxc) : line_const(C.c, s));
-            const float ux = ch * gx2, uy = ch * gy2;
-            const float tneg = XT ? xt_get(C, EPR_XT_TNEG, s, sxc) : line_const(C.tneg, s);
-            if (fabsf(ux) <= fsmax && fabsf(uy) <= fsmax && t >= tneg) {
-                int ix, iy;
-                const float2 d = floor_frac2(make_float2(ux, uy), ix, iy);
-                const int cx = lx - R + ix, cy = ly - R + iy;   // corner 00, tile-local
-                // all four corners have a slot (apron) when one is in the tile
-                if ((unsigned)(cx + 1) <= (unsigned)TW && (unsigned)(cy + 1) <= (unsigned)TH) {
-                    const float fs = XT ? xt_get(C, EPR_XT_F, s, sxc) : line_const(C.f, s);
-                    const float mus = XT ? xt_get(C, EPR_XT_MU, s, sxc) : line_const(C.mu, s);
-                    const float m = (fs * fxs) * exp2_approx((-mus * kLog2e) * t);   // 2^S f e^(-mu t)
-                    const float mx1 = m * d.x, mx0 = m - mx1;          // m dx, m (1 - dx)
-                    const float w = 1.f - d.y;
-                    const int idx = s * ACC + (cy + 1) * AP + (cx + kAccX);
-                    acc_add<MODE>(acc, idx, plane, mx0 * w, A);
-                    acc_add<MODE>(acc, idx + 1, plane, mx1 * w, A);
-                    acc_add<MODE>(acc, idx + AP, plane, mx0 * d.y, A);
-                    acc_add<MODE>(acc, idx + AP + 1, plane, mx1 * d.y, A);
-                }
-            } else {
-                far |= 1u << s;
-            }
-        }
-        if (far && (unsigned)(ly - R) < (unsigned)TH && (unsigned)(lx - R) < (unsigned)TW) {
-            const int sy = ty0 - R + ly, sx = tx0 - R + lx;
-            const int pos = atomicAdd(&s_far_n, 1);
-            if (pos < kFarList) {
-                s_far_idx[pos] = sy * nx + sx;
-                s_far_mask[pos] = far;
-            } else {   // list full: append to the global list directly
-                const int gpos = atomicAdd(&A.st[b].ovf_count[A.parity], 1);
-                if (gpos < C.ovf_cap) {
-                    A.ovf_idx[(size_t)b * C.ovf_cap + gpos] = sy * nx + sx;
-                    A.ovf_mask[(size_t)b * C.ovf_cap + gpos] = far;
-                    A.ovf_tg[(size_t)b * C.ovf_cap + gpos] = make_float4(t, gx2, gy2, 0.f);
-                } else {
-                    atomicOr(A.err, EPR_DEVERR_OVERFLOW);
-                }
-            }
-        }
-    };
-    // The scan: a thread takes kQuad vertically adjacent sources of one
-    // column (rows ly0 .. ly0 + kQuad - 1 of the region, padded to a multiple
-    // of kQuad; padding rows cannot reach the tile and are not owned by it),
-    // reusing the column's thickness values.  Sources 0, 1 and 2, 3 of the
-    // quad are the two lanes of packed arithmetic: the column's six values
-    // form the pairs (c0, c1), (c2, c3), (c4, c5), whose differences are the
-    // row gradients of both pairs.  The scan was bound by instruction issue
-    // (75 % active in a batch): the packed forms, the floor by rounding mode
-    // (FRND and F2I run at an eighth of the FMA rate) and one long-shift test
-    // per quad took it from 123 to 91 thread instructions per pixel, and the
-    // kernel from 142 to 103 us for eight 2048^2 projections; what bounds it
-    // now is the shared-memory data pipe (80 % busy: the loads of the staged
-    // window and the accumulator atomics).
-    // Work item (qy, lx) is advanced by kSplatThreads = dly quad rows +
-    // dlx columns.
-    const int nitem = RHq * RW;
-    const int dly = kSplatThreads / RW, dlx = kSplatThreads - dly * RW;
-    auto scan = [&](auto interior_tag) {
-        constexpr bool IN = decltype(interior_tag)::value;
-        int qy = tid / RW, lx = tid - (tid / RW) * RW;
-        for (int i = tid; i < nitem; i += kSplatThreads, lx += dlx,
-                 qy += dly + (lx >= RW ? 1 : 0), lx -= (lx >= RW ? RW : 0)) {
-            const int ly0 = qy * kQuad;
-            const float* tp = Ts + (ly0 + 1) * SWa + (lx + 1 + coff);   // source (ly0, lx)
-            float2 c[kQuad / 2 + 1], g_x[kQuad / 2], g_y[kQuad / 2];   // column pairs, twice the gradients
-#pragma unroll
-            for (int j = 0; j < kQuad / 2 + 1; ++j)
-                c[j] = make_float2(tp[(2 * j - 1) * SWa], tp[2 * j * SWa]);
-            const int sx = tx0 - R + lx;
-            if (!IN && (sx < 0 || sx >= nx)) continue;
-#pragma unroll
-            for (int j = 0; j < kQuad / 2; ++j) {
-                g_x[j] = sub2(make_float2(tp[2 * j * SWa + 1], tp[(2 * j + 1) * SWa + 1]),
-                              make_float2(tp[2 * j * SWa - 1], tp[(2 * j + 1) * SWa - 1]));
-                g_y[j] = sub2(c[j + 1], c[j]);
-                if constexpr (!IN) {   // one-sided differences are not halved
-                    if (sx == 0 || sx == nx - 1) g_x[j] = add2(g_x[j], g_x[j]);
-                    const int sy = ty0 - R + ly0 + 2 * j;
-                    if (sy == 0 || sy == ny - 1) g_y[j].x += g_y[j].x;
-                    if (sy + 1 == 0 || sy + 1 == ny - 1) g_y[j].y += g_y[j].y;
-                }
-            }
-            bool ok[kQuad];   // sources on the grid
-#pragma unroll
-            for (int j = 0; j < kQuad; ++j) ok[j] = IN || (unsigned)(ty0 - R + ly0 + j) < (unsigned)ny;
-            const float t[kQuad] = {c[0].y, c[1].x, c[1].y, c[2].x};
-            // no line's shift is long when that of the largest |c_s| is not;
-            // a NaN fails the test and goes to the source path
-            const float um = max_abs3(max_abs3(max_abs3(g_x[0].x, g_x[0].y, g_x[1].x), g_x[1].y, g_y[0].x),
-                                      g_y[0].y, max_abs3(g_y[1].x, g_y[1].y, 0.f));
-            const bool all_near = A.ch_max * um <= fsmax &&
-                                  min_nan(min_nan(t[0], t[1]), min_nan(t[2], t[3])) >= A.tneg_max;
-            if (XT || !all_near) {
-#pragma unroll 1
-                for (int j = 0; j < kQuad; ++j) {
-                    const bool hi = j >= 2, od = j & 1;
-                    const float2 gx = hi ? g_x[1] : g_x[0], gy = hi ? g_y[1] : g_y[0];
-                    const bool on = IN || (unsigned)(ty0 - R + ly0 + j) < (unsigned)ny;
-                    if (on) source(ly0 + j, lx, tp[j * SWa], od ? gx.y : gx.x, od ? gy.y : gy.x);
-                }
-                continue;
-            }
-#pragma unroll(NS ? NS : 1)
-            for (int s = 0; s < ns; ++s) {
-                const float2 ch = both(0.5f * C.c[s]);
-#pragma unroll
-                for (int j = 0; j < kQuad / 2; ++j) {
-                    int ix0, ix1, iy0, iy1;
-                    const float2 dx = floor_frac2(mul2(ch, g_x[j]), ix0, ix1);
-                    const float2 dy = floor_frac2(mul2(ch, g_y[j]), iy0, iy1);
-                    // corner 00, counted from the apron
-                    const int cx0 = lx - R + 1 + ix0, cx1 = lx - R + 1 + ix1;
-                    const int cy0 = ly0 + 2 * j - R + 1 + iy0, cy1 = ly0 + 2 * j - R + 2 + iy1;
-                    const bool in0 = ok[2 * j] && (unsigned)cx0 <= (unsigned)TW && (unsigned)cy0 <= (unsigned)TH;
-                    const bool in1 = ok[2 * j + 1] && (unsigned)cx1 <= (unsigned)TW && (unsigned)cy1 <= (unsigned)TH;
-                    if (in0 || in1) {
-                        const float mk = -C.mu[s] * kLog2e;
-                        // 2^S f e^(-mu t)
-                        const float2 m = mul2(both(C.f[s] * fxs),
-                                              make_float2(exp2_approx(mk * t[2 * j]), exp2_approx(mk * t[2 * j + 1])));
-                        const float2 mx1 = mul2(m, dx), mx0 = sub2(m, mx1);
-                        const float2 w = sub2(both(1.f), dy);
-                        const float2 v00 = mul2(mx0, w), v10 = mul2(mx1, w);
-                        const float2 v01 = mul2(mx0, dy), v11 = mul2(mx1, dy);
-                        if (in0) {
-                            const int idx = s * ACC + cy0 * AP + cx0 + kAccX - 1;
-                            acc_add<MODE>(acc, idx, plane, v00.x, A);
-                            acc_add<MODE>(acc, idx + 1, plane, v10.x, A);
-                            acc_add<MODE>(acc, idx + AP, plane, v01.x, A);
-                            acc_add<MODE>(acc, idx + AP + 1, plane, v11.x, A);
-                        }
-                        if (in1) {
-                            const int idx = s * ACC + cy1 * AP + cx1 + kAccX - 1;
-                            acc_add<MODE>(acc, idx, plane, v00.y, A);
-                            acc_add<MODE>(acc, idx + 1, plane, v10.y, A);
-                            acc_add<MODE>(acc, idx + AP, plane, v01.y, A);
-                            acc_add<MODE>(acc, idx + AP + 1, plane, v11.y, A);
-                        }
-                    }
-                }
-            }
-        }
-    };
-    if (interior) scan(std::true_type{});
-    else scan(std::false_type{});
-    float4 dreg[kDq];
-    if constexpr (RESID) {   // under way while the block meets at the barrier
-#pragma unroll
-        for (int k = 0; k < kDq; ++k) {
-            const int i4 = tid + k * kSplatThreads;
-            dreg[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (i4 < nq) {
-                const int ly = i4 / tw4, lx = (i4 - ly * tw4) << 2;
-                const int gy = ty0 + ly, gx = tx0 + lx;
-                if (gy < ny && gx < nx)
-                    dreg[k] = __ldg(reinterpret_cast<const float4*>(A.D + (size_t)b * npix + (size_t)gy * nx + gx));
-            }
-        }
-    }
-    __syncthreads();
-    epr_grid_release();
-
-    // far sources of this block: one reservation in the global list.  Each
-    // entry carries T and twice the gradient, formed from the staged window
-    // as in the scan (the same bits), so the overflow kernel reads no T.
-    const int nfar = s_far_n < kFarList ? s_far_n : kFarList;
-    if (nfar > 0) {
-        if (tid == 0) s_far_base = atomicAdd(&A.st[b].ovf_count[A.parity], nfar);
-        __syncthreads();
-        for (int e = tid; e < nfar; e += kSplatThreads) {
-            const int gpos = s_far_base + e;
-            if (gpos < C.ovf_cap) {
-                const int pix = s_far_idx[e];
-                const int sy = pix / nx, sx = pix - sy * nx;
-                const int ly = sy - ty0 + R, lx = sx - tx0 + R;   // in the source region
-                const float* tp = Ts + (ly + 1) * SWa + (lx + 1 + coff);
-                const float t = tp[0];
-                float gx2 = tp[1] - tp[-1], gy2 = tp[SWa] - tp[-SWa];
-                if (sx == 0 || sx == nx - 1) gx2 += gx2;
-                if (sy == 0 || sy == ny - 1) gy2 += gy2;
-                A.ovf_idx[(size_t)b * C.ovf_cap + gpos] = pix;
-                A.ovf_mask[(size_t)b * C.ovf_cap + gpos] = s_far_mask[e];
-                A.ovf_tg[(size_t)b * C.ovf_cap + gpos] = make_float4(t, gx2, gy2, 0.f);
-            } else {
-                atomicOr(A.err, EPR_DEVERR_OVERFLOW);
-            }
-        }
-    }
-
-    // flush: every pixel of the tile inside the grid, once, coalesced, four
-    // at a time
-    if constexpr (!DET) {
-        const uint4* a = reinterpret_cast<const uint4*>(acc);
-        const float inv = A.fxs_inv;
-#pragma unroll
-        for (int k = 0; k < kDq; ++k) {
-            const int i4 = tid + k * kSplatThreads;
-            if (i4 >= nq) continue;
-            const int ly = i4 / tw4, lx = (i4 - ly * tw4) << 2;
-            const int gy = ty0 + ly, gx = tx0 + lx;
-            if (gy >= ny || gx >= nx) continue;
-            const size_t o = (size_t)b * npix + (size_t)gy * nx + gx;
-            const int i0 = ((ly + 1) * AP + lx + kAccX) >> 2;
-            if constexpr (RESID) {
-                const uint4 v = a[i0];
-                const float4 d = dreg[k];
-                *reinterpret_cast<float4*>(A.P + o) =
-                    make_float4(d.x - (float)v.x * inv, d.y - (float)v.y * inv,
-                                d.z - (float)v.z * inv, d.w - (float)v.w * inv);
-            } else {
-                // sum <= 2 (2 reach + 3)^2 sum_s f_s: no overflow either
-                uint4 sum = make_uint4(0u, 0u, 0u, 0u);
-                for (int s = 0; s < ns; ++s) {
-                    const uint4 v = a[s * (ACC / 4) + i0];
-                    sum = make_uint4(sum.x + v.x, sum.y + v.y, sum.z + v.z, sum.w + v.w);
-                    if (ns > 1)
-                        *reinterpret_cast<float4*>(A.Ps + (size_t)s * npix + o + (size_t)b * (ns - 1) * npix) =
-                            make_float4((float)v.x * inv, (float)v.y * inv, (float)v.z * inv, (float)v.w * inv);
-                }
-                *reinterpret_cast<float4*>(A.P + o) = make_float4((float)sum.x * inv, (float)sum.y * inv,
-                                                                  (float)sum.z * inv, (float)sum.w * inv);
-            }
-        }
-    } else {
-        for (int i = tid; i < tile; i += kSplatThreads) {
-            const int ly = i / TW, lx = i & (TW - 1);
-            const int gy = ty0 + ly, gx = tx0 + lx;
-            if (gy >= ny || gx >= nx) continue;
-            const size_t o = (size_t)b * npix + (size_t)gy * nx + gx;
-            unsigned long long sum = 0ull;
-            for (int s = 0; s < ns; ++s) {
-                const unsigned long long q =
-                    acc_fx<MODE>(acc, s * ACC + (ly + 1) * AP + lx + kAccX, plane, A.fx_lo);
-                sum += q;
-                if (ns > 1) A.Psq[(size_t)s * npix + o + (size_t)b * (ns - 1) * npix] = q;
-            }
-            A.Pq[o] = sum;
-        }
-    }
-}
+using namespace eprsplat;
 
 // The long-shift sources of the overflow list, added with global atomics.
 template <bool DET, bool RESID, bool XT = false>
@@ -559,7 +68,7 @@ __global__ void __launch_bounds__(128) k_splat_overflow(const EprConsts C, const
                     atomicAdd(&A.P[(size_t)b * npix + o], -v);
                 } else {
                     atomicAdd(&A.P[(size_t)b * npix + o], v);
-                    if (ns > 1) atomicAdd(&A.Ps[((size_t)b * ns + s) * npix + o], v);
+                    if (ns > 1 && A.Ps) atomicAdd(&A.Ps[((size_t)b * ns + s) * npix + o], v);
                 }
             }
         }
@@ -571,15 +80,28 @@ __global__ void __launch_bounds__(128) k_splat_overflow(const EprConsts C, const
 // overflow sources are in: P <- D - P and P_s <- (D - P) P_s / P as float
 // maps, so that the adjoint gather reads one value per corner and line.  In
 // fixed-point mode the sums are read from the integer maps.
-// The float mode takes four pixels per thread and loads every line's P_s
-// before it stores any r_s (the stores could alias the later loads as far as
-// the compiler knows, which would serialise one memory round trip per line).
-__device__ __forceinline__ float split_one(float r, float p, float pl, float fs)
+//
+// Bound by memory (12 + 8 n_s bytes per pixel in float mode): four pixels per
+// thread, every line's P_s loaded before any r_s is stored (the stores could
+// alias the later loads as far as the compiler knows, which would serialise
+// one memory round trip per line).  The line count is bounded at compile time
+// by NSM, so the loads of 4 or 8 lines leave registers for enough warps, and r / P is
+// formed once per pixel: eight lines of a 2048^2 map 57 us with a division per
+// line and room for 16.
+template <bool DET>
+__device__ __forceinline__ float4 split_load(const float* f, const unsigned long long* q, size_t i)
 {
-    return (p > 1e-30f) ? r * (pl / p) : r * fs;
+    if constexpr (DET) {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(q + i);
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(q + i + 2);
+        return make_float4((float)a.x * EPR_FX_INV, (float)a.y * EPR_FX_INV, (float)b.x * EPR_FX_INV,
+                           (float)b.y * EPR_FX_INV);
+    } else {
+        return *reinterpret_cast<const float4*>(f + i);
+    }
 }
 
-template <bool DET, bool XT = false>
+template <bool DET, bool XT, int NSM>
 __global__ void __launch_bounds__(256) k_split(const EprConsts C, const SplatArgs A)
 {
     const int b = blockIdx.y;
@@ -588,52 +110,35 @@ __global__ void __launch_bounds__(256) k_split(const EprConsts C, const SplatArg
     epr_grid_release();
     const int ns = C.ns;
     const size_t npix = (size_t)C.nx * C.ny, pb = (size_t)b * npix;
-    if constexpr (!DET) {   // nx % 4 == 0: four pixels of one row per thread
-        const size_t n4 = npix / 4;
-        for (size_t q4 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q4 < n4;
-             q4 += (size_t)gridDim.x * blockDim.x) {
-            const size_t q = 4 * q4;
-            const float4 d = __ldg(reinterpret_cast<const float4*>(A.D + pb + q));
-            const float4 p = *reinterpret_cast<const float4*>(A.P + pb + q);
-            const float4 r = make_float4(d.x - p.x, d.y - p.y, d.z - p.z, d.w - p.w);
-            const int x = (int)(q % (size_t)C.nx);
-            float4 pl[EPR_MAX_LINES];
+    // nx % 4 == 0: four pixels of one row per thread
+    for (size_t q4 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q4 < npix / 4;
+         q4 += (size_t)gridDim.x * blockDim.x) {
+        const size_t q = 4 * q4;
+        const float4 d = __ldg(reinterpret_cast<const float4*>(A.D + pb + q));
+        const float4 p = split_load<DET>(A.P, A.Pq, pb + q);
+        float4 pl[NSM];
 #pragma unroll
-            for (int s = 0; s < EPR_MAX_LINES; ++s)
-                if (s < ns && ns > 1)
-                    pl[s] = *reinterpret_cast<const float4*>(A.Ps + (pb * ns) + (size_t)s * npix + q);
+        for (int s = 0; s < NSM; ++s)
+            if (s < ns && ns > 1) pl[s] = split_load<DET>(A.Ps, A.Psq, pb * ns + (size_t)s * npix + q);
+        const float4 r = make_float4(d.x - p.x, d.y - p.y, d.z - p.z, d.w - p.w);
+        const bool bx = p.x > 1e-30f, by = p.y > 1e-30f, bz = p.z > 1e-30f, bw = p.w > 1e-30f;
+        const float4 k = make_float4(bx ? r.x / p.x : r.x, by ? r.y / p.y : r.y, bz ? r.z / p.z : r.z,
+                                     bw ? r.w / p.w : r.w);
+        const int x = XT ? (int)(q % (size_t)C.nx) : 0;
 #pragma unroll
-            for (int s = 0; s < EPR_MAX_LINES; ++s) {
-                if (!(s < ns && ns > 1)) continue;
-                float4 o;
-                if constexpr (XT) {
-                    o = make_float4(split_one(r.x, p.x, pl[s].x, xt_get(C, EPR_XT_F, s, x)),
-                                    split_one(r.y, p.y, pl[s].y, xt_get(C, EPR_XT_F, s, x + 1)),
-                                    split_one(r.z, p.z, pl[s].z, xt_get(C, EPR_XT_F, s, x + 2)),
-                                    split_one(r.w, p.w, pl[s].w, xt_get(C, EPR_XT_F, s, x + 3)));
-                } else {
-                    const float fs = C.f[s];
-                    o = make_float4(split_one(r.x, p.x, pl[s].x, fs), split_one(r.y, p.y, pl[s].y, fs),
-                                    split_one(r.z, p.z, pl[s].z, fs), split_one(r.w, p.w, pl[s].w, fs));
-                }
-                *reinterpret_cast<float4*>(A.Ps + (pb * ns) + (size_t)s * npix + q) = o;
-            }
-            *reinterpret_cast<float4*>(A.P + pb + q) = r;
+        for (int s = 0; s < NSM; ++s) {
+            if (!(s < ns && ns > 1)) continue;
+            float4 f;
+            if constexpr (XT)
+                f = make_float4(xt_get(C, EPR_XT_F, s, x), xt_get(C, EPR_XT_F, s, x + 1),
+                                xt_get(C, EPR_XT_F, s, x + 2), xt_get(C, EPR_XT_F, s, x + 3));
+            else
+                f = make_float4(C.f[s], C.f[s], C.f[s], C.f[s]);
+            *reinterpret_cast<float4*>(A.Ps + pb * ns + (size_t)s * npix + q) =
+                make_float4(k.x * (bx ? pl[s].x : f.x), k.y * (by ? pl[s].y : f.y),
+                            k.z * (bz ? pl[s].z : f.z), k.w * (bw ? pl[s].w : f.w));
         }
-        return;
-    }
-    for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < npix;
-         q += (size_t)gridDim.x * blockDim.x) {
-        const float d = __ldg(&A.D[pb + q]);
-        const float p = DET ? (float)A.Pq[pb + q] * EPR_FX_INV : A.P[pb + q];
-        const float r = d - p;
-        for (int s = 0; ns > 1 && s < ns; ++s) {   // one line: r itself
-            const size_t o = (pb * ns) + (size_t)s * npix + q;
-            const float pl = DET ? (float)A.Psq[o] * EPR_FX_INV : A.Ps[o];
-            const float fs = XT ? xt_get(C, EPR_XT_F, s, (int)(q % (size_t)C.nx)) : line_const(C.f, s);
-            A.Ps[o] = split_one(r, p, pl, fs);
-        }
-        A.P[pb + q] = r;
+        *reinterpret_cast<float4*>(A.P + pb + q) = r;
     }
 }
 
@@ -642,14 +147,49 @@ __global__ void __launch_bounds__(256) k_split(const EprConsts C, const SplatArg
 // detector pixel and replicated to the fine pixels of its block, where it is
 // split over the lines with the fine weights P_s / P.  One thread per
 // detector pixel; P <- replicated residual, P_s <- split residuals.
-template <bool DET>
+//
+// OS is the factor at compile time for 2, 3 and 4 (0: any): the block's
+// values are then loaded together, as pairs or quads where they are aligned,
+// kept for the split, and written once.
+template <int OS>
+__device__ __forceinline__ void os_load(const float* p, float (&v)[OS])
+{
+    if constexpr (OS == 2) {
+        const float2 a = *reinterpret_cast<const float2*>(p);
+        v[0] = a.x;
+        v[1] = a.y;
+    } else if constexpr (OS == 4) {
+        const float4 a = *reinterpret_cast<const float4*>(p);
+        v[0] = a.x;
+        v[1] = a.y;
+        v[2] = a.z;
+        v[3] = a.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < OS; ++i) v[i] = p[i];
+    }
+}
+template <int OS>
+__device__ __forceinline__ void os_store(float* p, const float (&v)[OS])
+{
+    if constexpr (OS == 2) {
+        *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    } else if constexpr (OS == 4) {
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < OS; ++i) p[i] = v[i];
+    }
+}
+
+template <bool DET, int OS>
 __global__ void __launch_bounds__(256) k_split_os(const EprConsts C, const SplatArgs A)
 {
     const int b = blockIdx.y;
     epr_grid_wait();
     if (A.check_done && A.st[b].done) return;
     epr_grid_release();
-    const int ns = C.ns, os = C.os, nx = C.nx;
+    const int ns = C.ns, os = OS ? OS : C.os, nx = C.nx;
     const int nxd = C.nx / os, nyd = C.ny / os;
     const size_t npix = (size_t)C.nx * C.ny, pb = (size_t)b * npix;
     const size_t npd = (size_t)nxd * nyd;
@@ -658,6 +198,38 @@ __global__ void __launch_bounds__(256) k_split_os(const EprConsts C, const Splat
          qd += (size_t)gridDim.x * blockDim.x) {
         const int yd = (int)(qd / nxd), xd = (int)(qd - (size_t)yd * nxd);
         const size_t f0 = pb + (size_t)yd * os * nx + (size_t)xd * os;   // block corner
+        const float d = __ldg(&A.D[(size_t)b * npd + qd]);
+        if constexpr (OS > 0 && !DET) {
+            float p[OS][OS];
+#pragma unroll
+            for (int a = 0; a < OS; ++a) os_load<OS>(A.P + f0 + (size_t)a * nx, p[a]);
+            float sum = 0.f;
+#pragma unroll
+            for (int a = 0; a < OS; ++a)
+#pragma unroll
+                for (int c = 0; c < OS; ++c) sum += p[a][c];
+            const float r = d - sum * inv_o2;
+            for (int s = 0; ns > 1 && s < ns; ++s) {
+                const float fs = line_const(C.f, s);
+                float* ps = A.Ps + pb * ns + (size_t)s * npix + (f0 - pb);
+                float v[OS][OS];
+#pragma unroll
+                for (int a = 0; a < OS; ++a) os_load<OS>(ps + (size_t)a * nx, v[a]);
+#pragma unroll
+                for (int a = 0; a < OS; ++a) {
+#pragma unroll
+                    for (int c = 0; c < OS; ++c)
+                        v[a][c] = p[a][c] > 1e-30f ? r * (v[a][c] / p[a][c]) : r * fs;
+                    os_store<OS>(ps + (size_t)a * nx, v[a]);
+                }
+            }
+            float o[OS];
+#pragma unroll
+            for (int c = 0; c < OS; ++c) o[c] = r;
+#pragma unroll
+            for (int a = 0; a < OS; ++a) os_store<OS>(A.P + f0 + (size_t)a * nx, o);
+            continue;
+        }
         float mean;
         if constexpr (DET) {
             unsigned long long q = 0ull;
@@ -670,7 +242,7 @@ __global__ void __launch_bounds__(256) k_split_os(const EprConsts C, const Splat
                 for (int c = 0; c < os; ++c) sum += A.P[f0 + (size_t)a * nx + c];
             mean = sum * inv_o2;
         }
-        const float r = __ldg(&A.D[(size_t)b * npd + qd]) - mean;
+        const float r = d - mean;
         for (int a = 0; a < os; ++a)
             for (int c = 0; c < os; ++c) {
                 const size_t i = f0 + (size_t)a * nx + c;
@@ -730,111 +302,6 @@ __global__ void __launch_bounds__(256) k_bin_os(const EprConsts C, const SplatAr
     }
 }
 
-template <int NS, int MODE, bool RESID, int TH, int TW, int RC = 0, bool XT = false, int OCC = 0>
-cudaError_t launch_t(const EprConsts& C, const SplatArgs& A, dim3 grid, size_t smem, int batch,
-                     cudaStream_t stream)
-{
-    const bool pdl = C.pdl != 0;
-    const cudaError_t e = epr_launch_kernel(pdl, k_splat<NS, MODE, RESID, TH, TW, RC, XT, OCC>, grid,
-                                            dim3(splat_threads(NS)), smem, stream, C, A);
-    if (e != cudaSuccess) return e;
-    return epr_launch_kernel(pdl, k_splat_overflow<MODE != ACC_F32, RESID, XT>, dim3(128, batch),
-                             dim3(128), 0, stream, C, A);
-}
-
-// Tiles whose one-line residual kernel has a six-blocks-per-SM variant.
-template <int TH, int TW>
-constexpr bool has_occ6() { return TH * TW < 64 * 64; }
-
-template <int TH, int TW, int MODE>
-cudaError_t launch_fx(const EprConsts& C, const SplatArgs& A, dim3 grid, size_t smem, int batch,
-                      cudaStream_t stream)
-{
-    if (C.xt) return launch_t<0, MODE, false, TH, TW, 0, true>(C, A, grid, smem, batch, stream);
-    const bool r4 = MODE == ACC_FX2 && C.smax == 4;   // the default reach
-    if (C.ns == 1)
-        return r4 ? launch_t<1, MODE, false, TH, TW, MODE == ACC_FX2 ? 4 : 0>(C, A, grid, smem, batch, stream)
-                  : launch_t<1, MODE, false, TH, TW>(C, A, grid, smem, batch, stream);
-    return r4 ? launch_t<0, MODE, false, TH, TW, MODE == ACC_FX2 ? 4 : 0>(C, A, grid, smem, batch, stream)
-              : launch_t<0, MODE, false, TH, TW>(C, A, grid, smem, batch, stream);
-}
-
-template <int TH, int TW>
-cudaError_t launch_shape(const EprConsts& C, const SplatArgs& A, int resid, bool occ6, dim3 grid,
-                         size_t smem, int batch, cudaStream_t stream)
-{
-    const bool mono = C.ns == 1;
-    if (C.det)
-        return A.fx_lo > 0 ? launch_fx<TH, TW, ACC_FX2>(C, A, grid, smem, batch, stream)
-                           : launch_fx<TH, TW, ACC_FX64>(C, A, grid, smem, batch, stream);
-    if (C.xt)   // x-dependent spectrum: the generic kernels with per-column constants
-        return launch_t<0, ACC_F32, false, TH, TW, 0, true>(C, A, grid, smem, batch, stream);
-    if constexpr (has_occ6<TH, TW>()) {
-        if (resid && mono && occ6 && C.smax == 3)
-            return launch_t<1, ACC_F32, true, TH, TW, 3, false, 6>(C, A, grid, smem, batch, stream);
-        if (resid && mono && occ6 && C.smax == 4)
-            return launch_t<1, ACC_F32, true, TH, TW, 4, false, 6>(C, A, grid, smem, batch, stream);
-    }
-    if (resid && mono) {
-        switch (C.smax) {
-        case 3: return launch_t<1, ACC_F32, true, TH, TW, 3>(C, A, grid, smem, batch, stream);
-        case 4: return launch_t<1, ACC_F32, true, TH, TW, 4>(C, A, grid, smem, batch, stream);
-        case 6: return launch_t<1, ACC_F32, true, TH, TW, 6>(C, A, grid, smem, batch, stream);
-        default: return launch_t<1, ACC_F32, true, TH, TW>(C, A, grid, smem, batch, stream);
-        }
-    }
-    if (mono)
-        return C.smax == 4 ? launch_t<1, ACC_F32, false, TH, TW, 4>(C, A, grid, smem, batch, stream)
-                           : launch_t<1, ACC_F32, false, TH, TW>(C, A, grid, smem, batch, stream);
-    if (C.ns == 8)   // the common polychromatic counts with an unrolled line loop
-        return C.smax == 4 ? launch_t<8, ACC_F32, false, TH, TW, 4>(C, A, grid, smem, batch, stream)
-                           : launch_t<8, ACC_F32, false, TH, TW>(C, A, grid, smem, batch, stream);
-    if (C.ns == 4)
-        return C.smax == 4 ? launch_t<4, ACC_F32, false, TH, TW, 4>(C, A, grid, smem, batch, stream)
-                           : launch_t<4, ACC_F32, false, TH, TW>(C, A, grid, smem, batch, stream);
-    switch (C.smax) {
-    case 3: return launch_t<0, ACC_F32, false, TH, TW, 3>(C, A, grid, smem, batch, stream);
-    case 4: return launch_t<0, ACC_F32, false, TH, TW, 4>(C, A, grid, smem, batch, stream);
-    case 6: return launch_t<0, ACC_F32, false, TH, TW, 6>(C, A, grid, smem, batch, stream);
-    default: return launch_t<0, ACC_F32, false, TH, TW>(C, A, grid, smem, batch, stream);
-    }
-}
-
-template <int TH, int TW>
-cudaError_t init_shape()
-{
-    cudaError_t e = cudaSuccess;
-    auto allow = [&](auto kernel) { if (e == cudaSuccess) e = epr_allow_max_smem(kernel); };
-    allow(k_splat<1, ACC_FX2, false, TH, TW, 4>);
-    allow(k_splat<0, ACC_FX2, false, TH, TW, 4>);
-    allow(k_splat<1, ACC_FX2, false, TH, TW>);
-    allow(k_splat<0, ACC_FX2, false, TH, TW>);
-    allow(k_splat<1, ACC_FX64, false, TH, TW>);
-    allow(k_splat<0, ACC_FX64, false, TH, TW>);
-    allow(k_splat<1, ACC_F32, true, TH, TW>);
-    allow(k_splat<1, ACC_F32, true, TH, TW, 3>);
-    allow(k_splat<1, ACC_F32, true, TH, TW, 4>);
-    allow(k_splat<1, ACC_F32, true, TH, TW, 6>);
-    allow(k_splat<1, ACC_F32, false, TH, TW, 4>);
-    allow(k_splat<1, ACC_F32, false, TH, TW>);
-    allow(k_splat<0, ACC_F32, false, TH, TW>);
-    allow(k_splat<0, ACC_F32, false, TH, TW, 3>);
-    allow(k_splat<0, ACC_F32, false, TH, TW, 4>);
-    allow(k_splat<0, ACC_F32, false, TH, TW, 6>);
-    allow(k_splat<8, ACC_F32, false, TH, TW, 4>);
-    allow(k_splat<8, ACC_F32, false, TH, TW>);
-    allow(k_splat<4, ACC_F32, false, TH, TW, 4>);
-    allow(k_splat<4, ACC_F32, false, TH, TW>);
-    allow(k_splat<0, ACC_FX2, false, TH, TW, 0, true>);
-    allow(k_splat<0, ACC_FX64, false, TH, TW, 0, true>);
-    allow(k_splat<0, ACC_F32, false, TH, TW, 0, true>);
-    if constexpr (has_occ6<TH, TW>()) {
-        allow(k_splat<1, ACC_F32, true, TH, TW, 3, false, 6>);
-        allow(k_splat<1, ACC_F32, true, TH, TW, 4, false, 6>);
-    }
-    return e;
-}
-
 }  // namespace
 
 // Whether the six-blocks-per-SM residual splat exists for this tile and reach.
@@ -889,22 +356,32 @@ cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* 
     }
     const size_t smem = epr_splat_smem(C, TH, TW);
     dim3 grid((C.nx + TW - 1) / TW, (C.ny + TH - 1) / TH, batch);
+    const bool occ6 = W.splat_occ6 != 0;
     cudaError_t e;
-    if (TH == 64 && TW == 64) e = launch_shape<64, 64>(C, A, resid, W.splat_occ6 != 0, grid, smem, batch, stream);
-    else if (TH == 32 && TW == 64) e = launch_shape<32, 64>(C, A, resid, W.splat_occ6 != 0, grid, smem, batch, stream);
-    else if (TH == 64 && TW == 32) e = launch_shape<64, 32>(C, A, resid, W.splat_occ6 != 0, grid, smem, batch, stream);
-    else if (TH == 32 && TW == 32) e = launch_shape<32, 32>(C, A, resid, W.splat_occ6 != 0, grid, smem, batch, stream);
+    if (TH == 64 && TW == 64) e = epr_splat_launch_64x64(C, A, resid, occ6, grid, smem, stream);
+    else if (TH == 32 && TW == 64) e = epr_splat_launch_32x64(C, A, resid, occ6, grid, smem, stream);
+    else if (TH == 64 && TW == 32) e = epr_splat_launch_64x32(C, A, resid, occ6, grid, smem, stream);
+    else if (TH == 32 && TW == 32) e = epr_splat_launch_32x32(C, A, resid, occ6, grid, smem, stream);
     else return cudaErrorInvalidValue;
+    if (e != cudaSuccess) return e;
+    auto overflow = [&](auto kernel) {
+        e = epr_launch_kernel(C.pdl != 0, kernel, dim3(128, batch), dim3(128), 0, stream, C, A);
+    };
+    if (C.det && C.xt) overflow(k_splat_overflow<true, false, true>);
+    else if (C.det) overflow(k_splat_overflow<true, false>);
+    else if (C.xt) overflow(k_splat_overflow<false, false, true>);
+    else if (resid && C.ns == 1) overflow(k_splat_overflow<false, true>);
+    else overflow(k_splat_overflow<false, false>);
     epr_count_launch(2);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t epr_splat_init()
 {
-    cudaError_t e = init_shape<64, 64>();
-    if (e == cudaSuccess) e = init_shape<32, 64>();
-    if (e == cudaSuccess) e = init_shape<64, 32>();
-    if (e == cudaSuccess) e = init_shape<32, 32>();
+    cudaError_t e = epr_splat_init_64x64();
+    if (e == cudaSuccess) e = epr_splat_init_32x64();
+    if (e == cudaSuccess) e = epr_splat_init_64x32();
+    if (e == cudaSuccess) e = epr_splat_init_32x32();
     return e;
 }
 
@@ -922,17 +399,23 @@ cudaError_t epr_launch_split(const EprConsts& C, const EprWork& W, const float* 
     A.Psq = W.Psq;
     A.st = W.st;
     A.check_done = check_done;
-    const size_t npix = (size_t)C.nx * C.ny;
-    size_t blocks = (npix + 255) / 256;
+    const size_t n4 = (size_t)C.nx * C.ny / 4;
+    size_t blocks = (n4 + 255) / 256;
     if (blocks > 1216) blocks = 1216;   // 8 per SM on 152 SMs, grid-stride beyond
-    const dim3 grid((unsigned)blocks, batch);
-    cudaError_t e;
-    if (C.xt)
-        e = fixed_point ? epr_launch_kernel(C.pdl != 0, k_split<true, true>, grid, dim3(256), 0, stream, C, A)
-                        : epr_launch_kernel(C.pdl != 0, k_split<false, true>, grid, dim3(256), 0, stream, C, A);
-    else
-        e = fixed_point ? epr_launch_kernel(C.pdl != 0, k_split<true>, grid, dim3(256), 0, stream, C, A)
-                        : epr_launch_kernel(C.pdl != 0, k_split<false>, grid, dim3(256), 0, stream, C, A);
+    cudaError_t e = cudaSuccess;
+    auto go = [&](auto kernel) {
+        e = epr_launch_kernel(C.pdl != 0, kernel, dim3((unsigned)blocks, batch), dim3(256), 0, stream, C, A);
+    };
+    auto by_lines = [&](auto det, auto xt) {
+        constexpr bool DET = decltype(det)::value, XT = decltype(xt)::value;
+        if (C.ns <= 4) go(k_split<DET, XT, 4>);
+        else if (C.ns <= 8) go(k_split<DET, XT, 8>);
+        else go(k_split<DET, XT, 16>);
+    };
+    if (C.xt && fixed_point) by_lines(std::true_type{}, std::true_type{});
+    else if (C.xt) by_lines(std::false_type{}, std::true_type{});
+    else if (fixed_point) by_lines(std::true_type{}, std::false_type{});
+    else by_lines(std::false_type{}, std::false_type{});
     epr_count_launch(1);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -954,9 +437,12 @@ cudaError_t epr_launch_split_os(const EprConsts& C, const EprWork& W, const floa
     if (blocks > 1216) blocks = 1216;
     const dim3 grid((unsigned)blocks, batch), blk(256);
     const bool pdl = C.pdl != 0;
-    const cudaError_t e =
-        fixed_point ? epr_launch_kernel(pdl, k_split_os<true>, grid, blk, 0, stream, C, A)
-                    : epr_launch_kernel(pdl, k_split_os<false>, grid, blk, 0, stream, C, A);
+    cudaError_t e;
+    if (fixed_point) e = epr_launch_kernel(pdl, k_split_os<true, 0>, grid, blk, 0, stream, C, A);
+    else if (C.os == 2) e = epr_launch_kernel(pdl, k_split_os<false, 2>, grid, blk, 0, stream, C, A);
+    else if (C.os == 3) e = epr_launch_kernel(pdl, k_split_os<false, 3>, grid, blk, 0, stream, C, A);
+    else if (C.os == 4) e = epr_launch_kernel(pdl, k_split_os<false, 4>, grid, blk, 0, stream, C, A);
+    else e = epr_launch_kernel(pdl, k_split_os<false, 0>, grid, blk, 0, stream, C, A);
     epr_count_launch(1);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
