@@ -59,11 +59,10 @@ cudaError_t epr_col_init_tma(int ny);
 cudaError_t epr_launch_gather(const EprConsts& C, const float* T, const float* r, float* g, int line,
                               int batch, cudaStream_t stream);
 cudaError_t epr_launch_fx_to_float(const unsigned long long* q, float* out, size_t n, cudaStream_t stream);
-cudaError_t epr_launch_local(const EprConsts& C, const EprWork& W, const float* T, float* P, float* Ps,
-                             int order, int batch, int check_done, cudaStream_t stream);
-cudaError_t epr_local_init();
-cudaError_t epr_launch_wkb1(const EprConsts& C, const EprWork& W, const float* T, int fixed_point,
-                            int batch, int check_done, cudaStream_t stream);
+cudaError_t epr_launch_local(const EprConsts& C, const EprWork& W, const float* T, const float* D, float* P,
+                             float* Ps, int order, int batch, int check_done, cudaStream_t stream);
+cudaError_t epr_launch_wkb1(const EprConsts& C, const EprWork& W, const float* T, const float* D,
+                            int fixed_point, int batch, int check_done, cudaStream_t stream);
 cudaError_t epr_launch_col_kind(const EprConsts& C, const EprWork& W, int line, int batch, int kind,
                                 float kscale, cudaStream_t stream);
 int epr_sv_blocks();
@@ -84,8 +83,8 @@ cudaError_t epr_launch_sv_split_adj(const EprConsts& C, float* RSB, const float*
 cudaError_t epr_launch_sv_gT(const EprConsts& C, const float* vx, const float* vy, float* tn, int B,
                              cudaStream_t s);
 cudaError_t epr_launch_sv_accum(const double* part, size_t npix, int nslot, int slot, double* acc,
-size_t epr_vjp_part_len(int ns, int batch);
                                 int nacc, int slot_acc, double scale, int B, cudaStream_t s);
+size_t epr_vjp_part_len(int ns, int batch);
 cudaError_t epr_launch_vjp(const EprConsts& C, const float* T, const float* gbar, float* Tbar,
                            double* part, double* sums, int batch, cudaStream_t stream);
 
@@ -381,24 +380,45 @@ struct ProfScope {
     }
 };
 
+// The splat tile of a launch.  The default 64 x 64 tile has the smallest halo
+// (1.27 scanned sources per pixel at reach 4, 1.56 for 32 x 32), but a launch
+// with fewer of them than four per SM leaves SMs idle or with too few warps
+// to hide their latency; it takes 32 x 32 tiles.  Solve iteration of one line:
+// 256^2 30.0 -> 27.0 us, 512^2 30.3 -> 27.7, 1024^2 (256 large tiles) 42.8 ->
+// 38.8; 2048^2 (1024 large tiles) 70.7 with the large ones, 74.0 with the
+// small.  A tuned plan keeps the choice of its tuner.
+constexpr int kSplatMinTiles = 608;
+
+void splat_tile(const epr_plan_s* p, int batch, int* TH, int* TW)
+{
+    *TH = p->splat_TH;
+    *TW = p->splat_TW;
+    if (p->tuned || *TH != 64 || *TW != 64) return;
+    const long long tiles = (long long)((p->C.nx + 63) / 64) * ((p->C.ny + 63) / 64) * batch;
+    if (tiles < kSplatMinTiles) *TH = *TW = 32;
+}
+
 // One pass of the chosen forward model writing W.P (and W.Ps / W.Pq / W.Psq).
-// With D given (monochromatic float solve) W.P receives D - P instead of P.
-epr_status launch_forward(epr_plan_s* p, const float* T, const float* D, int parity, int batch,
-                          int model, int check_done, cudaStream_t s)
+// With D given W.P receives D - P instead of P (monochromatic float solve),
+// and the local and second-order models split it over the lines in W.Ps.
+epr_status launch_forward(epr_plan_s* p, const EprWork& W, const float* T, const float* D, int parity,
+                          int batch, int model, int check_done, cudaStream_t s)
 {
     if (model == EPR_MODEL_NONLOCAL || model == EPR_MODEL_NONLOCAL_WKB1) {
         {
             ProfScope ps(p, EPR_KERNEL_SPLAT, s);
-            EPR_TRY(epr_launch_splat(p->C, p->W, T, D, D != nullptr, parity, batch, p->splat_TH,
-                                     p->splat_TW, check_done, s));
+            int TH, TW;
+            splat_tile(p, batch, &TH, &TW);
+            const bool resid = D && model == EPR_MODEL_NONLOCAL;
+            EPR_TRY(epr_launch_splat(p->C, W, T, D, resid, parity, batch, TH, TW, check_done, s));
         }
         if (model == EPR_MODEL_NONLOCAL_WKB1) {   // second-order term: float P, P_s after it
             ProfScope ps(p, EPR_KERNEL_LOCAL, s);
-            EPR_TRY(epr_launch_wkb1(p->C, p->W, T, p->C.det, batch, check_done, s));
+            EPR_TRY(epr_launch_wkb1(p->C, W, T, D, p->C.det, batch, check_done, s));
         }
     } else {
         ProfScope ps(p, EPR_KERNEL_LOCAL, s);
-        EPR_TRY(epr_launch_local(p->C, p->W, T, p->W.P, p->W.Ps, model, batch, check_done, s));
+        EPR_TRY(epr_launch_local(p->C, W, T, D, W.P, W.Ps, model, batch, check_done, s));
     }
     return EPR_OK;
 }
@@ -424,21 +444,21 @@ epr_status launch_solve(epr_plan_s* p, const float* D, float* T, int batch, cons
     const bool nonlocal = model == EPR_MODEL_NONLOCAL || model == EPR_MODEL_NONLOCAL_WKB1;
     const int fwd_mode = nonlocal ? 0 : 1;
     // the residual D - P (and its split over the lines) is stored by the
-    // splat flush (plain non-local model, one line, float accumulation) or by
-    // the split kernel after the forward (several lines, fixed point, local
-    // closure, second-order non-local model)
+    // splat flush (plain non-local model, one line, float accumulation), by
+    // the stencil kernel of the local and second-order models, or by the split
+    // kernel after the forward (several lines, fixed point, oversampling)
     const bool nl = model == EPR_MODEL_NONLOCAL;   // P still in the splat's own format
-    const bool resid_in_splat = nl && C.ns == 1 && !C.det && C.os == 1 && !C.xt;
+    const bool resid_in_forward = C.os == 1 && (!nl || (C.ns == 1 && !C.det && !C.xt));
     const float eps = (float)(o->eps_I > 0 ? o->eps_I : 1e-8);
     for (int it = 0; it < o->n_iter; ++it) {
-        epr_status st = launch_forward(p, T, resid_in_splat ? D : nullptr, it & 1, batch, model, 1, s);
+        epr_status st = launch_forward(p, p->W, T, resid_in_forward ? D : nullptr, it & 1, batch, model, 1, s);
         if (st != EPR_OK) return st;
         if (C.os > 1) {
             ProfScope ps(p, EPR_KERNEL_OTHER, s);
             EPR_TRY(epr_launch_split_os(C, p->W, D, batch, nl && C.det, 1, s));
-        } else if (!resid_in_splat) {
+        } else if (!resid_in_forward) {
             ProfScope ps(p, EPR_KERNEL_OTHER, s);
-            EPR_TRY(epr_launch_split(C, p->W, D, batch, nl && C.det, 1, s));
+            EPR_TRY(epr_launch_split(C, p->W, D, batch, C.det, 1, s));
         }
         {
             ProfScope ps(p, EPR_KERNEL_ROW_FWD, s);
@@ -536,13 +556,13 @@ epr_status autotune_splat(epr_plan_s* p, const float* D, const float* T, int bat
             p->splat_TW = t[1];
             p->W.splat_occ6 = occ6;
             EPR_TRY(cudaMemsetAsync(p->W.st, 0, (size_t)batch * sizeof(EprProjState), s));
-            epr_status st = launch_forward(p, T, resid ? D : nullptr, 0, batch, EPR_MODEL_NONLOCAL, 0, s);
+            epr_status st = launch_forward(p, p->W, T, resid ? D : nullptr, 0, batch, EPR_MODEL_NONLOCAL, 0, s);
             if (st != EPR_OK) return st;
             float ms = 1e30f;   // the fastest of three repetitions of four forwards
             for (int rep = 0; rep < 3; ++rep) {
                 EPR_TRY(cudaEventRecord(e0, s));
                 for (int k = 0; k < 4; ++k) {
-                    st = launch_forward(p, T, resid ? D : nullptr, (k + 1) & 1, batch, EPR_MODEL_NONLOCAL,
+                    st = launch_forward(p, p->W, T, resid ? D : nullptr, (k + 1) & 1, batch, EPR_MODEL_NONLOCAL,
                                         0, s);
                     if (st != EPR_OK) return st;
                 }
@@ -817,11 +837,12 @@ int g_init_done[64];
 
 epr_status init_kernels(int dev, int nx, int ny)
 {
+    EPR_TRY(epr_row_init(nx));
+    EPR_TRY(epr_col_init_tma(ny));
     std::lock_guard<std::mutex> lk(g_init_mu);
     if (dev >= 0 && dev < 64 && g_init_done[dev]) return EPR_OK;
     EPR_TRY(epr_splat_init());
     EPR_TRY(epr_col_init());
-    EPR_TRY(epr_local_init());
     if (dev >= 0 && dev < 64) g_init_done[dev] = 1;
     return EPR_OK;
 }
@@ -835,8 +856,6 @@ const char* epr_status_string(epr_status s)
 {
     switch (s) {
     case EPR_OK: return "ok";
-    EPR_TRY(epr_row_init(nx));
-    EPR_TRY(epr_col_init_tma(ny));
     case EPR_ERR_INVALID_ARG: return "invalid argument";
     case EPR_ERR_UNSUPPORTED_SIZE:
         return "unsupported size (need 2^a 3^b, a >= 3, 16..4096; internal grids of an "
@@ -1000,9 +1019,23 @@ epr_status epr_forward(epr_plan_t p, const float* T, float* P, float* Ps, int ba
     if (st == EPR_OK && Ps) st = resolve(p, 2, Ps, nd * C.ns, false, s, &Psd, &sPs);
     if (st != EPR_OK) return st;
     EPR_TRY(cudaMemsetAsync(p->W.st, 0, (size_t)batch * sizeof(EprProjState), s));
-    st = launch_forward(p, Td, nullptr, 0, batch, model, 0, s);
-    if (st != EPR_OK) return st;
+    // on the detector grid the float models write the caller's maps (a line's
+    // prediction only where it is wanted): 4 lines of 2048^2 with P_s 97 us
+    // with a copy from the workspace.  Fixed point and oversampling convert
+    // from the workspace, and so does a call whose maps overlap.
     const bool fx = (model == EPR_MODEL_NONLOCAL) && C.det;
+    auto apart = [](const float* a, size_t na, const float* b, size_t nb) {
+        return !a || !b || a + na <= b || b + nb <= a;
+    };
+    const bool direct = C.os == 1 && !fx && apart(Td, n, Pd, n) && apart(Td, n, Psd, n * C.ns) &&
+                        apart(Pd, n, Psd, n * C.ns);
+    EprWork W = p->W;
+    if (direct) {
+        W.P = Pd;
+        if (C.ns > 1) W.Ps = Psd;
+    }
+    st = launch_forward(p, W, Td, nullptr, 0, batch, model, 0, s);
+    if (st != EPR_OK) return st;
     if (C.os > 1) {
         EPR_TRY(epr_launch_bin_os(C, p->W, fx, Pd, Psd, batch, s));
     } else if (fx) {
@@ -1011,12 +1044,14 @@ epr_status epr_forward(epr_plan_t p, const float* T, float* P, float* Ps, int ba
             if (C.ns > 1) EPR_TRY(epr_launch_fx_to_float(p->W.Psq, Psd, n * C.ns, s));
             else EPR_TRY(epr_launch_fx_to_float(p->W.Pq, Psd, n, s));
         }
-    } else {
+    } else if (!direct) {
         EPR_TRY(cudaMemcpyAsync(Pd, p->W.P, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
         if (Psd) {
             const float* src = C.ns > 1 ? p->W.Ps : p->W.P;
             EPR_TRY(cudaMemcpyAsync(Psd, src, n * C.ns * sizeof(float), cudaMemcpyDeviceToDevice, s));
         }
+    } else if (Psd && C.ns == 1) {
+        EPR_TRY(cudaMemcpyAsync(Psd, Pd, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
     }
     if (sP) EPR_TRY(cudaMemcpyAsync(P, Pd, nd * sizeof(float), cudaMemcpyDeviceToHost, s));
     if (sPs) EPR_TRY(cudaMemcpyAsync(Ps, Psd, nd * C.ns * sizeof(float), cudaMemcpyDeviceToHost, s));
@@ -1116,6 +1151,8 @@ epr_status epr_vjp(epr_plan_t p, const float* T, const float* gbar, float* Tbar,
     if (st == EPR_OK) st = resolve(p, 1, gbar, n, true, s, &gd, &sg);
     if (st == EPR_OK) st = resolve(p, 2, Tbar, n, false, s, &Tbd, &sTb);
     if (st != EPR_OK) return st;
+    const bool scalars = delta_bar || beta_bar || L_bar;
+    double* sums = p->vjp_part + (part_len - nsum);
     {
         ProfScope ps(p, EPR_KERNEL_OTHER, s);
         EPR_TRY(epr_launch_vjp(C, Td, gd, Tbd, p->vjp_part, scalars ? sums : nullptr, batch, s));
@@ -1143,8 +1180,6 @@ epr_status epr_vjp(epr_plan_t p, const float* T, const float* gbar, float* Tbar,
     return EPR_OK;
 }
 
-    const bool scalars = delta_bar || beta_bar || L_bar;
-    double* sums = p->vjp_part + (part_len - nsum);
 }  // extern "C"
 
 // --- reverse mode through the unrolled non-local solve ----------------------
@@ -1235,7 +1270,7 @@ epr_status sv_reverse_iteration(epr_plan_s* p, const float* D, const float* T, i
     const size_t npix = (size_t)C.nx * C.ny, m = (size_t)B * npix;
     // forward of this iteration, recomputed: P, P_s (float), r, r_s, g_s, h_s
     EPR_TRY(cudaMemsetAsync(p->W.st, 0, (size_t)B * sizeof(EprProjState), st));
-    epr_status es = launch_forward(p, T, nullptr, 0, B, EPR_MODEL_NONLOCAL, 0, st);
+    epr_status es = launch_forward(p, p->W, T, nullptr, 0, B, EPR_MODEL_NONLOCAL, 0, st);
     if (es != EPR_OK) return es;
     if (C.det) {
         EPR_TRY(epr_launch_fx_to_float(p->W.Pq, p->W.P, m, st));

@@ -1,7 +1,6 @@
 // Local O(L^2) forward closure (arXiv 2601.22793, Eq. 1) in pixel units,
 // and its diffraction-pressure term alone for the non-local model to second
-// order (k_wkb1, at the end),
-// per spectral line, summed over lines (Eq. 5):
+// order, per spectral line, summed over lines (Eq. 5):
 //   P_s = I - D_x(I u_x) - D_y(I u_y)                                    m = 1
 //       + 1/2 [D_xx(I u_x^2) + 2 D_x D_y(I u_x u_y) + D_yy(I u_y^2)]
 //       - eps^2/(4 p^4) [D_x(I D_x Q) + D_y(I D_y Q)]                      m = 2
@@ -10,336 +9,246 @@
 // [1, -2, 1] with the edge value replicated.  (eps grad phi = p u and the
 // physical derivative is D / p, which gives these pixel-unit forms.)
 //
-// One block computes a 32 x 32 output tile.  The nested derivatives reach 3
-// pixels, so the thickness is staged with a 3-pixel halo and every
-// intermediate field is evaluated in shared memory on a halo that shrinks by
-// one pixel per derivative.  Derivative stencils test the GLOBAL coordinate
-// for the edge rules, so values staged outside the grid are never used by
-// an in-grid output.
+// A warp owns a strip of columns and marches down its rows.  Every
+// intermediate field lives in registers, the last three rows of those that are
+// differentiated along y, and horizontal neighbours come by warp shuffle, so
+// there is no shared memory and no barrier.  The nested derivatives reach 3
+// pixels (2 for m = 1): 26 (28) of the 32 lanes are output columns, and a
+// strip of H rows computes H + 6.  The fields are bound by instruction issue:
+// the tile form this replaces staged every field in shared memory and spent
+// 440 (second-order term) and 620 (m = 2) thread instructions per pixel, most
+// of them on its index arithmetic, its barriers' phases and expm1.
+// Stencils test the GLOBAL coordinate for the edge rules, so values computed
+// outside the grid are never used by an in-grid output.  No atomics: the
+// result is the same on every run.
+//
+// In a solve (D given) the kernel also forms the residual and its split over
+// the lines, which would otherwise be a pass of its own over P and P_s.
 #include "epr_internal.cuh"
 
 namespace {
 
-constexpr int kLT = 32;            // output tile
-constexpr int kLH = 3;             // halo
-constexpr int kLE = kLT + 2 * kLH; // staged extent (38)
-constexpr int kLN = kLE * kLE;
-constexpr int kLocalThreads = 256;
+constexpr int kStencilThreads = 128;
 
-struct LocalArgs {
+enum { ST_LOCAL1 = 1, ST_LOCAL2 = 2, ST_WKB1 = 3 };
+
+struct StencilArgs {
     const float* T;
-    float* P;       // [B][ny][nx]
-    float* Ps;      // [B][ns][ny][nx] or NULL
+    const float* D;                  // solve: P <- D - P, P_s <- split residuals; else NULL
+    float* P;                        // [B][ny][nx] out (ST_WKB1: the splat's P in, float mode)
+    float* Ps;                       // [B][ns][ny][nx] (ns > 1), likewise, or NULL: not wanted
+    const unsigned long long* Pq;    // ST_WKB1: fixed-point sums of the splat (DET)
+    const unsigned long long* Psq;
     const EprProjState* st;
-    int order;
     int check_done;
+    int H, strips;                   // rows and strips of a projection
 };
 
-// Derivative stencils of a field given as a function of the staged index
-// (a shared array, or a product of shared arrays formed on the fly).
-template <class F>
-__device__ __forceinline__ float dX(F f, int l, int gx, int nx)
+// The sum of e^x - 1 over four arguments.  For |x| < 1/4 the Taylor series to
+// x^8 / 8! (the first omitted term is below 1.1e-11 |x|), whose rounding is
+// that of its last operations, as packed pairs; one test for all four.
+__device__ __forceinline__ float2 expm1_taylor(float2 x)
 {
-    if (gx == 0) return f(l + 1) - f(l);
-    if (gx == nx - 1) return f(l) - f(l - 1);
-    return 0.5f * (f(l + 1) - f(l - 1));
+    float2 p = fma2(x, both(1.f / 40320.f), both(1.f / 5040.f));
+    p = fma2(x, p, both(1.f / 720.f));
+    p = fma2(x, p, both(1.f / 120.f));
+    p = fma2(x, p, both(1.f / 24.f));
+    p = fma2(x, p, both(1.f / 6.f));
+    p = fma2(x, p, both(0.5f));
+    return fma2(mul2(x, x), p, x);
 }
-template <class F>
-__device__ __forceinline__ float dY(F f, int l, int gy, int ny)
+__device__ __noinline__ float expm1_sum4_any(float a, float b, float c, float d)
 {
-    if (gy == 0) return f(l + kLE) - f(l);
-    if (gy == ny - 1) return f(l) - f(l - kLE);
-    return 0.5f * (f(l + kLE) - f(l - kLE));
+    return (expm1f(a) + expm1f(b)) + (expm1f(c) + expm1f(d));
 }
-template <class F>
-__device__ __forceinline__ float dXX(F f, int l, int gx, int nx)
+__device__ __forceinline__ float expm1_sum4(float2 x, float2 y)
 {
-    const float lo = gx == 0 ? f(l) : f(l - 1);
-    const float hi = gx == nx - 1 ? f(l) : f(l + 1);
-    return lo - 2.f * f(l) + hi;
-}
-template <class F>
-__device__ __forceinline__ float dYY(F f, int l, int gy, int ny)
-{
-    const float lo = gy == 0 ? f(l) : f(l - kLE);
-    const float hi = gy == ny - 1 ? f(l) : f(l + kLE);
-    return lo - 2.f * f(l) + hi;
+    const float big = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y)));
+    if (!(big < 0.25f)) return expm1_sum4_any(x.x, x.y, y.x, y.y);
+    const float2 e = add2(expm1_taylor(x), expm1_taylor(y));   // a NaN argument stays one
+    return e.x + e.y;
 }
 
-struct Arr {
-    const float* a;
-    __device__ __forceinline__ float operator()(int l) const { return a[l]; }
+// Three consecutive rows of a field: m (row - 1), c (row), p (row + 1).
+struct Rows3 {
+    float m, c, p;
+    __device__ __forceinline__ void push(float v)
+    {
+        m = c;
+        c = p;
+        p = v;
+    }
 };
 
-// Shared fields: T, G_x, G_y, I (order 1); also Q, D_y(I u_x u_y), I D_x Q,
-// I D_y Q (order 2).  The fluxes I u and I u u are formed inside the stencils
-// from I and G.
-constexpr int local_fields(int order) { return order >= 2 ? 8 : 4; }
-
-template <int ORDER>
-__global__ void __launch_bounds__(kLocalThreads) k_local(const EprConsts C, const LocalArgs A)
+template <int MODE, bool DET>
+__global__ void __launch_bounds__(kStencilThreads, 8) k_stencil(const EprConsts C, const StencilArgs A)
 {
-    extern __shared__ __align__(16) float sm[];
-    float* Ts = sm;
-    float* GX = Ts + kLN;
-    float* GY = GX + kLN;
-    float* I = GY + kLN;
-    float* Q = I + kLN;       // order 2 only, as the three below
-    float* DYB = Q + kLN;
-    float* CXQ = DYB + kLN;
-    float* CYQ = CXQ + kLN;
-
+    constexpr int HALO = MODE == ST_LOCAL1 ? 2 : 3, OUT = 32 - 2 * HALO;
+    constexpr bool PRESSURE = MODE != ST_LOCAL1, LOCAL = MODE != ST_WKB1;
     const int nx = C.nx, ny = C.ny, ns = C.ns, b = blockIdx.z;
     epr_grid_wait();
     if (A.check_done && A.st[b].done) return;
     epr_grid_release();
-    const int ty0 = blockIdx.y * kLT, tx0 = blockIdx.x * kLT;
-    const int gy0 = ty0 - kLH, gx0 = tx0 - kLH;
-    const size_t npix = (size_t)nx * ny;
-    const float* Tb = A.T + (size_t)b * npix;
-    const int tid = threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const int w = (blockIdx.x * kStencilThreads + threadIdx.x) >> 5;
+    const int y0 = (w / A.strips) * A.H;
+    if (y0 >= ny) return;   // a whole warp
+    const int gx = (w % A.strips) * OUT - HALO + lane;
+    const int y1 = min(y0 + A.H, ny);   // rows y0 .. y1 - 1
+    const size_t npix = (size_t)nx * ny, pb = (size_t)b * npix;
+    const float* Tc = A.T + pb + min(max(gx, 0), nx - 1);   // this lane's column
+    const bool xl = gx <= 0, xh = gx >= nx - 1;
+    const float hsx = xl || xh ? 1.f : 0.5f;
+    const bool out = lane >= HALO && lane < 32 - HALO && gx < nx;
 
-    for (int i = tid; i < kLN; i += kLocalThreads) {
-        const int ly = i / kLE, lx = i - ly * kLE;
-        const int gy = min(max(gy0 + ly, 0), ny - 1), gx = min(max(gx0 + lx, 0), nx - 1);
-        Ts[i] = __ldg(&Tb[(size_t)gy * nx + gx]);
-    }
-    __syncthreads();
-    // gradient on the 2-pixel halo
-    for (int i = tid; i < kLN; i += kLocalThreads) {
-        const int ly = i / kLE, lx = i - ly * kLE;
-        if (ly < 1 || ly >= kLE - 1 || lx < 1 || lx >= kLE - 1) continue;
-        GX[i] = dX(Arr{Ts}, i, gx0 + lx, nx);
-        GY[i] = dY(Arr{Ts}, i, gy0 + ly, ny);
-    }
-    __syncthreads();
-
-    float pacc[kLT * kLT / kLocalThreads];
-#pragma unroll
-    for (int k = 0; k < kLT * kLT / kLocalThreads; ++k) pacc[k] = 0.f;
+    // horizontal neighbours, the edge value replicated
+    auto left = [&](float f) { const float v = __shfl_up_sync(0xffffffffu, f, 1); return xl ? f : v; };
+    auto right = [&](float f) { const float v = __shfl_down_sync(0xffffffffu, f, 1); return xh ? f : v; };
+    auto dX = [&](float f) { return (right(f) - left(f)) * hsx; };
+    auto dXX = [&](float f) { return left(f) - 2.f * f + right(f); };
+    auto dY = [&](const Rows3& f, int y) {
+        const bool lo = y == 0, hi = y == ny - 1;
+        return ((hi ? f.c : f.p) - (lo ? f.c : f.m)) * (lo || hi ? 1.f : 0.5f);
+    };
+    auto dYY = [&](const Rows3& f, int y) {
+        return (y == 0 ? f.c : f.m) - 2.f * f.c + (y == ny - 1 ? f.c : f.p);
+    };
+    auto ldT = [&](int y) { return __ldg(Tc + (size_t)min(max(y, 0), ny - 1) * nx); };
 
     for (int s = 0; s < ns; ++s) {
         const float fs = line_const(C.f, s), mus = line_const(C.mu, s);
         const float cs = line_const(C.c, s), qc = line_const(C.qc, s);
-        // fluxes I u_x, I u_y and I u_i u_j at staged index j
-        auto AX = [&](int j) { return I[j] * (cs * GX[j]); };
-        auto AY = [&](int j) { return I[j] * (cs * GY[j]); };
-        auto BXX = [&](int j) { const float ux = cs * GX[j]; return I[j] * ux * ux; };
-        auto BYY = [&](int j) { const float uy = cs * GY[j]; return I[j] * uy * uy; };
-        auto BXY = [&](int j) { return I[j] * (cs * GX[j]) * (cs * GY[j]); };
-        for (int i = tid; i < kLN; i += kLocalThreads) I[i] = fs * __expf(-mus * Ts[i]);
-        __syncthreads();
-        if constexpr (ORDER >= 2) {
-            // Q = (D_xx + D_yy) sqrt(I) / sqrt(I).  With sqrt(I) = sqrt(f) e^(-mu T / 2)
-            // each neighbour n contributes sqrt(I_n) / sqrt(I) - 1 = expm1(-mu (T_n - T) / 2)
-            // (a replicated edge neighbour contributes 0): the same quotient
-            // without the cancellation of second differences of a near-constant.
-            const float hm = -0.5f * mus;
-            for (int i = tid; i < kLN; i += kLocalThreads) {   // 1-pixel halo
-                const int ly = i / kLE, lx = i - ly * kLE;
-                if (ly < 1 || ly >= kLE - 1 || lx < 1 || lx >= kLE - 1) continue;
-                const int gx = gx0 + lx, gy = gy0 + ly;
-                const float t = Ts[i];
-                float q = 0.f;
-                if (gx > 0) q += expm1f(hm * (Ts[i - 1] - t));
-                if (gx < nx - 1) q += expm1f(hm * (Ts[i + 1] - t));
-                if (gy > 0) q += expm1f(hm * (Ts[i - kLE] - t));
-                if (gy < ny - 1) q += expm1f(hm * (Ts[i + kLE] - t));
-                Q[i] = I[i] > 0.f ? q : 0.f;
+        const float hm = -0.5f * mus;
+        // Row yl of T arrives at step yl; the fields I, u, Q and the fluxes are
+        // formed at row a = yl - 1, their first y derivatives and the flux of Q
+        // at row b = yl - 2, and the derivative of that flux at row c = yl - 3.
+        Rows3 t = {0.f, ldT(y0 - HALO), ldT(y0 - HALO + 1)};
+        Rows3 Q = {}, AY = {}, BYY = {}, BXY = {}, CYQ = {};
+        float Ib = 0.f, Ia = 0.f, Sc = 0.f, Sb = 0.f, Sa = 0.f;   // Sx: the terms known so far at row x
+        float ahead = ldT(y0 - HALO + 2), ahead2 = ldT(y0 - HALO + 3);
+#pragma unroll 3
+        for (int yl = y0 - HALO + 2; yl <= y1 - 1 + HALO; ++yl) {
+            const int a = yl - 1, bb = yl - 2;
+            t.push(ahead);   // rows a - 1, a, a + 1 after this push
+            ahead = ahead2;
+            ahead2 = ldT(yl + 2);
+            const float T0 = t.c, Tl = left(T0), Tr = right(T0);
+            const float Tu = a <= 0 ? T0 : t.m, Td = a >= ny - 1 ? T0 : t.p;
+            Ib = Ia;
+            Sc = Sb;
+            Sb = Sa;
+            Ia = fs * __expf(-mus * T0);
+            Sa = LOCAL ? Ia : 0.f;
+            if constexpr (LOCAL) {
+                const float ux = cs * ((Tr - Tl) * hsx), uy = cs * dY(t, a);
+                const float ax = Ia * ux, ay = Ia * uy;
+                AY.push(ay);
+                Sa -= dX(ax);
+                if constexpr (PRESSURE) {
+                    Sa += 0.5f * dXX(ax * ux);
+                    BYY.push(ay * uy);
+                    BXY.push(ax * uy);
+                }
+                Sb -= dY(AY, bb);
             }
-            __syncthreads();
-            for (int i = tid; i < kLN; i += kLocalThreads) {   // 2-pixel halo
-                const int ly = i / kLE, lx = i - ly * kLE;
-                if (ly < 2 || ly >= kLE - 2 || lx < 2 || lx >= kLE - 2) continue;
-                const int gx = gx0 + lx, gy = gy0 + ly;
-                DYB[i] = dY(BXY, i, gy, ny);
-                CXQ[i] = I[i] * dX(Arr{Q}, i, gx, nx);
-                CYQ[i] = I[i] * dY(Arr{Q}, i, gy, ny);
+            if constexpr (PRESSURE) {
+                // Q = (D_xx + D_yy) sqrt(I) / sqrt(I).  With sqrt(I) = sqrt(f) e^(-mu T / 2)
+                // each neighbour n contributes sqrt(I_n) / sqrt(I) - 1 = expm1(-mu (T_n - T) / 2)
+                // (a replicated edge neighbour contributes 0): the same quotient
+                // without the cancellation of second differences of a near-constant.
+                const float q = expm1_sum4(mul2(both(hm), sub2(make_float2(Tl, Tr), both(T0))),
+                                           mul2(both(hm), sub2(make_float2(Tu, Td), both(T0))));
+                Q.push(Ia > 0.f ? q : 0.f);
+                // the x derivatives of the two fluxes at row b are one
+                float fx = -qc * (Ib * dX(Q.c));
+                if constexpr (LOCAL) {
+                    Sb += 0.5f * dYY(BYY, bb);
+                    fx += dY(BXY, bb);
+                }
+                Sb += dX(fx);
+                CYQ.push(Ib * dY(Q, bb));
             }
-            __syncthreads();
+            const int yo = PRESSURE ? yl - 3 : bb;   // the row that is complete
+            const float p = PRESSURE ? Sc - qc * dY(CYQ, yo) : Sb;
+            if (!out || yo < y0 || yo >= y1) continue;
+            const size_t o = pb + (size_t)yo * nx + gx;
+            float tot = p;   // the prediction of all lines so far
+            if (s > 0) tot = A.P[o] + p;
+            else if constexpr (MODE == ST_WKB1) tot = (DET ? (float)A.Pq[o] * EPR_FX_INV : A.P[o]) + p;
+            if (ns > 1) {
+                const size_t os = pb * ns + (size_t)s * npix + (o - pb);
+                float ps = p;
+                if (A.Ps) {
+                    if constexpr (MODE == ST_WKB1) ps += DET ? (float)A.Psq[os] * EPR_FX_INV : A.Ps[os];
+                    A.Ps[os] = ps;
+                }
+            }
+            if (!A.D || s < ns - 1) {
+                A.P[o] = tot;
+                continue;
+            }
+            const float r = __ldg(&A.D[o]) - tot;
+            A.P[o] = r;
+            if (ns > 1) {   // this thread wrote every line's value of the pixel
+                const bool pos = tot > 1e-30f;
+                const float k = pos ? r / tot : r;
+                for (int l = 0; l < ns; ++l) {
+                    float* q = &A.Ps[pb * ns + (size_t)l * npix + (o - pb)];
+                    *q = k * (pos ? *q : line_const(C.f, l));
+                }
+            }
         }
-#pragma unroll
-        for (int k = 0; k < kLT * kLT / kLocalThreads; ++k) {
-            const int o = tid + k * kLocalThreads;
-            const int oy = o / kLT, ox = o - oy * kLT;
-            const int gy = ty0 + oy, gx = tx0 + ox;
-            if (gy >= ny || gx >= nx) continue;
-            const int i = (oy + kLH) * kLE + (ox + kLH);
-            float p = I[i] - dX(AX, i, gx, nx) - dY(AY, i, gy, ny);
-            if constexpr (ORDER >= 2) {
-                p += 0.5f * (dXX(BXX, i, gx, nx) + dYY(BYY, i, gy, ny)) + dX(Arr{DYB}, i, gx, nx);
-                p -= qc * (dX(Arr{CXQ}, i, gx, nx) + dY(Arr{CYQ}, i, gy, ny));
-            }
-            pacc[k] += p;
-            if (A.Ps) A.Ps[((size_t)b * ns + s) * npix + (size_t)gy * nx + gx] = p;
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int k = 0; k < kLT * kLT / kLocalThreads; ++k) {
-        const int o = tid + k * kLocalThreads;
-        const int oy = o / kLT, ox = o - oy * kLT;
-        const int gy = ty0 + oy, gx = tx0 + ox;
-        if (gy >= ny || gx >= nx) continue;
-        A.P[(size_t)b * npix + (size_t)gy * nx + gx] = pacc[k];
     }
 }
 
-// The non-local model to second order: the transport's prediction (P, P_s of
-// the splat, float or fixed point) minus the diffraction-pressure term of
-// Eq. 1 of every line, eps^2/(4 p^4) [D_x(I D_x Q) + D_y(I D_y Q)], with the
-// line's object intensity I = f_s exp(-mu_s T) at the same pixel and the
-// stencils and Q of the order-2 closure above.  Writes float P (and P_s for
-// several lines); the residual split reads them.  No atomics: the result is
-// the same on every run.
-struct Wkb1Args {
-    const float* T;
-    float* P;                        // [B][ny][nx] in (float mode) and out
-    float* Ps;                       // [B][ns][ny][nx] in/out (ns > 1)
-    const unsigned long long* Pq;    // fixed-point sums of the splat (DET)
-    const unsigned long long* Psq;
-    const EprProjState* st;
-    int check_done;
-};
-
-constexpr int kWkb1Fields = 5;   // T, I, Q, I D_x Q, I D_y Q
-
-template <bool DET>
-__global__ void __launch_bounds__(kLocalThreads) k_wkb1(const EprConsts C, const Wkb1Args A)
+template <int MODE, bool DET>
+cudaError_t launch_stencil(const EprConsts& C, StencilArgs& A, int batch, cudaStream_t stream)
 {
-    extern __shared__ __align__(16) float sm[];
-    float* Ts = sm;
-    float* I = Ts + kLN;
-    float* Q = I + kLN;
-    float* CXQ = Q + kLN;
-    float* CYQ = CXQ + kLN;
-    const int nx = C.nx, ny = C.ny, ns = C.ns, b = blockIdx.z;
-    epr_grid_wait();
-    if (A.check_done && A.st[b].done) return;
-    epr_grid_release();
-    const int ty0 = blockIdx.y * kLT, tx0 = blockIdx.x * kLT;
-    const int gy0 = ty0 - kLH, gx0 = tx0 - kLH;
-    const size_t npix = (size_t)nx * ny;
-    const float* Tb = A.T + (size_t)b * npix;
-    const int tid = threadIdx.x;
-    constexpr int KO = kLT * kLT / kLocalThreads;
-
-    for (int i = tid; i < kLN; i += kLocalThreads) {
-        const int ly = i / kLE, lx = i - ly * kLE;
-        const int gy = min(max(gy0 + ly, 0), ny - 1), gx = min(max(gx0 + lx, 0), nx - 1);
-        Ts[i] = __ldg(&Tb[(size_t)gy * nx + gx]);
-    }
-    float pacc[KO];
-#pragma unroll
-    for (int k = 0; k < KO; ++k) pacc[k] = 0.f;
-
-    for (int s = 0; s < ns; ++s) {
-        const float fs = line_const(C.f, s), mus = line_const(C.mu, s), qc = line_const(C.qc, s);
-        __syncthreads();   // Ts staged; the previous line's fields are consumed
-        for (int i = tid; i < kLN; i += kLocalThreads) I[i] = fs * __expf(-mus * Ts[i]);
-        // Q on the 1-pixel halo, as the order-2 closure forms it
-        const float hm = -0.5f * mus;
-        for (int i = tid; i < kLN; i += kLocalThreads) {
-            const int ly = i / kLE, lx = i - ly * kLE;
-            if (ly < 1 || ly >= kLE - 1 || lx < 1 || lx >= kLE - 1) continue;
-            const int gx = gx0 + lx, gy = gy0 + ly;
-            const float t = Ts[i];
-            float q = 0.f;
-            if (gx > 0) q += expm1f(hm * (Ts[i - 1] - t));
-            if (gx < nx - 1) q += expm1f(hm * (Ts[i + 1] - t));
-            if (gy > 0) q += expm1f(hm * (Ts[i - kLE] - t));
-            if (gy < ny - 1) q += expm1f(hm * (Ts[i + kLE] - t));
-            Q[i] = I[i] > 0.f ? q : 0.f;   // I[i] was written by this thread
-        }
-        __syncthreads();
-        for (int i = tid; i < kLN; i += kLocalThreads) {   // 2-pixel halo
-            const int ly = i / kLE, lx = i - ly * kLE;
-            if (ly < 2 || ly >= kLE - 2 || lx < 2 || lx >= kLE - 2) continue;
-            const int gx = gx0 + lx, gy = gy0 + ly;
-            CXQ[i] = I[i] * dX(Arr{Q}, i, gx, nx);
-            CYQ[i] = I[i] * dY(Arr{Q}, i, gy, ny);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < KO; ++k) {
-            const int o = tid + k * kLocalThreads;
-            const int oy = o / kLT, ox = o - oy * kLT;
-            const int gy = ty0 + oy, gx = tx0 + ox;
-            if (gy >= ny || gx >= nx) continue;
-            const int i = (oy + kLH) * kLE + (ox + kLH);
-            const float term = -qc * (dX(Arr{CXQ}, i, gx, nx) + dY(Arr{CYQ}, i, gy, ny));
-            pacc[k] += term;
-            if (ns > 1) {
-                const size_t o2 = ((size_t)b * ns + s) * npix + (size_t)gy * nx + gx;
-                const float ps = DET ? (float)A.Psq[o2] * EPR_FX_INV : A.Ps[o2];
-                A.Ps[o2] = ps + term;
-            }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < KO; ++k) {
-        const int o = tid + k * kLocalThreads;
-        const int oy = o / kLT, ox = o - oy * kLT;
-        const int gy = ty0 + oy, gx = tx0 + ox;
-        if (gy >= ny || gx >= nx) continue;
-        const size_t o2 = (size_t)b * npix + (size_t)gy * nx + gx;
-        const float p = DET ? (float)A.Pq[o2] * EPR_FX_INV : A.P[o2];
-        A.P[o2] = p + pacc[k];
-    }
+    constexpr int OUT = MODE == ST_LOCAL1 ? 28 : 26;
+    A.strips = (C.nx + OUT - 1) / OUT;
+    // 32 rows per strip (19 % of the rows are halo), 16 where that would leave
+    // fewer than 16 warps per SM
+    A.H = (long long)A.strips * ((C.ny + 31) / 32) * batch >= 152 * 16 ? 32 : 16;
+    const int warps = A.strips * ((C.ny + A.H - 1) / A.H);
+    const dim3 grid((warps * 32 + kStencilThreads - 1) / kStencilThreads, 1, batch);
+    const cudaError_t e = epr_launch_kernel(C.pdl != 0, k_stencil<MODE, DET>, grid, dim3(kStencilThreads), 0,
+                                            stream, C, A);
+    epr_count_launch(1);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace
 
-size_t epr_local_smem(int order) { return (size_t)local_fields(order) * kLN * sizeof(float); }
-
 // Second-order term of the non-local model, after the splat (one launch).
-// fixed_point = 1 reads the splat's integer sums.
-cudaError_t epr_launch_wkb1(const EprConsts& C, const EprWork& W, const float* T, int fixed_point,
-                            int batch, int check_done, cudaStream_t stream)
+// fixed_point = 1 reads the splat's integer sums.  With D (a solve) the
+// residual D - P and its split replace P and P_s.
+cudaError_t epr_launch_wkb1(const EprConsts& C, const EprWork& W, const float* T, const float* D,
+                            int fixed_point, int batch, int check_done, cudaStream_t stream)
 {
-    Wkb1Args A;
+    StencilArgs A = {};
     A.T = T;
+    A.D = D;
     A.P = W.P;
     A.Ps = W.Ps;
     A.Pq = W.Pq;
     A.Psq = W.Psq;
     A.st = W.st;
     A.check_done = check_done;
-    dim3 grid((C.nx + kLT - 1) / kLT, (C.ny + kLT - 1) / kLT, batch);
-    const size_t smem = (size_t)kWkb1Fields * kLN * sizeof(float);
-    const cudaError_t e =
-        fixed_point ? epr_launch_kernel(C.pdl != 0, k_wkb1<true>, grid, dim3(kLocalThreads), smem,
-                                        stream, C, A)
-                    : epr_launch_kernel(C.pdl != 0, k_wkb1<false>, grid, dim3(kLocalThreads), smem,
-                                        stream, C, A);
-    epr_count_launch(1);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return fixed_point ? launch_stencil<ST_WKB1, true>(C, A, batch, stream)
+                       : launch_stencil<ST_WKB1, false>(C, A, batch, stream);
 }
 
-cudaError_t epr_launch_local(const EprConsts& C, const EprWork& W, const float* T, float* P,
+// The local closure of order 1 or 2 (one launch); D as above.
+cudaError_t epr_launch_local(const EprConsts& C, const EprWork& W, const float* T, const float* D, float* P,
                              float* Ps, int order, int batch, int check_done, cudaStream_t stream)
 {
-    LocalArgs A;
+    StencilArgs A = {};
     A.T = T;
+    A.D = D;
     A.P = P;
     A.Ps = Ps;
     A.st = W.st;
-    A.order = order;
     A.check_done = check_done;
-    dim3 grid((C.nx + kLT - 1) / kLT, (C.ny + kLT - 1) / kLT, batch);
-    const cudaError_t e =
-        order >= 2 ? epr_launch_kernel(C.pdl != 0, k_local<2>, grid, dim3(kLocalThreads),
-                                       epr_local_smem(2), stream, C, A)
-                   : epr_launch_kernel(C.pdl != 0, k_local<1>, grid, dim3(kLocalThreads),
-                                       epr_local_smem(1), stream, C, A);
-    epr_count_launch(1);
-    return e != cudaSuccess ? e : cudaGetLastError();
-}
-
-cudaError_t epr_local_init()
-{
-    cudaError_t e = epr_allow_max_smem(k_local<1>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_local<2>);
-    if (e == cudaSuccess) e = epr_allow_max_smem(k_wkb1<false>);
-    return e != cudaSuccess ? e : epr_allow_max_smem(k_wkb1<true>);
+    return order >= 2 ? launch_stencil<ST_LOCAL2, false>(C, A, batch, stream)
+                      : launch_stencil<ST_LOCAL1, false>(C, A, batch, stream);
 }
