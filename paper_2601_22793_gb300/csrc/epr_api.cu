@@ -28,16 +28,13 @@
 
 // --- launchers from the other translation units -----------------------------
 cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* T, const float* D,
-                             int resid, int parity, int batch, int TH, int TW, int check_done,
-                             cudaStream_t stream);
+                             int parity, int batch, int TH, int TW, int check_done, cudaStream_t stream);
 size_t epr_splat_smem(const EprConsts& C, int TH, int TW);
 bool epr_splat_has_occ6(int TH, int TW, int reach);
 cudaError_t epr_splat_init();
 cudaError_t epr_launch_row_fwd(const EprConsts& C, const EprWork& W, int mode, const float* T,
                                const float* D, const float* G, int line0, int nl, int it,
                                float tol, int batch, int check_done, cudaStream_t stream);
-cudaError_t epr_launch_split(const EprConsts& C, const EprWork& W, const float* D, int batch,
-                             int fixed_point, int check_done, cudaStream_t stream);
 cudaError_t epr_launch_solve_begin(const EprConsts& C, const EprWork& W, const float* D, float* T,
                                    int batch, size_t npd, size_t npix, double scale,
                                    cudaStream_t stream);
@@ -265,6 +262,9 @@ epr_status ensure_workspace(epr_plan_s* p, int batch, int hist)
     if (e == cudaSuccess) e = dalloc(p, &W.ovf_idx, (size_t)nb * C.ovf_cap);
     if (e == cudaSuccess) e = dalloc(p, &W.ovf_mask, (size_t)nb * C.ovf_cap);
     if (e == cudaSuccess) e = dalloc(p, &W.ovf_tg, (size_t)nb * C.ovf_cap);
+    const size_t nclaim = C.ns > 1 && !C.det ? ((size_t)nb * npix + 31) / 32 : 0;
+    if (e == cudaSuccess && nclaim) e = dalloc(p, &W.claim, nclaim);
+    if (e == cudaSuccess && nclaim) e = cudaMemset(W.claim, 0, nclaim * sizeof(unsigned int));
     if (e == cudaSuccess) e = dalloc(p, &W.st, (size_t)nb);
     if (e == cudaSuccess) e = dalloc(p, &W.part_a, (size_t)nb * W.max_blocks);
     if (e == cudaSuccess) e = dalloc(p, &W.part_b, (size_t)nb * W.max_blocks);
@@ -399,8 +399,8 @@ void splat_tile(const epr_plan_s* p, int batch, int* TH, int* TW)
 }
 
 // One pass of the chosen forward model writing W.P (and W.Ps / W.Pq / W.Psq).
-// With D given W.P receives D - P instead of P (monochromatic float solve),
-// and the local and second-order models split it over the lines in W.Ps.
+// With D given (a solve on the detector grid) W.P receives the residual D - P
+// instead of P, and W.Ps its split over several lines.
 epr_status launch_forward(epr_plan_s* p, const EprWork& W, const float* T, const float* D, int parity,
                           int batch, int model, int check_done, cudaStream_t s)
 {
@@ -409,8 +409,8 @@ epr_status launch_forward(epr_plan_s* p, const EprWork& W, const float* T, const
             ProfScope ps(p, EPR_KERNEL_SPLAT, s);
             int TH, TW;
             splat_tile(p, batch, &TH, &TW);
-            const bool resid = D && model == EPR_MODEL_NONLOCAL;
-            EPR_TRY(epr_launch_splat(p->C, W, T, D, resid, parity, batch, TH, TW, check_done, s));
+            EPR_TRY(epr_launch_splat(p->C, W, T, model == EPR_MODEL_NONLOCAL ? D : nullptr, parity, batch, TH,
+                                     TW, check_done, s));
         }
         if (model == EPR_MODEL_NONLOCAL_WKB1) {   // second-order term: float P, P_s after it
             ProfScope ps(p, EPR_KERNEL_LOCAL, s);
@@ -443,22 +443,17 @@ epr_status launch_solve(epr_plan_s* p, const float* D, float* T, int batch, cons
     // with the identity
     const bool nonlocal = model == EPR_MODEL_NONLOCAL || model == EPR_MODEL_NONLOCAL_WKB1;
     const int fwd_mode = nonlocal ? 0 : 1;
-    // the residual D - P (and its split over the lines) is stored by the
-    // splat flush (plain non-local model, one line, float accumulation), by
-    // the stencil kernel of the local and second-order models, or by the split
-    // kernel after the forward (several lines, fixed point, oversampling)
-    const bool nl = model == EPR_MODEL_NONLOCAL;   // P still in the splat's own format
-    const bool resid_in_forward = C.os == 1 && (!nl || (C.ns == 1 && !C.det && !C.xt));
+    // the residual D - P and its split over the lines are stored by the splat
+    // or the stencil kernel; an oversampled solve forms them at detector
+    // resolution after the forward
+    const float* Dfwd = C.os == 1 ? D : nullptr;
     const float eps = (float)(o->eps_I > 0 ? o->eps_I : 1e-8);
     for (int it = 0; it < o->n_iter; ++it) {
-        epr_status st = launch_forward(p, p->W, T, resid_in_forward ? D : nullptr, it & 1, batch, model, 1, s);
+        epr_status st = launch_forward(p, p->W, T, Dfwd, it & 1, batch, model, 1, s);
         if (st != EPR_OK) return st;
         if (C.os > 1) {
             ProfScope ps(p, EPR_KERNEL_OTHER, s);
-            EPR_TRY(epr_launch_split_os(C, p->W, D, batch, nl && C.det, 1, s));
-        } else if (!resid_in_forward) {
-            ProfScope ps(p, EPR_KERNEL_OTHER, s);
-            EPR_TRY(epr_launch_split(C, p->W, D, batch, C.det, 1, s));
+            EPR_TRY(epr_launch_split_os(C, p->W, D, batch, model == EPR_MODEL_NONLOCAL && C.det, 1, s));
         }
         {
             ProfScope ps(p, EPR_KERNEL_ROW_FWD, s);
@@ -532,6 +527,7 @@ epr_status autotune_splat(epr_plan_s* p, const float* D, const float* T, int bat
 {
     p->tuned = true;
     const bool resid = p->C.ns == 1 && !p->C.det && p->C.os == 1 && !p->C.xt;
+    const float* Dfwd = p->C.os == 1 ? D : nullptr;   // as the solve runs it
     const int tiles[4][2] = {{64, 64}, {32, 64}, {64, 32}, {32, 32}};
     // the compile-time reaches, and the plan's own when it is none of them
     const int own = p->C.smax;
@@ -556,13 +552,13 @@ epr_status autotune_splat(epr_plan_s* p, const float* D, const float* T, int bat
             p->splat_TW = t[1];
             p->W.splat_occ6 = occ6;
             EPR_TRY(cudaMemsetAsync(p->W.st, 0, (size_t)batch * sizeof(EprProjState), s));
-            epr_status st = launch_forward(p, p->W, T, resid ? D : nullptr, 0, batch, EPR_MODEL_NONLOCAL, 0, s);
+            epr_status st = launch_forward(p, p->W, T, Dfwd, 0, batch, EPR_MODEL_NONLOCAL, 0, s);
             if (st != EPR_OK) return st;
             float ms = 1e30f;   // the fastest of three repetitions of four forwards
             for (int rep = 0; rep < 3; ++rep) {
                 EPR_TRY(cudaEventRecord(e0, s));
                 for (int k = 0; k < 4; ++k) {
-                    st = launch_forward(p, p->W, T, resid ? D : nullptr, (k + 1) & 1, batch, EPR_MODEL_NONLOCAL,
+                    st = launch_forward(p, p->W, T, Dfwd, (k + 1) & 1, batch, EPR_MODEL_NONLOCAL,
                                         0, s);
                     if (st != EPR_OK) return st;
                 }
@@ -775,12 +771,10 @@ epr_status solve_common(epr_plan_s* p, const float* D, float* T, int batch, int 
     if (p->opt.autotune && !p->tuned && model == EPR_MODEL_NONLOCAL && o->n_iter > 0) {
         st = autotune_splat(p, Dd, Td, batch, s);
         if (st != EPR_OK) return st;
-        // the column pass is timed on the residual of a plain forward (the
-        // monochromatic float solve's splat stores it in P; with several
-        // lines the split after the last forward of the splat tuner).  Not
-        // in fixed-point mode, whose results stay those of the default plan.
+        // the column pass is timed on the residual that the splat tuner's last
+        // forward left.  Not in fixed-point mode, whose results stay those of
+        // the default plan.
         if (p->C.os == 1 && !p->C.xt && !p->C.det) {
-            if (p->C.ns > 1) EPR_TRY(epr_launch_split(p->C, p->W, Dd, batch, 0, 0, s));
             st = autotune_col(p, Dd, Td, batch, s);
             if (st != EPR_OK) return st;
         }

@@ -79,6 +79,8 @@ struct EprWork {
     int* ovf_idx;        // [B][cap] source pixel index
     unsigned int* ovf_mask;   // [B][cap] lines that took the overflow path
     float4* ovf_tg;      // [B][cap] T and twice its gradient (x, y) at the source
+    unsigned int* claim; // [B ny nx / 32] pixels that long shifts reached, 0 between
+                         //    kernels (float mode, ns > 1)
     EprProjState* st;    // [B]
     double* part_a;      // [B][max_blocks] block partial sums of the inverse
     double* part_b;      // [B][max_blocks]    row pass (kappa)

@@ -7,16 +7,64 @@ namespace {
 
 using namespace eprsplat;
 
+// What the long-shift pass adds a contribution to.
+//   FAR_MODEL  P and P_s (a forward), float
+//   FAR_RESID  the residual D - P of one line (negative), float
+//   FAR_SPLIT  the split residuals r_s of several lines, float (see far_scale)
+//   FAR_FX     the fixed-point sums
+enum { FAR_MODEL = 0, FAR_RESID = 1, FAR_SPLIT = 2, FAR_FX = 3 };
+
+// Every corner pixel o on the grid, line s and contribution v of a list entry.
+template <bool XT, class F>
+__device__ __forceinline__ void far_corners(const EprConsts& C, int pix, unsigned int mask, float4 tg, F f)
+{
+    const int nx = C.nx, ny = C.ny;
+    const int sy = pix / nx, sx = pix - sy * nx;
+    const float t = tg.x;
+    for (int s = 0; s < C.ns; ++s) {
+        if (!((mask >> s) & 1u)) continue;
+        const float ch = 0.5f * (XT ? xt_get(C, EPR_XT_C, s, sx) : C.c[s]);
+        const float ux = ch * tg.y, uy = ch * tg.z;
+        const float fx = floorf(ux), fy = floorf(uy);
+        const float dx = ux - fx, dy = uy - fy;
+        const float fs = XT ? xt_get(C, EPR_XT_F, s, sx) : C.f[s];
+        const float mus = XT ? xt_get(C, EPR_XT_MU, s, sx) : C.mu[s];
+        const float m = fs * __expf(-mus * t);
+        const float w[4] = {(1.f - dx) * (1.f - dy), dx * (1.f - dy), (1.f - dx) * dy, dx * dy};
+        // corner coordinates in float first: a huge shift must not wrap an int
+        const float cxf = (float)sx + fx, cyf = (float)sy + fy;
+        for (int k = 0; k < 4; ++k) {
+            const float xf = cxf + (float)(k & 1), yf = cyf + (float)(k >> 1);
+            if (!(xf >= 0.f && xf < (float)nx && yf >= 0.f && yf < (float)ny)) continue;
+            f((size_t)(int)yf * nx + (int)xf, s, m * w[k]);
+        }
+    }
+}
+
+// The scale in which a pixel's split residuals hold its line predictions.
+// The splat flush of a several-line float solve stores r = D - P and r_s =
+// P_s k with k = r / P (never 0), so P_s = r_s / k, and P comes back as D - r.
+// Where no near source reaches the pixel (P = 0) r_s is r f_s; a contribution
+// is then added 2^20 times, which keeps its digits above those of r f_s.
+constexpr float kDarkScale = 1048576.f;
+__device__ __forceinline__ float far_scale(float d, float r, bool& lit)
+{
+    const float p = d - r;
+    lit = p > 1e-30f;
+    return lit ? split_ratio(r, p) : kDarkScale;
+}
+
 // The long-shift sources of the overflow list, added with global atomics.
-template <bool DET, bool RESID, bool XT = false>
-__global__ void __launch_bounds__(128) k_splat_overflow(const EprConsts C, const SplatArgs A)
+// FAR_SPLIT marks every pixel it touches in `claim` for k_overflow_fix.
+template <int TO, bool XT = false>
+__global__ void __launch_bounds__(128) k_splat_overflow(const __grid_constant__ EprConsts C, const SplatArgs A)
 {
     const int b = blockIdx.y;
     epr_grid_wait();
     if (A.check_done && A.st[b].done) return;
     epr_grid_release();
-    const int nx = C.nx, ny = C.ny, ns = C.ns;
-    const size_t npix = (size_t)nx * ny;
+    const int ns = C.ns;
+    const size_t npix = (size_t)C.nx * C.ny, pb = (size_t)b * npix;
     const int cnt_raw = A.st[b].ovf_count[A.parity];
     const int cnt = cnt_raw < C.ovf_cap ? cnt_raw : C.ovf_cap;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -41,104 +89,75 @@ __global__ void __launch_bounds__(128) k_splat_overflow(const EprConsts C, const
             mask = A.ovf_mask[(size_t)b * C.ovf_cap + e];
             tg = A.ovf_tg[(size_t)b * C.ovf_cap + e];
         }
-        const int sy = pix / nx, sx = pix - sy * nx;
-        const float t = tg.x;
-        for (int s = 0; s < ns; ++s) {
-            if (!((mask >> s) & 1u)) continue;
-            const float ch = 0.5f * (XT ? xt_get(C, EPR_XT_C, s, sx) : C.c[s]);
-            const float ux = ch * tg.y, uy = ch * tg.z;
-            const float fx = floorf(ux), fy = floorf(uy);
-            const float dx = ux - fx, dy = uy - fy;
-            const float fs = XT ? xt_get(C, EPR_XT_F, s, sx) : C.f[s];
-            const float mus = XT ? xt_get(C, EPR_XT_MU, s, sx) : C.mu[s];
-            const float m = fs * __expf(-mus * t);
-            const float w[4] = {(1.f - dx) * (1.f - dy), dx * (1.f - dy), (1.f - dx) * dy, dx * dy};
-            // corner coordinates in float first: a huge shift must not wrap an int
-            const float cxf = (float)sx + fx, cyf = (float)sy + fy;
-            for (int k = 0; k < 4; ++k) {
-                const float xf = cxf + (float)(k & 1), yf = cyf + (float)(k >> 1);
-                if (!(xf >= 0.f && xf < (float)nx && yf >= 0.f && yf < (float)ny)) continue;
-                const size_t o = (size_t)(int)yf * nx + (int)xf;
-                const float v = m * w[k];
-                if constexpr (DET) {
-                    const unsigned long long q = (unsigned long long)__float2ll_rn(v * EPR_FX_SCALE);
-                    atomicAdd(&A.Pq[(size_t)b * npix + o], q);
-                    if (ns > 1) atomicAdd(&A.Psq[((size_t)b * ns + s) * npix + o], q);
-                } else if constexpr (RESID) {
-                    atomicAdd(&A.P[(size_t)b * npix + o], -v);
-                } else {
-                    atomicAdd(&A.P[(size_t)b * npix + o], v);
-                    if (ns > 1 && A.Ps) atomicAdd(&A.Ps[((size_t)b * ns + s) * npix + o], v);
-                }
+        far_corners<XT>(C, pix, mask, tg, [&](size_t o, int s, float v) {
+            const size_t po = pb + o, ps = pb * ns + (size_t)s * npix + o;
+            if constexpr (TO == FAR_FX) {
+                const unsigned long long q = (unsigned long long)__float2ll_rn(v * EPR_FX_SCALE);
+                atomicAdd(&A.Pq[po], q);
+                if (ns > 1) atomicAdd(&A.Psq[ps], q);
+            } else if constexpr (TO == FAR_RESID) {
+                atomicAdd(&A.P[po], -v);
+            } else if constexpr (TO == FAR_SPLIT) {
+                bool lit;
+                const float k = far_scale(__ldg(&A.D[po]), A.P[po], lit);
+                atomicAdd(&A.Ps[ps], v * k);
+                atomicOr(&A.claim[po >> 5], 1u << (po & 31));
+            } else {
+                atomicAdd(&A.P[po], v);
+                if (ns > 1 && A.Ps) atomicAdd(&A.Ps[ps], v);
             }
-        }
+        });
     }
 }
 
-// The residual and its split over the lines (the weights P_s / P of the
-// "Iteration structure"; r f_s where P vanishes), once per pixel after the
-// overflow sources are in: P <- D - P and P_s <- (D - P) P_s / P as float
-// maps, so that the adjoint gather reads one value per corner and line.  In
-// fixed-point mode the sums are read from the integer maps.
-//
-// Bound by memory (12 + 8 n_s bytes per pixel in float mode): four pixels per
-// thread, every line's P_s loaded before any r_s is stored (the stores could
-// alias the later loads as far as the compiler knows, which would serialise
-// one memory round trip per line).  The line count is bounded at compile time
-// by NSM, so the loads of 4 or 8 lines leave registers for enough warps, and r / P is
-// formed once per pixel: eight lines of a 2048^2 map 57 us with a division per
-// line and room for 16.
-template <bool DET>
-__device__ __forceinline__ float4 split_load(const float* f, const unsigned long long* q, size_t i)
-{
-    if constexpr (DET) {
-        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(q + i);
-        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(q + i + 2);
-        return make_float4((float)a.x * EPR_FX_INV, (float)a.y * EPR_FX_INV, (float)b.x * EPR_FX_INV,
-                           (float)b.y * EPR_FX_INV);
-    } else {
-        return *reinterpret_cast<const float4*>(f + i);
-    }
-}
-
-template <bool DET, bool XT, int NSM>
-__global__ void __launch_bounds__(256) k_split(const EprConsts C, const SplatArgs A)
+// The residual and its split at the pixels that long-shift sources reached,
+// once they are all in: r = D - P and r_s = r P_s / P (r f_s where P
+// vanishes).  Fixed point forms them anew from the sums (every visitor of a
+// pixel writes the same values); float turns the pixel's split residuals back
+// into P_s, by the one visitor that takes its claim bit.  A few thousand
+// pixels instead of a pass over every map: the separate split of eight lines
+// of a 2048^2 map took 46 us.
+template <bool DET, bool XT = false>
+__global__ void __launch_bounds__(128) k_overflow_fix(const __grid_constant__ EprConsts C, const SplatArgs A)
 {
     const int b = blockIdx.y;
+    const int ns = C.ns, nx = C.nx;
+    const size_t npix = (size_t)nx * C.ny, pb = (size_t)b * npix;
+    // the list is the splat's, complete before the long-shift pass began
+    const int cnt_raw = A.st[b].ovf_count[A.parity];
+    const int cnt = cnt_raw < C.ovf_cap ? cnt_raw : C.ovf_cap;
     epr_grid_wait();
     if (A.check_done && A.st[b].done) return;
     epr_grid_release();
-    const int ns = C.ns;
-    const size_t npix = (size_t)C.nx * C.ny, pb = (size_t)b * npix;
-    // nx % 4 == 0: four pixels of one row per thread
-    for (size_t q4 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q4 < npix / 4;
-         q4 += (size_t)gridDim.x * blockDim.x) {
-        const size_t q = 4 * q4;
-        const float4 d = __ldg(reinterpret_cast<const float4*>(A.D + pb + q));
-        const float4 p = split_load<DET>(A.P, A.Pq, pb + q);
-        float4 pl[NSM];
-#pragma unroll
-        for (int s = 0; s < NSM; ++s)
-            if (s < ns && ns > 1) pl[s] = split_load<DET>(A.Ps, A.Psq, pb * ns + (size_t)s * npix + q);
-        const float4 r = make_float4(d.x - p.x, d.y - p.y, d.z - p.z, d.w - p.w);
-        const bool bx = p.x > 1e-30f, by = p.y > 1e-30f, bz = p.z > 1e-30f, bw = p.w > 1e-30f;
-        const float4 k = make_float4(bx ? r.x / p.x : r.x, by ? r.y / p.y : r.y, bz ? r.z / p.z : r.z,
-                                     bw ? r.w / p.w : r.w);
-        const int x = XT ? (int)(q % (size_t)C.nx) : 0;
-#pragma unroll
-        for (int s = 0; s < NSM; ++s) {
-            if (!(s < ns && ns > 1)) continue;
-            float4 f;
-            if constexpr (XT)
-                f = make_float4(xt_get(C, EPR_XT_F, s, x), xt_get(C, EPR_XT_F, s, x + 1),
-                                xt_get(C, EPR_XT_F, s, x + 2), xt_get(C, EPR_XT_F, s, x + 3));
-            else
-                f = make_float4(C.f[s], C.f[s], C.f[s], C.f[s]);
-            *reinterpret_cast<float4*>(A.Ps + pb * ns + (size_t)s * npix + q) =
-                make_float4(k.x * (bx ? pl[s].x : f.x), k.y * (by ? pl[s].y : f.y),
-                            k.z * (bz ? pl[s].z : f.z), k.w * (bw ? pl[s].w : f.w));
-        }
-        *reinterpret_cast<float4*>(A.P + pb + q) = r;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < cnt; e += gridDim.x * blockDim.x) {
+        const size_t at = (size_t)b * C.ovf_cap + e;
+        far_corners<XT>(C, A.ovf_idx[at], A.ovf_mask[at], A.ovf_tg[at], [&](size_t o, int, float) {
+            const size_t po = pb + o, ps = pb * ns + o;
+            const int x = XT ? (int)(o % (size_t)nx) : 0;
+            auto weight = [&](int l) { return XT ? xt_get(C, EPR_XT_F, l, x) : C.f[l]; };
+            const float d = __ldg(&A.D[po]);
+            float p = 0.f;
+            if constexpr (DET) {
+                p = (float)A.Pq[po] * EPR_FX_INV;
+                const float r = d - p, k = p > 1e-30f ? split_ratio(r, p) : r;
+                for (int l = 0; ns > 1 && l < ns; ++l)
+                    A.Ps[ps + l * npix] = k * (p > 1e-30f ? (float)A.Psq[ps + l * npix] * EPR_FX_INV : weight(l));
+                A.P[po] = r;
+            } else {
+                const unsigned int bit = 1u << (po & 31);
+                if (!(atomicAnd(&A.claim[po >> 5], ~bit) & bit)) return;   // another visitor's
+                bool lit;
+                const float r0 = A.P[po], k0 = far_scale(d, r0, lit);
+                auto line = [&](int l) {   // P_s with the long-shift contributions
+                    const float v = A.Ps[ps + l * npix];
+                    return lit ? v / k0 : fmaxf((v - r0 * weight(l)) * (1.f / kDarkScale), 0.f);
+                };
+                for (int l = 0; l < ns; ++l) p += line(l);
+                const float r = d - p, k = p > 1e-30f ? split_ratio(r, p) : r;
+                for (int l = 0; l < ns; ++l) A.Ps[ps + l * npix] = k * (p > 1e-30f ? line(l) : weight(l));
+                A.P[po] = r;
+            }
+        });
     }
 }
 
@@ -316,12 +335,13 @@ size_t epr_splat_smem(const EprConsts& C, int TH, int TW)
     return ((acc_bytes + 15) & ~size_t(15)) + (size_t)SH * (TW + 2 * HX) * sizeof(float);
 }
 
-// Host launcher: the tile kernel, then the overflow kernel (2 launches).
-// resid = 1 (mono float only): P receives D - P.  `parity` alternates the
-// overflow counter slot between consecutive splats of a solve.
+// Host launcher: the tile kernel, then the long-shift pass.  With D (a solve
+// on the detector grid) P receives D - P, P_s the split residuals, and where
+// the split needs the whole prediction of a pixel (several lines, fixed
+// point) a third launch redoes the pixels that long shifts reached.  `parity`
+// alternates the overflow counter slot between consecutive splats of a solve.
 cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* T, const float* D,
-                             int resid, int parity, int batch, int TH, int TW, int check_done,
-                             cudaStream_t stream)
+                             int parity, int batch, int TH, int TW, int check_done, cudaStream_t stream)
 {
     SplatArgs A;
     A.T = T;
@@ -335,6 +355,7 @@ cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* 
     A.ovf_tg = W.ovf_tg;
     A.st = W.st;
     A.err = W.err;
+    A.claim = W.claim;
     A.parity = parity & 1;
     A.check_done = check_done;
     {   // 2^(32 - S) >= 2 (2 reach + 3)^2: the largest pixel sum fits in uint32
@@ -357,6 +378,7 @@ cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* 
     const size_t smem = epr_splat_smem(C, TH, TW);
     dim3 grid((C.nx + TW - 1) / TW, (C.ny + TH - 1) / TH, batch);
     const bool occ6 = W.splat_occ6 != 0;
+    const int resid = D && C.ns == 1 && !C.det && !C.xt;   // its own kernels
     cudaError_t e;
     if (TH == 64 && TW == 64) e = epr_splat_launch_64x64(C, A, resid, occ6, grid, smem, stream);
     else if (TH == 32 && TW == 64) e = epr_splat_launch_32x64(C, A, resid, occ6, grid, smem, stream);
@@ -364,15 +386,32 @@ cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* 
     else if (TH == 32 && TW == 32) e = epr_splat_launch_32x32(C, A, resid, occ6, grid, smem, stream);
     else return cudaErrorInvalidValue;
     if (e != cudaSuccess) return e;
-    auto overflow = [&](auto kernel) {
+    auto go = [&](auto kernel) {
+        if (e != cudaSuccess) return;
         e = epr_launch_kernel(C.pdl != 0, kernel, dim3(128, batch), dim3(128), 0, stream, C, A);
+        epr_count_launch(1);
     };
-    if (C.det && C.xt) overflow(k_splat_overflow<true, false, true>);
-    else if (C.det) overflow(k_splat_overflow<true, false>);
-    else if (C.xt) overflow(k_splat_overflow<false, false, true>);
-    else if (resid && C.ns == 1) overflow(k_splat_overflow<false, true>);
-    else overflow(k_splat_overflow<false, false>);
-    epr_count_launch(2);
+    epr_count_launch(1);
+    if (C.det) {
+        if (C.xt) go(k_splat_overflow<FAR_FX, true>);
+        else go(k_splat_overflow<FAR_FX>);
+        if (D && C.xt) go(k_overflow_fix<true, true>);
+        else if (D) go(k_overflow_fix<true>);
+    } else if (resid) {
+        go(k_splat_overflow<FAR_RESID>);
+    } else if (D) {
+        if (C.xt) {
+            go(k_splat_overflow<FAR_SPLIT, true>);
+            go(k_overflow_fix<false, true>);
+        } else {
+            go(k_splat_overflow<FAR_SPLIT>);
+            go(k_overflow_fix<false>);
+        }
+    } else if (C.xt) {
+        go(k_splat_overflow<FAR_MODEL, true>);
+    } else {
+        go(k_splat_overflow<FAR_MODEL>);
+    }
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -383,41 +422,6 @@ cudaError_t epr_splat_init()
     if (e == cudaSuccess) e = epr_splat_init_64x32();
     if (e == cudaSuccess) e = epr_splat_init_32x32();
     return e;
-}
-
-// Residual split after the forward of a solve: fixed_point = 1 reads the
-// integer sums of the fixed-point splat, 0 the float maps (float splat,
-// local closure).
-cudaError_t epr_launch_split(const EprConsts& C, const EprWork& W, const float* D, int batch,
-                             int fixed_point, int check_done, cudaStream_t stream)
-{
-    SplatArgs A = {};
-    A.D = D;
-    A.P = W.P;
-    A.Ps = W.Ps;
-    A.Pq = W.Pq;
-    A.Psq = W.Psq;
-    A.st = W.st;
-    A.check_done = check_done;
-    const size_t n4 = (size_t)C.nx * C.ny / 4;
-    size_t blocks = (n4 + 255) / 256;
-    if (blocks > 1216) blocks = 1216;   // 8 per SM on 152 SMs, grid-stride beyond
-    cudaError_t e = cudaSuccess;
-    auto go = [&](auto kernel) {
-        e = epr_launch_kernel(C.pdl != 0, kernel, dim3((unsigned)blocks, batch), dim3(256), 0, stream, C, A);
-    };
-    auto by_lines = [&](auto det, auto xt) {
-        constexpr bool DET = decltype(det)::value, XT = decltype(xt)::value;
-        if (C.ns <= 4) go(k_split<DET, XT, 4>);
-        else if (C.ns <= 8) go(k_split<DET, XT, 8>);
-        else go(k_split<DET, XT, 16>);
-    };
-    if (C.xt && fixed_point) by_lines(std::true_type{}, std::true_type{});
-    else if (C.xt) by_lines(std::false_type{}, std::true_type{});
-    else if (fixed_point) by_lines(std::true_type{}, std::false_type{});
-    else by_lines(std::false_type{}, std::false_type{});
-    epr_count_launch(1);
-    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // Oversampled solve: the split at detector resolution (k_split_os).

@@ -33,9 +33,12 @@
 //    S = 24: a rounding error of at most 3e-8 per contribution, half an fp32
 //    ulp of a unit intensity.
 //  * Every destination pixel is written exactly once, with plain coalesced
-//    stores: no zero fill and no global atomics on the fast path.  In the
-//    monochromatic float solve the flush stores the residual D - P instead
-//    of P (the adjoint gather then reads one value per corner).
+//    stores: no zero fill and no global atomics on the fast path.  In a solve
+//    on the detector grid the flush stores the residual D - P instead of P
+//    and, for several lines, its split r_s = r P_s / P instead of P_s (the
+//    adjoint gather then reads one value per corner), so no pass over the maps
+//    is left between the splat and the gather; the pixels that long-shift
+//    sources reach afterwards are redone one by one (splat.cu).
 //  * A source-line with |u| > reach in either axis (or T below the bound
 //    above) is never splatted by the scan; the block that owns the source
 //    pixel appends it (with a bit mask of its long lines, its thickness and
@@ -63,7 +66,8 @@ struct SplatArgs {
     const float* T;          // [B][ny][nx]
     const float* D;          // [B][ny][nx] (residual output)
     float* P;                // [B][ny][nx]   P, or D - P (residual output)
-    float* Ps;               // [B][ns][ny][nx] or NULL: not wanted (float mode, ns > 1)
+    float* Ps;               // [B][ns][ny][nx] P_s, or r_s (residual output), or NULL:
+                             //    not wanted (float mode, ns > 1)
     unsigned long long* Pq;  // fixed-point mode
     unsigned long long* Psq;
     int* ovf_idx;
@@ -71,6 +75,7 @@ struct SplatArgs {
     float4* ovf_tg;          // (T, twice the gradient x, y, 0) of each entry
     EprProjState* st;
     unsigned int* err;
+    unsigned int* claim;     // [B ny nx / 32] bits, all 0 between solves (float mode, ns > 1)
     int parity;
     int check_done;
     float fxs, fxs_inv;      // float mode: scale 2^S of the uint32 accumulators
@@ -82,6 +87,14 @@ struct SplatArgs {
 constexpr int kFarList = 256;
 constexpr int kQuad = 4;   // sources per scan work item
 constexpr int kAccX = 4;   // accumulator column of tile column 0 (16-byte aligned rows)
+
+// r / P of the residual split, never 0, so that P_s stays recoverable from
+// r_s = P_s r / P (a residual below 1e-20 of P is one of 1e-20)
+__device__ __forceinline__ float split_ratio(float r, float p)
+{
+    const float k = r / p;
+    return fabsf(k) < 1e-20f ? 1e-20f : k;
+}
 
 }  // namespace eprsplat
 
@@ -226,7 +239,8 @@ k_splat(const __grid_constant__ EprConsts C, const SplatArgs A)
     constexpr int kDq = 4;   // float4 per thread: tiles up to 64 x 64
     constexpr int nq = tile >> 2;
     constexpr int tw4 = TW >> 2;
-    if constexpr (RESID) {
+    const bool split = !RESID && A.D != nullptr;   // a solve with several lines or in fixed point
+    if (RESID || split) {
         constexpr int kLine = TW / 32;   // 128-byte lines of a row
         if (tid < TH * kLine) {
             const int gy = ty0 + tid / kLine, gx = tx0 + 32 * (tid % kLine);
@@ -417,7 +431,7 @@ k_splat(const __grid_constant__ EprConsts C, const SplatArgs A)
     if (interior) scan(std::true_type{});
     else scan(std::false_type{});
     float4 dreg[kDq];
-    if constexpr (RESID) {   // under way while the block meets at the barrier
+    if (RESID || (split && !DET)) {   // under way while the block meets at the barrier
 #pragma unroll
         for (int k = 0; k < kDq; ++k) {
             const int i4 = tid + k * kSplatThreads;
@@ -466,8 +480,8 @@ k_splat(const __grid_constant__ EprConsts C, const SplatArgs A)
         const uint4* a = reinterpret_cast<const uint4*>(acc);
         const float inv = A.fxs_inv;
 #pragma unroll
-        for (int k = 0; k < kDq; ++k) {
-            const int i4 = tid + k * kSplatThreads;
+        for (int kk = 0; kk < kDq; ++kk) {
+            const int i4 = tid + kk * kSplatThreads;
             if (i4 >= nq) continue;
             const int ly = i4 / tw4, lx = (i4 - ly * tw4) << 2;
             const int gy = ty0 + ly, gx = tx0 + lx;
@@ -476,7 +490,7 @@ k_splat(const __grid_constant__ EprConsts C, const SplatArgs A)
             const int i0 = ((ly + 1) * AP + lx + kAccX) >> 2;
             if constexpr (RESID) {
                 const uint4 v = a[i0];
-                const float4 d = dreg[k];
+                const float4 d = dreg[kk];
                 *reinterpret_cast<float4*>(A.P + o) =
                     make_float4(d.x - (float)v.x * inv, d.y - (float)v.y * inv,
                                 d.z - (float)v.z * inv, d.w - (float)v.w * inv);
@@ -486,12 +500,31 @@ k_splat(const __grid_constant__ EprConsts C, const SplatArgs A)
                 for (int s = 0; s < ns; ++s) {
                     const uint4 v = a[s * (ACC / 4) + i0];
                     sum = make_uint4(sum.x + v.x, sum.y + v.y, sum.z + v.z, sum.w + v.w);
-                    if (ns > 1 && A.Ps)
-                        *reinterpret_cast<float4*>(A.Ps + (size_t)s * npix + o + (size_t)b * (ns - 1) * npix) =
-                            make_float4((float)v.x * inv, (float)v.y * inv, (float)v.z * inv, (float)v.w * inv);
                 }
-                *reinterpret_cast<float4*>(A.P + o) = make_float4((float)sum.x * inv, (float)sum.y * inv,
-                                                                  (float)sum.z * inv, (float)sum.w * inv);
+                float4 p = make_float4((float)sum.x * inv, (float)sum.y * inv, (float)sum.z * inv,
+                                       (float)sum.w * inv);
+                // what the lines' values are multiplied by: 1, or r / P
+                float4 k = make_float4(1.f, 1.f, 1.f, 1.f);
+                const bool bx = p.x > 1e-30f, by = p.y > 1e-30f, bz = p.z > 1e-30f, bw = p.w > 1e-30f;
+                if (split) {
+                    const float4 d = dreg[kk];
+                    const float4 r = make_float4(d.x - p.x, d.y - p.y, d.z - p.z, d.w - p.w);
+                    k = make_float4(bx ? split_ratio(r.x, p.x) : r.x, by ? split_ratio(r.y, p.y) : r.y,
+                                    bz ? split_ratio(r.z, p.z) : r.z, bw ? split_ratio(r.w, p.w) : r.w);
+                    p = r;
+                }
+                *reinterpret_cast<float4*>(A.P + o) = p;
+                for (int s = 0; ns > 1 && A.Ps && s < ns; ++s) {
+                    const uint4 q = a[s * (ACC / 4) + i0];
+                    float4 v = make_float4((float)q.x * inv, (float)q.y * inv, (float)q.z * inv, (float)q.w * inv);
+                    if (split) {   // f_s where P vanishes
+                        auto f = [&](int i) { return XT ? xt_get(C, EPR_XT_F, s, gx + i) : C.f[s]; };
+                        if (!(bx && by && bz && bw))
+                            v = make_float4(bx ? v.x : f(0), by ? v.y : f(1), bz ? v.z : f(2), bw ? v.w : f(3));
+                        v = make_float4(k.x * v.x, k.y * v.y, k.z * v.z, k.w * v.w);
+                    }
+                    *reinterpret_cast<float4*>(A.Ps + (size_t)s * npix + o + (size_t)b * (ns - 1) * npix) = v;
+                }
             }
         }
     } else {
@@ -508,6 +541,19 @@ k_splat(const __grid_constant__ EprConsts C, const SplatArgs A)
                 if (ns > 1) A.Psq[(size_t)s * npix + o + (size_t)b * (ns - 1) * npix] = q;
             }
             A.Pq[o] = sum;
+            if (split) {
+                const float p = (float)sum * EPR_FX_INV, r = __ldg(&A.D[o]) - p;
+                const bool lit = p > 1e-30f;
+                const float k = lit ? split_ratio(r, p) : r;
+                A.P[o] = r;
+                for (int s = 0; ns > 1 && s < ns; ++s) {
+                    const unsigned long long q =
+                        acc_fx<MODE>(acc, s * ACC + (ly + 1) * AP + lx + kAccX, plane, A.fx_lo);
+                    const float f = XT ? xt_get(C, EPR_XT_F, s, gx) : C.f[s];
+                    A.Ps[(size_t)s * npix + o + (size_t)b * (ns - 1) * npix] =
+                        k * (lit ? (float)q * EPR_FX_INV : f);
+                }
+            }
         }
     }
 }

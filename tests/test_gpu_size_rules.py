@@ -216,6 +216,34 @@ def test_split_line_counts(torch, E, oracle, lines, fixed):
         assert rel(host(T), Tref) <= 2e-5
 
 
+# several lines, or fixed point: pixels that long shifts reach are redone after
+# the splat has split their residual (reach 1 sends most sources that way and
+# leaves pixels that only they reach)
+@pytest.mark.parametrize("lines,fixed", [(1, True), (2, False), (2, True), (4, False), (8, False), (8, True),
+                                         (11, False)])
+@pytest.mark.parametrize("reach", [1, 4])
+def test_split_with_long_shifts(torch, E, oracle, lines, fixed, reach):
+    Es, d, b, w = spec(lines)
+    ln = oracle.Lines(Es, d, b, w, L, PIXEL)
+    T0 = phantom(96, 144) * 2.0
+    D = ph.poisson(oracle.forward(ln, phantom(96, 144, seed=12)), 1e4, 3).astype(np.float32)
+    D[40:44, 60:70] = oracle.forward(ln, T0)[40:44, 60:70]   # and pixels whose residual vanishes
+    Tref, info = oracle.solve(ln, D.astype(np.float64), T0=T0, n_iter=1, omega=0.4)
+    with E.Plan(144, 96, PIXEL, L, Es, d, b, w, deterministic=fixed, max_shift_px=reach) as p:
+        Dd = cuda(torch, np.stack([D, D]))
+        first = None
+        for _ in range(2):   # the second solve finds the workspace as the first left it
+            T = cuda(torch, np.stack([T0, T0]))
+            got = E.epr_solve_nonlocal(p.handle, Dd, T, batch=2, n_iter=1, omega=0.4, init=1)
+            assert (got["overflow_sources"] > 0) == (lines > 1 or reach == 1)   # one line: up to 2.4 px
+            for k in range(2):
+                assert rel(host(T[k]), Tref) <= 2e-5
+                assert abs(got["rho"][k] - info["rho"][0]) <= 1e-5 * info["rho"][0]
+            if fixed:
+                assert first is None or torch.equal(T, first)
+                first = T.clone()
+
+
 @pytest.mark.parametrize("os_", [2, 3, 4, 5])
 @pytest.mark.parametrize("lines", [1, 2])
 def test_oversampled_split_factors(torch, E, oracle, os_, lines):
