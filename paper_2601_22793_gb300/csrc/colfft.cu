@@ -251,7 +251,7 @@ cudaError_t epr_launch_col(const EprConsts& C, const EprWork& W, int line0, int 
         A.CW = cw;
         A.lgCW = cw == 2 ? 1 : 2;
         const ColKernel q = r8 ? k.radix8 : o5 ? k.occ5 : narrow ? k.narrow : k.wide;
-        e = epr_launch_kernel(pdl, q, dim3(C.half / cw, nl, batch), dim3(narrow ? k.threads2 : k.threads),
+        e = epr_launch_kernel(pdl, q, dim3(C.half / cw + (rho_it >= 0 ? 1 : 0), nl, batch), dim3(narrow ? k.threads2 : k.threads),
                               col_tma_smem(C.ny, cw), stream, C, A, maps[narrow ? 1 : 0]);
         done = true;
     }

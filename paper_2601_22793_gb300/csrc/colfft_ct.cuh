@@ -64,8 +64,9 @@ constexpr int col_min_blocks(int T)
     return b < 1 ? 1 : b > 16 ? 16 : b;
 }
 
-// Block 0 of the column pass of a solve (line 0) turns the forward row
+// One block of the column pass of a solve (line 0) turns the forward row
 // pass's partials into rho; the grid dependency wait has made them visible.
+// The bulk-copy pass launches one block more for it.
 __device__ __forceinline__ void col_finalize_rho(const ColArgs& A, int b, bool lead)
 {
     if (A.rho_it >= 0 && lead)
@@ -149,7 +150,12 @@ k_col_tma(const EprConsts C, const ColArgs A, const __grid_constant__ CUtensorMa
     const size_t base = ((size_t)__cvta_generic_to_shared(smem_raw) + 127) & ~size_t(127);
     float2* buf = reinterpret_cast<float2*>(smem_raw + (base - (size_t)__cvta_generic_to_shared(smem_raw)));
     const int b = blockIdx.z, sl = blockIdx.y, tid = threadIdx.x;
-    const int kx0 = blockIdx.x * CW;
+    const int kx0 = ((int)blockIdx.x - (A.rho_it >= 0 ? 1 : 0)) * CW;
+    if (A.rho_it >= 0 && blockIdx.x == 0) {   // the block that forms rho, in the first wave
+        epr_grid_wait();
+        if (!(A.check_done && A.st[b].done)) col_finalize_rho(A, b, sl == 0);
+        return;
+    }
     if (tid == 0) {
         epr_tma::mbar_init(&bar, 1);
         epr_tma::fence_async_shared();
@@ -165,7 +171,6 @@ k_col_tma(const EprConsts C, const ColArgs A, const __grid_constant__ CUtensorMa
         for (int i = 0; i < BOXES; ++i)
             epr_tma::load_2d(buf + i * BOXY * CW, &map, 2 * kx0, row0 + i * BOXY, &bar);
     }
-    col_finalize_rho(A, b, blockIdx.x == 0 && sl == 0);   // while the tile is in flight
     if (!epr_tma::mbar_wait(&bar, 0, kTmaWaitPolls)) {
         // the copy did not arrive: report, and wait once more (bounded) so
         // that no copy lands after the block has left

@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(512, 2) k_row_fwd(const EprConsts C, const Row
         cp_async_commit();
     }
     epr_grid_wait();
-    if constexpr (MODE != FWD_LOAD) fwd_finalize_kappa(A, b, blockIdx.x == 0);
+    if constexpr (MODE != FWD_LOAD) fwd_finalize_kappa(A, b, blockIdx.x == 0, (int)gridDim.x);
     if (A.check_done && A.st[b].done) {
         cp_async_wait_all();   // no copy may land after the block has left
         return;
@@ -464,7 +464,8 @@ cudaError_t epr_launch_row_fwd(const EprConsts& C, const EprWork& W, int mode, c
         e = epr_launch_kernel(pdl, kernel, grid, dim3(L.threads), L.smem, stream, C, A);
     };
     if (k) {
-        e = epr_launch_kernel(pdl, k, dim3(grid.x, grid.y, nl), dim3(threads), smem, stream, C, A);
+        e = epr_launch_kernel(pdl, k, dim3(grid.x + (A.fin ? 1 : 0), grid.y, nl), dim3(threads), smem, stream, C,
+                              A);
     } else if (mode == FWD_SOLVE_NL && C.xt) {   // per-column shift constants
         go(k_row_fwd<FWD_SOLVE_NL, false, true, 0, true>);
     } else if (mode == FWD_SOLVE_NL) {

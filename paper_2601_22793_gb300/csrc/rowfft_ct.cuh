@@ -66,17 +66,20 @@ using PR = eprfft::PadRow;   // shared layout of the packed rows
 // the first to the last: each kernel starts on the projections its
 // predecessor touched last, whose data are still in L2.
 __device__ __forceinline__ int row_batch_index() { return (int)(gridDim.y - 1 - blockIdx.y); }
-// Block 0 of a forward solve pass (line 0) turns the inverse pass's
+// One block of a forward solve pass (line 0) turns the inverse pass's nblk
 // partials of the previous iteration into kappa, the iteration count and
 // the convergence flag, unless the projection had already converged; the
 // grid dependency wait has made every partial visible.  The other blocks of
 // this pass may not see the flag: a projection that converges here runs this
 // pass and the splat before it once more, which changes nothing it keeps.
-__device__ __forceinline__ void fwd_finalize_kappa(const RowArgs& A, int b, bool lead)
+// The compile-time passes launch one block more for it (double-precision sums
+// of up to 2048 partials are a serial chain: 2.6 us of a 9.8 us pass over
+// 256^2 when a block did both).
+__device__ __forceinline__ void fwd_finalize_kappa(const RowArgs& A, int b, bool lead, int nblk)
 {
     if (A.fin && lead && !A.st[b].done)
         finalize_kappa(&A.st[b], A.part_a + (size_t)b * A.max_blocks,
-                       A.part_b + (size_t)b * A.max_blocks, (int)gridDim.x,
+                       A.part_b + (size_t)b * A.max_blocks, nblk,
                        A.hist ? A.hist + (size_t)b * A.hist_len : nullptr, A.hist_len, A.it - 1,
                        A.tol);
 }
@@ -226,7 +229,13 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
     const int ny = C.ny, tid = threadIdx.x;
     const size_t npix = (size_t)NX * ny;
     const size_t pb = (size_t)b * npix;
-    const int yb = blockIdx.x * RP * 2;
+    const int bx = (int)blockIdx.x - (A.fin ? 1 : 0);   // row block
+    const int yb = bx * RP * 2;
+    if (A.fin && blockIdx.x == 0) {   // the block that finishes the last iteration, in the first wave
+        epr_grid_wait();
+        if (sl == 0) fwd_finalize_kappa(A, b, true, (int)gridDim.x - 1);
+        return;
+    }
     float* Ts = reinterpret_cast<float*>(zs);   // aliases the FFT rows (see above)
     if constexpr (GATHER) {   // T is not written by the predecessor: fetch it before the wait
         const float* Tb = A.T + pb;
@@ -251,7 +260,6 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
         }
     }
     epr_grid_wait();
-    if (GATHER || !A.G) fwd_finalize_kappa(A, b, blockIdx.x == 0 && sl == 0);
     if (A.check_done && A.st[b].done) {
         cp_async_wait_all();   // no copy may land after the block has left
         return;
@@ -411,7 +419,7 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
     if (!norm) return;
     float rb = 0.f;
     block_sum2(ra, rb, red);   // |D - P|^2 partials; rho is formed by the column pass
-    store_partials(A.part_c + (size_t)b * A.max_blocks, nullptr, ra, rb);
+    if (tid == 0) A.part_c[(size_t)b * A.max_blocks + bx] = (double)ra;
 }
 
 // Z[k] = X0[k] + i X1[k] of the block's row pairs over the full rows, into
