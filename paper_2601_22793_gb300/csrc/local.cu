@@ -81,7 +81,7 @@ struct Rows3 {
 };
 
 template <int MODE, bool DET>
-__global__ void __launch_bounds__(kStencilThreads, 8) k_stencil(const EprConsts C, const StencilArgs A)
+__global__ void __launch_bounds__(kStencilThreads, 7) k_stencil(const EprConsts C, const StencilArgs A)
 {
     constexpr int HALO = MODE == ST_LOCAL1 ? 2 : 3, OUT = 32 - 2 * HALO;
     constexpr bool PRESSURE = MODE != ST_LOCAL1, LOCAL = MODE != ST_WKB1;
@@ -96,7 +96,10 @@ __global__ void __launch_bounds__(kStencilThreads, 8) k_stencil(const EprConsts 
     const int gx = (w % A.strips) * OUT - HALO + lane;
     const int y1 = min(y0 + A.H, ny);   // rows y0 .. y1 - 1
     const size_t npix = (size_t)nx * ny, pb = (size_t)b * npix;
-    const float* Tc = A.T + pb + min(max(gx, 0), nx - 1);   // this lane's column
+    // this lane's column of each map; offsets within a map fit in an int
+    const float* Tc = A.T + pb + min(max(gx, 0), nx - 1);
+    const float* Dc = A.D ? A.D + pb + gx : nullptr;
+    float* Pc = A.P + pb + gx;
     const bool xl = gx <= 0, xh = gx >= nx - 1;
     const float hsx = xl || xh ? 1.f : 0.5f;
     const bool out = lane >= HALO && lane < 32 - HALO && gx < nx;
@@ -113,7 +116,7 @@ __global__ void __launch_bounds__(kStencilThreads, 8) k_stencil(const EprConsts 
     auto dYY = [&](const Rows3& f, int y) {
         return (y == 0 ? f.c : f.m) - 2.f * f.c + (y == ny - 1 ? f.c : f.p);
     };
-    auto ldT = [&](int y) { return __ldg(Tc + (size_t)min(max(y, 0), ny - 1) * nx); };
+    auto ldT = [&](int y) { return __ldg(Tc + min(max(y, 0), ny - 1) * nx); };
 
     for (int s = 0; s < ns; ++s) {
         const float fs = line_const(C.f, s), mus = line_const(C.mu, s);
@@ -126,6 +129,16 @@ __global__ void __launch_bounds__(kStencilThreads, 8) k_stencil(const EprConsts 
         Rows3 Q = {}, AY = {}, BYY = {}, BXY = {}, CYQ = {};
         float Ib = 0.f, Ia = 0.f, Sc = 0.f, Sb = 0.f, Sa = 0.f;   // Sx: the terms known so far at row x
         float ahead = ldT(y0 - HALO + 2), ahead2 = ldT(y0 - HALO + 3);
+        // what the output rows need besides: D on the last line, and the
+        // prediction so far (the splat's, or the earlier lines')
+        const bool lastD = A.D && s == ns - 1;
+        const bool sofar = s > 0 || MODE == ST_WKB1;
+        auto ldD = [&](int y) { return lastD && out && y < y1 ? __ldg(Dc + y * nx) : 0.f; };
+        auto ldP = [&](int y) {
+            if (!(sofar && out && y < y1)) return 0.f;
+            return DET && s == 0 ? (float)A.Pq[pb + (size_t)y * nx + gx] * EPR_FX_INV : Pc[y * nx];
+        };
+        float d0 = 0.f, d1 = ldD(y0), p0 = 0.f, p1 = ldP(y0);   // rows yo, yo + 1
 #pragma unroll 3
         for (int yl = y0 - HALO + 2; yl <= y1 - 1 + HALO; ++yl) {
             const int a = yl - 1, bb = yl - 2;
@@ -169,31 +182,32 @@ __global__ void __launch_bounds__(kStencilThreads, 8) k_stencil(const EprConsts 
                 CYQ.push(Ib * dY(Q, bb));
             }
             const int yo = PRESSURE ? yl - 3 : bb;   // the row that is complete
+            if (yo >= y0) {
+                d0 = d1;
+                p0 = p1;
+                d1 = ldD(yo + 1);
+                p1 = ldP(yo + 1);
+            }
             const float p = PRESSURE ? Sc - qc * dY(CYQ, yo) : Sb;
             if (!out || yo < y0 || yo >= y1) continue;
-            const size_t o = pb + (size_t)yo * nx + gx;
-            float tot = p;   // the prediction of all lines so far
-            if (s > 0) tot = A.P[o] + p;
-            else if constexpr (MODE == ST_WKB1) tot = (DET ? (float)A.Pq[o] * EPR_FX_INV : A.P[o]) + p;
+            const float tot = p0 + p;   // the prediction of all lines so far
+            const size_t o = (size_t)yo * nx + gx;
             if (ns > 1) {
-                const size_t os = pb * ns + (size_t)s * npix + (o - pb);
+                const size_t os = pb * ns + (size_t)s * npix + o;
                 float ps = p;
                 if (A.Ps) {
                     if constexpr (MODE == ST_WKB1) ps += DET ? (float)A.Psq[os] * EPR_FX_INV : A.Ps[os];
                     A.Ps[os] = ps;
                 }
             }
-            if (!A.D || s < ns - 1) {
-                A.P[o] = tot;
-                continue;
-            }
-            const float r = __ldg(&A.D[o]) - tot;
-            A.P[o] = r;
+            const float r = d0 - tot;
+            Pc[yo * nx] = lastD ? r : tot;
+            if (!lastD) continue;
             if (ns > 1) {   // this thread wrote every line's value of the pixel
                 const bool pos = tot > 1e-30f;
                 const float k = pos ? r / tot : r;
                 for (int l = 0; l < ns; ++l) {
-                    float* q = &A.Ps[pb * ns + (size_t)l * npix + (o - pb)];
+                    float* q = &A.Ps[pb * ns + (size_t)l * npix + o];
                     *q = k * (pos ? *q : line_const(C.f, l));
                 }
             }
