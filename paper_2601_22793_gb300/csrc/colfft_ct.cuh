@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(NY * CW / EPT,
 k_col_tma(const EprConsts C, const ColArgs A, const __grid_constant__ CUtensorMap map)
 {
     constexpr int T = NY * CW / EPT;
+    static_assert(NY * CW % EPT == 0, "every element has a thread");
     constexpr int LGCW = CW == 2 ? 1 : CW == 4 ? 2 : 3;
     constexpr int BOXY = epr_col_box(NY, CW);
     constexpr int BOXES = NY / BOXY;

@@ -433,6 +433,26 @@ __device__ __forceinline__ void apply_twiddles(float2 (&v)[R], const float2* __r
     }
 }
 
+// Sequence m and index j of butterfly b = tid + k T of a stage with NR of them
+// per sequence.  Interleaved sequences (the columns of a tile) alternate with
+// b; sequences laid out one after another (rows, SJ = 1) take whole runs of
+// threads, so that a warp's accesses are contiguous and, where T divides NR, the
+// butterflies of one thread share their index, and with it the twiddles.
+template <int NR, int LGSEQ, int SJ, int T>
+__device__ __forceinline__ void ct_butterfly(int tid, int k, int& m, int& j)
+{
+    if constexpr (SJ == 1 && LGSEQ > 0 && NR % T == 0) {
+        m = k * T / NR;
+        j = tid + k * T % NR;
+    } else if constexpr (SJ == 1 && LGSEQ > 0) {
+        m = (unsigned)(tid + k * T) / NR;
+        j = (unsigned)(tid + k * T) % NR;
+    } else {
+        m = (tid + k * T) & ((1 << LGSEQ) - 1);
+        j = (tid + k * T) >> LGSEQ;
+    }
+}
+
 // Output map of a stage: out = post(value, e) with e = j * SJ + m * SM the
 // element's unpadded index; Identity leaves the value.
 struct Identity {
@@ -462,8 +482,8 @@ __device__ __forceinline__ void stage_ct(const float2* in, float2* buf, const fl
         const int b = tid + k * T;
         dst[k] = -1;
         if (NB % T == 0 || b < NB) {
-            const int m = b & (NSEQ - 1);
-            const int j = b >> LGSEQ;
+            int m, j;
+            ct_butterfly<NR, LGSEQ, SJ, T>(tid, k, m, j);
             const int jm = j % NS;
             const int jd = j / NS;
             const int base = m * SM;
@@ -621,21 +641,27 @@ __device__ __forceinline__ void stage_turn(float2* buf, const float2* __restrict
     __syncthreads();
 }
 
-// The first stage with its operands in registers: for one sequence (nseq =
-// 1) with EPT equal to the first radix R, thread tid's operands are elements
-// tid + r N / R, r < R, and the stage has no twiddles.  Writes its results to
-// buf (layout PAD) and synchronises; the caller has synchronised already if
-// buf aliases data that other threads still read.  Stages 1.. follow as
-// fft_ct<..., 1>.
-template <class PAD, int DIR, int N, int EPT, int SJ, int MAXR = 8>
+// The first stage with its operands in registers, for NSEQ sequences laid out
+// SM apart and N / R threads with the first radix R: v[m R + r] is element
+// tid + r N / R of sequence m, and the stage has no twiddles.  Writes its
+// results to buf (layout PAD) and synchronises; the caller has synchronised
+// already if buf aliases data that other threads still read.  Stages 1..
+// follow as fft_ct<..., 1>.
+template <class PAD, int DIR, int N, int NSEQ, int EPT, int SM, int MAXR = 8>
 __device__ __forceinline__ void stage0_regs(float2 (&v)[EPT], float2* buf, int tid)
 {
     constexpr int R = ct_radix(N, 0, MAXR);
-    static_assert(R == EPT && ct_n_stages(N, MAXR) > 1, "operands of the first stage in registers");
-    dft<R, DIR>(v);
-    const int dst = tid * R * SJ;   // (j / Ns) Ns R + (j mod Ns) with Ns = 1, j = tid
+    static_assert(R * NSEQ == EPT && ct_n_stages(N, MAXR) > 1, "operands of the first stage in registers");
+    const int dst = tid * R;   // (j / Ns) Ns R + (j mod Ns) with Ns = 1, j = tid
 #pragma unroll
-    for (int r = 0; r < R; ++r) buf[PAD::idx(dst + r * SJ)] = v[r];
+    for (int m = 0; m < NSEQ; ++m) {
+        float2 w[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) w[r] = v[m * R + r];
+        dft<R, DIR>(w);
+#pragma unroll
+        for (int r = 0; r < R; ++r) buf[PAD::idx(dst + r + m * SM)] = w[r];
+    }
     __syncthreads();
 }
 

@@ -457,6 +457,7 @@ cudaError_t epr_launch_row_fwd(const EprConsts& C, const EprWork& W, int mode, c
         }
     } else if (L.k) {
         smem = L.k->smem_plain;
+        threads = L.k->threads_plain;
         k = L.k->plain;
     }
     cudaError_t e = cudaSuccess;
@@ -506,6 +507,7 @@ cudaError_t epr_launch_row_inv(const EprConsts& C, const EprWork& W, int mode, f
         }
     } else if (L.k) {
         k = L.k->store;
+        threads = L.k->threads_plain;
         smem = L.k->smem_plain;
     }
     cudaError_t e = cudaSuccess;

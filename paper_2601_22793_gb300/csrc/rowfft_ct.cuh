@@ -51,6 +51,7 @@ struct RowKernels {
     RowKernel xfwd1, xfwdn, xinv1, xinvn;   // x-dependent spectrum
     size_t smem_fwd, smem_plain, smem_inv1, smem_invn1, smem_invn;   // invn1: one line on invn
     int threads16;         // one-line kernels with 16 elements per thread: their block, or 0
+    int threads_plain;     // block of plain and store
 };
 
 }  // namespace eprrow
@@ -153,8 +154,8 @@ __device__ __forceinline__ float2 log_ratio2(float2 t, float2 h, float om_f, flo
 }
 
 // blocks per SM that a block of T threads is bounded to: 64 registers, or 80
-// where `threads` is 768 (the several-line update of ragged lengths, whose
-// per-element row and column would spill)
+// where `threads` is 768 (the several-line update of ragged lengths with
+// several row pairs, whose per-element row and column would spill)
 // (a block of 352 or 384 threads fits three times into 1152)
 constexpr int row_min_blocks(int T, int threads = 1024)
 {
@@ -166,9 +167,18 @@ constexpr int row_min_blocks(int T, int threads = 1024)
 template <int NX>
 __host__ __device__ constexpr int ct_lg(int v) { return v <= 1 ? 0 : 1 + ct_lg<NX>(v / 2); }
 
-// packed row pair of element e (0 <= e < NX RP); NX may be 3 * 2^k with RP = 1
-template <int NX, int RP>
-__device__ __forceinline__ int row_of(int e) { return RP == 1 ? 0 : (int)((unsigned)e / NX); }
+// packed row pair m and column x of element tid + k T (0 <= that < NX RP)
+template <int NX, int RP, int T>
+__device__ __forceinline__ void row_of(int tid, int k, int& m, int& x)
+{
+    if constexpr (NX % T == 0) {   // the thread's elements of one k are one column's
+        m = k * T / NX;
+        x = tid + k * T % NX;
+    } else {
+        m = RP == 1 ? 0 : (int)((unsigned)(tid + k * T) / NX);
+        x = tid + k * T - m * NX;
+    }
+}
 
 // The gather of one pixel with any mapped point: corners outside the grid
 // read 0 (Eq. 4); a shift that is not finite or beyond the grid reads only 0.
@@ -211,11 +221,11 @@ __device__ __noinline__ float gather_guarded(const float* R, int y, int x, float
 // the plan's table.
 template <int NX, int RP, bool POLY, bool GATHER, bool OCC6 = false, bool XT = false, int EPT = kEPT>
 __global__ void __launch_bounds__(NX * RP / EPT, OCC6 ? 6 : (NX * RP / EPT == 256 && !POLY) ? 5
-                                                 : (EPT == 16 && NX * RP / EPT == 128) ? 7
                                                  : row_min_blocks(NX * RP / EPT))
 k_row_fwd_ct(const EprConsts C, const RowArgs A)
 {
     constexpr int T = NX * RP / EPT;
+    static_assert(NX * RP % EPT == 0 && RP * (NX / 2) % T == 0, "every element has a thread");
     constexpr int MAXR = row_maxr(EPT);   // radix-16 stages with 16 elements per thread
     constexpr int kRim = EPT <= kEPT ? 1 : 0;   // rows staged above and below the block's own
     constexpr int SM = NX + kPad;
@@ -279,8 +289,8 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
         float2 own[EPT];
 #pragma unroll
         for (int k = 0; k < EPT; ++k) {
-            const int e = tid + k * T;
-            const int m = row_of<NX, RP>(e), x = e - m * NX;
+            int m, x;
+            row_of<NX, RP, T>(tid, k, m, x);
             const float* q = Rt + (size_t)(yb + 2 * m) * NX + x;
             own[k] = make_float2(__ldg(q), __ldg(q + NX));
         }
@@ -313,9 +323,8 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
     // one element's loads and the next's.
     unsigned int rim = 0u;   // bits 2 k + r0
     auto shift2 = [&](int k, int& x, int& y0, float2& ux, float2& uy) {
-        const int e = tid + k * T;
-        const int m = row_of<NX, RP>(e);
-        x = e - m * NX;
+        int m;
+        row_of<NX, RP, T>(tid, k, m, x);
         y0 = yb + 2 * m;
         const float* tr = Ts + (2 * m + kRim) * NX + x;
         const float* tg = A.T + pb + (size_t)y0 * NX + x;   // the same pixel in memory
@@ -342,8 +351,8 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
 #pragma unroll
     for (int k = 0; k < EPT; ++k) {
         if constexpr (!GATHER) {   // identity back-transport of the local closure
-            const int e = tid + k * T;
-            const int m = row_of<NX, RP>(e), x = e - m * NX;
+            int m, x;
+            row_of<NX, RP, T>(tid, k, m, x);
             const size_t q = (size_t)(yb + 2 * m) * NX + x;
             vk[k] = make_float2(__ldg(Rb + q), __ldg(Rb + q + NX));
         } else {
@@ -380,15 +389,15 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
         }
     }
     if constexpr (GATHER) __syncthreads();   // every thickness read is done
-    if constexpr (RP == 1 && eprfft::ct_radix(NX, 0, MAXR) == EPT) {
-        // one row pair: vk[k] = element tid + k T, the first stage's operands
-        eprfft::stage0_regs<PR, -1, NX, EPT, 1, MAXR>(vk, zs, tid);
+    if constexpr (eprfft::ct_radix(NX, 0, MAXR) * RP == EPT && NX % T == 0) {
+        // vk[m R + r] = element tid + r T of pair m, the first stage's operands
+        eprfft::stage0_regs<PR, -1, NX, RP, EPT, SM, MAXR>(vk, zs, tid);
         eprfft::fft_ct<PR, -1, NX, EPT, LGRP, 1, SM, 1, MAXR>(zs, A.tw, tid);
     } else {
 #pragma unroll
         for (int k = 0; k < EPT; ++k) {
-            const int e = tid + k * T;
-            const int m = row_of<NX, RP>(e), x = e - m * NX;
+            int m, x;
+            row_of<NX, RP, T>(tid, k, m, x);
             zs[PR::idx(m * SM + x)] = vk[k];
         }
         __syncthreads();
@@ -428,8 +437,9 @@ template <int NX, int RP, int EPT>
 __device__ __forceinline__ void inv_unpack(const float2* __restrict__ Sb, float2* zs, int yb, int tid)
 {
     constexpr int T = NX * RP / EPT, HALF = NX / 2, SM = NX + kPad;
+    static_assert(NX * RP % EPT == 0 && RP * HALF % T == 0, "every element has a thread");
 #pragma unroll 2
-    for (int i0 = 0; i0 < RP * HALF; i0 += T) {   // T divides RP HALF: EPT is even
+    for (int i0 = 0; i0 < RP * HALF; i0 += T) {
         const int e = i0 + tid;
         const int m = e / HALF, k = e % HALF;
         const int y0 = yb + 2 * m;
@@ -511,7 +521,6 @@ struct InvUpdate1 {
 // it, so two 512-thread blocks fit on an SM.
 template <int NX, int RP, bool OCC6 = false, bool XT = false, int EPT = kEPT>
 __global__ void __launch_bounds__(NX * RP / EPT, OCC6 ? 6 : NX * RP / EPT == 256 ? 5
-                                                 : (EPT == 16 && NX * RP / EPT == 128) ? 7
                                                  : row_min_blocks(NX * RP / EPT))
 k_row_inv1(const EprConsts C, const RowArgs A)
 {
@@ -613,7 +622,7 @@ struct InvUpdatePoly {
 // pixel in shared memory (each thread owns its pixels); then T' = T - sum
 // and the kappa partial sums.
 template <int NX, int RP, bool XT = false, int EPT = kEPT>
-__global__ void __launch_bounds__(NX * RP / EPT, row_min_blocks(NX * RP / EPT, NX % 3 == 0 ? 768 : 1024))
+__global__ void __launch_bounds__(NX * RP / EPT, row_min_blocks(NX * RP / EPT, NX % 3 == 0 && RP > 1 ? 768 : 1024))
 k_row_invn(const EprConsts C, const RowArgs A)
 {
     constexpr int T = NX * RP / EPT;
@@ -728,9 +737,14 @@ constexpr RowKernels row_any()
     k.rp = RP;
     k.threads = NX * RP / EPT;
     k.fwdn = k_row_fwd_ct<NX, RP, true, true, false, false, EPT>;
-    k.plain = k_row_fwd_ct<NX, RP, true, false, false, false, EPT>;
     k.invn = k_row_invn<NX, RP, false, EPT>;
-    k.store = k_row_store<NX, RP, EPT>;
+    // the plain transforms hold nothing but the row: 16 elements per thread
+    // and radix-16 stages (2304 = 16 16 9 instead of 8 8 4 9) where that
+    // leaves a block of at least three warps
+    constexpr int EPTP = EPT == kEPT && RP == 1 && NX >= 1536 && NX % 16 == 0 ? 16 : EPT;
+    k.threads_plain = NX * RP / EPTP;
+    k.plain = k_row_fwd_ct<NX, RP, true, false, false, false, EPTP>;
+    k.store = k_row_store<NX, RP, EPTP>;
     k.smem_fwd = row_fwd_smem(NX, RP);
     k.smem_plain = row_fft_smem(NX, RP);
     k.smem_inv1 = k.smem_invn1 = row_inv_smem(NX, RP, 1);
