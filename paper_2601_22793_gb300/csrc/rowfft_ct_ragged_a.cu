@@ -12,9 +12,9 @@ const RowKernels kTable[] = {
     row_any<576, 2>(),
     row_any<648, 1>(),
     row_any<864, 2>(),
-    row_any<1296, 1>(),
-    row_any<2304, 1>(),
-    row_any<3888, 1>(),
+    row_full<1296, 1>(),
+    row_full<2304, 1>(),
+    row_full<3888, 1>(),
 };
 
 }  // namespace

@@ -12,8 +12,8 @@ const RowKernels kTable[] = {
     row_any<576, 1>(),
     row_any<768, 2>(),
     row_any<864, 1>(),
-    row_any<1728, 1>(),
-    row_any<2592, 1>(),
+    row_full<1728, 1>(),
+    row_full<2592, 1>(),
 };
 
 }  // namespace

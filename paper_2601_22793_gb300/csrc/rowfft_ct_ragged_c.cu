@@ -11,9 +11,9 @@ const RowKernels kTable[] = {
     row_any<432, 1>(),
     row_any<648, 2>(),
     row_any<768, 1>(),
-    row_any<1152, 1>(),
-    row_any<1944, 1>(),
-    row_any<3456, 1>(),
+    row_full<1152, 1>(),
+    row_full<1944, 1>(),
+    row_full<3456, 1>(),
 };
 
 }  // namespace
