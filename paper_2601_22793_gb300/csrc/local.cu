@@ -220,9 +220,10 @@ cudaError_t launch_stencil(const EprConsts& C, StencilArgs& A, int batch, cudaSt
 {
     constexpr int OUT = MODE == ST_LOCAL1 ? 28 : 26;
     A.strips = (C.nx + OUT - 1) / OUT;
-    // 32 rows per strip (19 % of the rows are halo), 16 where that would leave
-    // fewer than 16 warps per SM
-    A.H = (long long)A.strips * ((C.ny + 31) / 32) * batch >= 152 * 16 ? 32 : 16;
+    // 32 rows per strip (19 % of the rows computed are halo); fewer where that
+    // would leave under 8 warps per SM, since a strip's rows are a serial chain
+    A.H = 32;
+    while (A.H > 4 && (long long)A.strips * ((C.ny + A.H - 1) / A.H) * batch < 152 * 8) A.H /= 2;
     const int warps = A.strips * ((C.ny + A.H - 1) / A.H);
     const dim3 grid((warps * 32 + kStencilThreads - 1) / kStencilThreads, 1, batch);
     const cudaError_t e = epr_launch_kernel(C.pdl != 0, k_stencil<MODE, DET>, grid, dim3(kStencilThreads), 0,
