@@ -151,8 +151,8 @@ struct epr_plan_s {
     cudaGraphExec_t prof_exec;   // last profiled solve
     bool tuned;                  // autotuner has run
     // vector-Jacobian product workspace (allocated on first use)
-    double* vjp_part;      // block partials and their sums
-    double* h_vjp_part;    // pinned copy of the sums
+    double* vjp_part;      // block partials
+    double* h_vjp_part;    // their sums, pinned: written by the kernel itself
     int vjp_cap;
     // x-dependent spectrum: per-column constants on the device (C.xt points
     // here while a table is set) and the uniform preconditioner constants
@@ -1146,14 +1146,11 @@ epr_status epr_vjp(epr_plan_t p, const float* T, const float* gbar, float* Tbar,
     if (st == EPR_OK) st = resolve(p, 2, Tbar, n, false, s, &Tbd, &sTb);
     if (st != EPR_OK) return st;
     const bool scalars = delta_bar || beta_bar || L_bar;
-    double* sums = p->vjp_part + (part_len - nsum);
     {
         ProfScope ps(p, EPR_KERNEL_OTHER, s);
-        EPR_TRY(epr_launch_vjp(C, Td, gd, Tbd, p->vjp_part, scalars ? sums : nullptr, batch, s));
+        EPR_TRY(epr_launch_vjp(C, Td, gd, Tbd, p->vjp_part, scalars ? p->h_vjp_part : nullptr, batch, s));
     }
     if (sTb) EPR_TRY(cudaMemcpyAsync(Tbar, Tbd, n * sizeof(float), cudaMemcpyDeviceToHost, s));
-    if (scalars)
-        EPR_TRY(cudaMemcpyAsync(p->h_vjp_part, sums, nsum * sizeof(double), cudaMemcpyDeviceToHost, s));
     if (scalars || sTb) EPR_TRY(cudaStreamSynchronize(s));
     if (scalars) {
         const double p2 = p->pixel * p->pixel;

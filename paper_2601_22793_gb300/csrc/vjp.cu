@@ -17,22 +17,30 @@
 // A warp marches down a strip of 30 output columns (32 lanes): vx of the
 // neighbouring columns comes by warp shuffle and the last three rows of vy
 // stay in registers, so G^T needs no maps of vx and vy and no second pass.
-// Bound by the gather's loads (four corners per line and pixel, from L1 and
-// L2); the two-pass form it replaces also wrote and read vx, vy and Tbar and
-// kept its per-line sums in local memory.
+// The two-pass form it replaces also wrote and read vx, vy and Tbar and kept
+// its per-line sums in local memory.  Bound by the latency of the gather's
+// loads (four corners per line and pixel, from L1 and L2): long scoreboard is
+// the top stall, half of the issue slots are used.  The corners of all lines
+// are therefore loaded before the first is used, and the strips are cut so
+// that every resident warp has one.  1536 x 1024, 3 lines: 56 -> 34.5 us from
+// both, with the slopes taken from shared differences.
+#include <algorithm>
+
 #include "epr_internal.cuh"
 
 namespace {
 
 constexpr int kVjpThreads = 256;
-constexpr int kVjpRows = 32;       // rows of a strip unit
 constexpr int kVjpMaxBlocks = 608; // per projection: 4 per SM on 152 SMs
+
+constexpr int kVjpSlots = kVjpMaxBlocks * (kVjpThreads / 32);   // resident warps
 
 struct VjpArgs {
     const float* T;
     const float* gbar;
     float* Tbar;
     double* part;        // [B][kVjpMaxBlocks][2 ns]  (cbar_s, mubar_s) per block
+    int H;               // rows of a strip unit
     int strips, units;   // of one projection
 };
 
@@ -62,9 +70,10 @@ __device__ __noinline__ void vjp_corners(const float* G, int y, int x, float uy,
     }
 }
 
-// NSM: bound of the line count at compile time (the sums stay in registers)
+// NSM: the line count up to 4 (the corner loads of every line are then issued
+// together), a bound of it above (the sums stay in registers)
 template <int NSM>
-__global__ void __launch_bounds__(kVjpThreads) k_vjp(const __grid_constant__ EprConsts C, const VjpArgs A)
+__global__ void __launch_bounds__(kVjpThreads, NSM <= 8 ? 4 : 2) k_vjp(const __grid_constant__ EprConsts C, const VjpArgs A)
 {
     __shared__ float red[2 * NSM][kVjpThreads / 32];
     const int nx = C.nx, ny = C.ny, ns = C.ns, b = blockIdx.y;
@@ -76,7 +85,7 @@ __global__ void __launch_bounds__(kVjpThreads) k_vjp(const __grid_constant__ Epr
 #pragma unroll
     for (int s = 0; s < NSM; ++s) cacc[s] = macc[s] = 0.f;
     for (int w = blockIdx.x * (kVjpThreads / 32) + wid; w < A.units; w += gridDim.x * (kVjpThreads / 32)) {
-        const int y0 = (w / A.strips) * kVjpRows, y1 = min(y0 + kVjpRows, ny);
+        const int y0 = (w / A.strips) * A.H, y1 = min(y0 + A.H, ny);
         const int x = (w % A.strips) * 30 - 1 + lane;
         const bool on = x >= 0 && x < nx;                    // on the grid
         const bool own = on && lane >= 1 && lane < 31;       // an output column
@@ -101,36 +110,52 @@ __global__ void __launch_bounds__(kVjpThreads) k_vjp(const __grid_constant__ Epr
             float tb = 0.f, vx = 0.f, vy = 0.f;
             if (on && r >= 0 && r < ny) {
                 const bool mine = own && r >= y0 && r < y1;   // counted in the sums once
+                // the corners of up to four lines are on their way before the
+                // first is used
+                constexpr int K = NSM < 4 ? NSM : 4;
 #pragma unroll
-                for (int s = 0; s < NSM; ++s) {
-                    if (s >= ns) break;
-                    const float cs = C.c[s];
-                    const float ux = cs * gx, uy = cs * gy;
-                    int ix, iy;
-                    const float2 d = floor_frac2(make_float2(ux, uy), ix, iy);
-                    float dx = d.x, dy = d.y;
-                    const int cx = x + ix, cy = r + iy;
-                    float g[4];
-                    if ((unsigned)cx < (unsigned)(nx - 1) && (unsigned)cy < (unsigned)(ny - 1)) {
-                        const float* q = Gb + (size_t)cy * nx + cx;
-                        g[0] = __ldg(q);
-                        g[1] = __ldg(q + 1);
-                        g[2] = __ldg(q + nx);
-                        g[3] = __ldg(q + nx + 1);
-                    } else {
-                        vjp_corners(Gb, r, x, uy, ux, ny, nx, g, dx, dy);
+                for (int s0 = 0; s0 < NSM; s0 += K) {
+                    if (NSM > 4 && s0 >= ns) break;
+                    float g[K][4], dxs[K], dys[K];
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        if (NSM > 4 && s0 + k >= ns) break;
+                        const float cs = C.c[s0 + k];
+                        const float ux = cs * gx, uy = cs * gy;
+                        int ix, iy;
+                        const float2 d = floor_frac2(make_float2(ux, uy), ix, iy);
+                        dxs[k] = d.x;
+                        dys[k] = d.y;
+                        const int cx = x + ix, cy = r + iy;
+                        if ((unsigned)cx < (unsigned)(nx - 1) && (unsigned)cy < (unsigned)(ny - 1)) {
+                            const float* q = Gb + (cy * nx + cx);
+                            g[k][0] = __ldg(q);
+                            g[k][1] = __ldg(q + 1);
+                            g[k][2] = __ldg(q + nx);
+                            g[k][3] = __ldg(q + nx + 1);
+                        } else {
+                            vjp_corners(Gb, r, x, uy, ux, ny, nx, g[k], dxs[k], dys[k]);
+                        }
                     }
-                    const float a = (1.f - dy) * ((1.f - dx) * g[0] + dx * g[1]) +
-                                    dy * ((1.f - dx) * g[2] + dx * g[3]);
-                    const float Is = C.f[s] * __expf(-C.mu[s] * tc);
-                    const float ubx = Is * ((1.f - dy) * (g[1] - g[0]) + dy * (g[3] - g[2]));
-                    const float uby = Is * ((1.f - dx) * (g[2] - g[0]) + dx * (g[3] - g[1]));
-                    tb += -C.mu[s] * Is * a;
-                    vx += cs * ubx;
-                    vy += cs * uby;
-                    if (mine) {
-                        cacc[s] += ubx * gx + uby * gy;
-                        macc[s] += -tc * Is * a;
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        if (NSM > 4 && s0 + k >= ns) break;
+                        const int s = s0 + k;
+                        const float cs = C.c[s], dx = dxs[k], dy = dys[k];
+                        const float m = C.mu[s], Is = C.f[s] * __expf(-m * tc), ci = cs * Is;
+                        // the bilinear patch g00 + dx ex + dy ey + dx dy xy:
+                        // its value and its slopes, from differences of gbar
+                        const float g00 = g[k][0], ex = g[k][1] - g00, ey = g[k][2] - g00;
+                        const float xy = (g[k][3] - g[k][2]) - ex;
+                        const float slx = ex + dy * xy, sly = ey + dx * xy;
+                        const float Ia = Is * (g00 + dx * ex + dy * sly);
+                        tb -= m * Ia;
+                        vx += ci * slx;
+                        vy += ci * sly;
+                        if (mine) {
+                            cacc[s] += Is * (slx * gx + sly * gy);
+                            macc[s] -= tc * Ia;
+                        }
                     }
                 }
             }
@@ -184,11 +209,11 @@ __global__ void __launch_bounds__(256) k_vjp_sum(const double* part, int nblk, i
 
 }  // namespace
 
-// Doubles of workspace: the block partials, then the sums ([batch][2 ns]).
-size_t epr_vjp_part_len(int ns, int batch) { return (size_t)batch * (kVjpMaxBlocks + 1) * 2 * ns; }
+// Doubles of workspace: the block partials.
+size_t epr_vjp_part_len(int ns, int batch) { return (size_t)batch * kVjpMaxBlocks * 2 * ns; }
 
-// The gradient, and with `sums` (device, [batch][2 ns]: cbar_s, mubar_s) the
-// scalars.
+// The gradient, and with `sums` ([batch][2 ns]: cbar_s, mubar_s; pinned host
+// memory that the kernel writes itself) the scalars.
 cudaError_t epr_launch_vjp(const EprConsts& C, const float* T, const float* gbar, float* Tbar,
                            double* part, double* sums, int batch, cudaStream_t stream)
 {
@@ -198,12 +223,20 @@ cudaError_t epr_launch_vjp(const EprConsts& C, const float* T, const float* gbar
     A.Tbar = Tbar;
     A.part = part;
     A.strips = (C.nx + 29) / 30;
-    A.units = A.strips * ((C.ny + kVjpRows - 1) / kVjpRows);
+    // strips of 8 to 32 rows, as high as gives every resident warp (4 blocks
+    // per SM) one: a strip's rows are a serial chain of gathers, and each
+    // strip computes two more rows than it writes.  1536 x 1024, 3 lines:
+    // 11 rows 34.5 us, 22 rows 47.9, 16 rows 39.4 (before the shared slopes)
+    const long long rows = ((long long)A.strips * C.ny * batch + kVjpSlots - 1) / kVjpSlots;
+    A.H = (int)std::min(32LL, std::max(8LL, rows));
+    A.units = A.strips * ((C.ny + A.H - 1) / A.H);
     int nblk = (A.units + kVjpThreads / 32 - 1) / (kVjpThreads / 32);
     if (nblk > kVjpMaxBlocks) nblk = kVjpMaxBlocks;
     const dim3 grid(nblk, batch), blk(kVjpThreads);
     if (C.ns == 1) k_vjp<1><<<grid, blk, 0, stream>>>(C, A);
-    else if (C.ns <= 4) k_vjp<4><<<grid, blk, 0, stream>>>(C, A);
+    else if (C.ns == 2) k_vjp<2><<<grid, blk, 0, stream>>>(C, A);
+    else if (C.ns == 3) k_vjp<3><<<grid, blk, 0, stream>>>(C, A);
+    else if (C.ns == 4) k_vjp<4><<<grid, blk, 0, stream>>>(C, A);
     else if (C.ns <= 8) k_vjp<8><<<grid, blk, 0, stream>>>(C, A);
     else k_vjp<16><<<grid, blk, 0, stream>>>(C, A);
     epr_count_launch(1);

@@ -263,19 +263,22 @@ def test_oversampled_split_factors(torch, E, oracle, os_, lines):
         assert rel(host(T), Tref) <= 2e-5
 
 
-@pytest.mark.parametrize("nx,ny", [(16, 16), (24, 32), (32, 72), (64, 96), (96, 48)])
-@pytest.mark.parametrize("lines", [1, 3, 5])
-def test_gradient_at_strip_edges(torch, E, oracle, nx, ny, lines):
+# strips of 8 rows, then of 19 (the last cut short) and of 32
+@pytest.mark.parametrize("nx,ny,batch,lines", [(nx, ny, 2, n) for nx, ny in
+                                               [(16, 16), (24, 32), (32, 72), (64, 96), (96, 48)]
+                                               for n in (1, 2, 3, 4, 5)] +
+                         [(1024, 512, 5, 2), (1024, 512, 10, 1), (1024, 512, 10, 4)])
+def test_gradient_at_strip_edges(torch, E, oracle, nx, ny, batch, lines):
     Es, d, b, w = spec(lines)
     ln = oracle.Lines(Es, d, b, w, L, PIXEL)
     tau = phantom(ny, nx)
     g = ph.rng(7).normal(size=(ny, nx)).astype(np.float32)
     Tb, db, bb, lb = oracle.vjp(ln, tau, g)
     with E.Plan(nx, ny, PIXEL, L, Es, d, b, w) as p:
-        T, gd = cuda(torch, np.stack([tau, tau])), cuda(torch, np.stack([g, g]))
+        T, gd = cuda(torch, np.stack([tau] * batch)), cuda(torch, np.stack([g] * batch))
         out = torch.empty_like(T)
-        gdb, gbb, glb = E.epr_vjp(p.handle, T, gd, out, lines, batch=2)
-    assert rel(host(out), np.stack([Tb, Tb])) <= 1e-5
-    for k in range(2):
+        gdb, gbb, glb = E.epr_vjp(p.handle, T, gd, out, lines, batch=batch)
+    assert rel(host(out), np.stack([Tb] * batch)) <= 1e-5
+    for k in range(batch):
         for a, ref in ((gdb[k], db), (gbb[k], bb), (glb[k:k + 1], [lb])):
             assert np.allclose(a, ref, rtol=1e-3, atol=1e-5 * np.abs(np.asarray(ref)).max())
