@@ -337,6 +337,20 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
+// Rows of a strip for a kernel whose warps march down strips of columns: at
+// most `most` (the higher a strip, the smaller its halo's share), at least
+// `least`, and so that the strips of all projections fill the `slots` warps
+// that are resident at a time a whole number of times.
+inline int epr_strip_rows(int strips, int ny, int batch, int slots, int least, int most)
+{
+    const long long rows = (long long)strips * ny * batch;
+    const long long warps = slots * ((rows + (long long)slots * most - 1) / ((long long)slots * most));
+    int h = (int)((rows + warps - 1) / warps);
+    if (h < least) h = least;
+    while (h < most && (long long)strips * ((ny + h - 1) / h) * batch > warps) ++h;
+    return h;
+}
+
 // Kernel launch with the programmatic attribute when `pdl` is set.
 template <typename... KArgs, typename... Args>
 inline cudaError_t epr_launch_kernel(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block,

@@ -29,6 +29,8 @@
 namespace {
 
 constexpr int kStencilThreads = 128;
+constexpr int kStencilBlocks = 7;   // per SM: 72 registers a thread
+constexpr int kStencilSlots = 152 * kStencilBlocks * (kStencilThreads / 32);   // resident warps
 
 enum { ST_LOCAL1 = 1, ST_LOCAL2 = 2, ST_WKB1 = 3 };
 
@@ -81,7 +83,7 @@ struct Rows3 {
 };
 
 template <int MODE, bool DET>
-__global__ void __launch_bounds__(kStencilThreads, 7) k_stencil(const EprConsts C, const StencilArgs A)
+__global__ void __launch_bounds__(kStencilThreads, kStencilBlocks) k_stencil(const EprConsts C, const StencilArgs A)
 {
     constexpr int HALO = MODE == ST_LOCAL1 ? 2 : 3, OUT = 32 - 2 * HALO;
     constexpr bool PRESSURE = MODE != ST_LOCAL1, LOCAL = MODE != ST_WKB1;
@@ -220,10 +222,12 @@ cudaError_t launch_stencil(const EprConsts& C, StencilArgs& A, int batch, cudaSt
 {
     constexpr int OUT = MODE == ST_LOCAL1 ? 28 : 26;
     A.strips = (C.nx + OUT - 1) / OUT;
-    // 32 rows per strip (19 % of the rows computed are halo); fewer where that
-    // would leave under 8 warps per SM, since a strip's rows are a serial chain
-    A.H = 32;
-    while (A.H > 4 && (long long)A.strips * ((C.ny + A.H - 1) / A.H) * batch < 152 * 8) A.H /= 2;
+    // Strips that fill the resident warps a whole number of times.  One frame
+    // of 2048 x 2048 (39 rows and one wave; 32 rows made 1.2), ten second-order
+    // iterations: 1218 -> 1098 us; four of 1024 x 1024 (41 rows; 1.2 waves
+    // before), 20 iterations of order 2: 2053 -> 1870 us.  At most 48 rows: 64
+    // measured the same, 32 and 24 1.7 % slower per solve.
+    A.H = epr_strip_rows(A.strips, C.ny, batch, kStencilSlots, 4, 48);
     const int warps = A.strips * ((C.ny + A.H - 1) / A.H);
     const dim3 grid((warps * 32 + kStencilThreads - 1) / kStencilThreads, 1, batch);
     const cudaError_t e = epr_launch_kernel(C.pdl != 0, k_stencil<MODE, DET>, grid, dim3(kStencilThreads), 0,

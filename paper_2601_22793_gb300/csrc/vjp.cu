@@ -24,8 +24,6 @@
 // are therefore loaded before the first is used, and the strips are cut so
 // that every resident warp has one.  1536 x 1024, 3 lines: 56 -> 34.5 us from
 // both, with the slopes taken from shared differences.
-#include <algorithm>
-
 #include "epr_internal.cuh"
 
 namespace {
@@ -223,12 +221,10 @@ cudaError_t epr_launch_vjp(const EprConsts& C, const float* T, const float* gbar
     A.Tbar = Tbar;
     A.part = part;
     A.strips = (C.nx + 29) / 30;
-    // strips of 8 to 32 rows, as high as gives every resident warp (4 blocks
-    // per SM) one: a strip's rows are a serial chain of gathers, and each
-    // strip computes two more rows than it writes.  1536 x 1024, 3 lines:
-    // 11 rows 34.5 us, 22 rows 47.9, 16 rows 39.4 (before the shared slopes)
-    const long long rows = ((long long)A.strips * C.ny * batch + kVjpSlots - 1) / kVjpSlots;
-    A.H = (int)std::min(32LL, std::max(8LL, rows));
+    // a strip's rows are a serial chain of gathers, and each strip computes two
+    // more rows than it writes.  1536 x 1024, 3 lines: 11 rows (one strip per
+    // resident warp) 34.5 us, 22 rows 47.9
+    A.H = epr_strip_rows(A.strips, C.ny, batch, kVjpSlots, 8, 32);
     A.units = A.strips * ((C.ny + A.H - 1) / A.H);
     int nblk = (A.units + kVjpThreads / 32 - 1) / (kVjpThreads / 32);
     if (nblk > kVjpMaxBlocks) nblk = kVjpMaxBlocks;

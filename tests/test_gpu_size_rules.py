@@ -165,8 +165,9 @@ def test_forward_of_overlapping_maps(torch, E):
         assert torch.equal(buf[:2], Ps)
 
 
-# strips of 26 (28) and 30 columns, of 16 and 32 rows
-@pytest.mark.parametrize("nx,ny", [(16, 16), (24, 48), (32, 24), (64, 32), (96, 72), (144, 16), (288, 96)])
+# strips of 26 (28) columns, of 4 rows, then of 15 and of 43 (the last cut short)
+@pytest.mark.parametrize("nx,ny", [(16, 16), (24, 48), (32, 24), (64, 32), (96, 72), (144, 16), (288, 96),
+                                   (1024, 768), (2048, 1152)])
 @pytest.mark.parametrize("lines", [1, 3])
 @pytest.mark.parametrize("model", [1, 2, 3])
 def test_stencils_at_strip_edges(torch, E, oracle, nx, ny, lines, model):
