@@ -380,22 +380,31 @@ struct ProfScope {
     }
 };
 
-// The splat tile of a launch.  The default 64 x 64 tile has the smallest halo
-// (1.27 scanned sources per pixel at reach 4, 1.56 for 32 x 32), but a launch
-// with fewer of them than four per SM leaves SMs idle or with too few warps
-// to hide their latency; it takes 32 x 32 tiles.  Solve iteration of one line:
-// 256^2 30.0 -> 27.0 us, 512^2 30.3 -> 27.7, 1024^2 (256 large tiles) 42.8 ->
-// 38.8; 2048^2 (1024 large tiles) 70.7 with the large ones, 74.0 with the
-// small.  A tuned plan keeps the choice of its tuner.
-constexpr int kSplatMinTiles = 608;
-
+// The splat tile of a launch: the largest of the plan's default, 32 x 64 and
+// 32 x 32 whose blocks fill 4/5 of the resident ones (five per SM with one
+// line, two with several).  A larger tile scans a smaller halo (1.27 sources
+// per pixel for 64 x 64 at reach 4, 1.41 and 1.56), but too few blocks leave
+// SMs idle or with too few warps to hide their latency.  Solve iterations, us,
+// with 64 x 64, 32 x 64 and 32 x 32 tiles:
+//   one line      512^2 27.7 in place of 30.3 (32 x 32 for 64 x 64)
+//                 1024^2 33.9, 29.3, 29.0    1536 x 1024 40.5, 37.4, 38.0
+//                 2048^2 70.7, 71.6, 74.0
+//   several lines 512^2 (4) 37.5, 29.9, 28.6  768^2 (2) 39.8, 36.1, 37.1
+//                 1024^2 (2) 46.7, 47.8, 49.4
+//                 512^2 (8) -, 50.9, 44.6     768^2 (8) -, 91.7, 91.9
+// A tuned plan keeps the choice of its tuner, and reaches above 8 (where the
+// small tiles' halo is several times the tile) the default.
 void splat_tile(const epr_plan_s* p, int batch, int* TH, int* TW)
 {
     *TH = p->splat_TH;
     *TW = p->splat_TW;
-    if (p->tuned || *TH != 64 || *TW != 64) return;
-    const long long tiles = (long long)((p->C.nx + 63) / 64) * ((p->C.ny + 63) / 64) * batch;
-    if (tiles < kSplatMinTiles) *TH = *TW = 32;
+    if (p->tuned || p->C.smax > 8) return;
+    const long long least = (p->C.ns == 1 ? 5 : 2) * 152 * 4 / 5;
+    auto fills = [&](int h, int w) {
+        return (long long)((p->C.nx + w - 1) / w) * ((p->C.ny + h - 1) / h) * batch >= least;
+    };
+    if (*TH == 64 && !fills(64, 64)) *TH = 32;
+    if (*TH == 32 && *TW == 64 && !fills(32, 64)) *TW = 32;
 }
 
 // One pass of the chosen forward model writing W.P (and W.Ps / W.Pq / W.Psq).

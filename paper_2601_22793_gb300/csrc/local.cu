@@ -224,7 +224,7 @@ cudaError_t launch_stencil(const EprConsts& C, StencilArgs& A, int batch, cudaSt
     A.strips = (C.nx + OUT - 1) / OUT;
     // Strips that fill the resident warps a whole number of times.  One frame
     // of 2048 x 2048 (39 rows and one wave; 32 rows made 1.2), ten second-order
-    // iterations: 1218 -> 1098 us; four of 1024 x 1024 (41 rows; 1.2 waves
+    // iterations: 1218 -> 1098 us; four of 1024 x 1024 (40 rows; 1.2 waves
     // before), 20 iterations of order 2: 2053 -> 1870 us.  At most 48 rows: 64
     // measured the same, 32 and 24 1.7 % slower per solve.
     A.H = epr_strip_rows(A.strips, C.ny, batch, kStencilSlots, 4, 48);

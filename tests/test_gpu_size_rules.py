@@ -165,6 +165,23 @@ def test_forward_of_overlapping_maps(torch, E):
         assert torch.equal(buf[:2], Ps)
 
 
+# one line: 304 and 608 blocks are the fewest of 32 x 64 and 64 x 64 tiles;
+# several: 243.  Sizes on both sides of each line, and a ragged last tile.
+@pytest.mark.parametrize("nx,ny,batch,lines,fixed", [(1024, 576, 2, 1, False), (1152, 1152, 1, 1, False),
+                                                     (1152, 1152, 2, 1, True), (1536, 1296, 1, 3, False),
+                                                     (512, 512, 1, 2, False), (768, 648, 1, 2, True),
+                                                     (512, 512, 1, 8, False), (1024, 576, 1, 8, False)])
+def test_forward_tile_shapes(torch, E, oracle, nx, ny, batch, lines, fixed):
+    Es, d, b, w = spec(lines)
+    tau = phantom(ny, nx)
+    P, _, _ = oracle.forward(oracle.Lines(Es, d, b, w, L, PIXEL), tau, per_line=True)
+    with E.Plan(nx, ny, PIXEL, L, Es, d, b, w, deterministic=fixed) as p:
+        T = cuda(torch, np.stack([tau] * batch))
+        Pd = torch.empty_like(T)
+        E.epr_forward(p.handle, T, Pd, batch=batch)
+        assert rel(host(Pd), np.stack([P] * batch)) <= 2e-6
+
+
 # strips of 26 (28) columns, of 4 rows, then of 15 and of 43 (the last cut short)
 @pytest.mark.parametrize("nx,ny", [(16, 16), (24, 48), (32, 24), (64, 32), (96, 72), (144, 16), (288, 96),
                                    (1024, 768), (2048, 1152)])
