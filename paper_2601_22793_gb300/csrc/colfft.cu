@@ -176,8 +176,13 @@ const ColKernels* col_kernels(int ny)
 size_t col_tma_smem(int ny, int cw) { return 128 + (size_t)PC::len(ny * cw) * sizeof(float2); }
 
 // Launches with fewer wide tiles than this take the two-column tile: twice the
-// blocks, half the work in each.
-constexpr int kColMinBlocks = 304;
+// blocks, half the work in each, but a row of it is 16 bytes, half a sector.
+// Solve iterations, us, with wide and two-column tiles (wide tiles in
+// parentheses): 1024 rows 512 x 1024 (64) 22.7, 21.3; 1024^2 (128) 28.2, 28.9;
+// two of 1152 x 1728 (288) 70.7, 75.7; eight of 1024^2 (1024) 116, 121.  512
+// rows (512) 42.5, 40.8, (1024) 68.3, 67.3, (4096) 222, 226; 864 rows (256)
+// 41.3, 39.2; 256 rows (64) 16.7, 15.8, (1024) 46.2, 46.2, (8192) 253, 265.
+constexpr int col_wide_blocks(int ny) { return ny >= 1024 ? 128 : 1024; }
 
 }  // namespace
 
@@ -214,7 +219,8 @@ bool epr_col_make_map(const EprConsts& C, const float2* S, long long rows, CUten
     return true;
 }
 
-// rho_it >= 0 (a solve): block 0 also forms rho of iteration rho_it from the
+// rho_it >= 0 (a solve): a further block (block 0 of the passes without bulk
+// copies) forms rho of iteration rho_it from the
 // forward row pass's partials.
 cudaError_t epr_launch_col(const EprConsts& C, const EprWork& W, int line0, int nl, int batch,
                            int check_done, int cw_hint, int rho_it, cudaStream_t stream)
@@ -246,7 +252,7 @@ cudaError_t epr_launch_col(const EprConsts& C, const EprWork& W, int line0, int 
         const ColKernels& k = *col_kernels(C.ny);
         const CUtensorMap* maps = static_cast<const CUtensorMap*>(W.col_map);
         const bool r8 = k.radix8 && !W.col_radix16, o5 = k.occ5 && W.col_occ5;
-        const bool narrow = k.narrow && (long long)(C.half / k.cw) * nl * batch < kColMinBlocks;
+        const bool narrow = k.narrow && (long long)(C.half / k.cw) * nl * batch < col_wide_blocks(C.ny);
         const int cw = narrow ? 2 : k.cw;
         A.CW = cw;
         A.lgCW = cw == 2 ? 1 : 2;

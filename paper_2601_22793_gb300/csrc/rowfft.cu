@@ -382,10 +382,15 @@ void each_table(F f)
     }
 }
 
-// A block of several row pairs (256 threads) needs at least this many blocks
-// to be worth it; below, one pair per block spreads the rows over more SMs
-// (152).
-constexpr int kRowMinBlocks = 304;
+// Lengths up to 512 have blocks of several row pairs (96 to 128 threads) and of
+// one.  Fewer blocks of several than this (four per SM) leave SMs idle or with
+// too few warps: one pair per block is then the faster.  Solve iterations, us,
+// with several pairs and with one: 256^2 18.4, 15.1; 16 of 256^2 (512 blocks)
+// 29.8, 27.8; 32 (1024) 42.6, 44.1; four of 512^2 (512) 27.5, 26.6; 64 (8192)
+// 217, 243; eight of 384^2 (768) 34.3, 35.9.  Longer rows are one pair per
+// block at every count: two pairs (256 threads) took 115 for eight of 1024^2
+// where one takes 110, and 796 where it takes 697 for 16 of four lines.
+constexpr int kRowMinBlocks = 608;
 
 }  // namespace
 
@@ -395,19 +400,22 @@ struct EprRowLaunch {
     const RowKernels* k;    // compile-time kernels of this length and RP, or NULL
 };
 
-EprRowLaunch epr_row_config(const EprConsts& C, int batch)
+// solve: the passes of an iteration (of a plan with an x-dependent spectrum,
+// which not every length has compile-time kernels for).
+EprRowLaunch epr_row_config(const EprConsts& C, int batch, bool solve)
 {
     EprRowLaunch L = {};
-    int rp = 1;
-    while (rp * 2 * C.nx <= 2048 && (C.ny / 2) % (rp * 2) == 0) rp *= 2;
     const RowKernels *many = nullptr, *one = nullptr;
     each_table([&](const RowKernels& k) {
         if (k.nx != C.nx) return;
-        if (k.rp == rp && rp > 1) many = &k;
+        if (k.rp > 1 && (C.ny / 2) % k.rp == 0) many = &k;
         if (k.rp == 1) one = &k;
     });
-    if (many && (long long)(C.ny / (2 * rp)) * batch >= kRowMinBlocks) L.k = many;
+    int rp = 1;   // of the runtime-sized kernels
+    while (rp * 2 * C.nx <= 2048 && (C.ny / 2) % (rp * 2) == 0) rp *= 2;
+    if (many && (long long)(C.ny / (2 * many->rp)) * batch >= kRowMinBlocks) L.k = many;
     else if (one) L.k = one;
+    if (solve && C.xt && L.k && !L.k->xfwd1) L.k = nullptr;
     L.RP = L.k ? L.k->rp : rp;
     L.lgRP = 0;
     while ((1 << L.lgRP) < L.RP) ++L.lgRP;
@@ -427,7 +435,7 @@ cudaError_t epr_launch_row_fwd(const EprConsts& C, const EprWork& W, int mode, c
                                const float* D, const float* G, int line0, int nl, int it,
                                float tol, int batch, int check_done, cudaStream_t stream)
 {
-    const EprRowLaunch L = epr_row_config(C, batch);
+    const EprRowLaunch L = epr_row_config(C, batch, mode != FWD_LOAD);
     RowArgs A = {};
     A.T = T; A.D = D; A.G = mode == FWD_LOAD ? G : nullptr;
     A.P = W.P; A.Ps = W.Ps; A.Pq = W.Pq; A.Psq = W.Psq;
@@ -485,7 +493,7 @@ cudaError_t epr_launch_row_inv(const EprConsts& C, const EprWork& W, int mode, f
                                int line0, int nl, int it, float omega, float eps, float tol,
                                int batch, int check_done, cudaStream_t stream)
 {
-    const EprRowLaunch L = epr_row_config(C, batch);
+    const EprRowLaunch L = epr_row_config(C, batch, mode == INV_UPDATE);
     RowArgs A = {};
     A.Out = Out; A.S = W.S; A.st = W.st; A.part_a = W.part_a; A.part_b = W.part_b;
     A.hist_len = W.hist_len; A.max_blocks = W.max_blocks;
@@ -545,7 +553,7 @@ cudaError_t epr_launch_solve_begin(const EprConsts& C, const EprWork& W, const f
 }
 
 // Blocks of a row pass (the number of partials a reduction adds up).
-int epr_row_blocks(const EprConsts& C, int batch) { return C.ny / (2 * epr_row_config(C, batch).RP); }
+int epr_row_blocks(const EprConsts& C, int batch) { return C.ny / (2 * epr_row_config(C, batch, true).RP); }
 
 namespace {
 

@@ -14,8 +14,7 @@ constexpr RowKernels k2048()
 }
 
 const RowKernels kTable[] = {
-    row_full_xt<1024, 2>(),
-    row_any<1024, 1>(),
+    row_full_xt<1024, 1>(),
     k2048(),
 };
 

@@ -5,13 +5,11 @@
 namespace {
 
 const RowKernels kTable[] = {
-    row_any<144, 8>(),
+    row_any<144, 4>(),
     row_any<192, 1>(),
-    row_any<288, 4>(),
+    row_any<288, 2>(),
     row_any<384, 1>(),
-    row_any<576, 2>(),
     row_any<648, 1>(),
-    row_any<864, 2>(),
     row_full<1296, 1>(),
     row_full<2304, 1>(),
     row_full<3888, 1>(),

@@ -6,11 +6,10 @@ namespace {
 
 const RowKernels kTable[] = {
     row_any<144, 1>(),
-    row_any<216, 8>(),
+    row_any<216, 4>(),
     row_any<288, 1>(),
-    row_any<432, 4>(),
+    row_any<432, 2>(),
     row_any<576, 1>(),
-    row_any<768, 2>(),
     row_any<864, 1>(),
     row_full<1728, 1>(),
     row_full<2592, 1>(),

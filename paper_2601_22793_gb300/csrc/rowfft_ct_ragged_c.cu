@@ -5,12 +5,11 @@
 namespace {
 
 const RowKernels kTable[] = {
-    row_any<192, 8>(),
+    row_any<192, 4>(),
     row_any<216, 1>(),
-    row_any<384, 4>(),
+    row_any<384, 2>(),
     row_any<432, 1>(),
-    row_any<648, 2>(),
-    row_any<768, 1>(),
+    row_full<768, 1>(),
     row_full<1152, 1>(),
     row_full<1944, 1>(),
     row_full<3456, 1>(),

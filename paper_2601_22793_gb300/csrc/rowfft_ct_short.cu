@@ -5,11 +5,11 @@
 namespace {
 
 const RowKernels kTable[] = {
-    row_full<256, 8>(),
+    row_full<256, 4>(),
     row_any<256, 1, 4>(),
-    row_full<512, 4>(),
+    row_full<512, 2>(),
     row_any<512, 1, 4>(),
-    row_any<128, 16>(),
+    row_any<128, 8>(),
     row_any<128, 1, 4>(),
 };
 

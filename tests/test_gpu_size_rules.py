@@ -86,7 +86,7 @@ def test_precondition_every_length(torch, E, n, axis):
 
 # few blocks (one row pair each, narrow column tiles) and many of each length
 @pytest.mark.parametrize("nx,ny,lines", [(128, 48, 1), (144, 96, 2), (216, 24, 1), (256, 64, 1), (288, 72, 3),
-                                         (512, 32, 2), (648, 48, 1), (1024, 16, 1), (1296, 24, 1),
+                                         (512, 32, 2), (512, 512, 1), (648, 48, 1), (1024, 16, 1), (72, 1024, 2), (1296, 24, 1),
                                          (2048, 16, 1), (2304, 16, 2), (3456, 24, 1), (3888, 16, 2)])
 def test_solve_few_and_many_blocks(torch, E, oracle, nx, ny, lines):
     Es, d, b, w = spec(lines)
@@ -95,9 +95,9 @@ def test_solve_few_and_many_blocks(torch, E, oracle, nx, ny, lines):
     D = ph.poisson(oracle.forward(ln, tau), 1e4, 3).astype(np.float32)
     Tref, info = oracle.solve(ln, D.astype(np.float64), n_iter=3, omega=0.4)
     rp = 1   # row pairs of a large block, and the batch that fills the GPU with them
-    while 2 * rp * nx <= 2048 and (ny // 2) % (2 * rp) == 0:
+    while 2 * rp * nx <= 1152 and nx <= 512 and (ny // 2) % (2 * rp) == 0:
         rp *= 2
-    many = 304 // (ny // (2 * rp)) + 1 if rp > 1 else 3
+    many = 608 // (ny // (2 * rp)) + 1 if rp > 1 else 3
     for batch in (1, many):
         with E.Plan(nx, ny, PIXEL, L, Es, d, b, w) as p:
             Dd = cuda(torch, np.repeat(D[None], batch, 0))
