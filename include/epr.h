@@ -116,9 +116,9 @@ typedef struct {
                               maps, and epr_vjp and the batch API are not
                               available (EPR_ERR_INVALID_ARG). */
     int fft_radix;         /* largest radix of the column transforms: 0 = the
-                              default (8; with autotune the tuner may pick 16),
-                              8, or 16 (radix-16 stages where the 2048-row
-                              bulk-copy column pass has them).  Changes only
+                              default (16; with autotune the tuner may pick 8),
+                              8, or 16, for the 2048-row bulk-copy column pass
+                              (other lengths have one plan).  Changes only
                               the rounding of the preconditioner. */
     int reserved[4];       /* must be zero */
 } epr_options;

@@ -22,7 +22,7 @@ struct ColArgs {
     int CW, lgCW;
     int line0, nl;
     int check_done;
-    int rho_it;           // >= 0: block 0 forms rho of this iteration
+    int rho_it;           // >= 0: form rho of this iteration
     int nblk, max_blocks, hist_len;
     int kind;             // symbol of the generic pass: 0 = H = 1 / (1 + a),
                           // 1, 2 = kscale a / (1 + a)^2 (the derivatives of

@@ -14,8 +14,9 @@
 //   epilogue  unpack X0[k] = (Z[k] + conj Z[-k]) / 2, X1[k] = (Z[k] -
 //             conj Z[-k]) / 2i and store k < nx/2 with the real Nyquist
 //             value packed into the imaginary part of k = 0.
-// The block also stores its share of |D - P|^2; block 0 of the column pass
-// that follows adds the shares in a fixed order (deterministic) into rho.
+// The block also stores its share of |D - P|^2; a block of its own of the
+// column pass that follows adds the shares in a fixed order (deterministic)
+// into rho.
 //
 // Inverse row pass (C2R), the mirror image, fused with the update
 // ("Iterative inversion"): per line, I'_s = max(I_s + omega h_s, eps f_s),
@@ -23,8 +24,8 @@
 //   T' = - sum_s f_s mu_s ln(I'_s / f_s) / sum_s f_s mu_s^2,
 // evaluated as T' = T - sum_s w_s ln(1 + omega h_s / I_s) (w_s = f_s mu_s /
 // sum f mu^2), the same quantity without forming exp then log of values
-// near one.  Each block stores its shares of |T' - T|^2 and |T'|^2; block 0
-// of the next forward row pass (or a one-block kernel after the last
+// near one.  Each block stores its shares of |T' - T|^2 and |T'|^2; a block of
+// its own of the next forward row pass (or a one-block kernel after the last
 // iteration) adds them in a fixed order into kappa and retires the
 // projection when kappa <= tol.
 #include <mutex>
@@ -47,36 +48,15 @@ enum { INV_UPDATE = 0, INV_STORE = 1 };
 
 __device__ __forceinline__ int fdiv(int i, float inv_d) { return (int)(((float)i + 0.5f) * inv_d); }
 
-template <bool DET>
-__device__ __forceinline__ float ldP(const float* P, const unsigned long long* Pq, size_t i)
+// split residual of line s at detector pixel q of projection b (pb = b * npix)
+__device__ __forceinline__ float resid(const EprConsts& C, const RowArgs& A, size_t pb, size_t q, int s)
 {
-    if constexpr (DET) return (float)__ldg(&Pq[i]) * EPR_FX_INV;
-    else return __ldg(&P[i]);
-}
-
-// residual of line s at detector pixel q of projection b (pb = b * npix)
-template <bool DET, bool RESID>
-__device__ __forceinline__ float resid(const EprConsts& C, const RowArgs& A, size_t pb, size_t q,
-                                       int s)
-{
-    if constexpr (RESID) {   // the split residuals of the splat / split kernels
-        if (C.ns == 1) return __ldg(&A.P[pb + q]);
-        return __ldg(&A.Ps[pb * C.ns + (size_t)s * C.nx * C.ny + q]);
-    } else {
-        const float d = __ldg(&A.D[pb + q]);
-        const float p = ldP<DET>(A.P, A.Pq, pb + q);
-        const float r = d - p;
-        if (C.ns == 1) return r;
-        const size_t npix = (size_t)C.nx * C.ny;
-        const size_t ps = pb * C.ns + (size_t)s * npix + q;
-        const float pl = ldP<DET>(A.Ps, A.Psq, ps);
-        return (p > 1e-30f) ? r * (pl / p) : r * line_const(C.f, s);
-    }
+    if (C.ns == 1) return __ldg(&A.P[pb + q]);
+    return __ldg(&A.Ps[pb * C.ns + (size_t)s * C.nx * C.ny + q]);
 }
 
 // bilinear gather of line s's residual at (y + uy, x + ux); corners outside
 // the grid read 0 (Eq. 4)
-template <bool DET, bool RESID>
 __device__ __forceinline__ float gather_px(const EprConsts& C, const RowArgs& A, size_t pb, int y,
                                            int x, float uy, float ux, int s)
 {
@@ -91,13 +71,13 @@ __device__ __forceinline__ float gather_px(const EprConsts& C, const RowArgs& A,
     float r00 = 0.f, r10 = 0.f, r01 = 0.f, r11 = 0.f;
     if ((unsigned)cy < (unsigned)ny) {
         const size_t row = (size_t)cy * nx;
-        if (x0) r00 = resid<DET, RESID>(C, A, pb, row + cx, s);
-        if (x1) r10 = resid<DET, RESID>(C, A, pb, row + cx + 1, s);
+        if (x0) r00 = resid(C, A, pb, row + cx, s);
+        if (x1) r10 = resid(C, A, pb, row + cx + 1, s);
     }
     if ((unsigned)(cy + 1) < (unsigned)ny) {
         const size_t row = (size_t)(cy + 1) * nx;
-        if (x0) r01 = resid<DET, RESID>(C, A, pb, row + cx, s);
-        if (x1) r11 = resid<DET, RESID>(C, A, pb, row + cx + 1, s);
+        if (x0) r01 = resid(C, A, pb, row + cx, s);
+        if (x1) r11 = resid(C, A, pb, row + cx + 1, s);
     }
     const float top = r00 + dx * (r10 - r00);
     const float bot = r01 + dx * (r11 - r01);
@@ -105,7 +85,7 @@ __device__ __forceinline__ float gather_px(const EprConsts& C, const RowArgs& A,
 }
 
 // XT: an x-dependent spectrum, the shift constant read per object column.
-template <int MODE, bool DET, bool RESID, int NS, bool XT = false>
+template <int MODE, int NS, bool XT = false>
 __global__ void __launch_bounds__(512, 2) k_row_fwd(const EprConsts C, const RowArgs A)
 {
     extern __shared__ __align__(16) float2 zs[];
@@ -172,9 +152,9 @@ __global__ void __launch_bounds__(512, 2) k_row_fwd(const EprConsts C, const Row
                     else if (y == ny - 1) gy = t - tr[x - nx];
                     else gy = 0.5f * (tr[nx + x] - tr[x - nx]);
                     const float cs = XT ? xt_get(C, EPR_XT_C, s, x) : line_const(C.c, s);
-                    v[r0] = gather_px<DET, RESID>(C, A, pb, y, x, cs * gy, cs * gx, s);
+                    v[r0] = gather_px(C, A, pb, y, x, cs * gy, cs * gx, s);
                 } else if constexpr (MODE == FWD_SOLVE_LOCAL) {
-                    v[r0] = resid<DET, RESID>(C, A, pb, (size_t)y * nx + x, s);
+                    v[r0] = resid(C, A, pb, (size_t)y * nx + x, s);
                 } else {
                     v[r0] = __ldg(&A.G[pb + (size_t)y * nx + x]);
                 }
@@ -182,8 +162,7 @@ __global__ void __launch_bounds__(512, 2) k_row_fwd(const EprConsts C, const Row
                     if (sl == 0) {
                         const size_t q = (size_t)y * nx + x;
                         float r;
-                        if constexpr (RESID) r = __ldg(&A.P[pb + q]);
-                        else r = __ldg(&A.D[pb + q]) - ldP<DET>(A.P, A.Pq, pb + q);
+                        r = __ldg(&A.P[pb + q]);
                         ra += r * r;
                     }
                 }
@@ -429,7 +408,7 @@ EprRowLaunch epr_row_config(const EprConsts& C, int batch, bool solve)
 
 // mode: 0 = non-local solve, 1 = local solve, 2 = load real map G.
 // FWD_SOLVE_NL reads the residual D - P from P and the split residuals from P_s.
-// In a solve (it > 0) block 0 also finalises kappa of iteration it - 1
+// In a solve (it > 0) a further block finalises kappa of iteration it - 1
 // against tol.
 cudaError_t epr_launch_row_fwd(const EprConsts& C, const EprWork& W, int mode, const float* T,
                                const float* D, const float* G, int line0, int nl, int it,
@@ -438,7 +417,7 @@ cudaError_t epr_launch_row_fwd(const EprConsts& C, const EprWork& W, int mode, c
     const EprRowLaunch L = epr_row_config(C, batch, mode != FWD_LOAD);
     RowArgs A = {};
     A.T = T; A.D = D; A.G = mode == FWD_LOAD ? G : nullptr;
-    A.P = W.P; A.Ps = W.Ps; A.Pq = W.Pq; A.Psq = W.Psq;
+    A.P = W.P; A.Ps = W.Ps;
     A.S = W.S; A.st = W.st; A.part_a = W.part_a; A.part_b = W.part_b; A.part_c = W.part_c;
     A.hist = W.kappa_hist; A.hist_len = W.hist_len; A.max_blocks = W.max_blocks;
     A.tw = W.tw_x; A.RP = L.RP; A.lgRP = L.lgRP; A.line0 = line0; A.nl = nl; A.it = it;
@@ -449,7 +428,7 @@ cudaError_t epr_launch_row_fwd(const EprConsts& C, const EprWork& W, int mode, c
     const bool one = nl == 1, pdl = C.pdl != 0;
     // compile-time kernels: a line per grid z.  The residual D - P is in P
     // and, with several lines, the split residuals in P_s (written by the
-    // splat flush or the split kernel); the local closure back-transports with
+    // splat flush, the long-shift passes or the stencil kernel); the local closure back-transports with
     // the identity.
     RowKernel k = nullptr;
     size_t smem = 0;
@@ -476,14 +455,14 @@ cudaError_t epr_launch_row_fwd(const EprConsts& C, const EprWork& W, int mode, c
         e = epr_launch_kernel(pdl, k, dim3(grid.x + (A.fin ? 1 : 0), grid.y, nl), dim3(threads), smem, stream, C,
                               A);
     } else if (mode == FWD_SOLVE_NL && C.xt) {   // per-column shift constants
-        go(k_row_fwd<FWD_SOLVE_NL, false, true, 0, true>);
+        go(k_row_fwd<FWD_SOLVE_NL, 0, true>);
     } else if (mode == FWD_SOLVE_NL) {
-        if (one) go(k_row_fwd<FWD_SOLVE_NL, false, true, 1>);
-        else go(k_row_fwd<FWD_SOLVE_NL, false, true, 0>);
+        if (one) go(k_row_fwd<FWD_SOLVE_NL, 1>);
+        else go(k_row_fwd<FWD_SOLVE_NL, 0>);
     } else if (mode == FWD_SOLVE_LOCAL) {
-        go(k_row_fwd<FWD_SOLVE_LOCAL, false, true, 0>);
+        go(k_row_fwd<FWD_SOLVE_LOCAL, 0>);
     } else {
-        go(k_row_fwd<FWD_LOAD, false, false, 1>);
+        go(k_row_fwd<FWD_LOAD, 1>);
     }
     epr_count_launch(1);
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -595,14 +574,14 @@ cudaError_t allow_runtime_sized()
 {
     cudaError_t e = cudaSuccess;
     auto allow = [&](auto kernel) { if (e == cudaSuccess) e = epr_allow_max_smem(kernel); };
-    allow(k_row_fwd<FWD_SOLVE_NL, false, true, 1>);
-    allow(k_row_fwd<FWD_SOLVE_NL, false, true, 0>);
-    allow(k_row_fwd<FWD_SOLVE_LOCAL, false, true, 0>);
-    allow(k_row_fwd<FWD_LOAD, false, false, 1>);
+    allow(k_row_fwd<FWD_SOLVE_NL, 1>);
+    allow(k_row_fwd<FWD_SOLVE_NL, 0>);
+    allow(k_row_fwd<FWD_SOLVE_LOCAL, 0>);
+    allow(k_row_fwd<FWD_LOAD, 1>);
     allow(k_row_inv<INV_UPDATE, 1>);
     allow(k_row_inv<INV_UPDATE, 0>);
     allow(k_row_inv<INV_STORE, 1>);
-    allow(k_row_fwd<FWD_SOLVE_NL, false, true, 0, true>);
+    allow(k_row_fwd<FWD_SOLVE_NL, 0, true>);
     allow(k_row_inv<INV_UPDATE, 0, true>);
     return e;
 }

@@ -17,8 +17,6 @@ struct RowArgs {
     const float* D;          // [B][ny][nx]
     const float* P;          // [B][ny][nx]   P, or D - P when `resid`
     const float* Ps;         // [B][ns][ny][nx]
-    const unsigned long long* Pq;   // fixed-point mode
-    const unsigned long long* Psq;
     const float* G;          // [B][ny][nx] real input of a plain transform, else NULL
     float* Out;              // [B][ny][nx] real output (INV_STORE) or T (INV_UPDATE)
     float2* S;               // [B][nl][ny][nx/2]
@@ -32,7 +30,7 @@ struct RowArgs {
     int line0, nl;           // first physical line, number of lines handled
     int it, hist_len, max_blocks;
     int check_done;
-    int fin;                 // forward: block 0 finalises kappa of iteration it - 1
+    int fin;                 // forward: a further block finalises kappa of iteration it - 1
     float omega, eps, tol;
 };
 
