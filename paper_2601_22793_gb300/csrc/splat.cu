@@ -378,7 +378,11 @@ cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* 
     const size_t smem = epr_splat_smem(C, TH, TW);
     dim3 grid((C.nx + TW - 1) / TW, (C.ny + TH - 1) / TH, batch);
     const bool occ6 = W.splat_occ6 != 0;
-    const int resid = D && C.ns == 1 && !C.det && !C.xt;   // its own kernels
+    // one float line: P receives D - P and there is nothing to split, whichever
+    // kernel the tile ran (an x-dependent spectrum has the several-line one)
+    const bool mono = D && C.ns == 1 && !C.det;
+    const int resid = mono && !C.xt;   // its own kernels
+    if (D && !mono && !C.det && (!W.Ps || !W.claim)) return cudaErrorInvalidValue;
     cudaError_t e;
     if (TH == 64 && TW == 64) e = epr_splat_launch_64x64(C, A, resid, occ6, grid, smem, stream);
     else if (TH == 32 && TW == 64) e = epr_splat_launch_32x64(C, A, resid, occ6, grid, smem, stream);
@@ -397,8 +401,9 @@ cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* 
         else go(k_splat_overflow<FAR_FX>);
         if (D && C.xt) go(k_overflow_fix<true, true>);
         else if (D) go(k_overflow_fix<true>);
-    } else if (resid) {
-        go(k_splat_overflow<FAR_RESID>);
+    } else if (mono) {
+        if (C.xt) go(k_splat_overflow<FAR_RESID, true>);
+        else go(k_splat_overflow<FAR_RESID>);
     } else if (D) {
         if (C.xt) {
             go(k_splat_overflow<FAR_SPLIT, true>);
