@@ -276,6 +276,10 @@ epr_status ensure_workspace(epr_plan_s* p, int batch, int hist)
     if (e == cudaSuccess) e = cudaMemset(W.err, 0, sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMemset(W.rho_hist, 0, (size_t)nb * nh * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(W.kappa_hist, 0, (size_t)nb * nh * sizeof(double));
+    // the fills run on the default stream, which a non-blocking stream (those of
+    // a batch's size groups among them) does not wait for; a solve relies on the
+    // claim bits being 0 and does not clear them itself
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) {
         free_workspace(p);
         return cuda_status(e);

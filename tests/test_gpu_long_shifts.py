@@ -74,3 +74,27 @@ def test_xspec_solve_with_long_shifts(torch, E, oracle, lines, ny, nx, fixed):
         for k in range(2):
             assert rel(T[k].cpu().numpy(), Tref) <= 2e-5
             assert np.allclose(got["rho_hist"][k], info["rho"], rtol=1e-5)
+
+
+# the size groups of a batch run on streams of their own that do not wait for
+# the default stream: the marks of the first long-shift pass after an
+# allocation must not meet the clearing of the workspace
+def test_first_solve_after_an_allocation(torch, E, oracle):
+    Es, d, b, w = spec(4)
+    ln = oracle.Lines(Es, d, b, w, L, PIXEL)
+    shapes = [(256, 384), (384, 256), (128, 128), (256, 384)]
+    T0s = [phantom(ny, nx, 30 + i) * 2.0 for i, (ny, nx) in enumerate(shapes)]
+    Ds = [ph.poisson(oracle.forward(ln, phantom(ny, nx, 40 + i)), 1e4, i).astype(np.float32)
+          for i, (ny, nx) in enumerate(shapes)]
+    refs = [oracle.solve(ln, D.astype(np.float64), T0=T0, n_iter=1, omega=0.4)[0] for D, T0 in zip(Ds, T0s)]
+    Dd = [cuda(torch, D) for D in Ds]
+    for _ in range(4):
+        bh = E.epr_batch_create(PIXEL, L, Es, d, b, w, max_shift_px=1)
+        try:
+            Ts = [cuda(torch, T0) for T0 in T0s]
+            info = E.epr_solve_nonlocal_batched(bh, Dd, Ts, n_iter=1, omega=0.4, init=1)
+            assert info["overflow_sources"] > 0
+            for T, ref in zip(Ts, refs):
+                assert rel(T.cpu().numpy(), ref) <= 2e-5
+        finally:
+            E.epr_batch_destroy(bh)
