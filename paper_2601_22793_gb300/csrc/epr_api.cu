@@ -263,6 +263,7 @@ epr_status ensure_workspace(epr_plan_s* p, int batch, int hist)
     if (e == cudaSuccess) e = dalloc(p, &W.ovf_mask, (size_t)nb * C.ovf_cap);
     if (e == cudaSuccess) e = dalloc(p, &W.ovf_tg, (size_t)nb * C.ovf_cap);
     const size_t nclaim = C.ns > 1 && !C.det ? ((size_t)nb * npix + 31) / 32 : 0;
+    if (e == cudaSuccess && nclaim) e = dalloc(p, &W.Pnear, (size_t)nb * npix);
     if (e == cudaSuccess && nclaim) e = dalloc(p, &W.claim, nclaim);
     if (e == cudaSuccess && nclaim) e = cudaMemset(W.claim, 0, nclaim * sizeof(unsigned int));
     if (e == cudaSuccess) e = dalloc(p, &W.st, (size_t)nb);

@@ -79,6 +79,7 @@ struct EprWork {
     int* ovf_idx;        // [B][cap] source pixel index
     unsigned int* ovf_mask;   // [B][cap] lines that took the overflow path
     float4* ovf_tg;      // [B][cap] T and twice its gradient (x, y) at the source
+    float* Pnear;        // [B][ny][nx] P without the long shifts (float mode, ns > 1)
     unsigned int* claim; // [B ny nx / 32] pixels that long shifts reached, 0 between
                          //    kernels (float mode, ns > 1)
     EprProjState* st;    // [B]

@@ -42,16 +42,18 @@ __device__ __forceinline__ void far_corners(const EprConsts& C, int pix, unsigne
 }
 
 // The scale in which a pixel's split residuals hold its line predictions.
-// The splat flush of a several-line float solve stores r = D - P and r_s =
-// P_s k with k = r / P (never 0), so P_s = r_s / k, and P comes back as D - r.
-// Where no near source reaches the pixel (P = 0) r_s is r f_s; a contribution
-// is then added 2^20 times, which keeps its digits above those of r f_s.
-constexpr float kDarkScale = 1048576.f;
-__device__ __forceinline__ float far_scale(float d, float r, bool& lit)
+// The splat flush of a several-line float solve stores P (of the near sources),
+// r = D - P and r_s = k P_s with k = r / P (never 0), and a long-shift
+// contribution to P_s is added k times as large.  Where no near source reaches
+// the pixel (P = 0) r_s is r f_s; a contribution is then added 2^64 |r| times,
+// beside which r f_s is rounding error.  P is a map of its own because D - r
+// has lost its digits where D is much larger than P: the relative error of r_s
+// was 3e-4 at D = 1e4 P and of order 1 at D = 2e7 P.
+constexpr float kDarkScale = 18446744073709551616.f;
+__device__ __forceinline__ float far_scale(float r, float p)
 {
-    const float p = d - r;
-    lit = p > 1e-30f;
-    return lit ? split_ratio(r, p) : kDarkScale;
+    if (p > 1e-30f) return split_ratio(r, p);
+    return r != 0.f ? kDarkScale * fabsf(r) : 1.f;
 }
 
 // The long-shift sources of the overflow list, added with global atomics.
@@ -98,9 +100,9 @@ __global__ void __launch_bounds__(128) k_splat_overflow(const __grid_constant__ 
             } else if constexpr (TO == FAR_RESID) {
                 atomicAdd(&A.P[po], -v);
             } else if constexpr (TO == FAR_SPLIT) {
-                bool lit;
-                const float k = far_scale(__ldg(&A.D[po]), A.P[po], lit);
-                atomicAdd(&A.Ps[ps], v * k);
+                const float p = __ldg(&A.Pnear[po]);
+                atomicAdd(&A.Ps[ps], v * far_scale(__ldg(&A.D[po]) - p, p));
+                atomicAdd(&A.P[po], -v);
                 atomicOr(&A.claim[po >> 5], 1u << (po & 31));
             } else {
                 atomicAdd(&A.P[po], v);
@@ -110,13 +112,13 @@ __global__ void __launch_bounds__(128) k_splat_overflow(const __grid_constant__ 
     }
 }
 
-// The residual and its split at the pixels that long-shift sources reached,
-// once they are all in: r = D - P and r_s = r P_s / P (r f_s where P
-// vanishes).  Fixed point forms them anew from the sums (every visitor of a
-// pixel writes the same values); float turns the pixel's split residuals back
-// into P_s, by the one visitor that takes its claim bit.  A few thousand
-// pixels instead of a pass over every map: the separate split of eight lines
-// of a 2048^2 map took 46 us.
+// The split at the pixels that long-shift sources reached, once they are all
+// in: r_s = r P_s / P (r f_s where P vanishes).  Fixed point forms it and r
+// anew from the sums (every visitor of a pixel writes the same values).  Float
+// has r, and the lines' predictions in a common scale (far_scale): their shares
+// are the ratios to their sum.  The one visitor that takes the pixel's claim
+// bit writes them.  A few thousand pixels instead of a pass over every map: the
+// separate split of eight lines of a 2048^2 map took 46 us.
 template <bool DET, bool XT = false>
 __global__ void __launch_bounds__(128) k_overflow_fix(const __grid_constant__ EprConsts C, const SplatArgs A)
 {
@@ -136,9 +138,8 @@ __global__ void __launch_bounds__(128) k_overflow_fix(const __grid_constant__ Ep
             const int x = XT ? (int)(o % (size_t)nx) : 0;
             auto weight = [&](int l) { return XT ? xt_get(C, EPR_XT_F, l, x) : C.f[l]; };
             const float d = __ldg(&A.D[po]);
-            float p = 0.f;
             if constexpr (DET) {
-                p = (float)A.Pq[po] * EPR_FX_INV;
+                const float p = (float)A.Pq[po] * EPR_FX_INV;
                 const float r = d - p, k = p > 1e-30f ? split_ratio(r, p) : r;
                 for (int l = 0; ns > 1 && l < ns; ++l)
                     A.Ps[ps + l * npix] = k * (p > 1e-30f ? (float)A.Psq[ps + l * npix] * EPR_FX_INV : weight(l));
@@ -146,16 +147,17 @@ __global__ void __launch_bounds__(128) k_overflow_fix(const __grid_constant__ Ep
             } else {
                 const unsigned int bit = 1u << (po & 31);
                 if (!(atomicAnd(&A.claim[po >> 5], ~bit) & bit)) return;   // another visitor's
-                bool lit;
-                const float r0 = A.P[po], k0 = far_scale(d, r0, lit);
-                auto line = [&](int l) {   // P_s with the long-shift contributions
+                const float pn = __ldg(&A.Pnear[po]), r = A.P[po];
+                const bool lit = pn > 1e-30f;
+                auto line = [&](int l) {   // the scaled P_s with the long-shift contributions
                     const float v = A.Ps[ps + l * npix];
-                    return lit ? v / k0 : fmaxf((v - r0 * weight(l)) * (1.f / kDarkScale), 0.f);
+                    return lit ? v : fmaxf(__fsub_rn(v, __fmul_rn(d, weight(l))), 0.f);
                 };
-                for (int l = 0; l < ns; ++l) p += line(l);
-                const float r = d - p, k = p > 1e-30f ? split_ratio(r, p) : r;
-                for (int l = 0; l < ns; ++l) A.Ps[ps + l * npix] = k * (p > 1e-30f ? line(l) : weight(l));
-                A.P[po] = r;
+                double sum = 0.0;
+                for (int l = 0; l < ns; ++l) sum += (double)line(l);
+                const float all = (float)sum;
+                const bool any = lit || all > 1e-30f * far_scale(d, 0.f);
+                for (int l = 0; l < ns; ++l) A.Ps[ps + l * npix] = r * (any ? line(l) / all : weight(l));
             }
         });
     }
@@ -355,6 +357,7 @@ cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* 
     A.ovf_tg = W.ovf_tg;
     A.st = W.st;
     A.err = W.err;
+    A.Pnear = W.Pnear;
     A.claim = W.claim;
     A.parity = parity & 1;
     A.check_done = check_done;
@@ -382,7 +385,7 @@ cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* 
     // kernel the tile ran (an x-dependent spectrum has the several-line one)
     const bool mono = D && C.ns == 1 && !C.det;
     const int resid = mono && !C.xt;   // its own kernels
-    if (D && !mono && !C.det && (!W.Ps || !W.claim)) return cudaErrorInvalidValue;
+    if (D && !mono && !C.det && (!W.Ps || !W.Pnear || !W.claim)) return cudaErrorInvalidValue;
     cudaError_t e;
     if (TH == 64 && TW == 64) e = epr_splat_launch_64x64(C, A, resid, occ6, grid, smem, stream);
     else if (TH == 32 && TW == 64) e = epr_splat_launch_32x64(C, A, resid, occ6, grid, smem, stream);

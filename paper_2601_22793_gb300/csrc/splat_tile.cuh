@@ -75,6 +75,8 @@ struct SplatArgs {
     float4* ovf_tg;          // (T, twice the gradient x, y, 0) of each entry
     EprProjState* st;
     unsigned int* err;
+    float* Pnear;            // [B][ny][nx] P without the long shifts (residual output of
+                             //    several float lines)
     unsigned int* claim;     // [B ny nx / 32] bits, all 0 between solves (float mode, ns > 1)
     int parity;
     int check_done;
@@ -88,8 +90,8 @@ constexpr int kFarList = 256;
 constexpr int kQuad = 4;   // sources per scan work item
 constexpr int kAccX = 4;   // accumulator column of tile column 0 (16-byte aligned rows)
 
-// r / P of the residual split, never 0, so that P_s stays recoverable from
-// r_s = P_s r / P (a residual below 1e-20 of P is one of 1e-20)
+// r / P of the residual split, never 0, so that the shares P_s / P can still be
+// had from r_s = P_s r / P (r = 0 counts as 1e-20 P)
 __device__ __forceinline__ float split_ratio(float r, float p)
 {
     const float k = r / p;
@@ -509,6 +511,7 @@ k_splat(const __grid_constant__ EprConsts C, const SplatArgs A)
                 if (split) {
                     const float4 d = dreg[kk];
                     const float4 r = make_float4(d.x - p.x, d.y - p.y, d.z - p.z, d.w - p.w);
+                    if (ns > 1) *reinterpret_cast<float4*>(A.Pnear + o) = p;
                     k = make_float4(bx ? split_ratio(r.x, p.x) : r.x, by ? split_ratio(r.y, p.y) : r.y,
                                     bz ? split_ratio(r.z, p.z) : r.z, bw ? split_ratio(r.w, p.w) : r.w);
                     p = r;

@@ -98,3 +98,26 @@ def test_first_solve_after_an_allocation(torch, E, oracle):
                 assert rel(T.cpu().numpy(), ref) <= 2e-5
         finally:
             E.epr_batch_destroy(bh)
+
+
+# data far above the prediction (hot pixels, dark caustics): the split of a
+# pixel that long shifts reach needs the prediction itself, whose digits D - P
+# does not keep.  Absorption strong enough for predictions down to 1e-2, and
+# pixels that only long shifts reach.
+@pytest.mark.parametrize("lines", [2, 4, 5, 8])
+@pytest.mark.parametrize("level", [1.0, 1e3, 1e5, 1e7])
+def test_split_keeps_the_prediction(torch, E, oracle, lines, level):
+    Es, d, b, w = spec(lines)
+    b = b * 8.0
+    ln = oracle.Lines(Es, d, b, w, L, PIXEL)
+    T0 = phantom(96, 144) * 2.0
+    D = (level * ph.rng(4).uniform(0.9, 1.1, size=(96, 144))).astype(np.float32)
+    Tref, info = oracle.solve(ln, D.astype(np.float64), T0=T0, n_iter=1, omega=0.4)
+    with E.Plan(144, 96, PIXEL, L, Es, d, b, w, max_shift_px=1) as p:
+        T = cuda(torch, T0)
+        got = E.epr_solve_nonlocal(p.handle, cuda(torch, D), T, n_iter=1, omega=0.4, init=1)
+        assert got["overflow_sources"] > 0
+        err = rel(T.cpu().numpy(), Tref)
+        print("lines %d level %g: %.2e" % (lines, level, err))
+        assert err <= 2e-5
+        assert abs(got["rho"][0] - info["rho"][0]) <= 1e-5 * info["rho"][0]
