@@ -252,7 +252,8 @@ cudaError_t epr_launch_col(const EprConsts& C, const EprWork& W, int line0, int 
         const ColKernels& k = *col_kernels(C.ny);
         const CUtensorMap* maps = static_cast<const CUtensorMap*>(W.col_map);
         const bool r8 = k.radix8 && !W.col_radix16, o5 = k.occ5 && W.col_occ5;
-        const bool narrow = k.narrow && (long long)(C.half / k.cw) * nl * batch < col_wide_blocks(C.ny);
+        const long long tiles = (long long)(C.half / k.cw) * (C.det ? 1 : nl) * epr_rule_batch(C, batch);
+        const bool narrow = k.narrow && tiles < col_wide_blocks(C.ny);
         const int cw = narrow ? 2 : k.cw;
         A.CW = cw;
         A.lgCW = cw == 2 ? 1 : 2;

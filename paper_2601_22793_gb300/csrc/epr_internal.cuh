@@ -338,6 +338,11 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
+// The projections that a choice of kernel by the size of the launch may count:
+// in fixed-point mode one, so that a projection's plan, and with it every bit of
+// its result, is the same in whatever batch it is solved.
+inline int epr_rule_batch(const EprConsts& C, int batch) { return C.det ? 1 : batch; }
+
 // Rows of a strip for a kernel whose warps march down strips of columns: at
 // most `most` (the higher a strip, the smaller its halo's share), at least
 // `least`, and so that the strips of all projections fill the `slots` warps

@@ -227,7 +227,7 @@ cudaError_t launch_stencil(const EprConsts& C, StencilArgs& A, int batch, cudaSt
     // iterations: 1218 -> 1098 us; four of 1024 x 1024 (40 rows; 1.2 waves
     // before), 20 iterations of order 2: 2053 -> 1870 us.  At most 48 rows: 64
     // measured the same, 32 and 24 1.7 % slower per solve.
-    A.H = epr_strip_rows(A.strips, C.ny, batch, kStencilSlots, 4, 48);
+    A.H = epr_strip_rows(A.strips, C.ny, epr_rule_batch(C, batch), kStencilSlots, 4, 48);
     const int warps = A.strips * ((C.ny + A.H - 1) / A.H);
     const dim3 grid((warps * 32 + kStencilThreads - 1) / kStencilThreads, 1, batch);
     const cudaError_t e = epr_launch_kernel(C.pdl != 0, k_stencil<MODE, DET>, grid, dim3(kStencilThreads), 0,

@@ -392,7 +392,7 @@ EprRowLaunch epr_row_config(const EprConsts& C, int batch, bool solve)
     });
     int rp = 1;   // of the runtime-sized kernels
     while (rp * 2 * C.nx <= 2048 && (C.ny / 2) % (rp * 2) == 0) rp *= 2;
-    if (many && (long long)(C.ny / (2 * many->rp)) * batch >= kRowMinBlocks) L.k = many;
+    if (many && (long long)(C.ny / (2 * many->rp)) * epr_rule_batch(C, batch) >= kRowMinBlocks) L.k = many;
     else if (one) L.k = one;
     if (solve && C.xt && L.k && !L.k->xfwd1) L.k = nullptr;
     L.RP = L.k ? L.k->rp : rp;

@@ -224,7 +224,7 @@ cudaError_t epr_launch_vjp(const EprConsts& C, const float* T, const float* gbar
     // a strip's rows are a serial chain of gathers, and each strip computes two
     // more rows than it writes.  1536 x 1024, 3 lines: 11 rows (one strip per
     // resident warp) 34.5 us, 22 rows 47.9
-    A.H = epr_strip_rows(A.strips, C.ny, batch, kVjpSlots, 8, 32);
+    A.H = epr_strip_rows(A.strips, C.ny, epr_rule_batch(C, batch), kVjpSlots, 8, 32);
     A.units = A.strips * ((C.ny + A.H - 1) / A.H);
     int nblk = (A.units + kVjpThreads / 32 - 1) / (kVjpThreads / 32);
     if (nblk > kVjpMaxBlocks) nblk = kVjpMaxBlocks;
