@@ -285,7 +285,8 @@ epr_status epr_solve_local(epr_plan_t plan, const float* D, float* T, int batch,
                            const epr_solve_opts* opts, epr_solve_info* info, void* stream);
 
 /* The plan's kernel choices (not in the paper), as 9 host ints: splat tile
- * rows and columns, splat reach (px), column tile width (0 = the default
+ * rows and columns (0 0 = by the size of the launch, the default: no one tile
+ * is the plan's), splat reach (px), column tile width (0 = the default
  * pass), largest radix of the column transforms (8 or 16), row-pass blocks
  * per SM (5 or 6), blocks per SM of the radix-16 column pass (4 or 5),
  * blocks per SM of the one-line residual splat (5 or 6; 6 exists for tiles

@@ -149,7 +149,8 @@ struct epr_plan_s {
     int gkernels;
     bool has_graph;
     cudaGraphExec_t prof_exec;   // last profiled solve
-    bool tuned;                  // autotuner has run
+    bool tuned;                  // autotuner has run, or the choices were set
+    bool tile_fixed;             // splat_TH x splat_TW at every launch (tuned or set)
     // vector-Jacobian product workspace (allocated on first use)
     double* vjp_part;      // block partials
     double* h_vjp_part;    // their sums, pinned: written by the kernel itself
@@ -403,7 +404,7 @@ void splat_tile(const epr_plan_s* p, int batch, int* TH, int* TW)
 {
     *TH = p->splat_TH;
     *TW = p->splat_TW;
-    if (p->tuned || p->C.smax > 8) return;
+    if (p->tile_fixed || p->C.smax > 8) return;
     const long long least = (p->C.ns == 1 ? 5 : 2) * 152 * 4 / 5;
     auto fills = [&](int h, int w) {
         return (long long)((p->C.nx + w - 1) / w) * ((p->C.ny + h - 1) / h) * batch >= least;
@@ -539,7 +540,7 @@ epr_status collect_info(epr_plan_s* p, int batch, int n_iter, epr_solve_info* in
 // splat.
 epr_status autotune_splat(epr_plan_s* p, const float* D, const float* T, int batch, cudaStream_t s)
 {
-    p->tuned = true;
+    p->tuned = p->tile_fixed = true;
     const bool resid = p->C.ns == 1 && !p->C.det && p->C.os == 1 && !p->C.xt;
     const float* Dfwd = p->C.os == 1 ? D : nullptr;   // as the solve runs it
     const int tiles[4][2] = {{64, 64}, {32, 64}, {64, 32}, {32, 32}};
@@ -1550,8 +1551,8 @@ epr_status epr_plan_set_xspec(epr_plan_t p, const epr_xspec* tab)
 epr_status epr_plan_get_tuning(epr_plan_t p, int* out)
 {
     if (!p || !out) return EPR_ERR_INVALID_ARG;
-    out[0] = p->splat_TH;
-    out[1] = p->splat_TW;
+    out[0] = p->tile_fixed ? p->splat_TH : 0;   // 0 x 0: by the size of the launch
+    out[1] = p->tile_fixed ? p->splat_TW : 0;
     out[2] = p->C.smax;
     out[3] = p->col_cw;
     out[4] = p->W.col_radix16 ? 16 : 8;
@@ -1567,21 +1568,25 @@ epr_status epr_plan_set_tuning(epr_plan_t p, const int* in)
     if (!p || !in) return EPR_ERR_INVALID_ARG;
     const int th = in[0], tw = in[1], reach = in[2], cw = in[3], radix = in[4], occ = in[5];
     const int cocc = in[6], socc = in[7];
-    const bool tile_ok = (th == 64 || th == 32) && (tw == 64 || tw == 32);
+    const bool by_launch = th == 0 && tw == 0;
+    const bool tile_ok = by_launch || ((th == 64 || th == 32) && (tw == 64 || tw == 32));
     if (!tile_ok || reach < 1 || reach > EPR_MAX_SHIFT || !(cw == 0 || cw == 1 || cw == 2 || cw == 4) ||
         !(radix == 8 || radix == 16) || !(occ == 5 || occ == 6) || !(cocc == 4 || cocc == 5) ||
         (cocc == 5 && radix != 16) || !(socc == 5 || socc == 6) ||
-        (socc == 6 && !epr_splat_has_occ6(th, tw, reach)))
+        (socc == 6 && (by_launch || !epr_splat_has_occ6(th, tw, reach))))
         return EPR_ERR_INVALID_ARG;
     EprConsts C = p->C;
     C.smax = reach;
     if ((size_t)C.ns * th * tw * (C.det ? 8 : 4) > 65536) return EPR_ERR_INVALID_ARG;
     int optin = 0;
     EPR_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
-    if (epr_splat_smem(C, th, tw) + 4096 > (size_t)optin) return EPR_ERR_INVALID_ARG;
+    const int h = by_launch ? 32 : th, w = by_launch ? 32 : tw;   // the smallest tile must fit
+    if (epr_splat_smem(C, h, w) + 4096 > (size_t)optin) return EPR_ERR_INVALID_ARG;
     p->C.smax = reach;
+    p->tile_fixed = !by_launch;
     p->splat_TH = th;
     p->splat_TW = tw;
+    if (by_launch) choose_splat_tiles(p);
     p->col_cw = cw;
     p->W.col_radix16 = radix == 16;
     p->W.row_occ6 = occ == 6;

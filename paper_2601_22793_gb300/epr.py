@@ -230,7 +230,8 @@ def epr_plan_create(nx, ny, pixel_m, L_m, energy_keV, delta, beta, weights=None,
 
 
 def epr_plan_get_tuning(plan) -> dict:
-    """The plan's kernel choices (defaults, or the autotuner's)."""
+    """The plan's kernel choices (defaults, or the autotuner's).  A splat tile
+    of [0, 0] is chosen at each launch by its size."""
     v = (ctypes.c_int * 9)()
     _check(load().epr_plan_get_tuning(plan, v), "epr_plan_get_tuning")
     return {"splat_tile": [v[0], v[1]], "splat_reach": v[2], "col_tile_width": v[3],
