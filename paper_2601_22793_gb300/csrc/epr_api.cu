@@ -388,7 +388,8 @@ struct ProfScope {
 
 // The splat tile of a launch: the largest of the plan's default, 32 x 64 and
 // 32 x 32 whose blocks fill 4/5 of the resident ones (five per SM with one
-// line, two with several).  A larger tile scans a smaller halo (1.27 sources
+// line, two of the 512-thread blocks that several lines and an x-dependent
+// spectrum take).  A larger tile scans a smaller halo (1.27 sources
 // per pixel for 64 x 64 at reach 4, 1.41 and 1.56), but too few blocks leave
 // SMs idle or with too few warps to hide their latency.  Solve iterations, us,
 // with 64 x 64, 32 x 64 and 32 x 32 tiles:
@@ -398,6 +399,12 @@ struct ProfScope {
 //   several lines 512^2 (4) 37.5, 29.9, 28.6  768^2 (2) 39.8, 36.1, 37.1
 //                 1024^2 (2) 46.7, 47.8, 49.4
 //                 512^2 (8) -, 50.9, 44.6     768^2 (8) -, 91.7, 91.9
+//   one line, x-dependent   768^2 52.0, 48.9, 50.7   1024^2 33.1, 34.6, 38.2
+//                 1536 x 1024 72.0, 74.6, 79.4
+// In fixed point three 64 x 64 blocks of one line fit on an SM, not five; the
+// line for five is kept there, because the smaller tiles stay the better ones
+// up to it: 1024^2 35.6, 33.1, 31.6, 1536 x 1024 42.7, 41.8, 41.6, 1536^2 62.1,
+// 56.8, 58.4.
 // A tuned plan keeps the choice of its tuner, and reaches above 8 (where the
 // small tiles' halo is several times the tile) the default.
 void splat_tile(const epr_plan_s* p, int batch, int* TH, int* TW)
@@ -405,7 +412,7 @@ void splat_tile(const epr_plan_s* p, int batch, int* TH, int* TW)
     *TH = p->splat_TH;
     *TW = p->splat_TW;
     if (p->tile_fixed || p->C.smax > 8) return;
-    const long long least = (p->C.ns == 1 ? 5 : 2) * 152 * 4 / 5;
+    const long long least = (p->C.ns == 1 && !p->C.xt ? 5 : 2) * 152 * 4 / 5;
     auto fills = [&](int h, int w) {
         return (long long)((p->C.nx + w - 1) / w) * ((p->C.ny + h - 1) / h) * batch >= least;
     };

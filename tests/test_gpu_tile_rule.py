@@ -70,3 +70,27 @@ def test_default_tile_survives_a_tuning_round_trip(torch, E):
                 E.epr_plan_set_tuning(b.handle, dict(tun, splat_tile=bad))
         with pytest.raises(E.EprError):   # six blocks per SM belong to a tile
             E.epr_plan_set_tuning(b.handle, dict(tun, splat_blocks_per_sm=6))
+
+
+# an x-dependent spectrum runs two 512-thread blocks per SM with one line too:
+# 243 blocks of a tile fill the chip.  Sizes on both sides of the 32 x 64 and
+# the 64 x 64 line; the tile does not change a bit of the integer sums.
+@pytest.mark.parametrize("nx,ny,batch", [(512, 768, 1), (768, 768, 1), (1024, 768, 1), (1024, 1024, 1),
+                                         (512, 512, 4)])
+def test_xspec_tiles_of_one_line(torch, E, nx, ny, batch):
+    ells = ph.random_ellipsoids(ny, nx, 8, 8.0, 20.0, margin=4.0, seed=nx)
+    tau = ph.project_ellipsoids(ells, ny, nx, PIXEL).astype(np.float32)
+    X = np.array([0.0, nx - 1.0])
+    W, Dl, Bt = np.ones((1, 2)), ph.BONE[0] * np.array([[0.9, 1.1]]), ph.BONE[1] * np.array([[1.1, 0.9]])
+    with E.Plan(nx, ny, PIXEL, L, [80.0], [ph.BONE[0]], [ph.BONE[1]]) as p:
+        E.epr_plan_set_xspec(p.handle, X, W, Dl, Bt)
+        T = cuda(torch, np.stack([tau] * batch))
+        tun = E.epr_plan_get_tuning(p.handle)
+        got = []
+        for tile in ([0, 0], [64, 64], [32, 64], [64, 32], [32, 32]):
+            E.epr_plan_set_tuning(p.handle, dict(tun, splat_tile=tile))
+            P = torch.empty_like(T)
+            E.epr_forward(p.handle, T, P, batch=batch)
+            got.append(P)
+    for P in got[1:]:
+        assert torch.equal(P, got[0])
