@@ -35,8 +35,31 @@
 
 namespace eprfft {
 
+// Where the powers w^2 .. w^(R-1) of a stage's twiddle come from
+// (apply_twiddles).  A power from the table carries one rounding, but its loads
+// are scattered: lane j reads entry r j N / (Ns R).
+//   TREE  products of lower powers, from w alone, at most 4 roundings deep
+//   HALF  w^2, w^4 and w^8 from the table as well
+//   FINE  w, w^2, w^3 and every fourth power from the table
+//   FULL  every power from the table
+enum { TW_TREE = 0, TW_HALF = 1, TW_FINE = 2, TW_FULL = 3 };
+
+// Lengths whose passes take the more exact forms: those with a factor 9, and
+// the short ones with a factor 3 or below 256.  Their stages are many and of
+// mixed radix, and the tree's error in them is the larger one: relative error
+// of the filter at 1728 x 1728 5.1e-7 with TREE, 2.8e-7 with HALF rows and FINE
+// columns, 2.6e-7 with FULL; of a solve at 1728 x 1152 2.65e-7 with TREE,
+// 1.98e-7 with HALF rows and FULL columns (20 iterations of two lines 1983 and
+// 2028 us).  The powers of two from 256 on and 1536 and 3072, which carry the
+// large frames, keep TREE in a solve: 2048^2 takes 22 % more with FULL, four
+// lines of mixed sizes up to 3072 x 2048 3 to 10 %, and their error (2048
+// points: 1.8e-7 in radix 8, 2.5e-7 in radix 16) is well below the 4.2e-7 and
+// 6.5e-7 of a three-term recurrence of cos and sin.
+__host__ __device__ constexpr bool tw_exact(int n) { return n % 9 == 0 || (n % 3 == 0 && n < 1536) || n < 256; }
+
 // Each policy also states a period P and the address step of adding a
-// multiple c of P to an index: idx(i + c) = idx(i) + step(c) for every i.  A
+// multiple c of P to an index: idx(i + c) = idx(i) + step(c) for every i, and
+// how the passes that use it form their twiddles at length n.  A
 // stage whose operand stride is a multiple of P computes one address and adds
 // constants.
 struct PadRow {
@@ -47,6 +70,14 @@ struct PadRow {
     __host__ __device__ static __forceinline__ int len(int n) { return (n + 15) & ~15; }
     static constexpr int kPeriod = 128;   // the swizzle reads bits 0..6 only
     __host__ __device__ static constexpr int step(int c) { return c; }
+    __host__ __device__ static constexpr int tw(int n) { return tw_exact(n) ? TW_HALF : TW_TREE; }
+};
+
+// The rows of the plain transforms, the stand-alone filter's: no iteration
+// corrects their error.  FINE costs 2048^2 37.5 us for 32.6 with TREE, and FULL
+// 43.3 for another 1 % of the error.
+struct PadPlain : PadRow {
+    __host__ __device__ static constexpr int tw(int n) { return tw_exact(n) ? TW_FULL : TW_FINE; }
 };
 
 struct PadCol {
@@ -54,6 +85,7 @@ struct PadCol {
     __host__ __device__ static __forceinline__ int len(int n) { return n + 2 * (n >> 4) + 2; }
     static constexpr int kPeriod = 16;
     __host__ __device__ static constexpr int step(int c) { return c + 2 * (c >> 4); }
+    __host__ __device__ static constexpr int tw(int n) { return tw_exact(n) ? TW_FULL : TW_TREE; }
 };
 
 // Plain dense layout (a tile written by a bulk copy).
@@ -406,24 +438,25 @@ __host__ __device__ constexpr int ct_ns_rev(int n, int s, int maxr = 8)
     return v;
 }
 
-// v[r] *= w^r with w = exp(DIR 2 pi i i / N).  The powers come from products
-// of two lower ones (w^2 = w w, w^3 = w^2 w, w^4 = w^2 w^2, ...), so each is
-// at most 4 roundings deep: a transform of 2048 points is off by 1.8e-7 (radix
-// 8) and 2.5e-7 (radix 16) of its norm, where the three-term recurrence of
-// cos and sin (half the operations, 3 % of a 2048^2 solve) gives 4.2e-7 and
-// 6.5e-7: its error grows with r^2.  Taking w^4 and w^8 from the table as well
-// halves the error again and costs 3 %, in a kernel bound by its loads.
-template <int R, int DIR>
+__host__ __device__ constexpr bool tw_loaded(int mode, int r)
+{
+    return r == 1 || mode == TW_FULL || (mode == TW_HALF && (r & (r - 1)) == 0) ||
+           (mode == TW_FINE && (r < 4 || r % 4 == 0));
+}
+
+// v[r] *= w^r with w = exp(DIR 2 pi i i / N).  A power that is not loaded is the
+// product of two lower ones (TREE: w^2 = w w, w^3 = w^2 w, w^4 = w^2 w^2, ...).
+template <int R, int DIR, int MODE>
 __device__ __forceinline__ void apply_twiddles(float2 (&v)[R], const float2* __restrict__ tw, int i)
 {
     float2 p[R];
-    p[1] = __ldg(&tw[i]);
-    if (DIR > 0) p[1].y = -p[1].y;
-    v[1] = cmul(v[1], p[1]);
 #pragma unroll
-    for (int r = 2; r < R; ++r) {
-        const int h = r >= 8 ? 8 : r >= 4 ? 4 : 2;
-        if (h == r) {
+    for (int r = 1; r < R; ++r) {
+        const int h = MODE == TW_FINE ? r & ~3 : r >= 8 ? 8 : r >= 4 ? 4 : 2;
+        if (tw_loaded(MODE, r)) {
+            p[r] = __ldg(&tw[r * i]);
+            if (DIR > 0) p[r].y = -p[r].y;
+        } else if (h == r) {
             const float2 q = p[r / 2];
             p[r] = make_float2(q.x * q.x - q.y * q.y, (q.x + q.x) * q.y);
         } else {
@@ -496,7 +529,7 @@ __device__ __forceinline__ void stage_ct(const float2* in, float2* buf, const fl
                 for (int r = 0; r < R; ++r) v[k][r] = in[PADI::idx((j + r * NR) * SJ + base)];
             }
             if constexpr (NS > 1) {
-                apply_twiddles<R, DIR>(v[k], tw, jm * TWSTEP);
+                apply_twiddles<R, DIR, PADI::tw(N)>(v[k], tw, jm * TWSTEP);
             }
             dst[k] = (jd * NS * R + jm) * SJ + base;
         }
@@ -618,7 +651,7 @@ __device__ __forceinline__ void stage_turn(float2* buf, const float2* __restrict
 #pragma unroll
             for (int r = 0; r < R; ++r) v[k][r] = buf[PAD::idx((j + r * NR) * SJ + base)];
             if constexpr (NS > 1) {
-                apply_twiddles<R, DIRF>(v[k], tw, j * TWSTEP);
+                apply_twiddles<R, DIRF, PAD::tw(N)>(v[k], tw, j * TWSTEP);
             }
             j_of[k] = j;
             m_of[k] = m;

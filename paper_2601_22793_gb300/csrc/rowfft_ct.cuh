@@ -4,6 +4,8 @@
 // runtime-sized passes of the remaining lengths and describes the passes).
 #pragma once
 
+#include <type_traits>
+
 #include "epr_internal.cuh"
 #include "fft.cuh"
 
@@ -58,7 +60,8 @@ struct RowKernels {
 namespace {
 
 using namespace eprrow;
-using PR = eprfft::PadRow;   // shared layout of the packed rows
+using PR = eprfft::PadRow;    // shared layout of the packed rows
+using PP = eprfft::PadPlain;  // the same, of the plain transforms
 
 // Projection of a row-pass block.  The row passes walk the batch from the
 // last projection to the first (grid y), the splat and the column pass from
@@ -229,6 +232,7 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
     constexpr int SM = NX + kPad;
     constexpr int HALF = NX / 2;
     constexpr int LGRP = ct_lg<NX>(RP);
+    using PF = std::conditional_t<GATHER, PR, PP>;
     constexpr int kRowLines = (NX + 31) / 32;   // 128-byte lines of a row
     extern __shared__ __align__(16) float2 zs[];
     __shared__ float red[64];
@@ -389,8 +393,8 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
     if constexpr (GATHER) __syncthreads();   // every thickness read is done
     if constexpr (eprfft::ct_radix(NX, 0, MAXR) * RP == EPT && NX % T == 0) {
         // vk[m R + r] = element tid + r T of pair m, the first stage's operands
-        eprfft::stage0_regs<PR, -1, NX, RP, EPT, SM, MAXR>(vk, zs, tid);
-        eprfft::fft_ct<PR, -1, NX, EPT, LGRP, 1, SM, 1, MAXR>(zs, A.tw, tid);
+        eprfft::stage0_regs<PF, -1, NX, RP, EPT, SM, MAXR>(vk, zs, tid);
+        eprfft::fft_ct<PF, -1, NX, EPT, LGRP, 1, SM, 1, MAXR>(zs, A.tw, tid);
     } else {
 #pragma unroll
         for (int k = 0; k < EPT; ++k) {
@@ -399,7 +403,7 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
             zs[PR::idx(m * SM + x)] = vk[k];
         }
         __syncthreads();
-        eprfft::fft_ct<PR, -1, NX, EPT, LGRP, 1, SM, 0, MAXR>(zs, A.tw, tid);
+        eprfft::fft_ct<PF, -1, NX, EPT, LGRP, 1, SM, 0, MAXR>(zs, A.tw, tid);
     }
     epr_grid_release();
     float2* Sb = A.S + ((size_t)b * A.nl + sl) * (size_t)ny * HALF;
@@ -459,23 +463,23 @@ __device__ __forceinline__ void inv_unpack(const float2* __restrict__ Sb, float2
 // factor 3 run the reversed stage plan, whose last stage is the radix-8 one:
 // each thread then ends with one butterfly of 8 results instead of up to
 // three of 3, which the update would spill.
-template <int NX, int RP, int EPT, int MAXR>
+template <class PF, int NX, int RP, int EPT, int MAXR>
 __device__ __forceinline__ void inv_stages(float2* zs, const float2* tw, int tid)
 {
     constexpr int LGRP = ct_lg<NX>(RP), SM = NX + kPad, NST = eprfft::ct_n_stages(NX, MAXR);
     if constexpr (NX % 3 == 0)
-        eprfft::fft_ct_rev_stages<PR, +1, NX, EPT, LGRP, 1, SM, 0, NST - 1, MAXR>(zs, tw, tid);
+        eprfft::fft_ct_rev_stages<PF, +1, NX, EPT, LGRP, 1, SM, 0, NST - 1, MAXR>(zs, tw, tid);
     else
-        eprfft::fft_ct_stages<PR, +1, NX, EPT, LGRP, 1, SM, 0, NST - 1, MAXR>(zs, tw, tid);
+        eprfft::fft_ct_stages<PF, +1, NX, EPT, LGRP, 1, SM, 0, NST - 1, MAXR>(zs, tw, tid);
 }
-template <int NX, int RP, int EPT, int MAXR, class POST>
+template <class PF, int NX, int RP, int EPT, int MAXR, class POST>
 __device__ __forceinline__ void inv_last(float2* zs, const float2* tw, int tid, const POST& post)
 {
     constexpr int LGRP = ct_lg<NX>(RP), SM = NX + kPad;
     if constexpr (NX % 3 == 0)
-        eprfft::fft_ct_rev_last<PR, false, false, PR, +1, NX, EPT, LGRP, 1, SM, MAXR>(zs, tw, tid, post);
+        eprfft::fft_ct_rev_last<PF, false, false, PF, +1, NX, EPT, LGRP, 1, SM, MAXR>(zs, tw, tid, post);
     else
-        eprfft::fft_ct_last<PR, false, false, PR, +1, NX, EPT, LGRP, 1, SM, MAXR>(zs, tw, tid, post);
+        eprfft::fft_ct_last<PF, false, false, PF, +1, NX, EPT, LGRP, 1, SM, MAXR>(zs, tw, tid, post);
 }
 
 // The update of one result of the last inverse stage of a one-line block:
@@ -557,14 +561,14 @@ k_row_inv1(const EprConsts C, const RowArgs A)
         return;
     }
     inv_unpack<NX, RP, EPT>(A.S + (size_t)b * (size_t)ny * HALF, zs, yb, tid);
-    inv_stages<NX, RP, EPT, MAXR>(zs, A.tw, tid);
+    inv_stages<PR, NX, RP, EPT, MAXR>(zs, A.tw, tid);
     epr_grid_release();
     cp_async_wait_all();   // the thickness rows: visible to all after the last stage's barrier
     // the last stage hands each result to the update (no store, no barrier)
     const InvUpdate1<NX, SM, RP, XT, kStageT> up{C, Tsh, A.Out + pb + (size_t)yb * NX, C.mu[0],
                                                  C.wproj[0], A.omega / C.f[0], A.omega, A.eps,
                                                  {0.f, 0.f}, {0.f, 0.f}};
-    inv_last<NX, RP, EPT, MAXR>(zs, A.tw, tid, up);
+    inv_last<PR, NX, RP, EPT, MAXR>(zs, A.tw, tid, up);
     float da = up.da.x + up.da.y, db = up.db.x + up.db.y;
     block_sum2(da, db, red);   // kappa partials, finalised by the next forward pass
     store_partials(A.part_a + (size_t)b * A.max_blocks, A.part_b + (size_t)b * A.max_blocks, da, db);
@@ -655,7 +659,7 @@ k_row_invn(const EprConsts C, const RowArgs A)
     for (int sl = 0; sl < A.nl; ++sl) {
         const int s = A.line0 + sl;
         inv_unpack<NX, RP, EPT>(A.S + ((size_t)b * A.nl + sl) * (size_t)ny * HALF, zs, yb, tid);
-        inv_stages<NX, RP, EPT, row_maxr(EPT)>(zs, A.tw, tid);
+        inv_stages<PR, NX, RP, EPT, row_maxr(EPT)>(zs, A.tw, tid);
         if (sl == 0) {
             epr_grid_release();
             cp_async_wait_all();   // the thickness rows: visible after the last stage's barrier
@@ -668,7 +672,7 @@ k_row_invn(const EprConsts C, const RowArgs A)
         up.mus = line_const(C.mu, s);
         up.w = line_const(C.wproj, s);
         up.om_f = A.omega / line_const(C.f, s);
-        inv_last<NX, RP, EPT, row_maxr(EPT)>(zs, A.tw, tid, up);
+        inv_last<PR, NX, RP, EPT, row_maxr(EPT)>(zs, A.tw, tid, up);
     }
     float da = up.da.x + up.da.y, db = up.db.x + up.db.y;
     block_sum2(da, db, red);   // kappa partials, finalised by the next forward pass
@@ -702,10 +706,10 @@ k_row_store(const EprConsts C, const RowArgs A)
     const int yb = blockIdx.x * RP * 2;
     epr_grid_wait();
     inv_unpack<NX, RP, EPT>(A.S + (size_t)b * (size_t)ny * (NX / 2), zs, yb, tid);
-    inv_stages<NX, RP, EPT, row_maxr(EPT)>(zs, A.tw, tid);
+    inv_stages<PP, NX, RP, EPT, row_maxr(EPT)>(zs, A.tw, tid);
     epr_grid_release();
     const InvStore<NX, SM, RP> st{A.Out + (size_t)b * NX * ny + (size_t)yb * NX};
-    inv_last<NX, RP, EPT, row_maxr(EPT)>(zs, A.tw, tid, st);
+    inv_last<PP, NX, RP, EPT, row_maxr(EPT)>(zs, A.tw, tid, st);
 }
 
 // dynamic shared memory: the FFT rows; the forward gather aliases them with

@@ -1,0 +1,47 @@
+"""Errors against 64 bits, with bounds taken from the arithmetic."""
+import numpy as np
+import pytest
+
+from paper_2601_22793_gb300 import phantoms as ph
+
+pytestmark = pytest.mark.gpu
+
+PIXEL, L = 20e-6, 30.0
+
+
+@pytest.fixture(scope="module")
+def torch():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2601_22793_gb300 import build
+    build.build()
+    from paper_2601_22793_gb300 import epr
+    epr.load()
+    return torch
+
+
+@pytest.fixture(scope="module")
+def E():
+    from paper_2601_22793_gb300 import epr
+    return epr
+
+
+# The filter is four transforms along an axis.  Of one transform of up to 2592
+# points: at most 11.4 levels of additions, each off by 2.4e-8 rms (a rounding of
+# 2^-25 to 2^-24, uniform), and at most four layers of twiddle products, each off
+# by 5.5e-8 (the table's rounding and a complex product's):
+# sqrt(4 (11.4 2.4^2 + 4 5.5^2)) 1e-8 = 2.7e-7; the bound leaves 35 %.
+@pytest.mark.parametrize("n", [144, 384, 648, 768, 864, 1152, 1296, 1728, 2304, 2592])
+def test_filter_error_of_ragged_lengths(torch, E, n):
+    g = torch.randn(n, n, generator=torch.Generator(device="cuda").manual_seed(n), device="cuda")
+    mu = 2.0 * (2.0 * np.pi / (1.2398419843320026e-6 / 80e3)) * ph.BONE[1]
+    fy = torch.fft.fftfreq(n, PIXEL, dtype=torch.float64, device="cuda")[:, None]
+    fx = torch.fft.rfftfreq(n, PIXEL, dtype=torch.float64, device="cuda")[None]
+    H = mu / (mu + L * ph.BONE[0] * 4.0 * np.pi ** 2 * (fx * fx + fy * fy))
+    ref = torch.fft.irfft2(torch.fft.rfft2(g.double()) * H, s=(n, n))
+    with E.Plan(n, n, PIXEL, L, [80.0], [ph.BONE[0]], [ph.BONE[1]]) as p:
+        E.epr_precondition(p.handle, g)
+    err = ((g.double() - ref).norm() / ref.norm()).item()
+    print("filter %d: %.2e" % (n, err))
+    assert err <= 3.7e-7
