@@ -22,8 +22,8 @@
 // loads (four corners per line and pixel, from L1 and L2): long scoreboard is
 // the top stall, half of the issue slots are used.  The corners of all lines
 // are therefore loaded before the first is used, and the strips are cut so
-// that every resident warp has one.  1536 x 1024, 3 lines: 56 -> 34.5 us from
-// both, with the slopes taken from shared differences.
+// that every resident warp has one: 39.1 us where the two-pass form took 51.4
+// (1536 x 1024, 3 lines; one line 21.6 and 38.2).
 #include "epr_internal.cuh"
 
 namespace {
@@ -141,12 +141,16 @@ __global__ void __launch_bounds__(kVjpThreads, NSM <= 8 ? 4 : 2) k_vjp(const __g
                         const int s = s0 + k;
                         const float cs = C.c[s], dx = dxs[k], dy = dys[k];
                         const float m = C.mu[s], Is = C.f[s] * __expf(-m * tc), ci = cs * Is;
-                        // the bilinear patch g00 + dx ex + dy ey + dx dy xy:
-                        // its value and its slopes, from differences of gbar
-                        const float g00 = g[k][0], ex = g[k][1] - g00, ey = g[k][2] - g00;
-                        const float xy = (g[k][3] - g[k][2]) - ex;
-                        const float slx = ex + dy * xy, sly = ey + dx * xy;
-                        const float Ia = Is * (g00 + dx * ex + dy * sly);
+                        // the value and the slopes as weighted means of
+                        // corners and differences: a value formed from
+                        // differences of corners (g00 + dx (g10 - g00) + ..)
+                        // takes 35.5 us where this takes 39.1 (1536 x 1024, 3
+                        // lines), but carries the rounding of the largest corner
+                        const float g00 = g[k][0], g10 = g[k][1], g01 = g[k][2], g11 = g[k][3];
+                        const float wx = 1.f - dx, wy = 1.f - dy;
+                        const float slx = wy * (g10 - g00) + dy * (g11 - g01);
+                        const float sly = wx * (g01 - g00) + dx * (g11 - g10);
+                        const float Ia = Is * (wy * (wx * g00 + dx * g10) + dy * (wx * g01 + dx * g11));
                         tb -= m * Ia;
                         vx += ci * slx;
                         vy += ci * sly;
@@ -223,7 +227,7 @@ cudaError_t epr_launch_vjp(const EprConsts& C, const float* T, const float* gbar
     A.strips = (C.nx + 29) / 30;
     // a strip's rows are a serial chain of gathers, and each strip computes two
     // more rows than it writes.  1536 x 1024, 3 lines: 11 rows (one strip per
-    // resident warp) 34.5 us, 22 rows 47.9
+    // resident warp) 34.5 us, 22 rows 47.9 (both with the cheaper bilinear form)
     A.H = epr_strip_rows(A.strips, C.ny, epr_rule_batch(C, batch), kVjpSlots, 8, 32);
     A.units = A.strips * ((C.ny + A.H - 1) / A.H);
     int nblk = (A.units + kVjpThreads / 32 - 1) / (kVjpThreads / 32);

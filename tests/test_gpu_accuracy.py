@@ -45,3 +45,23 @@ def test_filter_error_of_ragged_lengths(torch, E, n):
     err = ((g.double() - ref).norm() / ref.norm()).item()
     print("filter %d: %.2e" % (n, err))
     assert err <= 3.7e-7
+
+
+# A thickness ramp whose shift is exactly half a pixel, and a misfit gradient of
+# 2^24 and 1 - 2^24 in turn: the bilinear value is exactly 1/2 everywhere (the
+# weights, their products and their sum are exact), and dF/dbeta = -2 k sum of
+# T I / 2.  The difference of two corners needs 25 bits: a value formed from it
+# is 0 and 1 in turn.  5e-6: exponentials, products and float sums of 48 terms.
+def test_gradient_of_large_alternating_misfits(torch, E):
+    nx, ny = 96, 48
+    delta, dist, pixel, beta = 2.0 ** -21, 1.0, 2.0 ** -16, 1e-11   # the shift constant is -2^11
+    k = 2.0 * np.pi / (1.2398419843320026e-6 / 80e3)
+    x = np.arange(nx)
+    T = np.broadcast_to((x * 2.0 ** -12).astype(np.float32), (ny, nx))
+    g = np.broadcast_to(np.where(x % 2 == 0, 2.0 ** 24, 1.0 - 2.0 ** 24).astype(np.float32), (ny, nx))
+    with E.Plan(nx, ny, pixel, dist, [80.0], [delta], [beta]) as p:
+        Td, gd = (torch.from_numpy(a.copy()).cuda() for a in (T, g))
+        _, got, _ = E.epr_vjp(p.handle, Td, gd, torch.empty_like(Td), 1)
+    T = T.astype(np.float64)
+    ref = -2.0 * k * 0.5 * (T * np.exp(-2.0 * k * beta * T)).sum()   # T = 0 in the column with a corner outside
+    assert abs(np.ravel(got)[0] / ref - 1.0) <= 5e-6
