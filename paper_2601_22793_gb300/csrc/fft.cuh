@@ -674,27 +674,20 @@ __device__ __forceinline__ void stage_turn(float2* buf, const float2* __restrict
     __syncthreads();
 }
 
-// The first stage with its operands in registers, for NSEQ sequences laid out
-// SM apart and N / R threads with the first radix R: v[m R + r] is element
-// tid + r N / R of sequence m, and the stage has no twiddles.  Writes its
-// results to buf (layout PAD) and synchronises; the caller has synchronised
-// already if buf aliases data that other threads still read.  Stages 1..
-// follow as fft_ct<..., 1>.
-template <class PAD, int DIR, int N, int NSEQ, int EPT, int SM, int MAXR = 8>
+// The first stage with its operands in registers: one sequence of N / R threads
+// with the first radix R, v[r] the element tid + r N / R, and no twiddles.
+// Writes its results to buf (layout PAD) and synchronises; the caller has
+// synchronised already if buf aliases data that other threads still read.
+// Stages 1.. follow as fft_ct<..., 1>.
+template <class PAD, int DIR, int N, int EPT, int MAXR = 8>
 __device__ __forceinline__ void stage0_regs(float2 (&v)[EPT], float2* buf, int tid)
 {
     constexpr int R = ct_radix(N, 0, MAXR);
-    static_assert(R * NSEQ == EPT && ct_n_stages(N, MAXR) > 1, "operands of the first stage in registers");
+    static_assert(R == EPT && ct_n_stages(N, MAXR) > 1, "operands of the first stage in registers");
+    dft<R, DIR>(v);
     const int dst = tid * R;   // (j / Ns) Ns R + (j mod Ns) with Ns = 1, j = tid
 #pragma unroll
-    for (int m = 0; m < NSEQ; ++m) {
-        float2 w[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) w[r] = v[m * R + r];
-        dft<R, DIR>(w);
-#pragma unroll
-        for (int r = 0; r < R; ++r) buf[PAD::idx(dst + r + m * SM)] = w[r];
-    }
+    for (int r = 0; r < R; ++r) buf[PAD::idx(dst + r)] = v[r];
     __syncthreads();
 }
 

@@ -391,9 +391,9 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
         }
     }
     if constexpr (GATHER) __syncthreads();   // every thickness read is done
-    if constexpr (eprfft::ct_radix(NX, 0, MAXR) * RP == EPT && NX % T == 0) {
-        // vk[m R + r] = element tid + r T of pair m, the first stage's operands
-        eprfft::stage0_regs<PF, -1, NX, RP, EPT, SM, MAXR>(vk, zs, tid);
+    if constexpr (RP == 1 && eprfft::ct_radix(NX, 0, MAXR) == EPT) {
+        // vk[r] = element tid + r T, the first stage's operands
+        eprfft::stage0_regs<PF, -1, NX, EPT, MAXR>(vk, zs, tid);
         eprfft::fft_ct<PF, -1, NX, EPT, LGRP, 1, SM, 1, MAXR>(zs, A.tw, tid);
     } else {
 #pragma unroll
