@@ -412,7 +412,7 @@ void splat_tile(const epr_plan_s* p, int batch, int* TH, int* TW)
     *TH = p->splat_TH;
     *TW = p->splat_TW;
     if (p->tile_fixed || p->C.smax > 8) return;
-    const long long least = (p->C.ns == 1 && !p->C.xt ? 5 : 2) * 152 * 4 / 5;
+    const long long least = (p->C.ns == 1 && !p->C.xt ? 5 : 2) * EPR_SMS * 4 / 5;
     auto fills = [&](int h, int w) {
         return (long long)((p->C.nx + w - 1) / w) * ((p->C.ny + h - 1) / h) * batch >= least;
     };

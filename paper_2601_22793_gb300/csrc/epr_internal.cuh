@@ -11,6 +11,7 @@
 
 #define EPR_MAX_LINES 16
 #define EPR_MAX_SHIFT 32
+#define EPR_SMS 152   // multiprocessors of the chip these kernels are written for
 
 // Device-side error bits (OR-ed into the plan's error word).
 #define EPR_DEVERR_OVERFLOW 1u

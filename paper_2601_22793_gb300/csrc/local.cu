@@ -30,7 +30,7 @@ namespace {
 
 constexpr int kStencilThreads = 128;
 constexpr int kStencilBlocks = 7;   // per SM: 72 registers a thread
-constexpr int kStencilSlots = 152 * kStencilBlocks * (kStencilThreads / 32);   // resident warps
+constexpr int kStencilSlots = EPR_SMS * kStencilBlocks * (kStencilThreads / 32);   // resident warps
 
 enum { ST_LOCAL1 = 1, ST_LOCAL2 = 2, ST_WKB1 = 3 };
 

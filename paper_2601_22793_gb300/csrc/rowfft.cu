@@ -369,7 +369,7 @@ void each_table(F f)
 // 217, 243; eight of 384^2 (768) 34.3, 35.9.  Longer rows are one pair per
 // block at every count: two pairs (256 threads) took 115 for eight of 1024^2
 // where one takes 110, and 796 where it takes 697 for 16 of four lines.
-constexpr int kRowMinBlocks = 608;
+constexpr int kRowMinBlocks = 4 * EPR_SMS;
 
 }  // namespace
 
@@ -522,7 +522,7 @@ cudaError_t epr_launch_solve_begin(const EprConsts& C, const EprWork& W, const f
                                    cudaStream_t stream)
 {
     size_t parts = (npix / 4 + 255) / 256;   // a float4 per thread, up to 4 blocks per SM
-    if (parts > 608) parts = 608;
+    if (parts > 4 * EPR_SMS) parts = 4 * EPR_SMS;
     if (parts > (size_t)W.max_blocks) parts = W.max_blocks;
     k_solve_begin<<<dim3((unsigned)parts, batch), 256, 0, stream>>>(D, npd, T, npix, W.part_a, W.max_blocks,
                                                                     W.st, W.err);

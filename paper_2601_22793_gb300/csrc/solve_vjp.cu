@@ -344,7 +344,7 @@ inline dim3 sv_grid(size_t npix, int nblk, int batch)
 }  // namespace
 
 // Blocks per projection of the reductions (the partial buffers hold this many).
-int epr_sv_blocks() { return 608; }   // 4 per SM on 152 SMs
+int epr_sv_blocks() { return 4 * EPR_SMS; }
 
 cudaError_t epr_launch_sv_split(const EprConsts& C, const float* D, const float* P, const float* Ps,
                                 float* r, float* RS, int B, cudaStream_t s)

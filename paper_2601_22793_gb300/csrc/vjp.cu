@@ -29,7 +29,7 @@
 namespace {
 
 constexpr int kVjpThreads = 256;
-constexpr int kVjpMaxBlocks = 608; // per projection: 4 per SM on 152 SMs
+constexpr int kVjpMaxBlocks = 4 * EPR_SMS;   // per projection
 
 constexpr int kVjpSlots = kVjpMaxBlocks * (kVjpThreads / 32);   // resident warps
 
