@@ -206,8 +206,10 @@ def kernel_bytes_per_px(ns: int) -> dict:
                   spectrum (4 B/px); col reads + writes the spectrum;
                   row_inv reads the spectrum and T, writes T'.
     n_s lines:    splat reads T and D, writes D - P and the split residuals
-                  r_s; row_fwd reads T and r_s, writes n_s spectra; col
-                  8 B/px/line; row_inv reads n_s spectra and T, writes T'."""
+                  r_s (and P, which only the passes over the long-shift
+                  sources read: not counted); row_fwd reads T and r_s, writes
+                  n_s spectra; col 8 B/px/line; row_inv reads n_s spectra and
+                  T, writes T'."""
     if ns == 1:
         return {"splat": 12, "row_fwd": 12, "col": 8, "row_inv": 12}
     return {"splat": 12 + 4 * ns, "row_fwd": 4 + 8 * ns, "col": 8 * ns, "row_inv": 8 + 4 * ns}

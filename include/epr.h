@@ -75,7 +75,9 @@ typedef struct {
                               overflow list and are added with global atomics. */
     int deterministic;     /* 1 = accumulate the splat in int64 fixed point
                               (value * 2^40, round to nearest even): results are
-                              bit-identical across runs.  0 (default) = the
+                              bit-identical across runs, and the same in
+                              whatever batch a projection is solved (kernels
+                              are then chosen by its size alone).  0 (default) = the
                               tile accumulators hold round(value * 2^S) in
                               uint32, S = 32 - ceil(log2(2 (2 max_shift_px + 3)^2))
                               (24 at the default reach), and the long-shift
@@ -333,8 +335,8 @@ epr_status epr_precondition_noalloc(float* g, int nx, int ny, double pixel_m, do
 
 /* Kernel kinds reported by epr_profile_read. */
 typedef enum {
-    EPR_KERNEL_SPLAT = 0,    /* forward transport (bilinear redistribution)   */
-    EPR_KERNEL_ROW_FWD = 1,  /* split + adjoint gather + R2C row FFT          */
+    EPR_KERNEL_SPLAT = 0,    /* forward transport, residual and its split     */
+    EPR_KERNEL_ROW_FWD = 1,  /* adjoint gather + R2C row FFT                  */
     EPR_KERNEL_COL = 2,      /* column FFT + Paganin filter + inverse         */
     EPR_KERNEL_ROW_INV = 3,  /* C2R row FFT + update + projection             */
     EPR_KERNEL_LOCAL = 4,    /* local closure stencil                         */

@@ -1,13 +1,19 @@
 // Host runtime of libepr: plans, device workspace, the C ABI of include/epr.h,
 // launch sequences of the solvers and their capture in CUDA graphs.
 //
-// One solver iteration (arXiv 2601.22793, "Iterative inversion") is four
+// One solver iteration (arXiv 2601.22793, "Iterative inversion") is five or six
 // kernels over the whole batch:
-//   splat     forward transport of all lines, P and P_s        (splat.cu)
-//   row_fwd   split + adjoint gather + R2C row FFT, rho share  (rowfft.cu)
-//   col       column FFT, Paganin filter, inverse column FFT   (colfft.cu)
-//   row_inv   C2R row FFT + update + projection, kappa share   (rowfft.cu)
-// The local solver replaces splat by the stencil closure (local.cu) and the
+//   splat     forward transport of all lines; the residual D - P and its split
+//             over the lines                                     (splat.cu)
+//   overflow  the sources shifted beyond the splat's reach       (splat.cu)
+//   fix       several lines or fixed point: the split of the pixels that these
+//             reach                                              (splat.cu)
+//   row_fwd   adjoint gather + R2C row FFT, rho share            (rowfft.cu)
+//   col       column FFT, Paganin filter, inverse column FFT     (colfft.cu)
+//   row_inv   C2R row FFT + update + projection, kappa share     (rowfft.cu)
+// The second-order model and an oversampled grid form the residual in a kernel
+// after these (local.cu, splat.cu).  The local solver replaces the transport by
+// the stencil closure (local.cu), which forms the residual itself, and the
 // gather by the identity.  The iteration loop is captured once per
 // (buffers, batch, options) into a CUDA graph and replayed.
 #include <math.h>
@@ -1100,8 +1106,7 @@ epr_status epr_precondition(epr_plan_t p, float* g, int line, int batch, void* s
 {
     if (!p || !g || batch <= 0 || line < 0 || line >= p->C.ns) return EPR_ERR_INVALID_ARG;
     if (!aligned16(g)) return EPR_ERR_INVALID_ARG;
-    // the stand-alone passes run the runtime-sized engine, whose blocks hold
-    // rows and columns of up to 4096 points
+    // rows and columns of up to 4096 points, the sides of a detector
     if (p->C.nx > 4096 || p->C.ny > 4096) return EPR_ERR_UNSUPPORTED_SIZE;
     EPR_TRY(cudaSetDevice(p->device));
     cudaStream_t s = (cudaStream_t)stream;

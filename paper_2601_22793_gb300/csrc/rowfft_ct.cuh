@@ -17,8 +17,8 @@ constexpr int kPad = 4;   // float2 padding between packed rows in shared memory
 struct RowArgs {
     const float* T;          // [B][ny][nx]
     const float* D;          // [B][ny][nx]
-    const float* P;          // [B][ny][nx]   P, or D - P when `resid`
-    const float* Ps;         // [B][ns][ny][nx]
+    const float* P;          // [B][ny][nx]   residual D - P
+    const float* Ps;         // [B][ns][ny][nx]   split residuals r_s (ns > 1)
     const float* G;          // [B][ny][nx] real input of a plain transform, else NULL
     float* Out;              // [B][ny][nx] real output (INV_STORE) or T (INV_UPDATE)
     float2* S;               // [B][nl][ny][nx/2]
@@ -88,7 +88,7 @@ __device__ __forceinline__ void fwd_finalize_kappa(const RowArgs& A, int b, bool
 
 // ln(1 + q) for |q| < 1/4 from ln(1 + q) = 2 atanh(z), z = q / (2 + q), and
 // the Taylor series of atanh: 2 z (1 + z^2/3 + z^4/5 + ... + z^10/11).  Here
-// |z| < 1/7, so the first omitted term, 2 |z|^13 / 13, is below 4e-12 |z|:
+// |z| < 1/7, so the first omitted term, 2 |z|^13 / 13, is below 1.2e-11 |z|:
 // the error is the rounding of the few operations.
 __device__ __forceinline__ float log1p_atanh(float q)
 {

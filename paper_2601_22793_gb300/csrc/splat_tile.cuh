@@ -314,10 +314,10 @@ k_splat(const __grid_constant__ EprConsts C, const SplatArgs A)
     // row gradients of both pairs.  The scan was bound by instruction issue
     // (75 % active in a batch): the packed forms, the floor by rounding mode
     // (FRND and F2I run at an eighth of the FMA rate) and one long-shift test
-    // per quad took it from 123 to 91 thread instructions per pixel, and the
-    // kernel from 142 to 103 us for eight 2048^2 projections; what bounds it
-    // now is the shared-memory data pipe (80 % busy: the loads of the staged
-    // window and the accumulator atomics).
+    // per quad took the kernel from 123 to 94 thread instructions per pixel and
+    // from 142 to 103 us for eight 2048^2 projections.  Instruction issue is
+    // still what bounds it (81 % active; the L1 data path, for the staged
+    // window and the accumulator atomics, 66 %).
     // Work item (qy, lx) is advanced by kSplatThreads = dly quad rows +
     // dlx columns.
     const int nitem = RHq * RW;
