@@ -318,7 +318,7 @@ epr_status epr_check_device_status(epr_plan_t plan, void* stream);
  * has no counterpart: this serves callers that cannot let a library call
  * cudaMalloc (their device memory is owned by their own pool allocator or
  * fixed at start-up, or an allocation's possible device synchronisation is
- * not acceptable).  Scratch lives in a static device array of 16 MiB + 64 KiB
+ * not acceptable).  Scratch lives in a static device array of 16 MiB + 256 KiB
  * that every GPU loading the library holds until the process exits; it
  * bounds batch * nx * ny to 4 Mi pixels (e.g. one 2048 x 2048 map), and a
  * larger request returns EPR_ERR_UNSUPPORTED_SIZE.  Every call looks up the

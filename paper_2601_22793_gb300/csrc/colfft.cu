@@ -100,6 +100,7 @@ k_col_ct(const EprConsts C, const ColArgs A)
 {
     constexpr int T = NY * CW / EPT;
     constexpr int LGCW = CW == 1 ? 0 : CW == 2 ? 1 : CW == 4 ? 2 : CW == 8 ? 3 : 4;
+    static_assert(!eprfft::tw_exact(NY), "table 0 alone is there");
     extern __shared__ __align__(16) float2 buf[];
     const int b = blockIdx.z, sl = blockIdx.y;
     epr_grid_wait();

@@ -15,7 +15,7 @@ namespace eprcol {
 struct ColArgs {
     float2* S;            // [B][nl][ny][nx/2]
     EprProjState* st;
-    const float2* tw;     // exp(-2 pi i t / ny)
+    const float2* tw;     // twiddle tables of length ny
     unsigned int* err;    // device error word
     const double* part_c; // [B][max_blocks] forward row pass partials
     double* rho_hist;     // [B][hist_len]

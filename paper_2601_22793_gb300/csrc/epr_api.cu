@@ -31,6 +31,7 @@
 #include <cuda.h>
 
 #include "epr_internal.cuh"
+#include "fft.cuh"
 
 // --- launchers from the other translation units -----------------------------
 cudaError_t epr_launch_splat(const EprConsts& C, const EprWork& W, const float* T, const float* D,
@@ -854,6 +855,28 @@ bool line_constants(epr_plan_s* p, double L_m, const double* delta, const double
     return true;
 }
 
+// The first `tables` twiddle tables of length n, from values formed in double.
+cudaError_t upload_twiddles(int n, int tables, float2** out)
+{
+    std::vector<float2> tw((size_t)tables * n);
+    for (int t = 0; t < n; ++t) {
+        const double a = -2.0 * kPi * (double)t / n;
+        tw[t] = make_float2((float)cos(a), (float)sin(a));
+    }
+    for (int tab = 1; tab < tables; ++tab) {
+        const eprfft::TwPlan p(n, tab);
+        for (int s = 1; s < p.stages; ++s)
+            for (int r = 1; r < p.r[s]; ++r) {
+                const int step = r * (n / (p.ns[s] * p.r[s]));
+                float2* to = tw.data() + (size_t)tab * n + r * p.ns[s];
+                for (int jm = 0; jm < p.ns[s]; ++jm) to[jm] = tw[jm * step];
+            }
+    }
+    cudaError_t e = cudaMalloc((void**)out, tw.size() * sizeof(float2));
+    if (e == cudaSuccess) e = cudaMemcpy(*out, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice);
+    return e;
+}
+
 std::mutex g_init_mu;
 int g_init_done[64];
 
@@ -964,20 +987,10 @@ epr_status epr_plan_create(epr_plan_t* out, int nx, int ny, double pixel_m, doub
         delete p;
         return st;
     }
-    // twiddle tables exp(-2 pi i t / n), built in double
-    std::vector<float2> tw(nx > ny ? nx : ny);
-    for (int t = 0; t < nx; ++t) {
-        const double a = -2.0 * kPi * (double)t / nx;
-        tw[t] = make_float2((float)cos(a), (float)sin(a));
-    }
-    e = cudaMalloc((void**)&p->tw_x, nx * sizeof(float2));
-    if (e == cudaSuccess) e = cudaMemcpy(p->tw_x, tw.data(), nx * sizeof(float2), cudaMemcpyHostToDevice);
-    for (int t = 0; t < ny; ++t) {
-        const double a = -2.0 * kPi * (double)t / ny;
-        tw[t] = make_float2((float)cos(a), (float)sin(a));
-    }
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p->tw_y, ny * sizeof(float2));
-    if (e == cudaSuccess) e = cudaMemcpy(p->tw_y, tw.data(), ny * sizeof(float2), cudaMemcpyHostToDevice);
+    // the plain row passes of every length read the stage tables, the columns
+    // those of an exact length
+    e = upload_twiddles(nx, eprfft::kTwTables, &p->tw_x);
+    if (e == cudaSuccess) e = upload_twiddles(ny, eprfft::tw_exact(ny) ? eprfft::kTwTables : 1, &p->tw_y);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         if (p->tw_x) cudaFree(p->tw_x);

@@ -91,8 +91,8 @@ struct EprWork {
     double* rho_hist;    // [B][hist_len]
     double* kappa_hist;  // [B][hist_len]
     unsigned int* err;   // device error word
-    const float2* tw_x;  // twiddles exp(-2 pi i t / nx), t < nx
-    const float2* tw_y;  // twiddles exp(-2 pi i t / ny), t < ny
+    const float2* tw_x;  // twiddle tables of length nx (kTwTables in fft.cuh)
+    const float2* tw_y;  // and of length ny
     int hist_len;        // columns of rho_hist / kappa_hist
     int max_blocks;      // columns of part_a / part_b / part_c
     const void* col_map; // host: CUtensorMap of S for the column pass's bulk

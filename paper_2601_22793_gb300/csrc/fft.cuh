@@ -35,32 +35,20 @@
 
 namespace eprfft {
 
-// Where the powers w^2 .. w^(R-1) of a stage's twiddle come from
-// (apply_twiddles).  A power from the table carries one rounding, but its loads
-// are scattered: lane j reads entry r j N / (Ns R).
-//   TREE  products of lower powers, from w alone, at most 4 roundings deep
-//   HALF  w^2, w^4 and w^8 from the table as well
-//   FINE  w, w^2, w^3 and every fourth power from the table
-//   FULL  every power from the table
-enum { TW_TREE = 0, TW_HALF = 1, TW_FINE = 2, TW_FULL = 3 };
-
-// Lengths whose passes take the more exact forms: those with a factor 9, and
-// the short ones with a factor 3 or below 256.  Their stages are many and of
-// mixed radix, and the tree's error in them is the larger one: relative error
-// of the filter at 1728 x 1728 5.1e-7 with TREE, 2.8e-7 with HALF rows and FINE
-// columns, 2.6e-7 with FULL; of a solve at 1728 x 1152 2.65e-7 with TREE,
-// 1.98e-7 with HALF rows and FULL columns (20 iterations of two lines 1983 and
-// 2028 us).  The powers of two from 256 on and 1536 and 3072, which carry the
-// large frames, keep TREE in a solve: 2048^2 takes 22 % more with FULL, four
-// lines of mixed sizes up to 3072 x 2048 3 to 10 %, and their error (2048
-// points: 1.8e-7 in radix 8, 2.5e-7 in radix 16) is well below the 4.2e-7 and
-// 6.5e-7 of a three-term recurrence of cos and sin.
+// Lengths whose passes read every power of a twiddle from a table (EXACT of
+// apply_twiddles): those with a factor 9, and the short ones with a factor 3 or
+// below 256.  Their stages are many and of mixed radix, and the error of powers
+// formed as products is the larger one there: of the filter at 1728 x 1728
+// 5.1e-7 where it is 2.6e-7 with the table, of a solve at 1728 x 1152 2.65e-7
+// and 1.98e-7.  The powers of two from 256 on and 1536 and 3072 keep the products
+// in a solve: 2048^2 takes 3367 us with them and 3388 with the table (256^2 347
+// and 355), and their error (2048 points: 1.8e-7 in radix 8, 2.5e-7 in radix 16)
+// is well below the 4.2e-7 and 6.5e-7 of a three-term recurrence of cos and sin.
 __host__ __device__ constexpr bool tw_exact(int n) { return n % 9 == 0 || (n % 3 == 0 && n < 1536) || n < 256; }
 
 // Each policy also states a period P and the address step of adding a
 // multiple c of P to an index: idx(i + c) = idx(i) + step(c) for every i, and
-// how the passes that use it form their twiddles at length n.  A
-// stage whose operand stride is a multiple of P computes one address and adds
+// whether the passes that use it read every twiddle power of length n.  A stage whose operand stride is a multiple of P computes one address and adds
 // constants.
 struct PadRow {
     __host__ __device__ static __forceinline__ int idx(int i)
@@ -70,14 +58,13 @@ struct PadRow {
     __host__ __device__ static __forceinline__ int len(int n) { return (n + 15) & ~15; }
     static constexpr int kPeriod = 128;   // the swizzle reads bits 0..6 only
     __host__ __device__ static constexpr int step(int c) { return c; }
-    __host__ __device__ static constexpr int tw(int n) { return tw_exact(n) ? TW_HALF : TW_TREE; }
+    __host__ __device__ static constexpr bool exact(int n) { return tw_exact(n); }
 };
 
 // The rows of the plain transforms, the stand-alone filter's: no iteration
-// corrects their error.  FINE costs 2048^2 37.5 us for 32.6 with TREE, and FULL
-// 43.3 for another 1 % of the error.
+// corrects their error (2048^2 33.7 us, 32.8 with products).
 struct PadPlain : PadRow {
-    __host__ __device__ static constexpr int tw(int n) { return tw_exact(n) ? TW_FULL : TW_FINE; }
+    __host__ __device__ static constexpr bool exact(int) { return true; }
 };
 
 struct PadCol {
@@ -85,7 +72,7 @@ struct PadCol {
     __host__ __device__ static __forceinline__ int len(int n) { return n + 2 * (n >> 4) + 2; }
     static constexpr int kPeriod = 16;
     __host__ __device__ static constexpr int step(int c) { return c + 2 * (c >> 4); }
-    __host__ __device__ static constexpr int tw(int n) { return tw_exact(n) ? TW_FULL : TW_TREE; }
+    __host__ __device__ static constexpr bool exact(int n) { return tw_exact(n); }
 };
 
 // Plain dense layout (a tile written by a bulk copy).
@@ -370,8 +357,8 @@ __device__ void fft(float2* buf, int N, int lgseq, int sj, int sm, const float2*
 // sequences (1 << LGSEQ), the strides SJ / SM and the elements per thread are
 // template parameters, so every stage is unrolled, strides fold into address
 // offsets, the first stage (Ns = 1) needs no twiddle, and a radix-R stage
-// loads one twiddle w = exp(DIR 2 pi i jm / (Ns R)) and forms w^2 .. w^(R-1)
-// as products (apply_twiddles).
+// loads w^1 .. w^(R-1), w = exp(DIR 2 pi i jm / (Ns R)), or w and forms the
+// others as products (apply_twiddles).
 // ---------------------------------------------------------------------------
 namespace eprfft {
 
@@ -438,23 +425,52 @@ __host__ __device__ constexpr int ct_ns_rev(int n, int s, int maxr = 8)
     return v;
 }
 
-__host__ __device__ constexpr bool tw_loaded(int mode, int r)
-{
-    return r == 1 || mode == TW_FULL || (mode == TW_HALF && (r & (r - 1)) == 0) ||
-           (mode == TW_FINE && (r < 4 || r % 4 == 0));
-}
+// Twiddle tables of length n, kTwTables of n entries each.  Table 0 holds
+// exp(-2 pi i t / n) at t.  The others belong to the stage plans of largest radix
+// 4, 8 and 16 and their reversals: the stage with Ns holds w^(r jm), w = exp(-2 pi
+// i / (Ns R)), at r Ns + jm (r = 1 .. R - 1, jm < Ns), so that the lanes of a warp
+// read consecutive entries.  The regions of a plan's stages follow one another
+// and end at n; the entries below the second stage's Ns are unused.  (From table
+// 0, whose lanes lie r n / (Ns R) entries apart, a filter of four 2304 x 1536 maps
+// took 122.6 us in place of 108.6, and a 2592 x 2304 solve 1209 in place of 1126.)
+constexpr int kTwTables = 7;
+__host__ __device__ constexpr int tw_table(int maxr, bool rev) { return (maxr >= 16 ? 5 : maxr >= 8 ? 3 : 1) + rev; }
 
-// v[r] *= w^r with w = exp(DIR 2 pi i i / N).  A power that is not loaded is the
-// product of two lower ones (TREE: w^2 = w w, w^3 = w^2 w, w^4 = w^2 w^2, ...).
-template <int R, int DIR, int MODE>
-__device__ __forceinline__ void apply_twiddles(float2 (&v)[R], const float2* __restrict__ tw, int i)
+struct TwPlan {
+    int n, stages, ns[16], r[16];
+    __host__ __device__ TwPlan(int n_, int tab) : n(n_), stages(0)
+    {
+        if (tab == 0) return;
+        const int maxr = tab >= 5 ? 16 : tab >= 3 ? 8 : 4;
+        const int count = ct_n_stages(n, maxr);
+        for (int v = 1; stages < count; v *= r[stages - 1]) {
+            ns[stages] = v;
+            r[stages] = tab % 2 == 0 ? ct_radix(n, count - 1 - stages, maxr) : ct_radix(n, stages, maxr);
+            ++stages;
+        }
+    }
+    // the entry of table 0 that entry e of this table repeats
+    __host__ __device__ int source(int e) const
+    {
+        if (stages == 0) return e;
+        for (int s = 1; s < stages; ++s)
+            if (e >= ns[s] && e < ns[s] * r[s]) return (e / ns[s]) * (e % ns[s]) * (n / (ns[s] * r[s]));
+        return 0;   // unused
+    }
+};
+
+// v[r] *= w^r with w = exp(DIR 2 pi i jm / (NS R)).  EXACT: every power from
+// table TAB.  Else from w alone, each other power a product of two lower ones
+// (w^2 = w w, w^3 = w^2 w, w^4 = w^2 w^2, ...), at most 4 roundings deep.
+template <int R, int DIR, bool EXACT, int N, int NS, int TAB>
+__device__ __forceinline__ void apply_twiddles(float2 (&v)[R], const float2* __restrict__ tw, int jm)
 {
     float2 p[R];
 #pragma unroll
     for (int r = 1; r < R; ++r) {
-        const int h = MODE == TW_FINE ? r & ~3 : r >= 8 ? 8 : r >= 4 ? 4 : 2;
-        if (tw_loaded(MODE, r)) {
-            p[r] = __ldg(&tw[r * i]);
+        const int h = r >= 8 ? 8 : r >= 4 ? 4 : 2;
+        if (EXACT || r == 1) {
+            p[r] = __ldg(tw + (EXACT ? TAB * N + r * NS + jm : jm * (N / (NS * R))));
             if (DIR > 0) p[r].y = -p[r].y;
         } else if (h == r) {
             const float2 q = p[r / 2];
@@ -497,7 +513,7 @@ struct Identity {
 // barrier, so in == buf works even when PADI != PAD.  STORE = false hands
 // each result to post only (post(value, e) for its side effects, nothing is
 // written); SYNC_END = false leaves out the closing barrier.
-template <class PADI, class PAD, int R, int DIR, int EPT, int N, int NS, int LGSEQ, int SJ, int SM,
+template <class PADI, class PAD, int R, int DIR, int EPT, int N, int NS, int LGSEQ, int SJ, int SM, int TAB,
           class POST = Identity, bool STORE = true, bool SYNC_END = true>
 __device__ __forceinline__ void stage_ct(const float2* in, float2* buf, const float2* __restrict__ tw,
                                          int tid, const POST& post = POST())
@@ -507,7 +523,6 @@ __device__ __forceinline__ void stage_ct(const float2* in, float2* buf, const fl
     constexpr int PER = (EPT + R - 1) / R;
     constexpr int NR = N / R;
     constexpr int NB = NR * NSEQ;
-    constexpr int TWSTEP = N / (NS * R);
     float2 v[PER][R];
     int dst[PER];
 #pragma unroll
@@ -529,7 +544,7 @@ __device__ __forceinline__ void stage_ct(const float2* in, float2* buf, const fl
                 for (int r = 0; r < R; ++r) v[k][r] = in[PADI::idx((j + r * NR) * SJ + base)];
             }
             if constexpr (NS > 1) {
-                apply_twiddles<R, DIR, PADI::tw(N)>(v[k], tw, jm * TWSTEP);
+                apply_twiddles<R, DIR, PADI::exact(N), N, NS, TAB>(v[k], tw, jm);
             }
             dst[k] = (jd * NS * R + jm) * SJ + base;
         }
@@ -562,7 +577,7 @@ template <class PAD, int DIR, int N, int EPT, int LGSEQ, int SJ, int SM, int S, 
 __device__ __forceinline__ void fft_ct_stages(float2* buf, const float2* __restrict__ tw, int tid)
 {
     if constexpr (S < SEND) {
-        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM>(buf, buf,
+        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, false)>(buf, buf,
                                                                                               tw, tid);
         fft_ct_stages<PAD, DIR, N, EPT, LGSEQ, SJ, SM, S + 1, SEND, MAXR>(buf, tw, tid);
     }
@@ -577,7 +592,7 @@ __device__ __forceinline__ void fft_ct_last(float2* buf, const float2* __restric
                                             const POST& post = POST())
 {
     constexpr int S = ct_n_stages(N, MAXR) - 1;
-    stage_ct<PAD, PADO, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM, POST, STORE,
+    stage_ct<PAD, PADO, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, false), POST, STORE,
              SYNC_END>(buf, buf, tw, tid, post);
 }
 
@@ -586,7 +601,7 @@ template <class PAD, int DIR, int N, int EPT, int LGSEQ, int SJ, int SM, int S, 
 __device__ __forceinline__ void fft_ct_rev_stages(float2* buf, const float2* __restrict__ tw, int tid)
 {
     if constexpr (S < SEND) {
-        stage_ct<PAD, PAD, ct_radix_rev(N, S, MAXR), DIR, EPT, N, ct_ns_rev(N, S, MAXR), LGSEQ, SJ, SM>(
+        stage_ct<PAD, PAD, ct_radix_rev(N, S, MAXR), DIR, EPT, N, ct_ns_rev(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, true)>(
             buf, buf, tw, tid);
         fft_ct_rev_stages<PAD, DIR, N, EPT, LGSEQ, SJ, SM, S + 1, SEND, MAXR>(buf, tw, tid);
     }
@@ -600,7 +615,7 @@ __device__ __forceinline__ void fft_ct_rev_last(float2* buf, const float2* __res
                                                 const POST& post = POST())
 {
     constexpr int S = ct_n_stages(N, MAXR) - 1;
-    stage_ct<PAD, PADO, ct_radix_rev(N, S, MAXR), DIR, EPT, N, ct_ns_rev(N, S, MAXR), LGSEQ, SJ, SM, POST,
+    stage_ct<PAD, PADO, ct_radix_rev(N, S, MAXR), DIR, EPT, N, ct_ns_rev(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, true), POST,
              STORE, SYNC_END>(buf, buf, tw, tid, post);
 }
 
@@ -611,7 +626,7 @@ __device__ __forceinline__ void fft_ct_from_stages(const float2* in, float2* buf
                                                    const float2* __restrict__ tw, int tid)
 {
     static_assert(SEND >= 1, "at least the first stage");
-    stage_ct<Dense, PAD, ct_radix(N, 0, MAXR), DIR, EPT, N, 1, LGSEQ, SJ, SM>(in, buf, tw, tid);
+    stage_ct<Dense, PAD, ct_radix(N, 0, MAXR), DIR, EPT, N, 1, LGSEQ, SJ, SM, 0>(in, buf, tw, tid);
     fft_ct_stages<PAD, DIR, N, EPT, LGSEQ, SJ, SM, 1, SEND, MAXR>(buf, tw, tid);
 }
 
@@ -637,7 +652,6 @@ __device__ __forceinline__ void stage_turn(float2* buf, const float2* __restrict
     constexpr int PER = (EPT + R - 1) / R;
     constexpr int NR = N / R;
     constexpr int NB = NR * NSEQ;
-    constexpr int TWSTEP = N / (NS * R);
     float2 v[PER][R];
     int j_of[PER], m_of[PER];
 #pragma unroll
@@ -651,7 +665,7 @@ __device__ __forceinline__ void stage_turn(float2* buf, const float2* __restrict
 #pragma unroll
             for (int r = 0; r < R; ++r) v[k][r] = buf[PAD::idx((j + r * NR) * SJ + base)];
             if constexpr (NS > 1) {
-                apply_twiddles<R, DIRF, PAD::tw(N)>(v[k], tw, j * TWSTEP);
+                apply_twiddles<R, DIRF, PAD::exact(N), N, NS, tw_table(MAXR, false)>(v[k], tw, j);
             }
             j_of[k] = j;
             m_of[k] = m;
@@ -700,11 +714,11 @@ __device__ __forceinline__ void fft_ct(float2* buf, const float2* __restrict__ t
 {
     static_assert(MAXR <= EPT, "a stage's butterfly holds MAXR elements of one thread");
     if constexpr (S + 1 < ct_n_stages(N, MAXR)) {
-        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM>(buf, buf,
+        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, false)>(buf, buf,
                                                                                               tw, tid);
         fft_ct<PAD, DIR, N, EPT, LGSEQ, SJ, SM, S + 1, MAXR>(buf, tw, tid, post);
     } else if constexpr (S + 1 == ct_n_stages(N, MAXR)) {
-        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM>(
+        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, false)>(
             buf, buf, tw, tid, post);
     }
 }
@@ -718,9 +732,9 @@ __device__ __forceinline__ void fft_ct_from(const float2* in, float2* buf, const
                                             int tid, const POST& post = POST())
 {
     if constexpr (ct_n_stages(N, MAXR) == 1) {
-        stage_ct<Dense, PAD, ct_radix(N, 0, MAXR), DIR, EPT, N, 1, LGSEQ, SJ, SM>(in, buf, tw, tid, post);
+        stage_ct<Dense, PAD, ct_radix(N, 0, MAXR), DIR, EPT, N, 1, LGSEQ, SJ, SM, 0>(in, buf, tw, tid, post);
     } else {
-        stage_ct<Dense, PAD, ct_radix(N, 0, MAXR), DIR, EPT, N, 1, LGSEQ, SJ, SM>(in, buf, tw, tid);
+        stage_ct<Dense, PAD, ct_radix(N, 0, MAXR), DIR, EPT, N, 1, LGSEQ, SJ, SM, 0>(in, buf, tw, tid);
         fft_ct<PAD, DIR, N, EPT, LGSEQ, SJ, SM, 1, MAXR>(buf, tw, tid, post);
     }
 }

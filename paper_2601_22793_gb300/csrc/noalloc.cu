@@ -8,7 +8,7 @@
 // cudaMalloc, which may synchronise the device, is not acceptable.
 // epr_precondition_noalloc serves them: it runs the same three kernels as
 // epr_precondition (forward row FFT, column filter, inverse row FFT) but
-// keeps its scratch -- the packed half spectrum and the two twiddle tables
+// keeps its scratch -- the packed half spectrum and the twiddle tables
 // -- in one file-scope __device__ array of fixed size.  It calls no
 // cudaMalloc, cudaFree or other allocating routine.
 //
@@ -24,13 +24,14 @@
 #include <mutex>
 
 #include "epr_internal.cuh"
+#include "fft.cuh"
 
 // Scratch: up to kNoallocPixels map pixels of half spectrum (4 bytes per
-// pixel) plus the twiddle tables of the two axes.
+// pixel) plus the twiddle tables of the two axes (rows: of every stage plan).
 namespace {
 constexpr size_t kNoallocPixels = (size_t)4 << 20;                 // 4 Mi pixels
 constexpr size_t kNoallocSpectrum = kNoallocPixels * 4;             // 16 MiB
-constexpr size_t kNoallocTwiddles = (size_t)2 * 4096 * sizeof(float2);
+constexpr size_t kNoallocTwiddles = (size_t)(eprfft::kTwTables + 1) * 4096 * sizeof(float2);
 constexpr size_t kNoallocBytes = kNoallocSpectrum + kNoallocTwiddles;
 }  // namespace
 
@@ -46,19 +47,22 @@ cudaError_t epr_launch_row_inv(const EprConsts& C, const EprWork& W, int mode, f
 cudaError_t epr_launch_col(const EprConsts& C, const EprWork& W, int line0, int nl, int batch,
                            int check_done, int cw_hint, int rho_it, cudaStream_t stream);
 cudaError_t epr_row_init(int nx);
+int epr_row_plain_radix(const EprConsts& C, int batch);
 cudaError_t epr_col_init();
 
 namespace {
 
-// exp(-2 pi i t / n) for t < n, in double then rounded (the table a plan
-// builds on the host), written into the scratch array
-__global__ void k_noalloc_twiddles(float2* tw, int n)
+// The tables a plan builds on the host, written into the scratch array: table 0,
+// and with grid y of 2 or 3 those of the stage plan of largest radix maxr and of
+// its reversal (which the inverse of lengths with a factor 3 runs).
+__global__ void k_noalloc_twiddles(float2* tw, int n, int maxr)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    const int tab = blockIdx.y == 0 ? 0 : eprfft::tw_table(maxr, blockIdx.y == 2);
     double s, c;
-    sincospi(-2.0 * (double)t / (double)n, &s, &c);
-    tw[t] = make_float2((float)c, (float)s);
+    sincospi(-2.0 * (double)eprfft::TwPlan(n, tab).source(e) / (double)n, &s, &c);
+    tw[(size_t)tab * n + e] = make_float2((float)c, (float)s);
 }
 
 // Device address of the scratch array.  In host code the array's name is
@@ -136,12 +140,14 @@ extern "C" epr_status epr_precondition_noalloc(float* g, int nx, int ny, double 
     EprWork W = {};
     W.S = reinterpret_cast<float2*>(base);
     float2* tw_x = reinterpret_cast<float2*>(base + kNoallocSpectrum);
-    float2* tw_y = tw_x + 4096;
+    float2* tw_y = tw_x + eprfft::kTwTables * 4096;
     W.tw_x = tw_x;
     W.tw_y = tw_y;
 
-    k_noalloc_twiddles<<<(nx + 255) / 256, 256, 0, s>>>(tw_x, nx);
-    k_noalloc_twiddles<<<(ny + 255) / 256, 256, 0, s>>>(tw_y, ny);
+    // the columns run a plain pass, which reads table 0
+    const int maxr = epr_row_plain_radix(C, batch);
+    k_noalloc_twiddles<<<dim3((nx + 255) / 256, maxr == 0 ? 1 : nx % 3 ? 2 : 3), 256, 0, s>>>(tw_x, nx, maxr);
+    k_noalloc_twiddles<<<(ny + 255) / 256, 256, 0, s>>>(tw_y, ny, 0);
     epr_count_launch(2);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = epr_launch_row_fwd(C, W, 2, nullptr, nullptr, g, 0, 1, 0, 0.f, batch, 0, s);

@@ -534,6 +534,14 @@ cudaError_t epr_launch_solve_begin(const EprConsts& C, const EprWork& W, const f
 // Blocks of a row pass (the number of partials a reduction adds up).
 int epr_row_blocks(const EprConsts& C, int batch) { return C.ny / (2 * epr_row_config(C, batch, true).RP); }
 
+// Largest radix of the plain row transforms of a launch (which stage table they
+// read); 0: the runtime-sized ones.
+int epr_row_plain_radix(const EprConsts& C, int batch)
+{
+    const EprRowLaunch L = epr_row_config(C, batch, false);
+    return L.k ? row_maxr(C.nx * L.RP / L.k->threads_plain) : 0;
+}
+
 namespace {
 
 // kappa of the last iteration of a solve (the forward pass of a following

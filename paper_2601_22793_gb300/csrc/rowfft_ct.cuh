@@ -27,7 +27,7 @@ struct RowArgs {
     double* part_b;
     double* part_c;          // [B][max_blocks] forward pass partials (rho)
     double* hist;            // kappa history (finalised by the forward pass)
-    const float2* tw;        // exp(-2 pi i t / nx)
+    const float2* tw;        // twiddle tables of length nx
     int RP, lgRP;            // row pairs per block
     int line0, nl;           // first physical line, number of lines handled
     int it, hist_len, max_blocks;
