@@ -44,12 +44,16 @@ namespace eprfft {
 // in a solve: 2048^2 takes 3367 us with them and 3388 with the table (256^2 347
 // and 355), and their error (2048 points: 1.8e-7 in radix 8, 2.5e-7 in radix 16)
 // is well below the 4.2e-7 and 6.5e-7 of a three-term recurrence of cos and sin.
-__host__ __device__ constexpr bool tw_exact(int n) { return n % 9 == 0 || (n % 3 == 0 && n < 1536) || n < 256; }
+__host__ __device__ constexpr bool tw_exact(int n)
+{
+    return n % 9 == 0 || (n % 3 == 0 && n < 1536) || n < 256;
+}
 
 // Each policy also states a period P and the address step of adding a
-// multiple c of P to an index: idx(i + c) = idx(i) + step(c) for every i, and
-// whether the passes that use it read every twiddle power of length n.  A stage whose operand stride is a multiple of P computes one address and adds
-// constants.
+// multiple c of P to an index: idx(i + c) = idx(i) + step(c) for every i.  A
+// stage whose operand stride is a multiple of P computes one address and adds
+// constants.  exact(n): whether the passes that use the policy read every
+// twiddle power of length n.
 struct PadRow {
     __host__ __device__ static __forceinline__ int idx(int i)
     {
@@ -434,7 +438,10 @@ __host__ __device__ constexpr int ct_ns_rev(int n, int s, int maxr = 8)
 // 0, whose lanes lie r n / (Ns R) entries apart, a filter of four 2304 x 1536 maps
 // took 122.6 us in place of 108.6, and a 2592 x 2304 solve 1209 in place of 1126.)
 constexpr int kTwTables = 7;
-__host__ __device__ constexpr int tw_table(int maxr, bool rev) { return (maxr >= 16 ? 5 : maxr >= 8 ? 3 : 1) + rev; }
+__host__ __device__ constexpr int tw_table(int maxr, bool rev)
+{
+    return (maxr >= 16 ? 5 : maxr >= 8 ? 3 : 1) + (rev ? 1 : 0);
+}
 
 struct TwPlan {
     int n, stages, ns[16], r[16];
@@ -454,7 +461,8 @@ struct TwPlan {
     {
         if (stages == 0) return e;
         for (int s = 1; s < stages; ++s)
-            if (e >= ns[s] && e < ns[s] * r[s]) return (e / ns[s]) * (e % ns[s]) * (n / (ns[s] * r[s]));
+            if (e >= ns[s] && e < ns[s] * r[s])
+                return (e / ns[s]) * (e % ns[s]) * (n / (ns[s] * r[s]));
         return 0;   // unused
     }
 };
@@ -512,9 +520,10 @@ struct Identity {
 // `buf` (layout PAD).  Every operand is read before the stage's first
 // barrier, so in == buf works even when PADI != PAD.  STORE = false hands
 // each result to post only (post(value, e) for its side effects, nothing is
-// written); SYNC_END = false leaves out the closing barrier.
-template <class PADI, class PAD, int R, int DIR, int EPT, int N, int NS, int LGSEQ, int SJ, int SM, int TAB,
-          class POST = Identity, bool STORE = true, bool SYNC_END = true>
+// written); SYNC_END = false leaves out the closing barrier.  TAB: the twiddle
+// table of the stage's plan.
+template <class PADI, class PAD, int R, int DIR, int EPT, int N, int NS, int LGSEQ, int SJ, int SM,
+          int TAB, class POST = Identity, bool STORE = true, bool SYNC_END = true>
 __device__ __forceinline__ void stage_ct(const float2* in, float2* buf, const float2* __restrict__ tw,
                                          int tid, const POST& post = POST())
 {
@@ -577,8 +586,8 @@ template <class PAD, int DIR, int N, int EPT, int LGSEQ, int SJ, int SM, int S, 
 __device__ __forceinline__ void fft_ct_stages(float2* buf, const float2* __restrict__ tw, int tid)
 {
     if constexpr (S < SEND) {
-        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, false)>(buf, buf,
-                                                                                              tw, tid);
+        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM,
+                 tw_table(MAXR, false)>(buf, buf, tw, tid);
         fft_ct_stages<PAD, DIR, N, EPT, LGSEQ, SJ, SM, S + 1, SEND, MAXR>(buf, tw, tid);
     }
 }
@@ -592,8 +601,8 @@ __device__ __forceinline__ void fft_ct_last(float2* buf, const float2* __restric
                                             const POST& post = POST())
 {
     constexpr int S = ct_n_stages(N, MAXR) - 1;
-    stage_ct<PAD, PADO, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, false), POST, STORE,
-             SYNC_END>(buf, buf, tw, tid, post);
+    stage_ct<PAD, PADO, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM,
+             tw_table(MAXR, false), POST, STORE, SYNC_END>(buf, buf, tw, tid, post);
 }
 
 // Stages S .. SEND - 1 of the reversed plan, no output map.
@@ -601,8 +610,8 @@ template <class PAD, int DIR, int N, int EPT, int LGSEQ, int SJ, int SM, int S, 
 __device__ __forceinline__ void fft_ct_rev_stages(float2* buf, const float2* __restrict__ tw, int tid)
 {
     if constexpr (S < SEND) {
-        stage_ct<PAD, PAD, ct_radix_rev(N, S, MAXR), DIR, EPT, N, ct_ns_rev(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, true)>(
-            buf, buf, tw, tid);
+        stage_ct<PAD, PAD, ct_radix_rev(N, S, MAXR), DIR, EPT, N, ct_ns_rev(N, S, MAXR), LGSEQ, SJ, SM,
+                 tw_table(MAXR, true)>(buf, buf, tw, tid);
         fft_ct_rev_stages<PAD, DIR, N, EPT, LGSEQ, SJ, SM, S + 1, SEND, MAXR>(buf, tw, tid);
     }
 }
@@ -615,8 +624,8 @@ __device__ __forceinline__ void fft_ct_rev_last(float2* buf, const float2* __res
                                                 const POST& post = POST())
 {
     constexpr int S = ct_n_stages(N, MAXR) - 1;
-    stage_ct<PAD, PADO, ct_radix_rev(N, S, MAXR), DIR, EPT, N, ct_ns_rev(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, true), POST,
-             STORE, SYNC_END>(buf, buf, tw, tid, post);
+    stage_ct<PAD, PADO, ct_radix_rev(N, S, MAXR), DIR, EPT, N, ct_ns_rev(N, S, MAXR), LGSEQ, SJ, SM,
+             tw_table(MAXR, true), POST, STORE, SYNC_END>(buf, buf, tw, tid, post);
 }
 
 // Stages 0 .. SEND - 1 of the transform with its input in a dense tile `in`
@@ -714,12 +723,12 @@ __device__ __forceinline__ void fft_ct(float2* buf, const float2* __restrict__ t
 {
     static_assert(MAXR <= EPT, "a stage's butterfly holds MAXR elements of one thread");
     if constexpr (S + 1 < ct_n_stages(N, MAXR)) {
-        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, false)>(buf, buf,
-                                                                                              tw, tid);
+        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM,
+                 tw_table(MAXR, false)>(buf, buf, tw, tid);
         fft_ct<PAD, DIR, N, EPT, LGSEQ, SJ, SM, S + 1, MAXR>(buf, tw, tid, post);
     } else if constexpr (S + 1 == ct_n_stages(N, MAXR)) {
-        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM, tw_table(MAXR, false)>(
-            buf, buf, tw, tid, post);
+        stage_ct<PAD, PAD, ct_radix(N, S, MAXR), DIR, EPT, N, ct_ns(N, S, MAXR), LGSEQ, SJ, SM,
+                 tw_table(MAXR, false)>(buf, buf, tw, tid, post);
     }
 }
 
