@@ -22,8 +22,8 @@
 // loads (four corners per line and pixel, from L1 and L2): long scoreboard is
 // the top stall, half of the issue slots are used.  The corners of all lines
 // are therefore loaded before the first is used, and the strips are cut so
-// that every resident warp has one: 39.1 us where the two-pass form took 51.4
-// (1536 x 1024, 3 lines; one line 21.6 and 38.2).
+// that every resident warp has one: 41.1 us where the two-pass form took 51.3
+// (1536 x 1024, 3 lines; one line 22.7 and 38.0).
 #include "epr_internal.cuh"
 
 namespace {
@@ -68,12 +68,26 @@ __device__ __noinline__ void vjp_corners(const float* G, int y, int x, float uy,
     }
 }
 
+// A sum of floats with its rounding error beside it (Knuth's two-sum).  The terms
+// of the scalars nearly cancel: with the lanes' sums added in plain float, dF/dbeta
+// was off by 12 % more than in the two-pass form, whose threads each added
+// fewer terms; without those roundings by 5 % less.  39.1 -> 41.1 us.
+struct Pair {
+    float s, c;
+    __device__ __forceinline__ void add(float s2, float c2)
+    {
+        const float t = s + s2, b = t - s;
+        c += c2 + ((s - (t - b)) + (s2 - b));
+        s = t;
+    }
+};
+
 // NSM: the line count up to 4 (the corner loads of every line are then issued
 // together), a bound of it above (the sums stay in registers)
 template <int NSM>
 __global__ void __launch_bounds__(kVjpThreads, NSM <= 8 ? 4 : 2) k_vjp(const __grid_constant__ EprConsts C, const VjpArgs A)
 {
-    __shared__ float red[2 * NSM][kVjpThreads / 32];
+    __shared__ double red[2 * NSM][kVjpThreads / 32];
     const int nx = C.nx, ny = C.ny, ns = C.ns, b = blockIdx.y;
     const size_t npix = (size_t)nx * ny, pb = (size_t)b * npix;
     const float* Tb = A.T + pb;
@@ -179,20 +193,20 @@ __global__ void __launch_bounds__(kVjpThreads, NSM <= 8 ? 4 : 2) k_vjp(const __g
     // deterministic block partials: warp shuffles, then warps in order
 #pragma unroll
     for (int s = 0; s < NSM; ++s) {
-        float c = cacc[s], m = macc[s];
+        Pair c = {cacc[s], 0.f}, m = {macc[s], 0.f};
         for (int o = 16; o > 0; o >>= 1) {
-            c += __shfl_down_sync(0xffffffffu, c, o);
-            m += __shfl_down_sync(0xffffffffu, m, o);
+            c.add(__shfl_down_sync(0xffffffffu, c.s, o), __shfl_down_sync(0xffffffffu, c.c, o));
+            m.add(__shfl_down_sync(0xffffffffu, m.s, o), __shfl_down_sync(0xffffffffu, m.c, o));
         }
         if (lane == 0) {
-            red[2 * s][wid] = c;
-            red[2 * s + 1][wid] = m;
+            red[2 * s][wid] = (double)c.s + (double)c.c;
+            red[2 * s + 1][wid] = (double)m.s + (double)m.c;
         }
     }
     __syncthreads();
     if (threadIdx.x < 2 * ns) {
         double acc = 0.0;
-        for (int i = 0; i < kVjpThreads / 32; ++i) acc += (double)red[threadIdx.x][i];
+        for (int i = 0; i < kVjpThreads / 32; ++i) acc += red[threadIdx.x][i];
         A.part[((size_t)b * kVjpMaxBlocks + blockIdx.x) * 2 * ns + threadIdx.x] = acc;
     }
 }

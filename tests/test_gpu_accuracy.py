@@ -65,3 +65,22 @@ def test_gradient_of_large_alternating_misfits(torch, E):
     T = T.astype(np.float64)
     ref = -2.0 * k * 0.5 * (T * np.exp(-2.0 * k * beta * T)).sum()   # T = 0 in the column with a corner outside
     assert abs(np.ravel(got)[0] / ref - 1.0) <= 5e-6
+
+
+# No shift (L = 0), unit intensity, a thickness ramp of 2^-12 per column and a
+# misfit gradient in every eighth row: dF/dL = -delta / p^2 times the sum of 2^-12
+# (g(x + 1) - g(x)), with nothing beyond the last column, which telescopes to
+# -2^-12 g(0) per row.  Every term is a multiple of 2^-12 that a float holds (up to
+# 2^23 of them); the sums of a warp's lanes are not.
+def test_gradient_scalars_that_cancel(torch, E):
+    nx, ny = 96, 48
+    delta, pixel, beta = 2.0 ** -21, 2.0 ** -16, 1e-19   # exp(-mu T) is 1
+    g = np.zeros((ny, nx), np.float32)
+    g[::8] = ph.rng(3).integers(-2 ** 22, 2 ** 22, size=(ny // 8, nx))
+    g[::8, 0] = 1.0
+    T = np.tile((np.arange(nx) * 2.0 ** -12).astype(np.float32), (ny, 1))
+    with E.Plan(nx, ny, pixel, 0.0, [80.0], [delta], [beta]) as p:
+        Td, gd = torch.from_numpy(T).cuda(), torch.from_numpy(g).cuda()
+        _, _, got = E.epr_vjp(p.handle, Td, gd, torch.empty_like(Td), 1)
+    ref = -delta / pixel ** 2 * (ny // 8) * (-2.0 ** -12)
+    assert abs(np.ravel(got)[0] / ref - 1.0) <= 1e-12
