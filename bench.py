@@ -386,7 +386,7 @@ def xspec_solve(epr, ph, torch, timeit):
     return {"workload": "ellipsoids_poly_2048, 1 projection, 8 lines, 50 iterations, 5-knot "
                         "x-dependent table", "ms_per_solve": round(ms_x, 3),
             "ms_per_solve_uniform_spectrum": round(ms_u, 3),
-            "note": "the x-dependent path runs the runtime-sized kernels with per-column constants"}
+            "note": "the x-dependent path runs the kernels with per-column constants"}
 
 
 # --------------------------------------------------------------------------

@@ -14,10 +14,11 @@
 // differentiated along y, and horizontal neighbours come by warp shuffle, so
 // there is no shared memory and no barrier.  The nested derivatives reach 3
 // pixels (2 for m = 1): 26 (28) of the 32 lanes are output columns, and a
-// strip of H rows computes H + 6.  The fields are bound by instruction issue:
-// the tile form this replaces staged every field in shared memory and spent
-// 440 (second-order term) and 620 (m = 2) thread instructions per pixel, most
-// of them on its index arithmetic, its barriers' phases and expm1.
+// strip of H rows computes H + 6.  221 (second-order term) and 304 (m = 2)
+// thread instructions per pixel; the tile form this replaces staged every field
+// in shared memory and spent 440 and 620, most of them on its index arithmetic,
+// its barriers' phases and expm1.  47 and 58 % of the issue slots are used: what
+// is left is the wait for the rows of T and P at 28 warps per SM.
 // Stencils test the GLOBAL coordinate for the edge rules, so values computed
 // outside the grid are never used by an in-grid output.  No atomics: the
 // result is the same on every run.

@@ -132,7 +132,7 @@ __device__ __forceinline__ float rcp_approx(float x)
 
 // log_ratio of two pixels of one column (packed): both above the floor with
 // |q| < 1/4 by the series of log1p_atanh, else one by one.  The update is
-// bound by instruction issue (78 % active); the packed form takes
+// bound by instruction issue (70 % active in a batch); the packed form takes
 // 21 arithmetic instructions for two pixels.
 __device__ __forceinline__ float2 log_ratio2(float2 t, float2 h, float om_f, float mus, float eps)
 {
@@ -317,7 +317,7 @@ k_row_fwd_ct(const EprConsts C, const RowArgs A)
     __syncthreads();
     float2 vk[EPT];   // the packed row pair values, stored once the thickness is dead
     // The gather of a row pair's two pixels (y0, x) and (y0 + 1, x), packed:
-    // 126 -> 92 thread instructions per pixel of this kernel, 148 -> 133 us for
+    // 126 -> 95 thread instructions per pixel of this kernel, 148 -> 135 us for
     // eight 2048^2 projections (with the loads ahead of the gather above).
     // Pixels whose four corners all lie on the grid load them unconditionally
     // on the spot; the others (the rim of the field) are flagged and redone
